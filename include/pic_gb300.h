@@ -60,7 +60,9 @@ extern "C" {
                         as an exact integer cell plus an FP32 in-cell offset      */
 
 /* schedules of the push (how uneven sub-cycle counts are spread over warps) */
-#define PIC_SCHED_PLAIN 0   /* one thread per particle, no binning               */
+#define PIC_SCHED_PLAIN 0   /* mixed form: one thread per particle, no binning;
+                               FP64 form: its sub-cycled particles are pushed in
+                               warps of equal k (the same bits)                   */
 #define PIC_SCHED_BINNED 1  /* m = 1 particles streamed; k > 0 particles compacted
                                by warp ballot into per-k queues and drained by
                                warps of equal k                                   */

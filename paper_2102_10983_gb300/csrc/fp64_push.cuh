@@ -1,0 +1,179 @@
+// Per-electron FP64 pieces shared by the FP64 kernels (push_f64.cu,
+// pic_sc1d.cu, study.cu): every result has the bits of the plain FP64
+// expression it replaces, but the FP64 unit (one per SM, 19 clocks per warp
+// instruction) only sees the multiplications and additions of the method.
+// Division and square root run on the integer pipes (fp64_int.cuh); so do the
+// floors, offsets, window tests and powers of two below, each of which would
+// take one to three of the unit's slots.
+#pragma once
+
+#include <math.h>
+
+#include "fp64_int.cuh"
+#include "pic_internal.h"
+
+namespace pic {
+
+// dt / 4^k: the exponent field lowered by 2k (ldexp's bits) while it stays
+// normal.
+__device__ __forceinline__ double pow4_down64(double dt, int k) {
+  const long long u = __double_as_longlong(dt);
+  if (((u >> 52) & 0x7ff) > 2 * k) return __longlong_as_double(u - ((long long)k << 53));
+  return ldexp(dt, -2 * k);
+}
+
+// G / 2^52 for 0 <= G < 2^52, exact.
+__device__ __forceinline__ double fix52(uint64_t G) {
+  const int lz = __clzll((long long)G);
+  const uint64_t bits = (G << (lz - 11)) + ((uint64_t)(uint32_t)(1033 - lz) << 52);
+  return G ? __longlong_as_double((long long)bits) : 0.0;
+}
+
+// A position in node units on both grids (E nodes at i, B nodes at i + 1/2):
+// the tent's lower nodes and the offsets from them.
+struct Coords64 {
+  int64_t je, jb;
+  double we, wb;
+};
+
+// floor(s), s - floor(s) and the same of s - 1/2.  For 1 <= s < 2^21 all four
+// are exact and read off the significand: the fraction as a 52-bit fixed-point
+// number, half a node being its top bit.  False outside that range (the caller
+// takes coords64_any).
+__device__ __forceinline__ bool coords64_fast(double s, Coords64& c) {
+  const uint64_t u = (uint64_t)__double_as_longlong(s);
+  const uint32_t h = (uint32_t)(u >> 32);
+  const int sh = (int)(h >> 20) - 1023;
+  const uint64_t G = (u << (sh & 31)) & 0xfffffffffffffull;
+  const int32_t j = (int32_t)(((h & 0xfffffu) | 0x100000u) >> ((20 - sh) & 31));
+  c.je = j;
+  c.we = fix52(G);
+  c.jb = j - ((G >> 51) ? 0 : 1);
+  c.wb = fix52(G ^ 0x8000000000000ull);
+  return h - 0x3ff00000u < 0x01500000u;
+}
+__device__ __forceinline__ void coords64_any(double s, Coords64& c) {
+  const double fe = floor(s), sb = s - 0.5, fb = floor(sb);
+  c.je = (int64_t)fe;
+  c.we = s - fe;
+  c.jb = (int64_t)fb;
+  c.wb = sb - fb;
+}
+
+// The criterion of Sec. IV decided in FP32 where that is safe.  c = |q/m| dt /
+// (2 Psi_max) (a normal FP32 number in [2^-60, 2^60], Psi_max not tiny; else
+// the host passes 0 and every electron takes the exact test): r = c |B| /
+// gamma carries a relative error below 2^-20, so away from the powers of four
+// by 2^-18 the comparisons of r are those of Psi / Psi_max.  Returns -1 where
+// it cannot tell (near a threshold, or anything not finite).
+__device__ __forceinline__ int criterion_f64_guess(float c, double b0, double px, double py, double pz,
+                                                   int k_max, bool& capped) {
+  const float b = fabsf((float)b0), x = (float)px, y = (float)py, z = (float)pz;
+  const float g2 = fmaf(x, x, fmaf(y, y, fmaf(z, z, 1.0f)));
+  float r = c * b * fp64i_rsqrt(g2);
+  if (!(g2 < 0x1p100f && r < 0x1p60f && c > 0.f)) return -1;
+  int k = 0;
+  while (r > 0x1.00004p0f && k < k_max) {
+    r *= 0.25f;
+    ++k;
+  }
+  capped = r > 1.0f;
+  // r <= 1 + 2^-18 here, or k = k_max; the last threshold not passed was 1,
+  // and a passed one left r > (1 + 2^-18) / 4
+  return fabsf(r - 1.0f) <= 0x1p-18f ? -1 : k;
+}
+
+// The exact test: Psi as the oracle forms it, k the smallest with
+// Psi / 4^k <= Psi_max.
+__device__ __forceinline__ int criterion_f64_exact(double qm_abs, double dt, double psi_max, int k_max,
+                                                   double b0, double px, double py, double pz,
+                                                   bool& capped) {
+  const double g0 = sqrt_rn(1.0 + (px * px + py * py + pz * pz));
+  double psi = div_rn(qm_abs * fabs(b0) * dt, 2.0 * g0);
+  int k = 0;
+  while (psi > psi_max && k < k_max) {
+    psi = psi * 0.25;
+    ++k;
+  }
+  capped = psi > psi_max;
+  return k;
+}
+
+__device__ __forceinline__ int criterion_f64(float c, double qm_abs, double dt, double psi_max,
+                                             int k_max, double b0, double px, double py, double pz,
+                                             bool& capped) {
+  int k = criterion_f64_guess(c, b0, px, py, pz, k_max, capped);
+  if (k < 0) k = criterion_f64_exact(qm_abs, dt, psi_max, k_max, b0, px, py, pz, capped);
+  return k;
+}
+
+// q/m times v: a sign for the electron (UNIT: |q/m| = 1).
+template <bool UNIT>
+__device__ __forceinline__ double times_qm(double qm, double v) {
+  if constexpr (UNIT)
+    return __longlong_as_double(__double_as_longlong(v) ^
+                                (__double_as_longlong(qm) & (long long)0x8000000000000000ull));
+  else
+    return qm * v;
+}
+
+// Momentum, with p_x^2 (which the next push of the sub-cycle needs again) and
+// p_z^2 (which no push changes: B is along z, E in the plane).
+struct Mom64 {
+  double x, y, z, x2, z2;
+};
+__device__ __forceinline__ Mom64 mom64(double x, double y, double z) {
+  return Mom64{x, y, z, x * x, z * z};
+}
+
+// Boris push in E = (0, ey, 0), B = (0, 0, bz) (Eqs. eq:p - eq:gamman) with
+// half = hp / 2, then x += h v_x (Eq. eq:x); gam: gamma after it.
+template <bool UNIT>
+static __device__ __noinline__ void push64_any(double ey, double bz, double half, double h, double qm,
+                                               Mom64* p, double* x, double* gam) {
+  const double dpy = times_qm<UNIT>(qm, ey) * half;
+  const double my = p->y + dpy;
+  const double gn = sqrt(1.0 + (p->x2 + my * my + p->z2));
+  const double tz = (times_qm<UNIT>(qm, bz) * half) / gn;
+  const double ppx = p->x + my * tz;
+  const double ppy = my - p->x * tz;
+  const double sz = (2.0 * tz) / (1.0 + tz * tz);
+  p->x = p->x + ppy * sz;
+  p->y = (my - ppx * sz) + dpy;
+  p->x2 = p->x * p->x;
+  *gam = sqrt(1.0 + (p->x2 + p->y * p->y + p->z2));
+  *x = *x + h * (p->x / *gam);
+}
+// The same bits with the integer roots and quotients, in one straight line (no
+// branch between the FP64 operations, so their latencies overlap what is
+// independent); operands outside those routines' domain are seen at the end
+// and the push is taken again by push64_any.
+template <bool UNIT>
+__device__ __forceinline__ void push64(double ey, double bz, double half, double h, double qm, Mom64& p,
+                                       double& x, double& gam) {
+  const double dpy = times_qm<UNIT>(qm, ey) * half;
+  const double my = p.y + dpy;
+  const double num = times_qm<UNIT>(qm, bz) * half;
+  double tz, sz, vx;
+  bool ok = div_sqrt_try(num, 1.0 + (p.x2 + my * my + p.z2), tz, nullptr);
+  const double ppx = p.x + my * tz;
+  const double ppy = my - p.x * tz;
+  ok &= div2_try(tz, 1.0 + tz * tz, sz);
+  Mom64 q;
+  q.x = p.x + ppy * sz;
+  q.y = (my - ppx * sz) + dpy;
+  q.z = p.z;
+  q.z2 = p.z2;
+  q.x2 = q.x * q.x;
+  double g;
+  ok &= div_sqrt_try(q.x, 1.0 + (q.x2 + q.y * q.y + q.z2), vx, &g);
+  if (ok) {
+    p = q;
+    x = x + h * vx;
+    gam = g;
+  } else {
+    push64_any<UNIT>(ey, bz, half, h, qm, &p, &x, &gam);
+  }
+}
+
+}  // namespace pic

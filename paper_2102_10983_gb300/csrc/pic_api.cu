@@ -50,6 +50,12 @@ struct pic_ctx {
   int64_t* dslot_i0 = nullptr;
   int32_t heavy_budget = 256;
   double* work = nullptr;  // FP64 form with PIC_DIAG_WORK: per-particle work of E
+  // FP64 form: node fields at t_n (4 W, optional), k > 0 electrons of a step
+  double* nodes64 = nullptr;
+  uint8_t* k_sub = nullptr;
+  int32_t* queue64 = nullptr;
+  int32_t* bin64 = nullptr;  // two sets of 32 counters, used in turn
+  int bin64_at = 0;
   int32_t* pred_queue = nullptr;
   const pic_mlp* mlp = nullptr;
   int32_t predict_every = 1;
@@ -103,7 +109,8 @@ static void free_all(pic_ctx* c) {
   void* ptrs[] = {c->x, c->px, c->py, c->pz, c->cell, c->frac, c->fpx, c->fpy, c->fpz,
                   c->status, c->ringE, c->ringB, c->staging, c->wtab64, c->wtab32,
                   c->dstats, c->queue, c->qcount, c->pred, c->pred_queue, c->half,
-                  c->coef, c->lag_step, c->lag_j, c->dslot_i0, c->work, c->feat};
+                  c->coef, c->lag_step, c->lag_j, c->dslot_i0, c->work, c->feat,
+                  c->nodes64, c->k_sub, c->queue64, c->bin64};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -269,6 +276,9 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     A((void**)&c->py, cap * 8);
     A((void**)&c->pz, cap * 8);
     if (prm->diagnostics == PIC_DIAG_WORK) A((void**)&c->work, cap * 8);
+    A((void**)&c->k_sub, cap);
+    A((void**)&c->queue64, cap * 4);
+    A((void**)&c->bin64, 64 * 4);
   }
   A((void**)&c->status, cap);
   // the mixed form's ring is mirrored (2R slots, see PushArgsMixed)
@@ -290,7 +300,14 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     return fail(nullptr, e == cudaErrorMemoryAllocation ? PIC_ENOMEM : PIC_ECUDA,
                 "pic_create: device allocation failed: %s", cudaGetErrorString(e));
   }
+  // the node fields save the FP64 push its gathers; without room for them it
+  // gathers the levels
+  if (!mixed && cudaMalloc((void**)&c->nodes64, (size_t)window_cells * 32) != cudaSuccess) {
+    c->nodes64 = nullptr;
+    cudaGetLastError();
+  }
   e = cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream);
+  if (e == cudaSuccess && c->bin64) e = cudaMemsetAsync(c->bin64, 0, 64 * 4, c->stream);
   if (e == cudaSuccess && c->qcount) e = cudaMemsetAsync(c->qcount, 0, 64 * 4, c->stream);
   if (e == cudaSuccess && c->pred) e = cudaMemsetAsync(c->pred, 0, cap, c->stream);
 
@@ -733,6 +750,7 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
   } else {
     memset(&base, 0, sizeof(base));
   }
+  const float crit64 = criterion_f64_scale(fabs(c->prm.qm), c->prm.dt, c->prm.psi_max);
   for (int64_t j = 0; j < n_steps; ++j) {
     const int64_t s = n + j;
     const int64_t J = J0 + j;  // the launch's index in the run
@@ -771,6 +789,16 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
       a.crit_row = wrows_total(c->prm.k_max) - 1;
       a.stats = c->dstats;
       a.work = c->work;
+      const int64_t i32 = ((int64_t)1 << 31) - 1;
+      a.lo_i = (int32_t)(lo < -i32 ? -i32 : lo > i32 ? i32 : lo);
+      a.hi_i = (int32_t)(hi < -i32 ? -i32 : hi > i32 ? i32 : hi);
+      a.crit_scale = crit64;
+      a.nodes = c->nodes64;
+      a.k_sub = c->k_sub;
+      a.queue = c->queue64;
+      a.bin = c->bin64 + 32 * c->bin64_at;
+      c->bin64_at ^= 1;
+      a.bin_next = c->bin64 + 32 * c->bin64_at;
       e = mark(ev0);
       if (e == cudaSuccess) e = launch_push_f64(a, p, c->stream, &launches);
     } else {

@@ -45,6 +45,13 @@ __host__ __device__ inline int64_t wrow(int k, int64_t j) {
 }
 inline int64_t wrows_total(int k_max) { return wrow(k_max + 1, 1) + 1; }  // + criterion row
 
+// The scale |q/m| dt / (2 Psi_max) of the FP64 kernels' FP32 criterion
+// (criterion_f64_guess), 0 where that test does not apply.
+inline float criterion_f64_scale(double qm_abs, double dt, double psi_max) {
+  const double c = qm_abs * dt / (2.0 * psi_max);
+  return (c >= 0x1p-60 && c <= 0x1p60 && psi_max >= 0x1p-500 && psi_max <= 0x1p500) ? (float)c : 0.0f;
+}
+
 // Arguments of the FP64 push (one macro step).
 struct PushArgsF64 {
   int64_t n;
@@ -56,6 +63,7 @@ struct PushArgsF64 {
   const double* E[kMaxOrder + 1];  // ring slot of level n-p+l, l = 0..p
   const double* B[kMaxOrder + 1];
   double lo, hi;  // s = x/dx must satisfy lo <= s < hi (and s - 1/2 too)
+  int32_t lo_i, hi_i;  // the same, clamped to 32 bits
   int64_t mask;   // W - 1
   double dt, inv_dx, psi_max, qm, qm_abs;
   int k_max;
@@ -63,6 +71,13 @@ struct PushArgsF64 {
   int64_t crit_row;
   DevStats* stats;
   double* work;  // nullptr, or per particle the accumulated work of E (App. B)
+  float crit_scale;   // criterion_f64_scale: 0 = the exact criterion only
+  double* nodes;      // nullptr, or 4 W: each node's fields at t_n (nodes_f64_kernel)
+  uint8_t* k_sub;     // per particle: k of the step where k > 0 (written every step)
+  int32_t* queue;     // particles with k > 0, grouped by k
+  int32_t* bin;       // [32] this step's counts and cursors, zero on entry
+  int32_t* bin_next;  // [32] the next step's: zeroed by this one
+  int sms;            // set by the launcher
 };
 
 // Arguments of the mixed-precision push.  Position = (cell + frac) * dx with

@@ -5,7 +5,7 @@
 // matches a serial FP64 evaluation of the same formulas bit for bit.  sqrt and
 // division are the IEEE correctly rounded double operations.
 //
-// One thread per particle, grid-stride.  Per macro step (Algorithm 1, Sec. IV):
+// Per particle and macro step (Algorithm 1, Sec. IV):
 //   criterion: Psi0 = |q/m| |B(x_n, t_n)| dt / (2 gamma), gamma of the stored
 //              momentum, B interpolated with the order-p weights at t_n;
 //              k = smallest k with Psi0/4^k <= Psi_max (capped at k_max);
@@ -14,6 +14,7 @@
 //   (Eqs. eq:Enp, eq:Bnp), Boris (Eqs. eq:p - eq:gamman), x += h v_x (Eq. eq:x).
 #include <math.h>
 
+#include "fp64_push.cuh"
 #include "pic_internal.h"
 
 namespace pic {
@@ -70,128 +71,380 @@ cudaError_t build_wtab_f64(double* wtab, int order, int k_max, int field_time, c
   return cudaGetLastError();
 }
 
-// Temporal sum at the two tent nodes (ascending level), then the tent weight.
+// ---------------------------------------------------------------- node sums at t_n
+
+// Per window node (position i & (W-1)): the temporal sums f_i of E_y and B_z at
+// theta = 1/2 and the steps f_{i+1} - f_i to the next node, as {E, dE, B, dB}.
+// The criterion's B_z and an m = 1 push's fields at a particle are then one
+// multiplication and one addition per grid, the bits of the full gather.
 template <int P>
-__device__ __forceinline__ double gather_f64(const double* const* lv, const double* w, double s,
-                                             int64_t mask) {
-  double fl = floor(s);
-  int64_t j = (int64_t)fl;
-  double frac = s - fl;
-  int64_t a0 = j & mask, a1 = (j + 1) & mask;
-  double f0 = w[0] * __ldg(lv[0] + a0);
-  double f1 = w[0] * __ldg(lv[0] + a1);
+__device__ __forceinline__ double tsum64(const double* const* lv, const double* w, int64_t c) {
+  double f = w[0] * __ldg(lv[0] + c);
 #pragma unroll
-  for (int l = 1; l <= P; ++l) {
-    f0 = f0 + w[l] * __ldg(lv[l] + a0);
-    f1 = f1 + w[l] * __ldg(lv[l] + a1);
-  }
-  return f0 + frac * (f1 - f0);
+  for (int l = 1; l <= P; ++l) f = f + w[l] * __ldg(lv[l] + c);
+  return f;
 }
 
 template <int P>
-__global__ void __launch_bounds__(256) push_f64_kernel(PushArgsF64 a) {
-  __shared__ unsigned long long sh[12];
-  if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
-  __syncthreads();
-  const int stride = 2 * (P + 1);
-  const double* wcrit = a.wtab + a.crit_row * stride + (P + 1);
-  const double* E[P + 1];
-  const double* B[P + 1];
+__global__ void __launch_bounds__(128) nodes_f64_kernel(PushArgsF64 a) {
+  const double* wE = a.wtab + wrow(0, 1) * (2 * (P + 1));
+  const double* wB = a.wtab + a.crit_row * (2 * (P + 1)) + (P + 1);
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c <= a.mask;
+       c += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t c1 = (c + 1) & a.mask;
+    const double e0 = tsum64<P>(a.E, wE, c), e1 = tsum64<P>(a.E, wE, c1);
+    const double b0 = tsum64<P>(a.B, wB, c), b1 = tsum64<P>(a.B, wB, c1);
+    reinterpret_cast<double2*>(a.nodes)[2 * c] = make_double2(e0, e1 - e0);
+    reinterpret_cast<double2*>(a.nodes)[2 * c + 1] = make_double2(b0, b1 - b0);
+  }
+}
+
+// ---------------------------------------------------------------- one sub-cycle
+
+// Node indices and offsets of s, and whether both grids' tents lie in the
+// window (lo <= s, s - 1/2 < hi; lo and hi are integers).
+__device__ __forceinline__ bool locate(const PushArgsF64& a, double s, Coords64& c) {
+  if (coords64_fast(s, c)) return c.jb >= a.lo_i && c.je < a.hi_i;  // jb <= je
+  const double sb = s - 0.5;
+  if (!(s >= a.lo && s < a.hi) || !(sb >= a.lo && sb < a.hi)) return false;
+  coords64_any(s, c);
+  return true;
+}
+
+// One grid's levels at the current node pair, and their temporal sums for the
+// next sub-step.
+template <int P>
+struct NodePair {
+  double v0[P + 1], v1[P + 1];
+  int32_t at = -1;  // masked index of the lower node
+  double f, d;      // f_i, f_{i+1} - f_i
+  __device__ __forceinline__ void load(const double* const* lv, int32_t node, int32_t mask) {
+    const int32_t next = (node + 1) & mask;
 #pragma unroll
-  for (int l = 0; l <= P; ++l) {
-    E[l] = a.E[l];
-    B[l] = a.B[l];
+    for (int l = 0; l <= P; ++l) {
+      v0[l] = __ldg(lv[l] + node);
+      v1[l] = __ldg(lv[l] + next);
+    }
+    at = node;
   }
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint8_t st = a.status[i];
-    if (st & PIC_STATUS_LOST) continue;
-    const int k_prev = st & 0x7f;
-    double pv0 = a.px[i], pv1 = a.py[i], pv2 = a.pz[i];
-    double xi = a.x[i];
+  __device__ __forceinline__ void sums(const double* w) {
+    double f0 = w[0] * v0[0], f1 = w[0] * v1[0];
+#pragma unroll
+    for (int l = 1; l <= P; ++l) {
+      f0 = f0 + w[l] * v0[l];
+      f1 = f1 + w[l] * v1[l];
+    }
+    f = f0;
+    d = f1 - f0;
+  }
+};
 
-    double s = xi * a.inv_dx;
-    double sb = s - 0.5;
-    if (!(s >= a.lo && s < a.hi) || !(sb >= a.lo && sb < a.hi)) {
-      a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
-      atomicAdd(&sh[11], 1ull);
-      continue;
-    }
-    double b0 = gather_f64<P>(B, wcrit, sb, a.mask);
-    double g0 = sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-    double psi = (a.qm_abs * fabs(b0) * a.dt) / (2.0 * g0);
-    int k = 0;
-    while (psi > a.psi_max && k < a.k_max) {
-      psi = psi * 0.25;
-      ++k;
-    }
-    const bool capped = psi > a.psi_max;
-    const int64_t m = (int64_t)1 << (2 * k);
-    const double h = ldexp(a.dt, -2 * k);
-    const double h_old = ldexp(a.dt, -2 * k_prev);
-    atomicAdd(&sh[k], 1ull);
-    atomicAdd(&sh[8], (unsigned long long)m);
-    if (k > 0) atomicAdd(&sh[9], (unsigned long long)m);
-    if (capped) atomicAdd(&sh[10], 1ull);
-
-    const double* wr = a.wtab + wrow(k, 1) * stride;
-    bool frozen = false;
-    double work = a.work ? a.work[i] : 0.0;
-    for (int64_t j = 1; j <= m; ++j, wr += stride) {
-      s = xi * a.inv_dx;
-      sb = s - 0.5;
-      if (!(s >= a.lo && s < a.hi) || !(sb >= a.lo && sb < a.hi)) {
-        frozen = true;
-        break;
-      }
-      const double ey = gather_f64<P>(E, wr, s, a.mask);
-      const double bz = gather_f64<P>(B, wr + (P + 1), sb, a.mask);
-      const double hp = (j == 1) ? 0.5 * (h_old + h) : h;
-      double vy_before = 0.0;
-      if (a.work) vy_before = pv1 / sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-      // Boris, E = (0, ey, 0), B = (0, 0, bz)
-      const double half = 0.5 * hp;
-      const double dpy = (a.qm * ey) * half;
-      const double mx = pv0, my = pv1 + dpy, mz = pv2;
-      const double gn = sqrt(1.0 + (mx * mx + my * my + mz * mz));
-      const double tz = ((a.qm * bz) * half) / gn;
-      const double ppx = mx + my * tz;
-      const double ppy = my - mx * tz;
-      const double sz = (2.0 * tz) / (1.0 + tz * tz);
-      const double qx = mx + ppy * sz;
-      const double qy = my - ppx * sz;
-      pv0 = qx;
-      pv1 = qy + dpy;
-      pv2 = mz;
-      const double g = sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-      // the work of E over this push (App. B): (q hp / 2) E . (v_before + v_after)
-      if (a.work) work = work + ((a.qm * hp) * 0.5) * (ey * (vy_before + pv1 / g));
-      xi = xi + h * (pv0 / g);
-    }
-    if (a.work) a.work[i] = work;
-    a.x[i] = xi;
-    a.px[i] = pv0;
-    a.py[i] = pv1;
-    a.pz[i] = pv2;
-    if (frozen) {
-      a.status[i] = (uint8_t)(k | PIC_STATUS_LOST);
-      atomicAdd(&sh[11], 1ull);
+// All 4^k sub-steps of one macro step of g electrons (g a power of two; entries
+// first .. of the queue, those from `end` on absent).  Lane l works on electron
+// l mod g, in 32 / g equal copies: every copy takes the electron's serial chain
+// (about 21 dependent FP64 operations of 64 clocks and five divisions and
+// roots per sub-step), which costs the FP64 unit nothing, its time being per
+// warp instruction.  What does not depend on where the electron goes while it
+// keeps its nodes -- the temporal sums at its nodes, 28 operations at order 3
+// -- the copies share: copy r forms those of the r-th sub-step to come, so a
+// warp pays for them once in 32 / g sub-steps, or when one of its electrons
+// changes node.
+template <int P, bool UNIT>
+__device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first, int64_t end, int g, int k,
+                                             unsigned long long* sh) {
+  constexpr int stride = 2 * (P + 1);
+  const int lane = threadIdx.x & 31, mine = lane & (g - 1), rows = 32 / g;
+  const int copy = lane / g;
+  const bool valid = first + mine < end;
+  const int64_t i = valid ? a.queue[first + mine] : 0;
+  const uint8_t st = valid ? a.status[i] : 0;
+  double xi = valid ? a.x[i] : 0.0;
+  Mom64 p = valid ? mom64(a.px[i], a.py[i], a.pz[i]) : Mom64{0.0, 0.0, 0.0, 0.0, 0.0};
+  const int m = 1 << (2 * k);
+  const int32_t mask = (int32_t)a.mask;
+  const double h = pow4_down64(a.dt, k), h_old = pow4_down64(a.dt, st & 0x7f);
+  double hp = 0.5 * (h_old + h);
+  double half = 0.5 * hp;
+  const double* w = a.wtab + wrow(k, 1) * stride;
+  const bool diag = a.work != nullptr;
+  double work = diag && valid ? a.work[i] : 0.0;
+  double vy = diag ? div_rn(p.y, sqrt_rn(1.0 + (p.x2 + p.y * p.y + p.z2))) : 0.0;
+  NodePair<P> E, B;
+  bool live = valid;
+  int have = 0, at = 0;  // the warp holds the sums of sub-steps at .. at + have - 1
+  double ef = 0.0, ed = 0.0, bf = 0.0, bd = 0.0;  // sub-step j's
+  auto take = [&](int r) {  // they are with copy r
+    if (rows > 1) {
+      const int src = mine + (r & (rows - 1)) * g;
+      ef = __shfl_sync(0xffffffffu, E.f, src);
+      ed = __shfl_sync(0xffffffffu, E.d, src);
+      bf = __shfl_sync(0xffffffffu, B.f, src);
+      bd = __shfl_sync(0xffffffffu, B.d, src);
     } else {
-      a.status[i] = (uint8_t)k;
+      ef = E.f;
+      ed = E.d;
+      bf = B.f;
+      bd = B.d;
+    }
+  };
+#pragma unroll 1
+  for (int j = 0; j < m; ++j) {
+    Coords64 c;
+    const bool in = live && locate(a, xi * a.inv_dx, c);
+    const int32_t ne = in ? (int32_t)(c.je & a.mask) : E.at, nb = in ? (int32_t)(c.jb & a.mask) : B.at;
+    live = in;
+    const bool moved = ne != E.at || nb != B.at;
+    if (__any_sync(0xffffffffu, moved || j >= at + have)) {
+      if (!__any_sync(0xffffffffu, live)) break;
+      if (moved) {
+        E.load(a.E, ne, mask);
+        B.load(a.B, nb, mask);
+      }
+      at = j;
+      have = rows;
+      const double* wr = w + (int64_t)(j + copy < m ? j + copy : m - 1) * stride;
+      E.sums(wr);
+      B.sums(wr + (P + 1));
+      take(0);
+    }
+    const double ey = ef + c.we * ed, bz = bf + c.wb * bd;
+    take(j + 1 - at);  // the next sub-step's, unless the electron changes node
+    if (live) {
+      double gam;
+      push64<UNIT>(ey, bz, half, h, a.qm, p, xi, gam);
+      if (diag) {  // (q hp / 2) E . (v_before + v_after) (App. B)
+        const double v = div_rn(p.y, gam);
+        work = work + ((a.qm * hp) * 0.5) * (ey * (vy + v));
+        vy = v;
+        hp = h;
+      }
+      half = 0.5 * h;
     }
   }
+  if (valid && copy == 0) {
+    if (diag) a.work[i] = work;
+    a.x[i] = xi;
+    a.px[i] = p.x;
+    a.py[i] = p.y;
+    a.status[i] = (uint8_t)(live ? k : k | PIC_STATUS_LOST);
+    if (!live) atomicAdd(&sh[11], 1ull);
+  }
+}
+
+// Block counters -> context counters: sh[0..7] the k histogram, sh[10] caps,
+// sh[11] lost.  Sub-step sums follow from the histogram (m = 4^k).
+__device__ __forceinline__ void flush_f64(unsigned long long* sh, DevStats* st) {
   __syncthreads();
   if (threadIdx.x < 12) {
     unsigned long long v = sh[threadIdx.x];
+    if (threadIdx.x == 8 || threadIdx.x == 9) {
+      v = 0;
+      for (int k = threadIdx.x == 8 ? 0 : 1; k < 8; ++k) v += sh[k] << (2 * k);
+    }
     if (v) {
-      unsigned long long* dst = threadIdx.x < 8 ? &a.stats->k_hist[threadIdx.x]
-                                : threadIdx.x == 8 ? &a.stats->substeps
-                                : threadIdx.x == 9 ? &a.stats->n_star
-                                : threadIdx.x == 10 ? &a.stats->clamped
-                                                    : &a.stats->lost;
+      unsigned long long* dst = threadIdx.x < 8 ? &st->k_hist[threadIdx.x]
+                                : threadIdx.x == 8 ? &st->substeps
+                                : threadIdx.x == 9 ? &st->n_star
+                                : threadIdx.x == 10 ? &st->clamped
+                                                    : &st->lost;
       atomicAdd(dst, v);
     }
   }
+}
+
+// ---------------------------------------------------------------- the three passes of a step
+//
+// A warp runs as long as its largest 4^k, and the FP64 unit takes an
+// instruction's 19 clocks however few lanes are active (one thread per
+// particle left 4.75 of 32 active on the a0 = 150 ensemble).  So:
+//  1. criterion_push_f64_kernel, one thread per particle in order: the
+//     criterion; m = 1 electrons are pushed at once, the others' k is noted;
+//  2. bin_f64_kernel: the noted electrons, grouped by k, largest first;
+//  3. subcycle_f64_kernel: warps take up to 32 of one k at a time, longest first.
+// Measured per step (order 3): 1,048,576 electrons of the a0 = 150 ensemble 6.2
+// ms as one thread per particle, 1.9 ms so (pass 1 0.09 ms = 25 FP64 slots per
+// warp, pass 2 6 us, the rest the longest chain: 1,024 sub-steps of 1.7 us,
+// 2.6 us before); 256 electrons at the a0 = 100 front 2.98 -> 1.2 ms, the chain
+// likewise.
+
+template <int P, bool UNIT>
+__global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) {
+  __shared__ unsigned long long sh[12];
+  if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
+  if (blockIdx.x == 0 && threadIdx.x < 32) a.bin_next[threadIdx.x] = 0;  // the next step's counts
+  __syncthreads();
+  unsigned k0 = 0, k1 = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint8_t st = a.status[i];
+    int k_sub = 0;
+    if (!(st & PIC_STATUS_LOST)) {
+      const double x = a.x[i];
+      Mom64 p = mom64(a.px[i], a.py[i], a.pz[i]);
+      Coords64 c;
+      if (!locate(a, x * a.inv_dx, c)) {
+        a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
+        atomicAdd(&sh[11], 1ull);
+      } else {
+        double ey, bz;
+        if (a.nodes) {
+          const double2 e = __ldg(reinterpret_cast<const double2*>(a.nodes) + 2 * (c.je & a.mask));
+          const double2 b = __ldg(reinterpret_cast<const double2*>(a.nodes) + 2 * (c.jb & a.mask) + 1);
+          ey = e.x + c.we * e.y;
+          bz = b.x + c.wb * b.y;
+        } else {
+          const double* wE = a.wtab + wrow(0, 1) * (2 * (P + 1));
+          const double* wB = a.wtab + a.crit_row * (2 * (P + 1)) + (P + 1);
+          const int64_t e0 = c.je & a.mask, b0 = c.jb & a.mask;
+          const double fe = tsum64<P>(a.E, wE, e0), fb = tsum64<P>(a.B, wB, b0);
+          ey = fe + c.we * (tsum64<P>(a.E, wE, (e0 + 1) & a.mask) - fe);
+          bz = fb + c.wb * (tsum64<P>(a.B, wB, (b0 + 1) & a.mask) - fb);
+        }
+        bool capped;
+        const int k = criterion_f64(a.crit_scale, a.qm_abs, a.dt, a.psi_max, a.k_max, bz, p.x, p.y, p.z,
+                                    capped);
+        if (capped) atomicAdd(&sh[10], 1ull);
+        if (k > 0) {
+          k_sub = k;
+          if (k == 1)
+            ++k1;
+          else
+            atomicAdd(&sh[k], 1ull);
+        } else {
+          ++k0;
+          const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
+          double vy = 0.0;
+          if (a.work) vy = div_rn(p.y, sqrt_rn(1.0 + (p.x2 + p.y * p.y + p.z2)));
+          double xn = x, g;
+          push64<UNIT>(ey, bz, 0.5 * hp, a.dt, a.qm, p, xn, g);
+          a.x[i] = xn;
+          if (a.work) a.work[i] = a.work[i] + ((a.qm * hp) * 0.5) * (ey * (vy + div_rn(p.y, g)));
+          a.px[i] = p.x;
+          a.py[i] = p.y;
+          a.status[i] = 0;
+        }
+      }
+    }
+    a.k_sub[i] = (uint8_t)k_sub;
+  }
+  const unsigned k0w = __reduce_add_sync(0xffffffffu, k0), k1w = __reduce_add_sync(0xffffffffu, k1);
+  if ((threadIdx.x & 31) == 0 && k0w) atomicAdd(&sh[0], (unsigned long long)k0w);
+  if ((threadIdx.x & 31) == 0 && k1w) atomicAdd(&sh[1], (unsigned long long)k1w);
+  flush_f64(sh, a.stats);
+  if (threadIdx.x > 0 && threadIdx.x < 8 && sh[threadIdx.x])
+    atomicAdd(&a.bin[threadIdx.x], (int32_t)sh[threadIdx.x]);
+}
+
+// bin[1..7]: the step's counts per k; bin[8 + k]: entries of k placed so far;
+// bin[16]: the sub-cycle kernel's item cursor.  Queue order: k = 7 first.
+__global__ void __launch_bounds__(256) bin_f64_kernel(PushArgsF64 a) {
+  __shared__ int cnt[8], base[8];
+  const int64_t n16 = (a.n + 15) / 16;
+  int64_t start[8];
+  start[7] = 0;
+#pragma unroll
+  for (int k = 6; k >= 1; --k) start[k] = start[k + 1] + a.bin[k + 1];
+  if (start[1] + a.bin[1] == 0) return;
+  for (int64_t v0 = (int64_t)blockIdx.x * blockDim.x; v0 < n16; v0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i0 = 16 * (v0 + threadIdx.x);
+    uint32_t w[4] = {0, 0, 0, 0};
+    if (i0 + 16 <= a.n) {
+      const uint4 q = *reinterpret_cast<const uint4*>(a.k_sub + i0);
+      w[0] = q.x; w[1] = q.y; w[2] = q.z; w[3] = q.w;
+    } else {
+      for (int q = 0; q < 16 && i0 + q < a.n; ++q) w[q >> 2] |= (uint32_t)a.k_sub[i0 + q] << (8 * (q & 3));
+    }
+    if (!__syncthreads_or((w[0] | w[1] | w[2] | w[3]) != 0)) continue;
+    if (threadIdx.x < 8) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    int off[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int k = (w[q >> 2] >> (8 * (q & 3))) & 7;
+      off[q] = k ? atomicAdd(&cnt[k], 1) : 0;
+    }
+    __syncthreads();
+    if (threadIdx.x > 0 && threadIdx.x < 8 && cnt[threadIdx.x])
+      base[threadIdx.x] = atomicAdd(&a.bin[8 + threadIdx.x], cnt[threadIdx.x]);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int k = (w[q >> 2] >> (8 * (q & 3))) & 7;
+      if (k) {
+        int64_t s = 0;
+#pragma unroll
+        for (int r = 1; r < 8; ++r)
+          if (r == k) s = start[r];
+        a.queue[s + base[k] + off[q]] = (int32_t)(i0 + q);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Electrons per warp for a k with `count` of them: few enough that every SM
+// gets a warp of them before any warp holds a second electron (a sub-cycle is
+// a latency-bound chain, so fewer electrons per warp cost nothing while units
+// are idle and save the temporal sums), at most 32.
+__device__ __forceinline__ int group_f64(int count, int sms) {
+  int g = 1;
+  while (g < 32 && count > g * sms) g *= 2;
+  return g;
+}
+
+// One warp per block: the few long chains of a step spread over the SMs.
+template <int P, bool UNIT>
+__global__ void __launch_bounds__(32) subcycle_f64_kernel(PushArgsF64 a) {
+  __shared__ unsigned long long sh[12];
+  if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
+  __syncwarp();
+  // cumulative work items and entries, k = 7 first
+  int64_t t = blockIdx.x;
+  for (;;) {
+    int64_t items = 0, entries = 0, first = -1, end = 0;
+    int k = 0, g = 1;
+#pragma unroll
+    for (int q = 7; q >= 1; --q) {
+      const int c = a.bin[q];
+      const int gq = group_f64(c, a.sms);
+      const int64_t n = (c + gq - 1) / gq;
+      if (first < 0 && t < items + n) {
+        k = q;
+        g = gq;
+        first = entries + (t - items) * gq;
+        end = entries + c;
+      }
+      items += n;
+      entries += c;
+    }
+    if (first < 0) break;
+    subcycle_f64<P, UNIT>(a, first, end, g, k, sh);
+    int next = 0;
+    if (threadIdx.x == 0) next = atomicAdd(&a.bin[16], 1);
+    t = (int64_t)gridDim.x + __shfl_sync(0xffffffffu, next, 0);
+  }
+  __syncwarp();
+  if (threadIdx.x == 0 && sh[11]) atomicAdd(&a.stats->lost, sh[11]);
+}
+
+template <int P, bool UNIT>
+static void launch_f64_p(PushArgsF64 a, int sms, cudaStream_t s, int* launches) {
+  a.sms = sms;
+  int n = 3;
+  if (a.nodes) {
+    const int64_t want = (a.mask + 128) / 128;
+    nodes_f64_kernel<P><<<(int)(want < sms * 8 ? want : sms * 8), 128, 0, s>>>(a);
+    ++n;
+  }
+  // small ensembles in small blocks: every SM's FP64 unit takes part
+  const int threads = a.n >= (int64_t)sms * 256 ? 256 : a.n >= (int64_t)sms * 64 ? 64 : 32;
+  const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)sms * 8;
+  criterion_push_f64_kernel<P, UNIT><<<(int)(want < cap ? want : cap), threads, 0, s>>>(a);
+  const int64_t vecs = (a.n + 4095) / 4096;
+  bin_f64_kernel<<<(int)(vecs < sms * 8 ? vecs : sms * 8), 256, 0, s>>>(a);
+  const int64_t most = (int64_t)sms * 12;
+  subcycle_f64_kernel<P, UNIT><<<(int)(a.n < most ? a.n : most), 32, 0, s>>>(a);
+  if (launches) *launches += n;
 }
 
 cudaError_t launch_push_f64(const PushArgsF64& a, int order, cudaStream_t s, int* launches) {
@@ -199,18 +452,15 @@ cudaError_t launch_push_f64(const PushArgsF64& a, int order, cudaStream_t s, int
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int64_t want = (a.n + 255) / 256;
-  int64_t cap = (int64_t)sms * 8;
-  int blocks = (int)(want < cap ? want : cap);
+  const bool unit = a.qm_abs == 1.0;
   switch (order) {
-    case 1: push_f64_kernel<1><<<blocks, 256, 0, s>>>(a); break;
-    case 2: push_f64_kernel<2><<<blocks, 256, 0, s>>>(a); break;
-    case 3: push_f64_kernel<3><<<blocks, 256, 0, s>>>(a); break;
-    case 4: push_f64_kernel<4><<<blocks, 256, 0, s>>>(a); break;
-    case 5: push_f64_kernel<5><<<blocks, 256, 0, s>>>(a); break;
+    case 1: unit ? launch_f64_p<1, true>(a, sms, s, launches) : launch_f64_p<1, false>(a, sms, s, launches); break;
+    case 2: unit ? launch_f64_p<2, true>(a, sms, s, launches) : launch_f64_p<2, false>(a, sms, s, launches); break;
+    case 3: unit ? launch_f64_p<3, true>(a, sms, s, launches) : launch_f64_p<3, false>(a, sms, s, launches); break;
+    case 4: unit ? launch_f64_p<4, true>(a, sms, s, launches) : launch_f64_p<4, false>(a, sms, s, launches); break;
+    case 5: unit ? launch_f64_p<5, true>(a, sms, s, launches) : launch_f64_p<5, false>(a, sms, s, launches); break;
     default: return cudaErrorInvalidValue;
   }
-  if (launches) ++*launches;
   return cudaGetLastError();
 }
 
