@@ -156,8 +156,8 @@ __device__ __forceinline__ double sqrt_rn(double a) {
 
 // The same without branches, for a caller that strings several together and
 // looks at the result's validity once (false: an operand or a result outside
-// the domain, the value is to be ignored): 2 a / b; and t / sqrt(a), which
-// starts from the root's own reciprocal, the root in *g if g is given.
+// the domain, the values are to be ignored): 2 a / b; and g = sqrt(a) with
+// t / g (TWO: and u / g), which start from the root's own reciprocal.
 __device__ __forceinline__ bool div2_try(double a, double b, double& q) {
   const uint64_t ub = (uint64_t)__double_as_longlong(b);
   const uint32_t hb = (uint32_t)(ub >> 32);
@@ -166,13 +166,15 @@ __device__ __forceinline__ bool div2_try(double a, double b, double& q) {
                        hb, q) &
          ((unsigned)(eb - 1) < 2046u);
 }
-__device__ __forceinline__ bool div_sqrt_try(double t, double a, double& q, double* g) {
+template <bool TWO>
+__device__ __forceinline__ bool div_sqrt_try(double t, double u, double a, double& qt, double& qu, double& g) {
   uint64_t sig;
   int field;
   float y;
-  const bool ok = fp64i_sqrt(a, sig, field, y);
-  if (g) *g = fp64i_pack(sig, field);
-  return ok & fp64i_quot<0>((uint64_t)__double_as_longlong(t), sig, field, y, 0u, q);
+  bool ok = fp64i_sqrt(a, sig, field, y);
+  g = fp64i_pack(sig, field);
+  if constexpr (TWO) ok &= fp64i_quot<0>((uint64_t)__double_as_longlong(u), sig, field, y, 0u, qu);
+  return ok & fp64i_quot<0>((uint64_t)__double_as_longlong(t), sig, field, y, 0u, qt);
 }
 
 }  // namespace pic

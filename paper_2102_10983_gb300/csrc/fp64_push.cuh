@@ -60,6 +60,47 @@ __device__ __forceinline__ void coords64_any(double s, Coords64& c) {
   c.wb = sb - fb;
 }
 
+// floor(s) and s - floor(s) on one grid, the same way.
+__device__ __forceinline__ void floor_frac64(double s, int64_t& j, double& w) {
+  const uint64_t u = (uint64_t)__double_as_longlong(s);
+  const uint32_t h = (uint32_t)(u >> 32);
+  const int sh = (int)(h >> 20) - 1023;
+  j = (int32_t)(((h & 0xfffffu) | 0x100000u) >> ((20 - sh) & 31));
+  w = fix52((u << (sh & 31)) & 0xfffffffffffffull);
+  if (h - 0x3ff00000u >= 0x01500000u) {
+    const double fl = floor(s);
+    j = (int64_t)fl;
+    w = s - fl;
+  }
+}
+
+// v 4^-k (ldexp's bits, which a multiplication by that power has too).
+__device__ __forceinline__ double scale_down64(double v, int k) {
+  return v == 0.0 ? v : pow4_down64(v, k);
+}
+__device__ __forceinline__ double half64(double v) {
+  const long long u = __double_as_longlong(v);
+  return ((u >> 52) & 0x7ff) > 1 ? __longlong_as_double(u - (1ll << 52)) : 0.5 * v;
+}
+
+// (double)q and __double2ll_rn(v) on the integer pipes.
+__device__ __forceinline__ double ll_to_double(int64_t q) {
+  if ((uint64_t)q >> 52) return (double)q;
+  const int lz = __clzll(q);
+  const uint64_t bits = ((uint64_t)q << (lz - 11)) + ((uint64_t)(uint32_t)(1085 - lz) << 52);
+  return q ? __longlong_as_double((long long)bits) : 0.0;
+}
+__device__ __forceinline__ int64_t double_to_ll(double v) {
+  const uint64_t u = (uint64_t)__double_as_longlong(v);
+  const int sh = 1075 - (int)((u >> 52) & 0x7ff);  // |v| = M 2^-sh
+  if (sh < 1) return __double2ll_rn(v);
+  const uint64_t M = fp64i_sig(u);
+  const int r = sh & 63;
+  // nearest, ties to even: half a unit less one, plus the quotient's last bit
+  const uint64_t q = sh > 53 ? 0ull : (M + (1ull << (r - 1)) - 1 + ((M >> r) & 1)) >> r;
+  return (int64_t)u < 0 ? -(int64_t)q : (int64_t)q;
+}
+
 // The criterion of Sec. IV decided in FP32 where that is safe.  c = |q/m| dt /
 // (2 Psi_max) (a normal FP32 number in [2^-60, 2^60], Psi_max not tiny; else
 // the host passes 0 and every electron takes the exact test): r = c |B| /
@@ -107,6 +148,89 @@ __device__ __forceinline__ int criterion_f64(float c, double qm_abs, double dt, 
   return k;
 }
 
+// One grid's levels at the current node pair, and their temporal sums for the
+// next sub-step.
+template <int P>
+struct NodePair {
+  double v0[P + 1], v1[P + 1];
+  int32_t at = -1;  // masked index of the lower node
+  double f, d;      // f_i, f_{i+1} - f_i
+  __device__ __forceinline__ void load(const double* const* lv, int32_t node, int32_t mask) {
+    const int32_t next = (node + 1) & mask;
+#pragma unroll
+    for (int l = 0; l <= P; ++l) {
+      v0[l] = __ldg(lv[l] + node);
+      v1[l] = __ldg(lv[l] + next);
+    }
+    at = node;
+  }
+  __device__ __forceinline__ void sums(const double* w) {
+    double f0 = w[0] * v0[0], f1 = w[0] * v1[0];
+#pragma unroll
+    for (int l = 1; l <= P; ++l) {
+      f0 = f0 + w[l] * v0[l];
+      f1 = f1 + w[l] * v1[l];
+    }
+    f = f0;
+    d = f1 - f0;
+  }
+};
+
+// Electrons per warp for a k with `count` of them: few enough that every SM
+// gets a warp of them before any warp holds a second electron (a sub-cycle is
+// a latency-bound chain, so fewer electrons per warp cost nothing while units
+// are idle and save the temporal sums), at most 32.
+__device__ __forceinline__ int group_f64(int count, int sms) {
+  int g = 1;
+  while (g < 32 && count > g * sms) g *= 2;
+  return g;
+}
+
+// Work item t of the binned electrons (bin[1..7]: their counts, k = 7 first in
+// the queue): entries first .. of the queue (those from `end` on absent), g of
+// them, all of one k.  False past the last item.
+__device__ __forceinline__ bool item_f64(const int32_t* bin, int sms, int64_t t, int64_t& first,
+                                         int64_t& end, int& k, int& g) {
+  int64_t items = 0, entries = 0;
+  first = -1;
+#pragma unroll
+  for (int q = 7; q >= 1; --q) {
+    const int c = bin[q];
+    const int gq = group_f64(c, sms);
+    const int64_t n = (c + gq - 1) / gq;
+    if (first < 0 && t < items + n) {
+      k = q;
+      g = gq;
+      first = entries + (t - items) * gq;
+      end = entries + c;
+    }
+    items += n;
+    entries += c;
+  }
+  return first >= 0;
+}
+
+// Block counters -> context counters: sh[0..7] the k histogram, sh[10] caps,
+// sh[11] lost.  Sub-step sums follow from the histogram (m = 4^k).
+__device__ __forceinline__ void flush_f64(unsigned long long* sh, DevStats* st) {
+  __syncthreads();
+  if (threadIdx.x < 12) {
+    unsigned long long v = sh[threadIdx.x];
+    if (threadIdx.x == 8 || threadIdx.x == 9) {
+      v = 0;
+      for (int k = threadIdx.x == 8 ? 0 : 1; k < 8; ++k) v += sh[k] << (2 * k);
+    }
+    if (v) {
+      unsigned long long* dst = threadIdx.x < 8 ? &st->k_hist[threadIdx.x]
+                                : threadIdx.x == 8 ? &st->substeps
+                                : threadIdx.x == 9 ? &st->n_star
+                                : threadIdx.x == 10 ? &st->clamped
+                                                    : &st->lost;
+      atomicAdd(dst, v);
+    }
+  }
+}
+
 // q/m times v: a sign for the electron (UNIT: |q/m| = 1).
 template <bool UNIT>
 __device__ __forceinline__ double times_qm(double qm, double v) {
@@ -126,54 +250,59 @@ __device__ __forceinline__ Mom64 mom64(double x, double y, double z) {
   return Mom64{x, y, z, x * x, z * z};
 }
 
-// Boris push in E = (0, ey, 0), B = (0, 0, bz) (Eqs. eq:p - eq:gamman) with
-// half = hp / 2, then x += h v_x (Eq. eq:x); gam: gamma after it.
-template <bool UNIT>
-static __device__ __noinline__ void push64_any(double ey, double bz, double half, double h, double qm,
-                                               Mom64* p, double* x, double* gam) {
+// Boris push in E = (ex, ey, 0), B = (0, 0, bz) (Eqs. eq:p - eq:gamman) with
+// half = hp / 2, and the velocity after it.  EX: with E_x (and v_y wanted).
+struct Push64 {
+  double vx, vy, gam;
+};
+template <bool UNIT, bool EX>
+static __device__ __noinline__ Push64 push64_any(double ex, double ey, double bz, double half, double qm,
+                                                 Mom64* p) {
+  const double dpx = EX ? times_qm<UNIT>(qm, ex) * half : 0.0;
   const double dpy = times_qm<UNIT>(qm, ey) * half;
-  const double my = p->y + dpy;
-  const double gn = sqrt(1.0 + (p->x2 + my * my + p->z2));
+  const double mx = EX ? p->x + dpx : p->x, my = p->y + dpy;
+  const double gn = sqrt(1.0 + (mx * mx + my * my + p->z2));
   const double tz = (times_qm<UNIT>(qm, bz) * half) / gn;
-  const double ppx = p->x + my * tz;
-  const double ppy = my - p->x * tz;
+  const double ppx = mx + my * tz;
+  const double ppy = my - mx * tz;
   const double sz = (2.0 * tz) / (1.0 + tz * tz);
-  p->x = p->x + ppy * sz;
+  p->x = EX ? (mx + ppy * sz) + dpx : mx + ppy * sz;
   p->y = (my - ppx * sz) + dpy;
   p->x2 = p->x * p->x;
-  *gam = sqrt(1.0 + (p->x2 + p->y * p->y + p->z2));
-  *x = *x + h * (p->x / *gam);
+  Push64 r;
+  r.gam = sqrt(1.0 + (p->x2 + p->y * p->y + p->z2));
+  r.vx = p->x / r.gam;
+  r.vy = EX ? p->y / r.gam : 0.0;
+  return r;
 }
 // The same bits with the integer roots and quotients, in one straight line (no
 // branch between the FP64 operations, so their latencies overlap what is
 // independent); operands outside those routines' domain are seen at the end
 // and the push is taken again by push64_any.
-template <bool UNIT>
-__device__ __forceinline__ void push64(double ey, double bz, double half, double h, double qm, Mom64& p,
-                                       double& x, double& gam) {
+template <bool UNIT, bool EX>
+__device__ __forceinline__ Push64 push64(double ex, double ey, double bz, double half, double qm, Mom64& p) {
+  const double dpx = EX ? times_qm<UNIT>(qm, ex) * half : 0.0;
   const double dpy = times_qm<UNIT>(qm, ey) * half;
+  const double mx = EX ? p.x + dpx : p.x, mx2 = EX ? mx * mx : p.x2;
   const double my = p.y + dpy;
   const double num = times_qm<UNIT>(qm, bz) * half;
-  double tz, sz, vx;
-  bool ok = div_sqrt_try(num, 1.0 + (p.x2 + my * my + p.z2), tz, nullptr);
-  const double ppx = p.x + my * tz;
-  const double ppy = my - p.x * tz;
+  double tz, sz, none;
+  bool ok = div_sqrt_try<false>(num, 0.0, 1.0 + (mx2 + my * my + p.z2), tz, none, none);
+  const double ppx = mx + my * tz;
+  const double ppy = my - mx * tz;
   ok &= div2_try(tz, 1.0 + tz * tz, sz);
   Mom64 q;
-  q.x = p.x + ppy * sz;
+  q.x = EX ? (mx + ppy * sz) + dpx : mx + ppy * sz;
   q.y = (my - ppx * sz) + dpy;
   q.z = p.z;
   q.z2 = p.z2;
   q.x2 = q.x * q.x;
-  double g;
-  ok &= div_sqrt_try(q.x, 1.0 + (q.x2 + q.y * q.y + q.z2), vx, &g);
-  if (ok) {
-    p = q;
-    x = x + h * vx;
-    gam = g;
-  } else {
-    push64_any<UNIT>(ey, bz, half, h, qm, &p, &x, &gam);
-  }
+  Push64 r;
+  r.vy = 0.0;
+  ok &= div_sqrt_try<EX>(q.x, q.y, 1.0 + (q.x2 + q.y * q.y + q.z2), r.vx, r.vy, r.gam);
+  if (!ok) return push64_any<UNIT, EX>(ex, ey, bz, half, qm, &p);
+  p = q;
+  return r;
 }
 
 }  // namespace pic

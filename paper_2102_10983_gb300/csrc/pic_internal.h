@@ -52,6 +52,15 @@ inline float criterion_f64_scale(double qm_abs, double dt, double psi_max) {
   return (c >= 0x1p-60 && c <= 0x1p60 && psi_max >= 0x1p-500 && psi_max <= 0x1p500) ? (float)c : 0.0f;
 }
 
+// The electrons of a step that sub-cycle: k_sub[i] = their k (else 0), bin[1..7]
+// the counts per k, bin[8..15] places taken so far, bin[16] the item cursor.
+struct BinF64 {
+  int64_t n;
+  const uint8_t* k_sub;
+  int32_t* queue;
+  int32_t* bin;
+};
+
 // Arguments of the FP64 push (one macro step).
 struct PushArgsF64 {
   int64_t n;
@@ -234,6 +243,8 @@ cudaError_t launch_from_mixed(const int32_t* cell, const float* frac, const floa
 // Launchers (return cudaError_t of the launch).
 cudaError_t build_wtab_f64(double* wtab, int order, int k_max, int field_time, cudaStream_t s);
 cudaError_t build_wtab_f32(float* wtab, const double* wtab64, int64_t count, cudaStream_t s);
+// Groups the particles whose k_sub is set by k, k = 7 first (push_f64.cu).
+cudaError_t launch_bin_f64(const BinF64& a, int sms, cudaStream_t s);
 cudaError_t launch_push_f64(const PushArgsF64& a, int order, cudaStream_t s, int* launches);
 cudaError_t launch_push_mixed(const PushArgsMixed& a, int order, int schedule, int sm_count,
                               cudaStream_t s, int* launches);

@@ -8,16 +8,22 @@
 // which threads add their contributions does not change a bit either.
 //
 // Per macro step n (state: x at t_n, p at t_n - h_old/2):
-//   push_deposit_kernel<P>: one thread per electron.  Criterion of Sec. IV
-//     (|B_z| at x_n, t_n, gamma of the stored momentum; smallest k with
-//     Psi0/4^k <= Psi_max); m = 4^k sub-steps of h = dt/4^k, the first with
-//     (h_old + h)/2; each sub-step gathers E_x, E_y, B_z with the order-p
-//     weights of Sec. VI (tabulated per (k, j)) and the tent (Eqs. eq:Enp,
-//     eq:Bnp), takes the Boris push with E = (E_x, E_y, 0) (Eqs. eq:p -
-//     eq:gamman) and moves x by h v_x (Eq. eq:x).  It adds (h/dt) v_y S(x_mid)
-//     of every sub-step to per-node FP64 sums in registers, and at the end of
-//     the macro step one rounded fixed-point value per node to J_y, and the
-//     charge flux of its move (start -> end or frozen position) to J_x.
+//   push and deposit: criterion of Sec. IV (|B_z| at x_n, t_n, gamma of the
+//     stored momentum; smallest k with Psi0/4^k <= Psi_max); m = 4^k sub-steps
+//     of h = dt/4^k, the first with (h_old + h)/2; each sub-step gathers E_x,
+//     E_y, B_z with the order-p weights of Sec. VI (tabulated per (k, j)) and
+//     the tent (Eqs. eq:Enp, eq:Bnp), takes the Boris push with E = (E_x, E_y,
+//     0) (Eqs. eq:p - eq:gamman) and moves x by h v_x (Eq. eq:x).  It adds
+//     (h/dt) v_y S(x_mid) of every sub-step to per-node FP64 sums, and at the
+//     end of the macro step one rounded fixed-point value per node to J_y, and
+//     the charge flux of its move (start -> end or frozen position) to J_x.
+//     As in push_f64.cu: node fields at t_n once per step (nodes_kernel), the
+//     m = 1 electrons in order (push_deposit_kernel), the others in warps of
+//     equal k (subcycle_deposit_kernel), and roots, quotients, floors and
+//     conversions off the FP64 unit, which bounds the kernels (19 clocks per
+//     warp instruction).  1,760,600 electrons, 20,000 cells, a0 = 150: 1.58 ms
+//     per step as one kernel on that unit alone, 0.49 ms so (0.25 the m = 1
+//     pass at ~48 slots per warp, 0.24 the sub-cycles).
 //   field_kernel: E_y^{n+1} (Eq. eq:Ey with -dt J_y; Mur at both ends),
 //     E_x^{n+1} = E_x^n - dt J_x, B_z^{n+3/2} (Eq. eq:Bz); also clears the
 //     other parity's accumulators for the next step.
@@ -29,6 +35,7 @@
 
 #include <vector>
 
+#include "fp64_push.cuh"
 #include "pic_internal.h"
 #include "pic_sc1d.h"
 
@@ -54,36 +61,25 @@ struct Sc1dArgs {
   const double* wtab;
   int64_t crit_row;
   DevStats* stats;
+  float crit_scale;   // criterion_f64_scale
+  double2* nodes;     // [M][3]: {f, f_next - f} of E_x, E_y, B_z at t_n
+  uint8_t* k_sub;     // as in PushArgsF64
+  int32_t* queue;
+  int32_t* bin;
+  int32_t* bin_next;
+  int sms;
 };
-
-// Field of one grid at coordinate u (node units of that grid), weights w over
-// the P+1 levels in ascending time: temporal sums at the two tent nodes, then
-// the tent weight.
-template <int P>
-__device__ __forceinline__ double gather(const double* const* lv, const double* w, double u) {
-  const double fl = floor(u);
-  const int64_t j = (int64_t)fl + 2;
-  const double frac = u - fl;
-  double f0 = w[0] * lv[0][j];
-  double f1 = w[0] * lv[0][j + 1];
-#pragma unroll
-  for (int l = 1; l <= P; ++l) {
-    f0 = f0 + w[l] * lv[l][j];
-    f1 = f1 + w[l] * lv[l][j + 1];
-  }
-  return f0 + frac * (f1 - f0);
-}
 
 __device__ __forceinline__ bool inside(double s, int32_t n_cells) {
   return s >= 0.5 && s < (double)n_cells - 0.5;
 }
 
-// Node charges of Q at s: r0 at node floor(s), r1 at floor(s)+1, r0 + r1 = Q.
-__device__ __forceinline__ void split(int64_t Q, double s, int64_t& i, int64_t& r0, int64_t& r1) {
-  const double fl = floor(s);
-  i = (int64_t)fl;
-  r1 = __double2ll_rn((double)Q * (s - fl));
-  r0 = Q - r1;
+// Tent nodes and offsets of s on both grids; false outside the interior.
+__device__ __forceinline__ bool locate(const Sc1dArgs& a, double s, Coords64& c) {
+  if (coords64_fast(s, c)) return c.jb < a.n_cells - 1;  // s >= 1; s < N - 1/2
+  if (!inside(s, a.n_cells)) return false;
+  coords64_any(s, c);
+  return true;
 }
 
 // a[idx] += v; an index outside [0, M) (only a non-finite position could
@@ -92,138 +88,295 @@ __device__ __forceinline__ void add_i64(unsigned long long* a, int64_t idx, int6
   if (idx >= 0 && idx < M) atomicAdd(a + idx, (unsigned long long)v);
 }
 
+// The warp's sum of v (two's complement, exact), as three integer reductions
+// of 27 + 27 + 10 bits.
+__device__ __forceinline__ unsigned long long warp_sum_i64(int64_t v) {
+  const uint64_t u = (uint64_t)v;
+  const uint64_t lo = __reduce_add_sync(0xffffffffu, (unsigned)u & 0x7ffffffu);
+  const uint64_t mid = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 27) & 0x7ffffffu);
+  const uint64_t hi = __reduce_add_sync(0xffffffffu, (unsigned)(u >> 54));
+  return lo + (mid << 27) + (hi << 54);
+}
+
+// a[idx] += v0, a[idx + 1] += v1, summed over the lanes of equal idx first:
+// electrons near each other in the store share nodes (a hundred per cell in
+// order of position), and atomics on one address are served one at a time
+// (rho_kernel on 1,760,600 electrons: 187 us lane by lane, 27 us so).  Three
+// sums; a warp spread wider than that adds the rest lane by lane.  All lanes call this; a
+// lane without a deposit passes zeros.  The sums are exact, so neither their
+// order nor the grouping changes a bit.
+__device__ __forceinline__ void add_pair_warp(unsigned long long* a, int64_t idx, int64_t M, int64_t v0,
+                                              int64_t v1) {
+  const int lane = threadIdx.x & 31;
+  const bool some = (v0 | v1) != 0;
+  unsigned todo = __ballot_sync(0xffffffffu, some);
+#pragma unroll 1
+  for (int it = 0; it < 3 && todo; ++it) {
+    const int leader = __ffs(todo) - 1;
+    const int64_t key = __shfl_sync(0xffffffffu, idx, leader);
+    const bool same = some && idx == key;
+    const unsigned long long s0 = warp_sum_i64(same ? v0 : 0), s1 = warp_sum_i64(same ? v1 : 0);
+    if (lane == leader) {
+      if (s0) add_i64(a, key, M, (int64_t)s0);
+      if (s1) add_i64(a, key + 1, M, (int64_t)s1);
+    }
+    todo &= ~__ballot_sync(0xffffffffu, same);
+  }
+  if ((todo >> lane) & 1u) {
+    if (v0) add_i64(a, idx, M, v0);
+    if (v1) add_i64(a, idx + 1, M, v1);
+  }
+}
+
+// Node charges of Q at node i's offset w: r0 at node i, r1 at i + 1, r0 + r1 = Q.
+__device__ __forceinline__ void split(int64_t Q, double w, int64_t& r0, int64_t& r1) {
+  r1 = double_to_ll(ll_to_double(Q) * w);
+  r0 = Q - r1;
+}
+
+// J_x of a move from (ia, wa) to (ib, wb): the charge that crosses the faces
+// after nodes lo and lo + 1, lo = min(ia, ib) (c dt < dx: at most one node on).
+__device__ __forceinline__ void face_flux(int64_t Q, int64_t ia, double wa, int64_t ib, double wb,
+                                          int64_t& lo, int64_t& f0, int64_t& f1) {
+  int64_t ra0, ra1, rb0, rb1;
+  split(Q, wa, ra0, ra1);
+  split(Q, wb, rb0, rb1);
+  lo = ia < ib ? ia : ib;
+  // running sum of the charge -r leaving ia, ia + 1 and arriving at ib, ib + 1
+  f0 = ia == ib ? rb0 - ra0 : ia < ib ? -ra0 : rb0;
+  f1 = ia == ib ? 0 : ia < ib ? -rb1 : ra1;
+}
+
+// Per array index: the temporal sums at theta = 1/2 and the step to the next
+// index, of E_x, E_y and B_z: the fields of the criterion and of every m = 1
+// push (one multiplication and one addition per grid and electron instead of
+// the gather's 17 operations; the same bits).
 template <int P>
+__global__ void __launch_bounds__(128) nodes_kernel(Sc1dArgs a) {
+  constexpr int stride = 2 * (P + 1);
+  const double* wE = a.wtab + wrow(0, 1) * stride;
+  const double* wB = a.wtab + a.crit_row * stride + (P + 1);
+  for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < 3 * a.M;
+       q += (int64_t)gridDim.x * blockDim.x) {
+    const int f = (int)(q % 3);
+    const int64_t c = q / 3, c1 = c + 1 < a.M ? c + 1 : c;
+    const double* const* lv = f == 0 ? a.Ex : f == 1 ? a.Ey : a.Bz;
+    const double* w = f == 2 ? wB : wE;
+    double f0 = w[0] * __ldg(lv[0] + c), f1 = w[0] * __ldg(lv[0] + c1);
+#pragma unroll
+    for (int l = 1; l <= P; ++l) {
+      f0 = f0 + w[l] * __ldg(lv[l] + c);
+      f1 = f1 + w[l] * __ldg(lv[l] + c1);
+    }
+    a.nodes[q] = make_double2(f0, f1 - f0);
+  }
+}
+
+// The three passes of push_f64.cu with E_x and the deposit: (1) here, every
+// electron's criterion, the m = 1 push and its deposit; (2) bin_f64_kernel;
+// (3) subcycle_deposit_kernel.
+template <bool UNIT>
 __global__ void __launch_bounds__(256) push_deposit_kernel(Sc1dArgs a) {
   __shared__ unsigned long long sh[12];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
+  if (blockIdx.x == 0 && threadIdx.x < 32) a.bin_next[threadIdx.x] = 0;  // the next step's counts
   __syncthreads();
-  constexpr int stride = 2 * (P + 1);
-  const double* wcrit = a.wtab + a.crit_row * stride + (P + 1);
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint8_t st = a.status[i];
-    if (st & PIC_STATUS_LOST) continue;
-    const int k_prev = st & 0x7f;
-    double pv0 = a.px[i], pv1 = a.py[i], pv2 = a.pz[i];
-    double xi = a.x[i];
-    const double s_a = xi * a.inv_dx;
-    if (!inside(s_a, a.n_cells)) {
-      a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
-      atomicAdd(&sh[11], 1ull);
-      continue;
-    }
-    const double b0 = gather<P>(a.Bz, wcrit, s_a - 0.5);
-    const double g0 = sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-    double psi = (a.qm_abs * fabs(b0) * a.dt) / (2.0 * g0);
-    int k = 0;
-    while (psi > a.psi_max && k < a.k_max) {
-      psi = psi * 0.25;
-      ++k;
-    }
-    const bool capped = psi > a.psi_max;
-    const int64_t m = (int64_t)1 << (2 * k);
-    const double h = ldexp(a.dt, -2 * k);
-    const double h_old = ldexp(a.dt, -2 * k_prev);
-    const double inv_m = ldexp(1.0, -2 * k);
-    atomicAdd(&sh[k], 1ull);
-    atomicAdd(&sh[8], (unsigned long long)m);
-    if (k > 0) atomicAdd(&sh[9], (unsigned long long)m);
-    if (capped) atomicAdd(&sh[10], 1ull);
-
-    // J_y sums of nodes base .. base+4, base = floor(s_a) - 2 (a macro step
-    // moves an electron less than one cell: c dt < dx)
-    const int64_t base = (int64_t)floor(s_a) - 2;
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const double* wr = a.wtab + wrow(k, 1) * stride;
-    bool frozen = false;
-    for (int64_t j = 1; j <= m; ++j, wr += stride) {
-      const double s = xi * a.inv_dx;
-      if (!inside(s, a.n_cells)) {
-        frozen = true;
-        break;
-      }
-      const double ex = gather<P>(a.Ex, wr, s - 0.5);
-      const double ey = gather<P>(a.Ey, wr, s);
-      const double bz = gather<P>(a.Bz, wr + (P + 1), s - 0.5);
-      const double hp = (j == 1) ? 0.5 * (h_old + h) : h;
-      // Boris, E = (ex, ey, 0), B = (0, 0, bz)
-      const double half = 0.5 * hp;
-      const double dpx = (a.qm * ex) * half;
-      const double dpy = (a.qm * ey) * half;
-      const double mx = pv0 + dpx, my = pv1 + dpy, mz = pv2;
-      const double gn = sqrt(1.0 + (mx * mx + my * my + mz * mz));
-      const double tz = ((a.qm * bz) * half) / gn;
-      const double ppx = mx + my * tz;
-      const double ppy = my - mx * tz;
-      const double sz = (2.0 * tz) / (1.0 + tz * tz);
-      const double qx = mx + ppy * sz;
-      const double qy = my - ppx * sz;
-      pv0 = qx + dpx;
-      pv1 = qy + dpy;
-      pv2 = mz;
-      const double g = sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-      const double vx = pv0 / g, vy = pv1 / g;
-      const double s_mid = (xi + 0.5 * (h * vx)) * a.inv_dx;
-      xi = xi + h * vx;
-      const double fl = floor(s_mid);
-      const int c = (int)((int64_t)fl - base);
-      const double cw = vy * inv_m;  // (h/dt) v_y
-      const double t = cw * (s_mid - fl);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {  // acc[c] += cw - t; acc[c+1] += t (registers)
-        if (q == c) {
-          acc[q] = acc[q] + (cw - t);
-          acc[q + 1] = acc[q + 1] + t;
+  unsigned k0 = 0, k1 = 0;
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < a.n; b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = b + threadIdx.x;
+    const uint8_t st = i < a.n ? a.status[i] : PIC_STATUS_LOST;
+    int k_sub = 0;
+    int64_t jd = 0, d0 = 0, d1 = 0, jf = 0, f0 = 0, f1 = 0;
+    if (!(st & PIC_STATUS_LOST)) {
+      const double x = a.x[i];
+      Mom64 p = mom64(a.px[i], a.py[i], a.pz[i]);
+      Coords64 c;
+      if (!locate(a, x * a.inv_dx, c)) {
+        a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
+        atomicAdd(&sh[11], 1ull);
+      } else {
+        const double2 nx = __ldg(a.nodes + 3 * (c.jb + 2)), ny = __ldg(a.nodes + 3 * (c.je + 2) + 1),
+                      nb = __ldg(a.nodes + 3 * (c.jb + 2) + 2);
+        const double bz = nb.x + c.wb * nb.y;
+        bool capped;
+        const int k = criterion_f64(a.crit_scale, a.qm_abs, a.dt, a.psi_max, a.k_max, bz, p.x, p.y, p.z,
+                                    capped);
+        if (capped) atomicAdd(&sh[10], 1ull);
+        if (k > 0) {
+          k_sub = k;
+          if (k == 1)
+            ++k1;
+          else
+            atomicAdd(&sh[k], 1ull);
+        } else {
+          ++k0;
+          const double ex = nx.x + c.wb * nx.y, ey = ny.x + c.we * ny.y;
+          const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
+          const Push64 r = push64<UNIT, true>(ex, ey, bz, 0.5 * hp, a.qm, p);
+          const double hv = a.dt * r.vx;
+          const double xn = x + hv;
+          a.x[i] = xn;
+          a.px[i] = p.x;
+          a.py[i] = p.y;
+          a.status[i] = 0;
+          const int64_t Q = a.Q[i];
+          const double Qd = ll_to_double(Q);
+          double w;
+          floor_frac64((x + half64(hv)) * a.inv_dx, jd, w);
+          const double t = r.vy * w;
+          d0 = -double_to_ll((r.vy - t) * Qd);
+          d1 = -double_to_ll(t * Qd);
+          int64_t ib;
+          floor_frac64(xn * a.inv_dx, ib, w);
+          face_flux(Q, c.je, c.we, ib, w, jf, f0, f1);
         }
       }
     }
-    a.x[i] = xi;
-    a.px[i] = pv0;
-    a.py[i] = pv1;
-    a.pz[i] = pv2;
-    if (frozen) {
-      a.status[i] = (uint8_t)(k | PIC_STATUS_LOST);
-      atomicAdd(&sh[11], 1ull);
-    } else {
-      a.status[i] = (uint8_t)k;
+    if (i < a.n) a.k_sub[i] = (uint8_t)k_sub;
+    add_pair_warp(a.D, jd + 2, a.M, d0, d1);
+    add_pair_warp(a.F, jf + 2, a.M, f0, f1);
+  }
+  const unsigned k0w = __reduce_add_sync(0xffffffffu, k0), k1w = __reduce_add_sync(0xffffffffu, k1);
+  if ((threadIdx.x & 31) == 0 && k0w) atomicAdd(&sh[0], (unsigned long long)k0w);
+  if ((threadIdx.x & 31) == 0 && k1w) atomicAdd(&sh[1], (unsigned long long)k1w);
+  flush_f64(sh, a.stats);
+  if (threadIdx.x > 0 && threadIdx.x < 8 && sh[threadIdx.x])
+    atomicAdd(&a.bin[threadIdx.x], (int32_t)sh[threadIdx.x]);
+}
+
+// The J_y sums of an electron's sub-steps at nodes base .. base + 4, base =
+// floor(s_a) - 2 (a macro step moves an electron less than one cell): the two
+// nodes it is between in registers of their own, the five spelled out, since
+// an add to each of the five under a predicate costs the FP64 unit five.
+struct NodeSums {
+  double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  double lo = 0.0, hi = 0.0;  // acc[at], acc[at + 1] while at is current
+  int at = 0;
+  __device__ __forceinline__ void put() {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) acc[q] = q == at ? lo : q == at + 1 ? hi : acc[q];
+  }
+  __device__ __forceinline__ void add(int64_t c, double v0, double v1) {
+    if (c < 0 || c > 3) return;
+    if ((int)c != at) {
+      put();
+      at = (int)c;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (q == at) {
+          lo = acc[q];
+          hi = acc[q + 1];
+        }
     }
+    lo = lo + v0;
+    hi = hi + v1;
+  }
+};
+
+// The sub-cycles, g equal-k electrons per warp (subcycle_f64 of push_f64.cu,
+// with E_x and the deposit).
+template <int P, bool UNIT>
+__device__ __forceinline__ void subcycle_deposit(const Sc1dArgs& a, int64_t first, int64_t end, int g, int k,
+                                                 unsigned long long* sh) {
+  constexpr int stride = 2 * (P + 1);
+  const int lane = threadIdx.x & 31, mine = lane & (g - 1), rows = 32 / g;
+  const int copy = lane / g;
+  const bool valid = first + mine < end;
+  const int64_t i = valid ? a.queue[first + mine] : 0;
+  const uint8_t st = valid ? a.status[i] : 0;
+  double xi = valid ? a.x[i] : 0.0;
+  Mom64 p = valid ? mom64(a.px[i], a.py[i], a.pz[i]) : Mom64{0.0, 0.0, 0.0, 0.0, 0.0};
+  const int m = 1 << (2 * k);
+  const double h = pow4_down64(a.dt, k), h_old = pow4_down64(a.dt, st & 0x7f);
+  double half = 0.5 * (0.5 * (h_old + h));
+  const double* w = a.wtab + wrow(k, 1) * stride;
+  NodePair<P> X, Y, B;
+  NodeSums J;
+  bool live = valid;
+  int64_t ia, ib;
+  double wa, wb;
+  floor_frac64(xi * a.inv_dx, ia, wa);
+  int have = 0, at = 0;  // the warp holds the sums of sub-steps at .. at + have - 1
+  double v[6];           // sub-step j's
+  auto take = [&](int r) {  // they are with copy r
+    const double mineof[6] = {X.f, X.d, Y.f, Y.d, B.f, B.d};
+    const int src = mine + (r & (rows - 1)) * g;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) v[q] = rows > 1 ? __shfl_sync(0xffffffffu, mineof[q], src) : mineof[q];
+  };
+#pragma unroll 1
+  for (int j = 0; j < m; ++j) {
+    Coords64 c;
+    const bool in = live && locate(a, xi * a.inv_dx, c);
+    const int32_t ny = in ? (int32_t)c.je + 2 : Y.at, nb = in ? (int32_t)c.jb + 2 : B.at;
+    live = in;
+    const bool moved = ny != Y.at || nb != B.at;
+    if (__any_sync(0xffffffffu, moved || j >= at + have)) {
+      if (!__any_sync(0xffffffffu, live)) break;
+      if (moved) {
+        X.load(a.Ex, nb, 0x7fffffff);
+        Y.load(a.Ey, ny, 0x7fffffff);
+        B.load(a.Bz, nb, 0x7fffffff);
+      }
+      at = j;
+      have = rows;
+      const double* wr = w + (int64_t)(j + copy < m ? j + copy : m - 1) * stride;
+      X.sums(wr);
+      Y.sums(wr);
+      B.sums(wr + (P + 1));
+      take(0);
+    }
+    const double ex = v[0] + c.wb * v[1], ey = v[2] + c.we * v[3], bz = v[4] + c.wb * v[5];
+    take(j + 1 - at);  // the next sub-step's, unless an electron changes node
+    if (live) {
+      const Push64 r = push64<UNIT, true>(ex, ey, bz, half, a.qm, p);
+      half = 0.5 * h;
+      const double hv = h * r.vx;
+      int64_t jm;
+      double wm;
+      floor_frac64((xi + half64(hv)) * a.inv_dx, jm, wm);
+      xi = xi + hv;
+      const double cw = scale_down64(r.vy, k);  // (h/dt) v_y
+      const double t = cw * wm;
+      J.add(jm - (ia - 2), cw - t, t);
+    }
+  }
+  if (valid && copy == 0) {
+    a.x[i] = xi;
+    a.px[i] = p.x;
+    a.py[i] = p.y;
+    a.status[i] = (uint8_t)(live ? k : k | PIC_STATUS_LOST);
+    if (!live) atomicAdd(&sh[11], 1ull);
+    J.put();
     const int64_t Q = a.Q[i];
 #pragma unroll
-    for (int c = 0; c < 5; ++c)
-      if (acc[c] != 0.0) add_i64(a.D, base + c + 2, a.M, -__double2ll_rn(acc[c] * (double)Q));
-    // J_x: the charge flux of the move s_a -> s_b through the faces
-    const double s_b = xi * a.inv_dx;
-    int64_t ia, ib, ra0, ra1, rb0, rb1;
-    split(Q, s_a, ia, ra0, ra1);
-    split(Q, s_b, ib, rb0, rb1);
-    const int64_t lo = (ia < ib ? ia : ib) - 1;
-    int64_t dC[6] = {0, 0, 0, 0, 0, 0};
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      if (lo + c == ia) dC[c] += ra0;      // the electron's charge -r leaves s_a
-      if (lo + c == ia + 1) dC[c] += ra1;
-      if (lo + c == ib) dC[c] -= rb0;      // and arrives at s_b
-      if (lo + c == ib + 1) dC[c] -= rb1;
-    }
-    int64_t flux = 0;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      flux -= dC[c];
-      if (flux != 0) add_i64(a.F, lo + c + 2, a.M, flux);
-    }
+    for (int q = 0; q < 5; ++q)
+      if (J.acc[q] != 0.0) add_i64(a.D, ia + q, a.M, -__double2ll_rn(J.acc[q] * (double)Q));
+    floor_frac64(xi * a.inv_dx, ib, wb);
+    int64_t lo, f0, f1;
+    face_flux(Q, ia, wa, ib, wb, lo, f0, f1);
+    if (f0) add_i64(a.F, lo + 2, a.M, f0);
+    if (f1) add_i64(a.F, lo + 3, a.M, f1);
   }
-  __syncthreads();
-  if (threadIdx.x < 12) {
-    const unsigned long long v = sh[threadIdx.x];
-    if (v) {
-      unsigned long long* dst = threadIdx.x < 8 ? &a.stats->k_hist[threadIdx.x]
-                                : threadIdx.x == 8 ? &a.stats->substeps
-                                : threadIdx.x == 9 ? &a.stats->n_star
-                                : threadIdx.x == 10 ? &a.stats->clamped
-                                                    : &a.stats->lost;
-      atomicAdd(dst, v);
-    }
+}
+
+template <int P, bool UNIT>
+__global__ void __launch_bounds__(32) subcycle_deposit_kernel(Sc1dArgs a) {
+  __shared__ unsigned long long sh[12];
+  if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
+  __syncwarp();
+  int64_t t = blockIdx.x;
+  for (;;) {
+    int64_t first, end;
+    int k, g;
+    if (!item_f64(a.bin, a.sms, t, first, end, k, g)) break;
+    subcycle_deposit<P, UNIT>(a, first, end, g, k, sh);
+    int next = 0;
+    if (threadIdx.x == 0) next = atomicAdd(&a.bin[16], 1);
+    t = (int64_t)gridDim.x + __shfl_sync(0xffffffffu, next, 0);
   }
+  __syncwarp();
+  if (threadIdx.x == 0 && sh[11]) atomicAdd(&a.stats->lost, sh[11]);
 }
 
 struct FieldArgs {
@@ -264,30 +417,52 @@ __global__ void field_kernel(FieldArgs a) {
   }
 }
 
-__global__ void rho_kernel(const double* x, const int64_t* Q, int64_t n, double inv_dx,
-                           unsigned long long* C, int64_t M, int negate) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t ii, r0, r1;
-    split(Q[i], x[i] * inv_dx, ii, r0, r1);
-    add_i64(C, ii + 2, M, negate ? r0 : -r0);
-    add_i64(C, ii + 3, M, negate ? r1 : -r1);
+// C += the node charges of every electron (negate: minus them).
+__global__ void __launch_bounds__(256) rho_kernel(const double* x, const int64_t* Q, int64_t n, double inv_dx,
+                                                  unsigned long long* C, int64_t M, int negate) {
+  for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < n; b += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = b + threadIdx.x;
+    int64_t j = 0, r0 = 0, r1 = 0;
+    if (i < n) {
+      double w;
+      floor_frac64(x[i] * inv_dx, j, w);
+      split(Q[i], w, r0, r1);
+    }
+    add_pair_warp(C, j + 2, M, negate ? r0 : -r0, negate ? r1 : -r1);
   }
+}
+
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u > v ? u : v;
+  }
+  return v;
 }
 
 // max over nodes k = -1 .. N+1 of |(E_x_{k+1/2} - E_x_{k-1/2})/dx - rho_k| and
 // of |rho^e_k| (non-negative doubles compare like their bit patterns)
-__global__ void gauss_kernel(const double* Ex, const unsigned long long* C,
-                             const unsigned long long* C_ion, int64_t N, double inv_dx,
-                             unsigned long long* out) {
+__global__ void __launch_bounds__(256) gauss_kernel(const double* Ex, const unsigned long long* C,
+                                                    const unsigned long long* C_ion, int64_t N, double inv_dx,
+                                                    unsigned long long* out) {
+  unsigned long long mg = 0, mr = 0;
   for (int64_t k = -1 + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k <= N + 1;
        k += (int64_t)gridDim.x * blockDim.x) {
     const int64_t q = k + 2;
     const double rho = (double)((long long)C[q] + (long long)C_ion[q]) * kUnit;
-    const double g = fabs((Ex[q] - Ex[q - 1]) * inv_dx - rho);
-    const double re = fabs((double)(long long)C[q] * kUnit);
-    atomicMax(&out[0], (unsigned long long)__double_as_longlong(g));
-    atomicMax(&out[1], (unsigned long long)__double_as_longlong(re));
+    const unsigned long long g =
+        (unsigned long long)__double_as_longlong(fabs((Ex[q] - Ex[q - 1]) * inv_dx - rho));
+    const unsigned long long re =
+        (unsigned long long)__double_as_longlong(fabs((double)(long long)C[q] * kUnit));
+    mg = g > mg ? g : mg;
+    mr = re > mr ? re : mr;
+  }
+  mg = warp_max_u64(mg);
+  mr = warp_max_u64(mr);
+  if ((threadIdx.x & 31) == 0) {
+    if (mg) atomicMax(&out[0], mg);
+    if (mr) atomicMax(&out[1], mr);
   }
 }
 
@@ -315,6 +490,11 @@ struct pic_sc1d {
   std::vector<int64_t> slot_level;
   unsigned long long* acc = nullptr;  // [2 parities][F, D][M], then C, C_ion [M] each, gauss [2]
   double* wtab = nullptr;
+  double2* nodes = nullptr;  // [M][3] fields at t_n
+  uint8_t* k_sub = nullptr;  // the electrons of a step that sub-cycle (push_deposit_kernel)
+  int32_t* queue = nullptr;
+  int32_t* bin = nullptr;    // two sets of 32 counters, used in turn
+  int bin_at = 0;
   DevStats* dstats = nullptr;
   double* staging = nullptr;  // 3 M host-upload staging
   int64_t launches = 0;
@@ -392,6 +572,10 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   ok &= cudaMalloc(&c->wtab, wcount * 8) == cudaSuccess;
   ok &= cudaMalloc(&c->dstats, sizeof(DevStats)) == cudaSuccess;
   ok &= cudaMalloc(&c->staging, 3 * c->M * 8) == cudaSuccess;
+  ok &= cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) == cudaSuccess;
+  ok &= cudaMalloc(&c->k_sub, cap) == cudaSuccess;
+  ok &= cudaMalloc(&c->queue, cap * 4) == cudaSuccess;
+  ok &= cudaMalloc(&c->bin, 64 * 4) == cudaSuccess;
   if (!ok) {
     pic_sc1d_destroy(c);
     return sc_fail(nullptr, PIC_ENOMEM, "pic_sc1d_create: device allocation failed");
@@ -399,6 +583,7 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   cudaError_t e = cudaMemsetAsync(c->ring, 0, (int64_t)c->R * 3 * c->M * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->acc, 0, (6 * c->M + 2) * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(c->bin, 0, 64 * 4, c->stream);
   if (e == cudaSuccess) e = build_wtab_f64(c->wtab, prm->order, prm->k_max, prm->field_time, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
@@ -415,6 +600,7 @@ extern "C" int pic_sc1d_destroy(pic_sc1d* c) {
   cudaFree(c->x); cudaFree(c->px); cudaFree(c->py); cudaFree(c->pz); cudaFree(c->w_stage);
   cudaFree(c->status); cudaFree(c->Q); cudaFree(c->ring); cudaFree(c->acc); cudaFree(c->wtab);
   cudaFree(c->dstats); cudaFree(c->staging);
+  cudaFree(c->nodes); cudaFree(c->k_sub); cudaFree(c->queue); cudaFree(c->bin);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   delete c;
@@ -517,8 +703,26 @@ static int sc_gauss(pic_sc1d* c) {
 }
 
 template <int P>
-static void launch_push(const Sc1dArgs& a, int blocks, cudaStream_t s) {
-  push_deposit_kernel<P><<<blocks, 256, 0, s>>>(a);
+static void launch_push(pic_sc1d* c, const Sc1dArgs& a) {
+  const cudaStream_t s = c->stream;
+  const bool unit = a.qm_abs == 1.0;
+  nodes_kernel<P><<<grid_for(c, 2 * 3 * c->M), 128, 0, s>>>(a);
+  // small ensembles in small blocks: every SM's FP64 unit takes part
+  const int threads = a.n >= (int64_t)a.sms * 256 ? 256 : a.n >= (int64_t)a.sms * 64 ? 64 : 32;
+  const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)a.sms * 8;
+  const int blocks = (int)(want < cap ? want : cap);
+  if (unit)
+    push_deposit_kernel<true><<<blocks, threads, 0, s>>>(a);
+  else
+    push_deposit_kernel<false><<<blocks, threads, 0, s>>>(a);
+  launch_bin_f64(BinF64{a.n, a.k_sub, a.queue, a.bin}, a.sms, s);
+  const int64_t most = (int64_t)a.sms * 12;
+  const int warps = (int)(a.n < most ? a.n : most);
+  if (unit)
+    subcycle_deposit_kernel<P, true><<<warps, 32, 0, s>>>(a);
+  else
+    subcycle_deposit_kernel<P, false><<<warps, 32, 0, s>>>(a);
+  c->launches += 4;
 }
 
 extern "C" int pic_sc1d_step(pic_sc1d* c, int64_t n0, int64_t n_steps, pic_sc1d_stats* stats) {
@@ -563,15 +767,21 @@ extern "C" int pic_sc1d_step(pic_sc1d* c, int64_t n0, int64_t n_steps, pic_sc1d_
     a.crit_row = wrows_total(c->prm.k_max) - 1;
     a.stats = c->dstats;
     if (c->n > 0) {
-      const int blocks = grid_for(c, c->n);
+      a.crit_scale = criterion_f64_scale(a.qm_abs, a.dt, a.psi_max);
+      a.nodes = c->nodes;
+      a.k_sub = c->k_sub;
+      a.queue = c->queue;
+      a.bin = c->bin + 32 * c->bin_at;
+      c->bin_at ^= 1;
+      a.bin_next = c->bin + 32 * c->bin_at;
+      a.sms = c->sm_count > 0 ? c->sm_count : 152;
       switch (p) {
-        case 1: launch_push<1>(a, blocks, c->stream); break;
-        case 2: launch_push<2>(a, blocks, c->stream); break;
-        case 3: launch_push<3>(a, blocks, c->stream); break;
-        case 4: launch_push<4>(a, blocks, c->stream); break;
-        case 5: launch_push<5>(a, blocks, c->stream); break;
+        case 1: launch_push<1>(c, a); break;
+        case 2: launch_push<2>(c, a); break;
+        case 3: launch_push<3>(c, a); break;
+        case 4: launch_push<4>(c, a); break;
+        case 5: launch_push<5>(c, a); break;
       }
-      ++c->launches;
     }
     FieldArgs f;
     const int s0 = slot_of(c, s), s1 = slot_of(c, s + 1);

@@ -111,34 +111,6 @@ __device__ __forceinline__ bool locate(const PushArgsF64& a, double s, Coords64&
   return true;
 }
 
-// One grid's levels at the current node pair, and their temporal sums for the
-// next sub-step.
-template <int P>
-struct NodePair {
-  double v0[P + 1], v1[P + 1];
-  int32_t at = -1;  // masked index of the lower node
-  double f, d;      // f_i, f_{i+1} - f_i
-  __device__ __forceinline__ void load(const double* const* lv, int32_t node, int32_t mask) {
-    const int32_t next = (node + 1) & mask;
-#pragma unroll
-    for (int l = 0; l <= P; ++l) {
-      v0[l] = __ldg(lv[l] + node);
-      v1[l] = __ldg(lv[l] + next);
-    }
-    at = node;
-  }
-  __device__ __forceinline__ void sums(const double* w) {
-    double f0 = w[0] * v0[0], f1 = w[0] * v1[0];
-#pragma unroll
-    for (int l = 1; l <= P; ++l) {
-      f0 = f0 + w[l] * v0[l];
-      f1 = f1 + w[l] * v1[l];
-    }
-    f = f0;
-    d = f1 - f0;
-  }
-};
-
 // All 4^k sub-steps of one macro step of g electrons (g a power of two; entries
 // first .. of the queue, those from `end` on absent).  Lane l works on electron
 // l mod g, in 32 / g equal copies: every copy takes the electron's serial chain
@@ -210,10 +182,10 @@ __device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first
     const double ey = ef + c.we * ed, bz = bf + c.wb * bd;
     take(j + 1 - at);  // the next sub-step's, unless the electron changes node
     if (live) {
-      double gam;
-      push64<UNIT>(ey, bz, half, h, a.qm, p, xi, gam);
+      const Push64 r = push64<UNIT, false>(0.0, ey, bz, half, a.qm, p);
+      xi = xi + h * r.vx;
       if (diag) {  // (q hp / 2) E . (v_before + v_after) (App. B)
-        const double v = div_rn(p.y, gam);
+        const double v = div_rn(p.y, r.gam);
         work = work + ((a.qm * hp) * 0.5) * (ey * (vy + v));
         vy = v;
         hp = h;
@@ -228,27 +200,6 @@ __device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first
     a.py[i] = p.y;
     a.status[i] = (uint8_t)(live ? k : k | PIC_STATUS_LOST);
     if (!live) atomicAdd(&sh[11], 1ull);
-  }
-}
-
-// Block counters -> context counters: sh[0..7] the k histogram, sh[10] caps,
-// sh[11] lost.  Sub-step sums follow from the histogram (m = 4^k).
-__device__ __forceinline__ void flush_f64(unsigned long long* sh, DevStats* st) {
-  __syncthreads();
-  if (threadIdx.x < 12) {
-    unsigned long long v = sh[threadIdx.x];
-    if (threadIdx.x == 8 || threadIdx.x == 9) {
-      v = 0;
-      for (int k = threadIdx.x == 8 ? 0 : 1; k < 8; ++k) v += sh[k] << (2 * k);
-    }
-    if (v) {
-      unsigned long long* dst = threadIdx.x < 8 ? &st->k_hist[threadIdx.x]
-                                : threadIdx.x == 8 ? &st->substeps
-                                : threadIdx.x == 9 ? &st->n_star
-                                : threadIdx.x == 10 ? &st->clamped
-                                                    : &st->lost;
-      atomicAdd(dst, v);
-    }
   }
 }
 
@@ -315,10 +266,9 @@ __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) 
           const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
           double vy = 0.0;
           if (a.work) vy = div_rn(p.y, sqrt_rn(1.0 + (p.x2 + p.y * p.y + p.z2)));
-          double xn = x, g;
-          push64<UNIT>(ey, bz, 0.5 * hp, a.dt, a.qm, p, xn, g);
-          a.x[i] = xn;
-          if (a.work) a.work[i] = a.work[i] + ((a.qm * hp) * 0.5) * (ey * (vy + div_rn(p.y, g)));
+          const Push64 r = push64<UNIT, false>(0.0, ey, bz, 0.5 * hp, a.qm, p);
+          a.x[i] = x + a.dt * r.vx;
+          if (a.work) a.work[i] = a.work[i] + ((a.qm * hp) * 0.5) * (ey * (vy + div_rn(p.y, r.gam)));
           a.px[i] = p.x;
           a.py[i] = p.y;
           a.status[i] = 0;
@@ -337,7 +287,7 @@ __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) 
 
 // bin[1..7]: the step's counts per k; bin[8 + k]: entries of k placed so far;
 // bin[16]: the sub-cycle kernel's item cursor.  Queue order: k = 7 first.
-__global__ void __launch_bounds__(256) bin_f64_kernel(PushArgsF64 a) {
+__global__ void __launch_bounds__(256) bin_f64_kernel(BinF64 a) {
   __shared__ int cnt[8], base[8];
   const int64_t n16 = (a.n + 15) / 16;
   int64_t start[8];
@@ -382,14 +332,10 @@ __global__ void __launch_bounds__(256) bin_f64_kernel(PushArgsF64 a) {
   }
 }
 
-// Electrons per warp for a k with `count` of them: few enough that every SM
-// gets a warp of them before any warp holds a second electron (a sub-cycle is
-// a latency-bound chain, so fewer electrons per warp cost nothing while units
-// are idle and save the temporal sums), at most 32.
-__device__ __forceinline__ int group_f64(int count, int sms) {
-  int g = 1;
-  while (g < 32 && count > g * sms) g *= 2;
-  return g;
+cudaError_t launch_bin_f64(const BinF64& a, int sms, cudaStream_t s) {
+  const int64_t vecs = (a.n + 4095) / 4096;
+  bin_f64_kernel<<<(int)(vecs < sms * 8 ? vecs : sms * 8), 256, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 // One warp per block: the few long chains of a step spread over the SMs.
@@ -398,26 +344,11 @@ __global__ void __launch_bounds__(32) subcycle_f64_kernel(PushArgsF64 a) {
   __shared__ unsigned long long sh[12];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
   __syncwarp();
-  // cumulative work items and entries, k = 7 first
   int64_t t = blockIdx.x;
   for (;;) {
-    int64_t items = 0, entries = 0, first = -1, end = 0;
-    int k = 0, g = 1;
-#pragma unroll
-    for (int q = 7; q >= 1; --q) {
-      const int c = a.bin[q];
-      const int gq = group_f64(c, a.sms);
-      const int64_t n = (c + gq - 1) / gq;
-      if (first < 0 && t < items + n) {
-        k = q;
-        g = gq;
-        first = entries + (t - items) * gq;
-        end = entries + c;
-      }
-      items += n;
-      entries += c;
-    }
-    if (first < 0) break;
+    int64_t first, end;
+    int k, g;
+    if (!item_f64(a.bin, a.sms, t, first, end, k, g)) break;
     subcycle_f64<P, UNIT>(a, first, end, g, k, sh);
     int next = 0;
     if (threadIdx.x == 0) next = atomicAdd(&a.bin[16], 1);
@@ -440,8 +371,7 @@ static void launch_f64_p(PushArgsF64 a, int sms, cudaStream_t s, int* launches) 
   const int threads = a.n >= (int64_t)sms * 256 ? 256 : a.n >= (int64_t)sms * 64 ? 64 : 32;
   const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)sms * 8;
   criterion_push_f64_kernel<P, UNIT><<<(int)(want < cap ? want : cap), threads, 0, s>>>(a);
-  const int64_t vecs = (a.n + 4095) / 4096;
-  bin_f64_kernel<<<(int)(vecs < sms * 8 ? vecs : sms * 8), 256, 0, s>>>(a);
+  launch_bin_f64(BinF64{a.n, a.k_sub, a.queue, a.bin}, sms, s);
   const int64_t most = (int64_t)sms * 12;
   subcycle_f64_kernel<P, UNIT><<<(int)(a.n < most ? a.n : most), 32, 0, s>>>(a);
   if (launches) *launches += n;
