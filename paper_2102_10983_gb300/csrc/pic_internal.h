@@ -47,7 +47,7 @@ inline int64_t wrows_total(int k_max) { return wrow(k_max + 1, 1) + 1; }  // + c
 
 // The scale |q/m| dt / (2 Psi_max) of the FP64 kernels' FP32 criterion
 // (criterion_f64_guess), 0 where that test does not apply.
-inline float criterion_f64_scale(double qm_abs, double dt, double psi_max) {
+__host__ __device__ inline float criterion_f64_scale(double qm_abs, double dt, double psi_max) {
   const double c = qm_abs * dt / (2.0 * psi_max);
   return (c >= 0x1p-60 && c <= 0x1p60 && psi_max >= 0x1p-500 && psi_max <= 0x1p500) ? (float)c : 0.0f;
 }

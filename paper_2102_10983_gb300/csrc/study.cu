@@ -4,14 +4,19 @@
 // the field sampled on the grid (the "perfectly propagating PIC" of Sec. III):
 // E_y at nodes i dx and times n dt, B_z at (i + 1/2) dx and (n + 1/2) dt.
 //
-// One thread per electron of a case (a0, dt, dx, Psi_max, order, ...), one
-// warp per CTA, x0 = j lambda / n_electrons; each thread integrates its whole
-// trajectory with the method (Algorithm 1 of Sec. IV, order-p Lagrange in
-// time of Sec. VI, tent in space, Boris), in FP64 compiled with -fmad=false in
-// the order of a serial evaluation.  The field values a gather needs are
-// computed from the formula (the device's exp, sin, cos) and cached per grid
-// for the current node pair and level window: a macro step that keeps the
-// nodes computes only the newest level, a sub-step none.
+// One warp per electron: each integrates its whole trajectory with the method
+// (Algorithm 1 of Sec. IV, order-p Lagrange in time of Sec. VI, tent in space,
+// Boris), in FP64 compiled with -fmad=false in the order of a serial
+// evaluation.  A trajectory is one serial chain, and the FP64 unit takes 19
+// clocks for a warp instruction with one active lane as with 32, so a warp of
+// 32 electrons (as this once was) ran all of them as long as its largest 4^k,
+// at 2 us per sub-step.  Here the chain is taken by every lane alike and the
+// work beside it is dealt to the lanes: the field at the nodes about the
+// electron (the formula's exp, sin, cos: one evaluation of the warp per macro
+// step serves all levels, grids and nodes, and the diagnostic's a), the
+// Lagrange weights and the temporal sums of 32 sub-steps at a time.  Orders 1,
+// 3 and 5, a0 = 5, lambda/75, 64 electrons each, 2,000 macro steps: 264 ms
+// with 32 electrons per warp, 25 ms so.
 //
 // Per electron and macro step (Sec. IV, Eqs. R error, gamma error): R = gamma
 // - p_x, the energy error |gamma - gamma_th| / gamma_th with gamma_th = 1 +
@@ -24,185 +29,232 @@
 
 #include <vector>
 
+#include "fp64_push.cuh"
 #include "pic_internal.h"
 
 namespace pic {
 namespace {
 
-__device__ __forceinline__ double a_of(const pic_study_case& q, double xi) {
-  const double d = xi - q.xi0;
-  return q.a0 * exp(-(d * d) / (2.0 * q.sigma * q.sigma)) * sin(xi);
-}
-
-// E_y = B_z = -da/dxi (Eq. laser5)
-__device__ __forceinline__ double field_of(const pic_study_case& q, double xi) {
-  const double d = xi - q.xi0;
-  const double env = exp(-(d * d) / (2.0 * q.sigma * q.sigma));
-  double sn, cs;
-  sincos(xi, &sn, &cs);  // one argument reduction for both
-  return -(q.a0 * env * (cs - (d / (q.sigma * q.sigma)) * sn));
-}
-
-// The rounded reciprocals of the integer denominators prod_{k != j} (j - k),
-// formed once per electron (the same values the weights' definition rounds).
-__device__ void lagrange_inv_den(int p, double* inv_den) {
-  for (int j = 0; j <= p; ++j) {
-    long long den = 1;
-    for (int k = 0; k <= p; ++k)
-      if (k != j) den *= (long long)(j - k);
-    inv_den[j] = 1.0 / (double)den;
-  }
-}
-
-__device__ void lagrange(int p, bool is_e, double theta, const double* inv_den, double* w) {
+// prod_{k != j} (c_k + theta) times the rounded reciprocal of the integer
+// denominator, c_k = p-k-1/2 (E) or p-k-1 (B).
+template <int P>
+__device__ __forceinline__ void lagrange(bool is_e, double theta, double* w) {
   const double c_off = is_e ? -0.5 : -1.0;
-  for (int j = 0; j <= p; ++j) {
+#pragma unroll
+  for (int j = 0; j <= P; ++j) {
     double num = 1.0;
     bool first = true;
-    for (int k = 0; k <= p; ++k) {
+    int den = 1;
+#pragma unroll
+    for (int k = 0; k <= P; ++k) {
       if (k == j) continue;
-      const double factor = ((double)(p - k) + c_off) + theta;
-      if (first) {
-        num = factor;
-        first = false;
-      } else {
-        num = num * factor;
-      }
+      const double factor = ((double)(P - k) + c_off) + theta;
+      num = first ? factor : num * factor;
+      first = false;
+      den *= j - k;
     }
-    w[j] = num * inv_den[j];
+    w[j] = num * (1.0 / (double)den);
   }
 }
 
-// The field values of one grid at its current node pair (j, j + 1) for the
-// levels n - p .. n (E: times (n - p + l) dt; B: + dt/2), computed on demand.
-template <int P>
-struct GridCache {
-  double v0[P + 1], v1[P + 1];
-  double j = -1e300;  // node of v0 (a node index, held as a double)
-  int64_t n = INT64_MIN;
+// theta of the j-th (0-based) of 4^k sub-steps.
+__device__ __forceinline__ double theta_of(int field_time, int j, int k) {
+  const double inv_m = scale_down64(1.0, k);
+  return field_time == 0 ? 0.5 + (double)j * inv_m : ((double)j + 0.5) * inv_m;
+}
 
-  __device__ void ensure(const pic_study_case& q, bool is_b, double j_new, int64_t n_new) {
-    if (j_new == j && n_new == n) return;
-    const double off = is_b ? 0.5 : 0.0;
-    const double x0 = (j_new + off) * q.dx, x1 = ((j_new + 1.0) + off) * q.dx;
-    if (j_new == j && n_new == n + 1) {  // same nodes, the window moves up one level
+__device__ __forceinline__ int mod_pos(int64_t a, int m) {
+  const int r = (int)(a % m);
+  return r < 0 ? r + m : r;
+}
+
+// The field about the electron: per grid (E: times n dt, nodes i dx; B: both
+// half a step on) the values at three nodes base .. base + 2 and levels n-P ..
+// n, one per lane (two at order 5), node i and level l in the slot (i mod 3, l
+// mod (P + 1)), so that a step on replaces the oldest level only and a node on
+// the hindmost node; and a copy in shared memory for the lanes to read.
+template <int P>
+struct FieldTile {
+  static constexpr int kPerGrid = 3 * (P + 1), kSlots = 2 * kPerGrid;
+  static constexpr int kPer = (kSlots + 31) / 32;  // slots per lane; lane 31's last is free
+  int64_t node[kPer], level[kPer];
+
+  __device__ __forceinline__ void init() {
 #pragma unroll
-      for (int l = 0; l < P; ++l) {
-        v0[l] = v0[l + 1];
-        v1[l] = v1[l + 1];
-      }
-      const double t = ((double)n_new + off) * q.dt;
-      v0[P] = field_of(q, t - x0);
-      v1[P] = field_of(q, t - x1);
-    } else {
+    for (int t = 0; t < kPer; ++t) node[t] = level[t] = INT64_MIN;
+  }
+  // Bring the tile to nodes je .. je + 2 (E), jb .. jb + 2 (B) and levels n-P
+  // .. n.  The free slot evaluates a(xi_diag), returned to every lane.
+  __device__ __forceinline__ double fill(const pic_study_case& q, double* sm, int64_t je, int64_t jb, int64_t n,
+                                         double xi_diag) {
+    const int lane = threadIdx.x;
+    const double ss = q.sigma * q.sigma, s2 = 2.0 * q.sigma * q.sigma;
+    double a = 0.0;
+    __syncwarp();
 #pragma unroll
-      for (int l = 0; l <= P; ++l) {
-        const double t = ((double)(n_new - P + l) + off) * q.dt;
-        v0[l] = field_of(q, t - x0);
-        v1[l] = field_of(q, t - x1);
+    for (int t = 0; t < kPer; ++t) {
+      const int slot = lane + 32 * t;
+      const bool used = slot < kSlots, is_b = slot >= kPerGrid;
+      const int r = is_b ? slot - kPerGrid : slot;
+      const int64_t j = is_b ? jb : je;
+      const int64_t i = j + (r / (P + 1) + 3 - mod_pos(j, 3)) % 3;
+      const int64_t l = n - (mod_pos(n, P + 1) + (P + 1) - r % (P + 1)) % (P + 1);
+      const bool stale = used && (node[t] != i || level[t] != l);
+      const bool diag = t == kPer - 1 && lane == 31;
+      if (stale || diag) {
+        const double off = is_b ? 0.5 : 0.0;
+        const double xi = diag ? xi_diag
+                               : (ll_to_double(l) + off) * q.dt - (ll_to_double(i) + off) * q.dx;
+        const double d = xi - q.xi0;
+        const double env = q.a0 * exp(div_rn(-(d * d), s2));
+        double sn, cs;
+        sincos(xi, &sn, &cs);  // one argument reduction for both
+        if (stale) {
+          sm[slot] = -(env * (cs - div_rn(d, ss) * sn));  // E_y = B_z = -da/dxi (Eq. laser5)
+          node[t] = i;
+          level[t] = l;
+        } else {
+          a = env * sn;
+        }
       }
     }
-    j = j_new;
-    n = n_new;
+    __syncwarp();
+    return __shfl_sync(0xffffffffu, a, 31);
+  }
+  // The values at nodes j, j + 1 of one grid, levels ascending.
+  __device__ __forceinline__ void read(const double* sm, bool is_b, int64_t j, int64_t n, double* v0,
+                                       double* v1) const {
+    const double* g = sm + (is_b ? kPerGrid : 0);
+    const int a = mod_pos(j, 3);
+    const double* r0 = g + a * (P + 1);
+    const double* r1 = g + (a == 2 ? 0 : a + 1) * (P + 1);
+    int l = mod_pos(n - P, P + 1);
+#pragma unroll
+    for (int q = 0; q <= P; ++q) {
+      v0[q] = r0[l];
+      v1[q] = r1[l];
+      l = l == P ? 0 : l + 1;
+    }
   }
 };
 
-// Temporal sums at the two tent nodes (ascending level), then the tent weight.
-template <int P>
-__device__ __forceinline__ double gather(GridCache<P>& c, const pic_study_case& q, bool is_b,
-                                         int64_t n, const double* w, double u) {
-  const double fl = floor(u);
-  const double frac = u - fl;
-  c.ensure(q, is_b, fl, n);
-  double f0 = w[0] * c.v0[0];
-  double f1 = w[0] * c.v1[0];
-#pragma unroll
-  for (int l = 1; l <= P; ++l) {
-    f0 = f0 + w[l] * c.v0[l];
-    f1 = f1 + w[l] * c.v1[l];
-  }
-  return f0 + frac * (f1 - f0);
-}
-
-__device__ __forceinline__ void atomic_max_pos(unsigned long long* a, double v) {
-  atomicMax(a, (unsigned long long)__double_as_longlong(v));  // v >= 0
-}
-
-template <int P>
-__device__ void study_electron(const pic_study_case& q, double x0, double* out_eps_r,
-                               double* out_eps_e, double* out_gmax, int64_t* n_star,
-                               int64_t* substeps, int64_t* k_hist) {
+template <int P, bool UNIT>
+__device__ __forceinline__ void study_electron(const pic_study_case& q, double x0, double* sm,
+                                               double* out_eps_r, double* out_eps_e, double* out_gmax,
+                                               int64_t* n_star, int64_t* substeps, int64_t* k_count) {
+  const int lane = threadIdx.x;
   const double dt = q.dt, inv_dx = 1.0 / q.dx;
-  double wB_half[P + 1], wE[P + 1], wB[P + 1], inv_den[P + 1];
-  lagrange_inv_den(P, inv_den);
-  lagrange(P, false, 0.5, inv_den, wB_half);
-  GridCache<P> cE, cB;
-  double pv0 = 0.0, pv1 = 0.0, pv2 = 0.0;
+  const double qm_abs = fabs(q.qm);
+  const float scale = criterion_f64_scale(qm_abs, dt, q.psi_max);
+  // the lane's weights for k <= 2: lanes 0 .. 15 the rows of k = 2, 16 .. 19
+  // those of k = 1, the rest theta = 1/2 (k = 0 and the criterion)
+  double wE0[P + 1], wB0[P + 1];
+  {
+    const double th = lane < 16 ? theta_of(q.field_time, lane, 2)
+                      : lane < 20 ? theta_of(q.field_time, lane - 16, 1) : 0.5;
+    lagrange<P>(true, th, wE0);
+    lagrange<P>(false, th, wB0);
+  }
+  FieldTile<P> tile;
+  tile.init();
+  NodePair<P> E, B;
+  Mom64 p = mom64(0.0, 0.0, 0.0);
   double xi = x0;
   int k_prev = 0;
   double eps_r = 0.0, eps_e = 0.0, gmax = 1.0;
-  int64_t ns = 0, sub = 0;
+  int64_t ns = 0, sub = 0, count = 0;
+  double xi_diag = q.xi0, g_diag = 1.0;  // the last step's momentum phase and gamma
+  auto locate = [&](Coords64& c) {
+    const double s = xi * inv_dx;
+    if (!coords64_fast(s, c)) coords64_any(s, c);
+  };
+  auto diagnose = [&](double a) {  // |gamma - gamma_th| / gamma_th of the step before
+    const double g_th = 1.0 + 0.5 * a * a;
+    const double de = div_rn(fabs(g_diag - g_th), g_th);
+    if (de > eps_e) eps_e = de;
+  };
   for (int64_t n = 0; n < q.n_steps; ++n) {
-    double s = xi * inv_dx;
-    const double b0 = gather<P>(cB, q, true, n, wB_half, s - 0.5);
-    const double g0 = sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-    double psi = (fabs(q.qm) * fabs(b0) * dt) / (2.0 * g0);
-    int k = 0;
-    while (psi > q.psi_max && k < q.k_max) {
-      psi = psi * 0.25;
-      ++k;
-    }
-    const int64_t m = (int64_t)1 << (2 * k);
-    const double h = ldexp(dt, -2 * k);
-    const double h_old = ldexp(dt, -2 * k_prev);
-    const double inv_m = ldexp(1.0, -2 * k);
-    k_hist[k] += 1;
+    Coords64 c;
+    locate(c);
+    const double a = tile.fill(q, sm, c.je, c.jb, n, xi_diag);
+    if (n > 0) diagnose(a);
+    int64_t je = c.je, jb = c.jb, te = je, tb = jb;  // the electron's nodes and the tile's
+    tile.read(sm, false, je, n, E.v0, E.v1);
+    tile.read(sm, true, jb, n, B.v0, B.v1);
+    E.sums(wE0);
+    B.sums(wB0);
+    const double b0 = __shfl_sync(0xffffffffu, B.f, 31) + c.wb * __shfl_sync(0xffffffffu, B.d, 31);
+    bool capped;
+    const int k = criterion_f64(scale, qm_abs, dt, q.psi_max, q.k_max, b0, p.x, p.y, p.z, capped);
+    const int m = 1 << (2 * k);
+    const double h = pow4_down64(dt, k), h_old = pow4_down64(dt, k_prev);
+    if (lane == k) ++count;
     sub += m;
     if (k > 0) ns += m;
-    double g = g0;
-    for (int64_t j = 1; j <= m; ++j) {
-      const double theta = (q.field_time == 0) ? 0.5 + (double)(j - 1) * inv_m
-                                                : ((double)(j - 1) + 0.5) * inv_m;
-      lagrange(P, true, theta, inv_den, wE);
-      lagrange(P, false, theta, inv_den, wB);
-      s = xi * inv_dx;
-      const double ey = gather<P>(cE, q, false, n, wE, s);
-      const double bz = gather<P>(cB, q, true, n, wB, s - 0.5);
-      const double hp = (j == 1) ? 0.5 * (h_old + h) : h;
-      // Boris, E = (0, ey, 0), B = (0, 0, bz)
-      const double half = 0.5 * hp;
-      const double dpy = (q.qm * ey) * half;
-      const double mx = pv0, my = pv1 + dpy, mz = pv2;
-      const double gn = sqrt(1.0 + (mx * mx + my * my + mz * mz));
-      const double tz = ((q.qm * bz) * half) / gn;
-      const double ppx = mx + my * tz;
-      const double ppy = my - mx * tz;
-      const double sz = (2.0 * tz) / (1.0 + tz * tz);
-      const double qx = mx + ppy * sz;
-      const double qy = my - ppx * sz;
-      pv0 = qx;
-      pv1 = qy + dpy;
-      pv2 = mz;
-      g = sqrt(1.0 + (pv0 * pv0 + pv1 * pv1 + pv2 * pv2));
-      xi = xi + h * (pv0 / g);
+    double half = 0.5 * (0.5 * (h_old + h));
+    double wE[P + 1], wB[P + 1];
+#pragma unroll
+    for (int l = 0; l <= P; ++l) {
+      wE[l] = wE0[l];
+      wB[l] = wB0[l];
+    }
+    const int first = k == 0 ? 31 : k == 1 ? 16 : 0;  // the lane with the first sub-step's sums
+    Push64 r;
+    for (int j = 0; j < m; ++j) {
+      if (j > 0) locate(c);
+      const bool moved = c.je != je || c.jb != jb;
+      if (k > 2 && (j & 31) == 0) {  // the next 32 sub-steps' weights
+        const double th = theta_of(q.field_time, j + lane, k);
+        lagrange<P>(true, th, wE);
+        lagrange<P>(false, th, wB);
+      }
+      if (moved) {
+        // one node on is in the tile; anything else (a step of more than a
+        // node, c dt > dx, or a turn back) is evaluated anew
+        if (c.je < te || c.je > te + 1 || c.jb < tb || c.jb > tb + 1) {
+          te = c.je;
+          tb = c.jb;
+          tile.fill(q, sm, te, tb, n, xi_diag);
+        }
+        je = c.je;
+        jb = c.jb;
+        tile.read(sm, false, je, n, E.v0, E.v1);
+        tile.read(sm, true, jb, n, B.v0, B.v1);
+      }
+      if (moved || (k > 2 && (j & 31) == 0)) {
+        E.sums(wE);
+        B.sums(wB);
+      }
+      const int src = first + (j & 31);
+      const double ey = __shfl_sync(0xffffffffu, E.f, src) + c.we * __shfl_sync(0xffffffffu, E.d, src);
+      const double bz = __shfl_sync(0xffffffffu, B.f, src) + c.wb * __shfl_sync(0xffffffffu, B.d, src);
+      r = push64<UNIT, false>(0.0, ey, bz, half, q.qm, p);
+      half = 0.5 * h;
+      xi = xi + h * r.vx;
     }
     k_prev = k;
-    const double R = g - pv0;
-    const double dR = fabs(R - 1.0);
+    const double dR = fabs((r.gam - p.x) - 1.0);
     if (dR > eps_r) eps_r = dR;
-    const double t_p = (double)(n + 1) * dt - 0.5 * h;
-    const double x_p = xi - 0.5 * h * (pv0 / g);
-    const double a = a_of(q, t_p - x_p);
-    const double g_th = 1.0 + 0.5 * a * a;
-    const double de = fabs(g - g_th) / g_th;
-    if (de > eps_e) eps_e = de;
-    if (g > gmax) gmax = g;
+    if (r.gam > gmax) gmax = r.gam;
+    const double t_p = ll_to_double(n + 1) * dt - 0.5 * h;
+    xi_diag = t_p - (xi - 0.5 * h * r.vx);
+    g_diag = r.gam;
+  }
+  if (q.n_steps > 0) {
+    Coords64 c;
+    locate(c);
+    diagnose(tile.fill(q, sm, c.je, c.jb, q.n_steps, xi_diag));
   }
   *out_eps_r = eps_r;
   *out_eps_e = eps_e;
   *out_gmax = gmax;
   *n_star = ns;
   *substeps = sub;
+  *k_count = count;
+}
+
+__device__ __forceinline__ void atomic_max_pos(unsigned long long* a, double v) {
+  atomicMax(a, (unsigned long long)__double_as_longlong(v));  // v >= 0
 }
 
 struct StudyAcc {
@@ -211,35 +263,43 @@ struct StudyAcc {
   unsigned long long k_hist[8];
 };
 
-// One warp per CTA: block b runs electrons 32 (b % per_case) .. + 31 of case
-// b / per_case, so a case of 64 electrons spreads over two SMs (the FP64 pipe
-// of one SM is the bound: ~2 DFMA per clock); every order in one launch, so
-// the cases of all orders run at once.
+template <int P>
+__device__ __forceinline__ void study_order(const pic_study_case& q, double x0, double* sm, double* er,
+                                            double* ee, double* gm, int64_t* ns, int64_t* sub, int64_t* kc) {
+  if (fabs(q.qm) == 1.0)
+    study_electron<P, true>(q, x0, sm, er, ee, gm, ns, sub, kc);
+  else
+    study_electron<P, false>(q, x0, sm, er, ee, gm, ns, sub, kc);
+}
+
+// One warp per CTA and electron: block b runs electron b mod per_case of case
+// b / per_case; every order in one launch, so the cases of all orders run at
+// once.
 __global__ void __launch_bounds__(32) study_kernel(const pic_study_case* cases, pic_study_result* out,
                                                    StudyAcc* acc, int per_case) {
+  __shared__ double sm[FieldTile<kMaxOrder>::kSlots];
   const int c = blockIdx.x / per_case;
   const pic_study_case q = cases[c];
-  const int e = (blockIdx.x % per_case) * 32 + (int)threadIdx.x;
+  const int e = blockIdx.x % per_case;
   if (e >= q.n_electrons) return;
   const double x0 = (2.0 * M_PI) * (double)e / (double)q.n_electrons;
   double er, ee, gm;
-  int64_t ns, sub;
-  int64_t kh[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  int64_t ns, sub, kc;
   switch (q.order) {
-    case 1: study_electron<1>(q, x0, &er, &ee, &gm, &ns, &sub, kh); break;
-    case 2: study_electron<2>(q, x0, &er, &ee, &gm, &ns, &sub, kh); break;
-    case 3: study_electron<3>(q, x0, &er, &ee, &gm, &ns, &sub, kh); break;
-    case 4: study_electron<4>(q, x0, &er, &ee, &gm, &ns, &sub, kh); break;
-    default: study_electron<5>(q, x0, &er, &ee, &gm, &ns, &sub, kh); break;
+    case 1: study_order<1>(q, x0, sm, &er, &ee, &gm, &ns, &sub, &kc); break;
+    case 2: study_order<2>(q, x0, sm, &er, &ee, &gm, &ns, &sub, &kc); break;
+    case 3: study_order<3>(q, x0, sm, &er, &ee, &gm, &ns, &sub, &kc); break;
+    case 4: study_order<4>(q, x0, sm, &er, &ee, &gm, &ns, &sub, &kc); break;
+    default: study_order<5>(q, x0, sm, &er, &ee, &gm, &ns, &sub, &kc); break;
   }
   StudyAcc& A = acc[c];
+  if (threadIdx.x < 8 && kc) atomicAdd(&A.k_hist[threadIdx.x], (unsigned long long)kc);
+  if (threadIdx.x > 0) return;
   atomic_max_pos(&A.eps_r, er);
   atomic_max_pos(&A.eps_e, ee);
   atomic_max_pos(&A.gmax, gm);
   atomicAdd(&A.n_star_sum, (unsigned long long)ns);
   atomicAdd(&A.substeps_sum, (unsigned long long)sub);
-  for (int k = 0; k < 8; ++k)
-    if (kh[k]) atomicAdd(&A.k_hist[k], (unsigned long long)kh[k]);
   if (e == 0) {
     pic_study_result& r = out[c];
     r.eps_dephasing_first = er;
@@ -290,10 +350,8 @@ extern "C" int pic_study_run(const pic_study_case* cases, int32_t n_cases, pic_s
   if (e == cudaSuccess) e = cudaMemsetAsync(dacc, 0, sizeof(StudyAcc) * n_cases, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(dout, 0, sizeof(pic_study_result) * n_cases, st);
   int per_case = 1;
-  for (int32_t i = 0; i < n_cases; ++i) {
-    const int w = (cases[i].n_electrons + 31) / 32;
-    per_case = w > per_case ? w : per_case;
-  }
+  for (int32_t i = 0; i < n_cases; ++i)
+    per_case = cases[i].n_electrons > per_case ? cases[i].n_electrons : per_case;
   if (e == cudaSuccess) {
     study_kernel<<<(unsigned)(n_cases * per_case), 32, 0, st>>>(dcases, dout, dacc, per_case);
     e = cudaGetLastError();
