@@ -22,6 +22,7 @@ LIB = os.path.join(HERE, "_build", "libpic_gb300.so")
 GENCODE = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = {
     "pic_api.cu": [],
+    "convert.cu": ["-fmad=false"],
     "push_f64.cu": ["-fmad=false"],
     "push_mixed.cu": [],
     "push_noalloc.cu": [],

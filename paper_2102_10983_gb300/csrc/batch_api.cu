@@ -158,6 +158,8 @@ extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t 
     d.qm = (float)s.qm;
     d.qm_abs = fabsf((float)s.qm);
     d.inv_dx = (float)(1.0 / s.dx);
+    d.dx = s.dx;
+    d.inv_dx64 = 1.0 / s.dx;
     d.k_max = s.k_max;
     d.field_time = s.field_time;
     d.ringE = b->ring + (size_t)q * 2 * (2 * (size_t)ring_levels) * window_cells;
@@ -234,31 +236,32 @@ extern "C" int pic_batch_particles_write(pic_batch* b, const double* x, const do
     BATCH_TRY(b, cudaMemcpyAsync(b->status, status, (size_t)b->n_total, kin, b->stream));
   else
     BATCH_TRY(b, cudaMemsetAsync(b->status, 0, (size_t)b->n_total, b->stream));
-  // staged per ensemble (each its own dx)
-  double* st = nullptr;
-  const int64_t biggest = [&] {
-    int64_t m = 0;
-    for (auto& q : b->ens_h) m = q.n_particles > m ? q.n_particles : m;
-    return m;
-  }();
-  if (where == PIC_HOST && biggest > 0) BATCH_TRY(b, cudaMalloc((void**)&st, sizeof(double) * 4 * biggest));
-  for (int q = 0; q < b->n_ens; ++q) {
-    const EnsDev& d = b->ens_dev_h[q];
-    if (d.count == 0) continue;
-    const double* src[4] = {x + d.first, px + d.first, py + d.first, pz + d.first};
-    if (where == PIC_HOST) {
-      for (int c = 0; c < 4; ++c)
-        BATCH_TRY(b, cudaMemcpyAsync(st + c * d.count, src[c], sizeof(double) * d.count,
-                                     cudaMemcpyHostToDevice, b->stream));
-      for (int c = 0; c < 4; ++c) src[c] = st + c * d.count;
-    }
-    BATCH_TRY(b, launch_to_mixed(src[0], src[1], src[2], src[3], b->cell + d.first, b->frac + d.first,
-                                 b->px + d.first, b->py + d.first, b->pz + d.first,
-                                 1.0 / b->ens_h[q].dx, d.count, b->stream));
+  // all ensembles in one launch (each its own dx); host arrays in stages
+  const MixedStore m{b->cell, b->frac, b->px, b->py, b->pz};
+  if (where == PIC_DEVICE) {
+    BATCH_TRY(b, launch_to_mixed_batch(x, px, py, pz, m, b->ens_dev, b->n_ens, 0, b->n_total, b->stream));
     ++b->launches;
-    if (where == PIC_HOST) BATCH_TRY(b, cudaStreamSynchronize(b->stream));
+  } else if (b->n_total > 0) {
+    const int64_t stage = b->n_total < ((int64_t)1 << 22) ? b->n_total : (int64_t)1 << 22;
+    const int64_t pitch = (stage + 1) & ~(int64_t)1;
+    double* st = nullptr;
+    BATCH_TRY(b, cudaMalloc((void**)&st, sizeof(double) * 4 * pitch));
+    const double* src[4] = {x, px, py, pz};
+    cudaError_t e = cudaSuccess;
+    for (int64_t off = 0; off < b->n_total && e == cudaSuccess; off += stage) {
+      const int64_t n = b->n_total - off < stage ? b->n_total - off : stage;
+      for (int c = 0; c < 4 && e == cudaSuccess; ++c)
+        e = cudaMemcpyAsync(st + c * pitch, src[c] + off, sizeof(double) * n, cudaMemcpyHostToDevice, b->stream);
+      if (e == cudaSuccess)
+        e = launch_to_mixed_batch(st, st + pitch, st + 2 * pitch, st + 3 * pitch,
+                                  MixedStore{m.cell + off, m.frac + off, m.px + off, m.py + off, m.pz + off},
+                                  b->ens_dev, b->n_ens, off, n, b->stream);
+      ++b->launches;
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    cudaFree(st);
+    if (e != cudaSuccess) return bfail(b, PIC_ECUDA, cudaGetErrorString(e));
   }
-  if (st) cudaFree(st);
   BATCH_TRY(b, cudaStreamSynchronize(b->stream));
   return PIC_OK;
 }
@@ -272,18 +275,12 @@ extern "C" int pic_batch_particles_read(pic_batch* b, double* x, double* px, dou
   double* st = nullptr;
   if (where == PIC_HOST && b->n_total > 0)
     BATCH_TRY(b, cudaMalloc((void**)&st, sizeof(double) * 4 * b->n_total));
-  for (int q = 0; q < b->n_ens; ++q) {
-    const EnsDev& d = b->ens_dev_h[q];
-    if (d.count == 0) continue;
-    double* dst[4] = {x ? x + d.first : nullptr, px ? px + d.first : nullptr,
-                      py ? py + d.first : nullptr, pz ? pz + d.first : nullptr};
-    if (where == PIC_HOST)
-      for (int c = 0; c < 4; ++c) dst[c] = st + c * b->n_total + d.first;
-    BATCH_TRY(b, launch_from_mixed(b->cell + d.first, b->frac + d.first, b->px + d.first,
-                                   b->py + d.first, b->pz + d.first, dst[0], dst[1], dst[2], dst[3],
-                                   b->ens_h[q].dx, d.count, b->stream));
-    ++b->launches;
-  }
+  double* dst[4] = {x, px, py, pz};
+  if (where == PIC_HOST)
+    for (int c = 0; c < 4; ++c) dst[c] = st + c * b->n_total;
+  BATCH_TRY(b, launch_from_mixed_batch(MixedStore{b->cell, b->frac, b->px, b->py, b->pz}, dst[0], dst[1], dst[2],
+                                       dst[3], b->ens_dev, b->n_ens, b->n_total, b->stream));
+  ++b->launches;
   if (where == PIC_HOST) {
     double* outs[4] = {x, px, py, pz};
     for (int c = 0; c < 4; ++c)

@@ -118,67 +118,30 @@ static void free_all(pic_ctx* c) {
 // ---------------------------------------------------------------- small kernels
 
 // Write a window of W nodes starting at global node i0 into a ring slot,
-// circularly: node i goes to position i & (W-1).  dslot_i0 (optional): the
-// device copy of the slots' window origins, updated in stream order.
+// circularly: node i goes to position i & (W-1).  mirror: the distance to a
+// second copy (the mixed form's ring holds each level twice), 0 for none.
+// dslot_i0 (optional): the device copy of the slots' window origins, updated
+// in stream order.
 template <typename T>
 __global__ void scatter_level_kernel(T* slotE, T* slotB, const double* Ey, const double* Bz,
-                                     int64_t i0, int64_t W, int64_t* dslot_i0, int32_t slot) {
+                                     int64_t i0, int64_t W, int64_t mirror, int64_t* dslot_i0,
+                                     int32_t slot) {
   if (dslot_i0 && blockIdx.x == 0 && threadIdx.x == 0) dslot_i0[slot] = i0;
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < W;
        c += (int64_t)gridDim.x * blockDim.x) {
     int64_t pos = (i0 + c) & (W - 1);
-    slotE[pos] = (T)Ey[c];
-    slotB[pos] = (T)Bz[c];
+    const T e = (T)Ey[c], b = (T)Bz[c];
+    slotE[pos] = e;
+    slotB[pos] = b;
+    if (mirror) {
+      slotE[pos + mirror] = e;
+      slotB[pos + mirror] = b;
+    }
   }
 }
 
-// x -> (cell, frac) with x = (cell + frac) dx, frac in [0, 1); p rounded to FP32.
-__global__ void to_mixed_kernel(const double* x, const double* px, const double* py,
-                                const double* pz, int32_t* cell, float* frac, float* fpx,
-                                float* fpy, float* fpz, double inv_dx, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    double s = x[i] * inv_dx;
-    double fl = floor(s);
-    double fr = s - fl;
-    float f = (float)fr;
-    if (f >= 1.0f) { f = 0.0f; fl += 1.0; }
-    cell[i] = (int32_t)fl;
-    frac[i] = f;
-    fpx[i] = (float)px[i];
-    fpy[i] = (float)py[i];
-    fpz[i] = (float)pz[i];
-  }
-}
-
-__global__ void from_mixed_kernel(const int32_t* cell, const float* frac, const float* fpx,
-                                  const float* fpy, const float* fpz, double* x, double* px,
-                                  double* py, double* pz, double dx, int64_t n) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    if (x) x[i] = ((double)cell[i] + (double)frac[i]) * dx;
-    if (px) px[i] = (double)fpx[i];
-    if (py) py[i] = (double)fpy[i];
-    if (pz) pz[i] = (double)fpz[i];
-  }
-}
-
-cudaError_t pic::launch_to_mixed(const double* x, const double* px, const double* py,
-                                 const double* pz, int32_t* cell, float* frac, float* fpx,
-                                 float* fpy, float* fpz, double inv_dx, int64_t n, cudaStream_t s) {
-  const int64_t want = (n + 255) / 256;
-  to_mixed_kernel<<<(int)(want < 152 * 16 ? (want > 0 ? want : 1) : 152 * 16), 256, 0, s>>>(
-      x, px, py, pz, cell, frac, fpx, fpy, fpz, inv_dx, n);
-  return cudaGetLastError();
-}
-
-cudaError_t pic::launch_from_mixed(const int32_t* cell, const float* frac, const float* fpx,
-                                   const float* fpy, const float* fpz, double* x, double* px,
-                                   double* py, double* pz, double dx, int64_t n, cudaStream_t s) {
-  const int64_t want = (n + 255) / 256;
-  from_mixed_kernel<<<(int)(want < 152 * 16 ? (want > 0 ? want : 1) : 152 * 16), 256, 0, s>>>(
-      cell, frac, fpx, fpy, fpz, x, px, py, pz, dx, n);
-  return cudaGetLastError();
+static MixedStore mixed_store(const pic_ctx* c, int64_t off = 0) {
+  return MixedStore{c->cell + off, c->frac + off, c->fpx + off, c->fpy + off, c->fpz + off};
 }
 
 static int grid_for(const pic_ctx* c, int64_t n) {
@@ -419,10 +382,8 @@ extern "C" int pic_particles_write(pic_ctx* c, const double* x, const double* px
   }
   const double inv_dx = 1.0 / c->prm.dx;
   if (where == PIC_DEVICE) {
-    to_mixed_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(x, px, py, pz, c->cell, c->frac, c->fpx,
-                                                            c->fpy, c->fpz, inv_dx, n);
+    CUDA_TRY(c, launch_to_mixed(x, px, py, pz, mixed_store(c), inv_dx, n, c->stream));
     ++c->launches;
-    CUDA_TRY(c, cudaGetLastError());
     return PIC_OK;
   }
   const int64_t chunk = c->staging_len / 4;
@@ -433,11 +394,9 @@ extern "C" int pic_particles_write(pic_ctx* c, const double* x, const double* px
     CUDA_TRY(c, cudaMemcpyAsync(s + chunk, px + off, cnt * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(s + 2 * chunk, py + off, cnt * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(c, cudaMemcpyAsync(s + 3 * chunk, pz + off, cnt * 8, cudaMemcpyHostToDevice, c->stream));
-    to_mixed_kernel<<<grid_for(c, cnt), 256, 0, c->stream>>>(
-        s, s + chunk, s + 2 * chunk, s + 3 * chunk, c->cell + off, c->frac + off, c->fpx + off,
-        c->fpy + off, c->fpz + off, inv_dx, cnt);
+    CUDA_TRY(c, launch_to_mixed(s, s + chunk, s + 2 * chunk, s + 3 * chunk, mixed_store(c, off), inv_dx, cnt,
+                                c->stream));
     ++c->launches;
-    CUDA_TRY(c, cudaGetLastError());
   }
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   return PIC_OK;
@@ -460,20 +419,16 @@ extern "C" int pic_particles_read(pic_ctx* c, double* x, double* px, double* py,
       if (dst[q])
         CUDA_TRY(c, cudaMemcpyAsync(dst[q], src[q], (size_t)n * 8, kind_out(where), c->stream));
   } else if (where == PIC_DEVICE) {
-    from_mixed_kernel<<<grid_for(c, n), 256, 0, c->stream>>>(c->cell, c->frac, c->fpx, c->fpy,
-                                                              c->fpz, x, px, py, pz, c->prm.dx, n);
+    CUDA_TRY(c, launch_from_mixed(mixed_store(c), x, px, py, pz, c->prm.dx, n, c->stream));
     ++c->launches;
-    CUDA_TRY(c, cudaGetLastError());
   } else {
     const int64_t chunk = c->staging_len / 4;
     double* s = c->staging;
     for (int64_t off = 0; off < n; off += chunk) {
       const int64_t cnt = (n - off < chunk) ? n - off : chunk;
-      from_mixed_kernel<<<grid_for(c, cnt), 256, 0, c->stream>>>(
-          c->cell + off, c->frac + off, c->fpx + off, c->fpy + off, c->fpz + off, s, s + chunk,
-          s + 2 * chunk, s + 3 * chunk, c->prm.dx, cnt);
+      CUDA_TRY(c, launch_from_mixed(mixed_store(c, off), s, s + chunk, s + 2 * chunk, s + 3 * chunk,
+                                    c->prm.dx, cnt, c->stream));
       ++c->launches;
-      CUDA_TRY(c, cudaGetLastError());
       double* dst[4] = {x, px, py, pz};
       for (int q = 0; q < 4; ++q)
         if (dst[q])
@@ -513,19 +468,11 @@ extern "C" int pic_fields_upload(pic_ctx* c, int64_t level, int64_t i0, const do
   if (c->prm.precision == PIC_FP64) {
     double* sE = (double*)c->ringE + (int64_t)slot * W;
     double* sB = (double*)c->ringB + (int64_t)slot * W;
-    scatter_level_kernel<double><<<blocks, 256, 0, c->stream>>>(sE, sB, e, b, i0, W, nullptr, 0);
+    scatter_level_kernel<double><<<blocks, 256, 0, c->stream>>>(sE, sB, e, b, i0, W, 0, nullptr, 0);
   } else {
-    for (int copy = 0; copy < 2; ++copy) {
-      float* sE = (float*)c->ringE + ((int64_t)slot + (int64_t)copy * c->R) * W;
-      float* sB = (float*)c->ringB + ((int64_t)slot + (int64_t)copy * c->R) * W;
-      scatter_level_kernel<float><<<blocks, 256, 0, c->stream>>>(
-          sE, sB, e, b, i0, W, copy == 0 ? c->dslot_i0 : nullptr, slot);
-      ++c->launches;
-    }
-    CUDA_TRY(c, cudaGetLastError());
-    c->slot_level[slot] = level;
-    c->slot_i0[slot] = i0;
-    return PIC_OK;
+    float* sE = (float*)c->ringE + (int64_t)slot * W;
+    float* sB = (float*)c->ringB + (int64_t)slot * W;
+    scatter_level_kernel<float><<<blocks, 256, 0, c->stream>>>(sE, sB, e, b, i0, W, c->R * W, c->dslot_i0, slot);
   }
   ++c->launches;
   CUDA_TRY(c, cudaGetLastError());

@@ -181,6 +181,7 @@ struct EnsDev {
   const float* ringE;  // mirrored ring of this ensemble (2R slots x W)
   const float* ringB;
   const int64_t* slot_i0;  // [R] window origin of each ring slot
+  double dx, inv_dx64;     // the cell and its reciprocal in FP64 (loading and reading particles)
   int64_t first, count;    // particle range in the concatenated store
   int64_t chunk_first;     // index of its first stream chunk
 };
@@ -233,12 +234,24 @@ int batch_max_blocks_per_sm(int order);
 cudaError_t launch_batch_scatter(const EnsDev* ens, int32_t n_ens, int64_t slot, int64_t R,
                                  int64_t W, const double* Ey, const double* Bz, const int64_t* i0,
                                  int64_t* slot_i0_all, cudaStream_t s);
+// The mixed form's particle arrays (momenta and position) from some particle on.
+struct MixedStore {
+  int32_t* cell;
+  float *frac, *px, *py, *pz;
+};
+// FP64 arrays <-> the mixed layout (convert.cu): n particles of one problem; of
+// a batch, particles off .. off + n - 1 of the concatenated store, x .. pz (and
+// what they point to) starting at particle off.  Outputs of launch_from_*
+// may be NULL.
 cudaError_t launch_to_mixed(const double* x, const double* px, const double* py, const double* pz,
-                            int32_t* cell, float* frac, float* fpx, float* fpy, float* fpz,
-                            double inv_dx, int64_t n, cudaStream_t s);
-cudaError_t launch_from_mixed(const int32_t* cell, const float* frac, const float* fpx,
-                              const float* fpy, const float* fpz, double* x, double* px, double* py,
-                              double* pz, double dx, int64_t n, cudaStream_t s);
+                            const MixedStore& m, double inv_dx, int64_t n, cudaStream_t s);
+cudaError_t launch_from_mixed(const MixedStore& m, double* x, double* px, double* py, double* pz,
+                              double dx, int64_t n, cudaStream_t s);
+cudaError_t launch_to_mixed_batch(const double* x, const double* px, const double* py, const double* pz,
+                                  const MixedStore& m, const EnsDev* ens, int32_t n_ens, int64_t off,
+                                  int64_t n, cudaStream_t s);
+cudaError_t launch_from_mixed_batch(const MixedStore& m, double* x, double* px, double* py, double* pz,
+                                    const EnsDev* ens, int32_t n_ens, int64_t n, cudaStream_t s);
 
 // Launchers (return cudaError_t of the launch).
 cudaError_t build_wtab_f64(double* wtab, int order, int k_max, int field_time, cudaStream_t s);
