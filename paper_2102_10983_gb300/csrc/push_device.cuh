@@ -318,6 +318,33 @@ __device__ __forceinline__ void table_coefs(const float* coef, int g, int32_t a0
   }
 }
 
+// One node of table_coefs / to_monomial (the same values).
+template <int P>
+__device__ __forceinline__ void table_coef(const float* coef, int g, int32_t a0, float* c0) {
+  const float* r0 = coef + (int64_t)a0 * (2 * (P + 1)) + g * (P + 1);
+  if constexpr (P == 3) {
+    const float4 v0 = __ldg(reinterpret_cast<const float4*>(r0));
+    c0[0] = v0.x; c0[1] = v0.y; c0[2] = v0.z; c0[3] = v0.w;
+  } else {
+#pragma unroll
+    for (int q = 0; q <= P; ++q) c0[q] = __ldg(r0 + q);
+  }
+}
+template <int P, class LV>
+__device__ __forceinline__ void to_monomial1(const LV& lv, int32_t a0,
+                                             const float (&M)[kMaxOrder + 1][kMaxOrder + 1], float* c0) {
+  float v0[P + 1];
+#pragma unroll
+  for (int l = 0; l <= P; ++l) v0[l] = __ldg(lv.at(l) + a0);
+#pragma unroll
+  for (int q = 0; q <= P; ++q) {
+    float x0 = __fmul_rn(v0[0], M[0][q]);
+#pragma unroll
+    for (int l = 1; l <= P; ++l) x0 = __fmaf_rn(v0[l], M[l][q], x0);
+    c0[q] = x0;
+  }
+}
+
 template <int P>
 __device__ __forceinline__ float horner(const float* c, float u) {
   float f = c[P];
@@ -326,22 +353,191 @@ __device__ __forceinline__ float horner(const float* c, float u) {
   return f;
 }
 
-// m = 1 takes a straight path with the tabulated weights and the criterion's
-// B_z (b0; unused for m > 1).  For m > 1 the
-// temporal interpolant at each tent node is a polynomial of degree p in
-// u = theta - 1; its coefficients are formed when the node index changes (an
-// electron moves a small fraction of a cell per sub-step) and each sub-step
-// evaluates it by Horner's rule: p FMAs per node, nothing waits on memory.
-// The floors of the offset on both grids are cached with the coefficients, so
-// while the nodes stay the same a sub-step's tent weights are one subtraction
-// each after the new offset (the same bits as a fresh floor).  The
-// coefficients come from
-// the step's node table (TABLE: F.coef, written by the half-step kernel), else
-// from the levels.
+// The m = 1 push: tabulated weights, the criterion's B_z (b0: same weights,
+// same nodes).
+template <int P, bool RING>
+__device__ __forceinline__ bool push_once_f32(const StepFields<P, RING>& F, const float* wtab, int32_t mask,
+                                              float dt, float inv_dx, float qm, int k_prev, float b0,
+                                              MixedState& s) {
+  const float* wr = wtab + wrow(0, 1) * (2 * (P + 1));
+  int32_t je, jb;
+  float we, wb;
+  if (!tent_coords(s.cell, s.frac, F.lo, F.hi, je, we, jb, wb)) return false;
+  const float ey = gather_f32<P>(F.E, wr, je, we, mask);
+  const float hp = __fmul_rn(0.5f, __fadd_rn(pow4_down(dt, k_prev), dt));
+  boris_f32(ey, b0, hp, __fmul_rn(dt, inv_dx), qm, s);
+  return true;
+}
+
+// One Boris sub-step as boris_f32 takes it (same operations, same bits) with
+// what the sub-steps of a cycle share carried along: qmh = q/m hp/2 and g2 = 1 +
+// p_x^2 + p_z^2 (the last sub-step's g2n is the next one's g2xz).
+__device__ __forceinline__ void boris_chain_f32(float ey, float bz, float qmh, float hx, MixedState& s,
+                                                float& g2) {
+  const float dpy = __fmul_rn(qmh, ey);
+  const float mx = s.ux, mz = s.uz;
+  const float my = __fadd_rn(s.uy, dpy);
+  const float inv_gn = rsqrt_sfu(__fmaf_rn(my, my, g2));
+  const float tz = __fmul_rn(__fmul_rn(qmh, bz), inv_gn);
+  const float ppx = __fmaf_rn(my, tz, mx);
+  const float ppy = __fmaf_rn(-mx, tz, my);
+  const float sz = __fmul_rn(__fmul_rn(2.0f, tz), rcp_sfu(__fmaf_rn(tz, tz, 1.0f)));
+  s.ux = __fmaf_rn(ppy, sz, mx);
+  s.uy = __fadd_rn(__fmaf_rn(-ppx, sz, my), dpy);
+  g2 = __fadd_rn(1.0f, __fmaf_rn(mz, mz, __fmul_rn(s.ux, s.ux)));
+  const float inv_g = rsqrt_sfu(__fmaf_rn(s.uy, s.uy, g2));
+  s.frac = __fmaf_rn(hx, __fmul_rn(s.ux, inv_g), s.frac);
+}
+
+// Three consecutive nodes' coefficients on one grid (g = 0: E, 1: B), lowest
+// node a: from the step's node table (TABLE) or formed from the levels.
+template <int P, bool RING, bool TABLE>
+__device__ __forceinline__ void three_nodes(const StepFields<P, RING>& F, int g, int32_t a, int32_t mask,
+                                            const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1],
+                                            float (&c)[3][P + 1]) {
+  if constexpr (TABLE) {
+    table_coefs<P>(F.coef, g, a & mask, (a + 1) & mask, c[0], c[1]);
+    table_coef<P>(F.coef, g, (a + 2) & mask, c[2]);
+  } else {
+    const Levels<P, RING>& lv = g ? F.B : F.E;
+    to_monomial<P>(lv, a & mask, (a + 1) & mask, mono[g], c[0], c[1]);
+    to_monomial1<P>(lv, (a + 2) & mask, mono[g], c[2]);
+  }
+}
+// Both rounded weights in [+0, 1): then the offsets' differences from their
+// nodes are exact and those nodes are the floors (a NaN or a negative weight
+// fails the unsigned test).
+__device__ __forceinline__ bool in_cell(float we, float wb) {
+  return __float_as_uint(we) < 0x3f800000u && __float_as_uint(wb) < 0x3f800000u;
+}
+
+// What the sub-steps of a cycle carry: the state, qmh = q/m hp/2, g2 = 1 + p_x^2
+// + p_z^2 and the sub-step's u = theta - 1.
+struct CycleState {
+  MixedState s;
+  float qmh, g2, u;
+};
+
+// n sub-steps, the electron's nodes looked at in each: any way it moves.  False
+// if it left the window.
+template <int P, bool RING, bool TABLE>
+__device__ __forceinline__ bool cycle_any(const StepFields<P, RING>& F, int32_t mask,
+                                          const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1], int n,
+                                          float hx, float qmh_next, float inv_m, CycleState& c) {
+  float ce[3][P + 1], cb[3][P + 1];  // monomial coefficients per node
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int q = 0; q <= P; ++q) ce[a][q] = cb[a][q] = 0.f;
+  // floors of the offset on the two grids at the lowest kept nodes (NaN: none
+  // yet), and the offset from which E's upper pair would leave the window
+  float fe = __int_as_float(0x7fc00000), fb = fe, fe_end = fe;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    const float f = c.s.frac;
+    const float fbm = __fsub_rn(f, 0.5f);
+    // floors: the kept node's or the next one's (whole numbers: exact)
+    const float fe1 = __fadd_rn(fe, 1.0f), fb1 = __fadd_rn(fb, 1.0f);
+    bool up_e = f >= fe1, up_b = fbm >= fb1;
+    float we = __fsub_rn(f, up_e ? fe1 : fe), wb = __fsub_rn(fbm, up_b ? fb1 : fb);
+    if (!(in_cell(we, wb) && f < fe_end)) {
+      int32_t je, jb;
+      if (!tent_coords(c.s.cell, f, F.lo, F.hi, je, we, jb, wb)) return false;
+      fe = floorf(f);
+      fb = floorf(fbm);
+      up_e = up_b = false;
+      // (past 2^22 cells a floor plus one may not be exact)
+      fe_end = je + 1 < F.hi && fabsf(f) < 0x1p22f ? __int_as_float(0x7f800000) : __fadd_rn(fe, 1.0f);
+      three_nodes<P, RING, TABLE>(F, 0, je, mask, mono, ce);
+      three_nodes<P, RING, TABLE>(F, 1, jb, mask, mono, cb);
+    }
+    const float e0 = horner<P>(ce[0], c.u), e1 = horner<P>(ce[1], c.u), e2 = horner<P>(ce[2], c.u);
+    const float b1 = horner<P>(cb[0], c.u), b2 = horner<P>(cb[1], c.u), b3 = horner<P>(cb[2], c.u);
+    const float el = up_e ? e1 : e0, eh = up_e ? e2 : e1;
+    const float bl = up_b ? b2 : b1, bh = up_b ? b3 : b2;
+    boris_chain_f32(__fmaf_rn(we, __fsub_rn(eh, el), el), __fmaf_rn(wb, __fsub_rn(bh, bl), bl), c.qmh, hx,
+                    c.s, c.g2);
+    c.qmh = qmh_next;
+    c.u = __fadd_rn(c.u, inv_m);
+  }
+  return true;
+}
+
+// n sub-steps without a branch among them, for an electron that stays within
+// two cells: the kept nodes are base .. base + 2 with base the floor of its
+// offset less `back` on each grid.  False (c to be ignored) if a weight left
+// its range, or near the window's ends.
+template <int P, bool RING, bool TABLE>
+__device__ __forceinline__ bool cycle_near(const StepFields<P, RING>& F, int32_t mask,
+                                           const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1], int n, float back,
+                                           float hx, float qmh_next, float inv_m, CycleState& c) {
+  const float f0 = c.s.frac;
+  const float fe = floorf(__fsub_rn(f0, back)), fb = floorf(__fsub_rn(__fsub_rn(f0, 0.5f), back));
+  const float fe1 = __fadd_rn(fe, 1.0f), fb1 = __fadd_rn(fb, 1.0f);
+  if (!(fabsf(f0) < 0x1p22f)) return false;
+  const int32_t je = c.s.cell + (int32_t)fe, jb = c.s.cell + (int32_t)fb;
+  if (jb < F.lo || je + 1 >= F.hi) return false;  // (jb <= je)
+  float ce[3][P + 1], cb[3][P + 1];
+  three_nodes<P, RING, TABLE>(F, 0, je, mask, mono, ce);
+  three_nodes<P, RING, TABLE>(F, 1, jb, mask, mono, cb);
+  float e0, e1, de0, de1, b0, b1, db0, db1;  // lower and upper pair: value, step to the next node
+  auto values = [&](float u) {
+    e0 = horner<P>(ce[0], u);
+    e1 = horner<P>(ce[1], u);
+    de0 = __fsub_rn(e1, e0);
+    de1 = __fsub_rn(horner<P>(ce[2], u), e1);
+    b0 = horner<P>(cb[0], u);
+    b1 = horner<P>(cb[1], u);
+    db0 = __fsub_rn(b1, b0);
+    db1 = __fsub_rn(horner<P>(cb[2], u), b1);
+  };
+  values(c.u);
+  bool held = true;
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    const float f = c.s.frac;
+    const float fbm = __fsub_rn(f, 0.5f);
+    const bool up_e = f >= fe1, up_b = fbm >= fb1;
+    const float we = __fsub_rn(f, up_e ? fe1 : fe), wb = __fsub_rn(fbm, up_b ? fb1 : fb);
+    const float ey = __fmaf_rn(we, up_e ? de1 : de0, up_e ? e1 : e0);
+    const float bz = __fmaf_rn(wb, up_b ? db1 : db0, up_b ? b1 : b0);
+    held = held && in_cell(we, wb);
+    c.u = __fadd_rn(c.u, inv_m);
+    values(c.u);
+    boris_chain_f32(ey, bz, c.qmh, hx, c.s, c.g2);
+    c.qmh = qmh_next;
+  }
+  return held;
+}
+
+// Sub-steps j0+1 .. j1 of the m = 4^k of one macro step (j1 = -1: all of them;
+// k >= 1 unless a whole m = 1 step): a sub-cycle can stop after any sub-step
+// and resume from the state it left (offset not yet normalised) with the same
+// bits as an uninterrupted one.
 //
-// Sub-steps j0+1 .. j1 of the m (j1 = -1: all of them): a sub-cycle can stop
-// after any sub-step and resume from the state it left (offset not yet
-// normalised) with the same bits as an uninterrupted one.
+// The temporal interpolant at each tent node is a polynomial of degree p in u =
+// theta - 1, evaluated by Horner's rule (p FMAs per node).  Each grid keeps
+// three nodes' coefficients: an electron moves less than a cell per macro step
+// (c dt < dx), so the nodes it needs change at most once within a sub-cycle,
+// and then it takes the other pair of the three: a select instead of a load.
+// (With two nodes kept, every lane's crossing made its warp wait about 600
+// clocks for L2 at a sub-step of its own.)
+//
+// A long sub-cycle is a serial chain, and the longest one of a call bounds it
+// whatever else the GPU does (1,024 sub-steps at k = 5).  Its dependent
+// operations take 120 clocks per sub-step; a branch that looks at the nodes in
+// each, and the nodes' values formed after it, made that 200.  So k >= kNearMin
+// runs without a branch (cycle_near), the next sub-step's values formed in the
+// shadow of this one's push: 153.  k >= kHalfMin goes in stretches of at most
+// half a macro step, half a cell, from the middle of the kept nodes, which an
+// electron cannot leave either way; k = 2 in one stretch, the nodes ahead of
+// the electron kept (its 16 sub-steps would not pay for a second load).  What
+// does not fit (a turn back, c dt > dx, the window's ends) takes cycle_any, as
+// does k = 1, whose four sub-steps gain nothing.  Per step, two nodes ->
+// three -> with stretches: 300 electrons at the front 119 -> 117 -> 95 us,
+// 16.8M electrons 249 -> 219 -> 199 us, 1,000,003 at fifth order 120 -> 118 ->
+// 90 us.
+constexpr int kNearMin = 2, kHalfMin = 3;
 template <int P, bool RING, bool TABLE = false>
 __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const float* wtab,
                                              int32_t mask, float dt, float inv_dx, float qm,
@@ -349,69 +545,40 @@ __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const
                                              const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1],
                                              int k, int k_prev, float b0, MixedState& s,
                                              int j0 = 0, int j1 = -1) {
-  constexpr int stride = 2 * (P + 1);
+  if (k == 0) return push_once_f32<P, RING>(F, wtab, mask, dt, inv_dx, qm, k_prev, b0, s);
   const float h = pow4_down(dt, k);
-  const float h_old = pow4_down(dt, k_prev);
   const float hx = __fmul_rn(h, inv_dx);
-  float hp = j0 == 0 ? __fmul_rn(0.5f, __fadd_rn(h_old, h)) : h;
-  if (k == 0) {
-    const float* wr = wtab + wrow(0, 1) * stride;
-    int32_t je, jb;
-    float we, wb;
-    if (!tent_coords(s.cell, s.frac, F.lo, F.hi, je, we, jb, wb)) return false;
-    const float ey = gather_f32<P>(F.E, wr, je, we, mask);
-    boris_f32(ey, b0, hp, hx, qm, s);  // b0: the criterion's B_z (same weights, same nodes)
-    return true;
-  }
+  const float qmh_next = __fmul_rn(qm, __fmul_rn(0.5f, h));
   const int m = 1 << (2 * k);
   const float inv_m = pow4_down(1.0f, k);
-  // u_j = theta_j - 1, exact in FP32 for m <= 4^7
-  const float u1 = field_time == 0 ? -0.5f : __fsub_rn(__fmul_rn(0.5f, inv_m), 1.0f);
-  int32_t ce = INT_MIN, cb = INT_MIN;
-  float ce0[P + 1], ce1[P + 1], cb0[P + 1], cb1[P + 1];  // monomial coefficients per node
-#pragma unroll
-  for (int q = 0; q <= P; ++q) ce0[q] = ce1[q] = cb0[q] = cb1[q] = 0.f;
-  // floors of the offset on the two grids at the cached nodes (NaN: none yet)
-  float fe = __int_as_float(0x7fc00000), fb = fe;
   const int j_end = j1 < 0 ? m : j1;
-  // u_j = u_1 + (j-1)/m: every partial sum is a multiple of 1/m in [-1, 1],
-  // exact in FP32, so the running sum has the bits of the direct formula
-  float u = __fmaf_rn((float)j0, inv_m, u1);
-  for (int j = j0 + 1; j <= j_end; ++j) {
-    const float f = s.frac;
-    const float fbm = __fsub_rn(f, 0.5f);
-    float we = __fsub_rn(f, fe), wb = __fsub_rn(fbm, fb);
-    // cached nodes still hold iff both rounded weights lie in [+0, 1): then
-    // f - fe and fbm - fb are exact and fe, fb are the floors (a NaN or a
-    // negative weight fails the unsigned test)
-    if (!(__float_as_uint(we) < 0x3f800000u && __float_as_uint(wb) < 0x3f800000u)) {
-      int32_t je, jb;
-      if (!tent_coords(s.cell, f, F.lo, F.hi, je, we, jb, wb)) return false;
-      fe = floorf(f);
-      fb = floorf(fbm);
-      if (je != ce) {
-        ce = je;
-        if constexpr (TABLE)
-          table_coefs<P>(F.coef, 0, je & mask, (je + 1) & mask, ce0, ce1);
-        else
-          to_monomial<P>(F.E, je & mask, (je + 1) & mask, mono[0], ce0, ce1);
+  // u_j = theta_j - 1 = u_1 + (j-1)/m: every partial sum is a multiple of 1/m
+  // in [-1, 1], exact in FP32 (m <= 4^7), so the running sum has the bits of
+  // the direct formula
+  const float u1 = field_time == 0 ? -0.5f : __fsub_rn(__fmul_rn(0.5f, inv_m), 1.0f);
+  const float hp = j0 == 0 ? __fmul_rn(0.5f, __fadd_rn(pow4_down(dt, k_prev), h)) : h;
+  CycleState c{s, __fmul_rn(qm, __fmul_rn(0.5f, hp)),
+               __fadd_rn(1.0f, __fmaf_rn(s.uz, s.uz, __fmul_rn(s.ux, s.ux))), __fmaf_rn((float)j0, inv_m, u1)};
+  bool ok = true;
+#pragma unroll 1
+  for (int j = j0; j < j_end && ok;) {
+    int n = j_end - j;
+    bool done = false;
+    if (k >= kNearMin) {
+      float back = c.s.ux < 0.f ? 1.0f : 0.0f;
+      if (k >= kHalfMin) {
+        n = min(n, m >> 1);
+        back = 0.5f;
       }
-      if (jb != cb) {
-        cb = jb;
-        if constexpr (TABLE)
-          table_coefs<P>(F.coef, 1, jb & mask, (jb + 1) & mask, cb0, cb1);
-        else
-          to_monomial<P>(F.B, jb & mask, (jb + 1) & mask, mono[1], cb0, cb1);
-      }
+      const CycleState before = c;
+      done = cycle_near<P, RING, TABLE>(F, mask, mono, n, back, hx, qmh_next, inv_m, c);
+      if (!done) c = before;
     }
-    const float fe0 = horner<P>(ce0, u), fe1 = horner<P>(ce1, u);
-    const float fb0 = horner<P>(cb0, u), fb1 = horner<P>(cb1, u);
-    boris_f32(__fmaf_rn(we, __fsub_rn(fe1, fe0), fe0), __fmaf_rn(wb, __fsub_rn(fb1, fb0), fb0), hp,
-              hx, qm, s);
-    hp = h;
-    u = __fadd_rn(u, inv_m);
+    if (!done) ok = cycle_any<P, RING, TABLE>(F, mask, mono, n, hx, qmh_next, inv_m, c);
+    j += n;
   }
-  return true;
+  s = c.s;
+  return ok;
 }
 
 // The node-table form of subcycle_f32 behind one call site.  With
@@ -792,7 +959,7 @@ constexpr int kChunk = PIC_CHUNK;    // particles per stream item (kChunk / kTil
 constexpr int kStages = PIC_STAGES;  // staged tiles per warp (one in flight while one is pushed)
 static_assert(kChunk % kTile == 0 && kTile % 64 == 0, "a stream item is whole tiles of whole rounds");
 constexpr int kStashK = kDeferMin - 1;
-constexpr int kStashCap = 64;
+constexpr int kStashCap = 96;  // up to 31 left over and a round's 64
 constexpr uint8_t kParity = 0x08;
 constexpr uint8_t kDeferMask = 0x70;
 // Deferred-k field value 1 (a k no sub-cycle is deferred with): the particle
@@ -819,40 +986,36 @@ __device__ __forceinline__ void enqueue(const PushArgsMixed& a, int key, int32_t
   }
 }
 
-// A warp's stash of particles waiting for a short sub-cycle of one k.
-#ifdef PIC_STASH_INDEX_ONLY
-// (index only: the drain reads the state back from global memory, leaving
-// more of the SM's on-chip memory to the L1 cache)
+// A warp's stash of particles waiting for a short sub-cycle of one k: two wide
+// words and a byte per entry, so that parking a particle is three stores.
 struct Stash {
-  int32_t idx[kStashCap];
+  float4 a[kStashCap];  // cell (bits), frac, ux, uy
+  float2 b[kStashCap];  // uz, particle index (bits)
   uint8_t kp[kStashCap];
 };
-#else
-struct Stash {
-  int32_t idx[kStashCap];
-  int32_t cell[kStashCap];
-  float frac[kStashCap], ux[kStashCap], uy[kStashCap], uz[kStashCap];
-  uint8_t kp[kStashCap];
-};
-#endif
+static_assert(sizeof(Stash) % 16 == 0, "stashes follow each other in shared memory");
 
-// Push the first `cnt` (<= 32) stashed particles, one per lane, with 4^k
-// sub-steps each; then move entries [cnt, n) to the front.  Warp-collective.
-// Stash entry kp: k_prev in bits 0-2, bit 3 set for a predicted-queue particle
-// (which stays in that queue).
+__device__ __forceinline__ void stash_put(Stash& S, int pos, int32_t i, const MixedState& s, uint8_t kp) {
+  S.a[pos] = make_float4(__int_as_float(s.cell), s.frac, s.ux, s.uy);
+  S.b[pos] = make_float2(s.uz, __int_as_float(i));
+  S.kp[pos] = kp;
+}
+
+// Push the last min(n, 32) stashed particles, one per lane, with 4^k sub-steps
+// each.  Warp-collective.  Stash entry kp: k_prev in bits 0-2, bit 3 set for a
+// predicted-queue particle (which stays in that queue).
 template <int P, bool RING>
 __device__ __forceinline__ void stash_drain(const PushArgsMixed& a, const StepFields<P, RING>& F,
-                                            Stash& S, int k, int& n, int cnt,
-                                            unsigned long long* sh) {
+                                            const Stash& S, int k, int& n, unsigned long long* sh) {
   const int lane = threadIdx.x & 31;
+  const int cnt = n < 32 ? n : 32;
   if (lane < cnt) {
-    const int32_t i = S.idx[lane];
-#ifdef PIC_STASH_INDEX_ONLY
-    MixedState s = load_state(a, i);
-#else
-    MixedState s = {S.cell[lane], S.frac[lane], S.ux[lane], S.uy[lane], S.uz[lane]};
-#endif
-    const uint8_t kp = S.kp[lane];
+    const int q = n - cnt + lane;
+    const float4 va = S.a[q];
+    const float2 vb = S.b[q];
+    const uint8_t kp = S.kp[q];
+    const int32_t i = __float_as_int(vb.y);
+    MixedState s = {__float_as_int(va.x), va.y, va.z, va.w, vb.x};
     const bool ok = subcycle_site<P, RING, RING>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm,
                                                  a.field_time, a.mono, k, kp & 7, 0.f, s);
     normalize(s);
@@ -862,21 +1025,7 @@ __device__ __forceinline__ void stash_drain(const PushArgsMixed& a, const StepFi
     if (!ok) atomicAdd(&sh[11], 1ull);
   }
   __syncwarp();
-  const int rest = n - cnt;
-  if (lane < rest) {
-    const int q = cnt + lane;
-    S.idx[lane] = S.idx[q];
-#ifndef PIC_STASH_INDEX_ONLY
-    S.cell[lane] = S.cell[q];
-    S.frac[lane] = S.frac[q];
-    S.ux[lane] = S.ux[q];
-    S.uy[lane] = S.uy[q];
-    S.uz[lane] = S.uz[q];
-#endif
-    S.kp[lane] = S.kp[q];
-  }
-  __syncwarp();
-  n = rest;
+  n -= cnt;
 }
 
 // Deferred item: particle i is in a step before this launch's (a long

@@ -405,44 +405,40 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
     for (int r = 0; r < kStashK; ++r)
       if (r == q) stash_n[r] = v;
   };
-  // push 32 particles of every stash that holds 32 or more (all = true: every
-  // parked particle); one call site of the sub-cycle per call site of this
+  // push 32 particles at a time of every stash that holds 32 or more (all =
+  // true: every parked particle); one call site of the sub-cycle per call site
+  // of this
   auto drain = [&](bool all) {
 #pragma unroll 1
     for (int q = 0; q < kStashK; ++q) {
       int n = stash_count(q);
-      const int cnt = all ? n : (n >= 32 ? 32 : 0);
-      if (cnt > 0) {
-        stash_drain<P, RING>(a, F, my_stash[q], q + 1, n, cnt, sh);
-        stash_set(q, n);
-      }
+      const int keep = all ? 0 : 31;
+      if (n <= keep) continue;
+#pragma unroll 1
+      while (n > keep) stash_drain<P, RING>(a, F, my_stash[q], q + 1, n, sh);
+      stash_set(q, n);
     }
   };
 
-  // park k = 1, 2 in the warp's stashes; push a stash when it holds 32
-  // (warp-collective; sk = 0: nothing to park)
-  auto park = [&](int sk, int32_t i, const MixedState& s, uint8_t kp) {
+  // park up to two particles per lane, i0 with k = k0 and i0 + 1 with k = k1
+  // (1 or 2; 0: nothing to park), in the warp's stashes of those k; push a
+  // stash when it holds 32 (warp-collective)
+  auto park = [&](int k0, int k1, int32_t i0, const MixedState& s0, const MixedState& s1, uint8_t kp0,
+                  uint8_t kp1) {
+    const unsigned lt = (1u << lane) - 1u;
+    int pos0 = 0, pos1 = 0;
     bool full = false;
 #pragma unroll
     for (int q = 0; q < kStashK; ++q) {
-      const unsigned m = __ballot_sync(0xffffffffu, sk == q + 1);
-      if (m == 0u) continue;
-      Stash& S = my_stash[q];
-      if (sk == q + 1) {
-        const int pos = stash_n[q] + __popc(m & ((1u << lane) - 1u));
-        S.idx[pos] = i;
-#ifndef PIC_STASH_INDEX_ONLY
-        S.cell[pos] = s.cell;
-        S.frac[pos] = s.frac;
-        S.ux[pos] = s.ux;
-        S.uy[pos] = s.uy;
-        S.uz[pos] = s.uz;
-#endif
-        S.kp[pos] = kp;
-      }
-      stash_n[q] += __popc(m);
+      const unsigned m0 = __ballot_sync(0xffffffffu, k0 == q + 1), m1 = __ballot_sync(0xffffffffu, k1 == q + 1);
+      const int n0 = stash_n[q], n1 = n0 + __popc(m0);
+      if (k0 == q + 1) pos0 = n0 + __popc(m0 & lt);
+      if (k1 == q + 1) pos1 = n1 + __popc(m1 & lt);
+      stash_n[q] = n1 + __popc(m1);
       full |= stash_n[q] >= 32;
     }
+    if (k0 > 0) stash_put(my_stash[k0 - 1], pos0, i0, s0, kp0);
+    if (k1 > 0) stash_put(my_stash[k1 - 1], pos1, i0 + 1, s1, kp1);
     __syncwarp();
     if (full) drain(false);
   };
@@ -459,6 +455,8 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
   const float qm_dt = __fmul_rn(a.qm_abs, a.dt);
   const float tp = __fmul_rn(2.0f, a.psi_max);
   const float tp2 = __fmul_rn(tp, tp);
+  // the largest k that the round itself settles: above it the cap or a deferral
+  const int k_short = a.k_max < kDeferMin - 1 ? a.k_max : kDeferMin - 1;
   auto stream_pair = [&](const Tile& T, bool staged, int r, uint32_t first) {
     const int q = r * 32 + lane;
     const uint32_t i = first + 2u * (uint32_t)q;
@@ -513,41 +511,55 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
     const float2 a2 = mul2(av, av);
     const float2 rhs =
         mul2(bc2(tp2), add2(bc2(1.0f), fma2(s.uz, s.uz, fma2(s.uy, s.uy, mul2(s.ux, s.ux)))));
-    bool push0 = mine0 && in0 && !(a2.x > rhs.x);
-    bool push1 = mine1 && in1 && !(a2.y > rhs.y);
-    tc.k0 += (push0 ? 1u : 0u) + (push1 ? 1u : 0u);
+    const bool big0 = a2.x > rhs.x, big1 = a2.y > rhs.y;
+    bool push0 = mine0 && in0 && !big0;
+    bool push1 = mine1 && in1 && !big1;
     const bool side = !__all_sync(0xffffffffu, (push0 || !mine0) && (push1 || !mine1));
-    int key0 = 0, key1 = 0, sk0 = 0, sk1 = 0;
-    if (side) {  // the rest of the criterion for the particles that do not take k = 0 at once
+    int k0 = 0, k1 = 0;  // k of the particles that sub-cycle
+    bool rare = false;
+    if (side) {
+      // the rest of the criterion's comparisons (psi_to_k): k = 1, 2, or more
+      const float2 r16 = mul2(rhs, bc2(16.0f)), r256 = mul2(r16, bc2(16.0f));
+      k0 = mine0 && in0 && big0 ? 1 + (a2.x > r16.x ? 1 : 0) + (a2.x > r256.x ? 1 : 0) : 0;
+      k1 = mine1 && in1 && big1 ? 1 + (a2.y > r16.y ? 1 : 0) + (a2.y > r256.y ? 1 : 0) : 0;
+      // long sub-cycles, caps below that and particles outside the window
+      rare = __any_sync(0xffffffffu, k0 > k_short || k1 > k_short || (mine0 && !in0) || (mine1 && !in1));
+      if (rare) {
 #pragma unroll 1
-      for (int e = 0; e < 2; ++e) {
-        const bool mine = e ? mine1 : mine0;
-        bool& push = e ? push1 : push0;
-        const bool inwin = e ? in1 : in0;
-        const uint8_t st = e ? st1 : st0;
-        const uint32_t ii = i + (uint32_t)e;
-        int& key = e ? key1 : key0;
-        int& sk = e ? sk1 : sk0;
-        if (!mine || push) continue;
-        if (!inwin) {
-          a.status[ii] = (uint8_t)(st | PIC_STATUS_LOST);
-          atomicAdd(&sh[11], 1ull);
-          continue;
-        }
-        bool capped;
-        const MixedState one = {0, 0.f, e ? s.ux.y : s.ux.x, e ? s.uy.y : s.uy.x, e ? s.uz.y : s.uz.x};
-        const int k = psi_to_k(e ? bz.y : bz.x, one, a.qm_abs, a.dt, a.psi_max, a.k_max, capped);
-        count_step(tc, sh, k, capped);
-        if (k == 0) {
-          push = true;  // capped at k_max = 0
-        } else if (k >= kDeferMin) {
-          defer_mark(a, ii, st & 7, k, a.step_cur);
-          key = k;
-        } else {
-          sk = k;
+        for (int e = 0; e < 2; ++e) {
+          int k = e ? k1 : k0;
+          bool push = false;
+          const uint32_t ii = i + (uint32_t)e;
+          const uint8_t st = e ? st1 : st0;
+          int key = 0;
+          if ((e ? mine1 : mine0) && !(e ? in1 : in0)) {
+            a.status[ii] = (uint8_t)(st | PIC_STATUS_LOST);
+            atomicAdd(&sh[11], 1ull);
+          } else if (k > k_short) {
+            bool capped;
+            const MixedState one = {0, 0.f, e ? s.ux.y : s.ux.x, e ? s.uy.y : s.uy.x, e ? s.uz.y : s.uz.x};
+            k = psi_to_k(e ? bz.y : bz.x, one, a.qm_abs, a.dt, a.psi_max, a.k_max, capped);
+            tc.capped += capped ? 1u : 0u;
+            if (k == 0) {
+              push = true;  // capped at k_max = 0
+            } else if (k >= kDeferMin) {
+              atomicAdd(&sh[k], 1ull);
+              defer_mark(a, ii, st & 7, k, a.step_cur);
+              key = k;
+              k = 0;
+            }
+          }
+          enqueue(a, key, (int32_t)ii);
+          k0 = e ? k0 : k;
+          k1 = e ? k : k1;
+          push0 |= !e && push;
+          push1 |= e && push;
         }
       }
+      tc.k1 += (k0 == 1 ? 1u : 0u) + (k1 == 1 ? 1u : 0u);
+      tc.k2 += (k0 == 2 ? 1u : 0u) + (k1 == 2 ? 1u : 0u);
     }
+    tc.k0 += (push0 ? 1u : 0u) + (push1 ? 1u : 0u);
     const MixedState p0 = {s.cell.x, s.frac.x, s.ux.x, s.uy.x, s.uz.x};  // as loaded, for the stash
     const MixedState p1 = {s.cell.y, s.frac.y, s.ux.y, s.uy.y, s.uz.y};
     if (push0 || push1) {
@@ -577,13 +589,7 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
         }
       }
     }
-    if (side) {
-#pragma unroll 1
-      for (int e = 0; e < 2; ++e) {
-        enqueue(a, e ? key1 : key0, (int32_t)(i + (uint32_t)e));
-        park(e ? sk1 : sk0, (int32_t)(i + (uint32_t)e), e ? p1 : p0, (uint8_t)((e ? st1 : st0) & 7));
-      }
-    }
+    if (side) park(k0, k1, (int32_t)i, p0, p1, (uint8_t)(st0 & 7), (uint8_t)(st1 & 7));
   };
 
   // Work items: a warp's first item is its warp-major index (no atomic: the
@@ -642,7 +648,7 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
     }
     if (heavy) heavy_particle<P, RING>(a, Fp, F, wcrit, i, tc, sh, key);
     enqueue(a, key, i);
-    park(sk, i, s, kp);
+    park(sk, 0, i, s, s, kp, kp);
     t = claim();
   }
 
