@@ -16,7 +16,8 @@ struct pic_mlp {
   float* G = nullptr;     // gradient
   float* M1 = nullptr;    // Adam first moment
   float* M2 = nullptr;    // Adam second moment
-  float* loss = nullptr;  // device scalar
+  float* part = nullptr;  // the gradient kernel's partial results per block
+  float* loss = nullptr;  // pinned host memory the device writes: a step's loss needs no copy
   int step = 0;
   int sm_count = 0;
   cudaStream_t stream = nullptr;
@@ -47,17 +48,20 @@ extern "C" int pic_mlp_create(uint64_t seed, void* stream, pic_mlp** out) {
   float** bufs[] = {&m->P, &m->G, &m->M1, &m->M2};
   for (float** b : bufs)
     if (e == cudaSuccess) e = cudaMalloc((void**)b, (size_t)np * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&m->loss, sizeof(float));
-  if (e != cudaSuccess) {
-    for (float** b : bufs)
-      if (*b) cudaFree(*b);
-    if (m->loss) cudaFree(m->loss);
-    delete m;
-    return mlp_fail(PIC_ENOMEM, "pic_mlp_create: device allocation failed");
-  }
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&m->sm_count, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&m->part, mlp_partial_floats(m->sm_count) * sizeof(float));
+  if (e == cudaSuccess) e = cudaHostAlloc((void**)&m->loss, sizeof(float), cudaHostAllocMapped);
+  if (e != cudaSuccess) {
+    for (float** b : bufs)
+      if (*b) cudaFree(*b);
+    if (m->part) cudaFree(m->part);
+    if (m->loss) cudaFreeHost(m->loss);
+    delete m;
+    cudaGetLastError();
+    return mlp_fail(PIC_ENOMEM, "pic_mlp_create: device allocation failed");
+  }
   std::vector<float> h(np, 0.f);
   uint64_t x = seed;
   auto next = [&]() {
@@ -81,7 +85,8 @@ extern "C" int pic_mlp_create(uint64_t seed, void* stream, pic_mlp** out) {
   if (e == cudaSuccess) e = cudaMemset(m->M2, 0, (size_t)np * sizeof(float));
   if (e != cudaSuccess) {
     for (float** b : bufs) cudaFree(*b);
-    cudaFree(m->loss);
+    cudaFree(m->part);
+    cudaFreeHost(m->loss);
     delete m;
     return mlp_fail(PIC_ECUDA, "pic_mlp_create: initialisation failed");
   }
@@ -96,7 +101,8 @@ extern "C" int pic_mlp_destroy(pic_mlp* m) {
   cudaFree(m->G);
   cudaFree(m->M1);
   cudaFree(m->M2);
-  cudaFree(m->loss);
+  cudaFree(m->part);
+  cudaFreeHost(m->loss);
   delete m;
   return PIC_OK;
 }
@@ -118,23 +124,16 @@ extern "C" int pic_mlp_params(pic_mlp* m, float* buf, int32_t set, int32_t where
   return PIC_OK;
 }
 
-static int grad_into(pic_mlp* m, const float* phi, const uint8_t* label, int64_t n) {
-  MLP_TRY(cudaMemsetAsync(m->G, 0, (size_t)mlp_param_count() * sizeof(float), m->stream));
-  MLP_TRY(cudaMemsetAsync(m->loss, 0, sizeof(float), m->stream));
-  MLP_TRY(launch_mlp_grad(m->P, phi, label, n, m->G, m->loss, m->sm_count, m->stream));
-  return PIC_OK;
-}
-
 extern "C" int pic_mlp_grad(pic_mlp* m, const float* phi, const uint8_t* label, int64_t n,
                             float* grad_out, float* loss_out) {
   if (!m || !phi || !label || n <= 0) return mlp_fail(PIC_EINVAL, "pic_mlp_grad: bad argument");
-  int rc = grad_into(m, phi, label, n);
-  if (rc != PIC_OK) return rc;
+  MLP_TRY(launch_mlp_grad(m->P, phi, label, n, m->part, m->sm_count, m->stream));
+  MLP_TRY(launch_mlp_finish(m->part, n, m->G, m->loss, nullptr, nullptr, nullptr, 0.f, 1, m->sm_count, m->stream));
   if (grad_out)
     MLP_TRY(cudaMemcpyAsync(grad_out, m->G, (size_t)mlp_param_count() * sizeof(float),
                             cudaMemcpyDeviceToHost, m->stream));
-  if (loss_out) MLP_TRY(cudaMemcpyAsync(loss_out, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
   MLP_TRY(cudaStreamSynchronize(m->stream));
+  if (loss_out) *loss_out = *(volatile float*)m->loss;
   return PIC_OK;
 }
 
@@ -142,13 +141,12 @@ extern "C" int pic_mlp_train_step(pic_mlp* m, const float* phi, const uint8_t* l
                                   float lr, float* loss_out) {
   if (!m || !phi || !label || n <= 0 || !(lr > 0))
     return mlp_fail(PIC_EINVAL, "pic_mlp_train_step: bad argument");
-  int rc = grad_into(m, phi, label, n);
-  if (rc != PIC_OK) return rc;
+  MLP_TRY(launch_mlp_grad(m->P, phi, label, n, m->part, m->sm_count, m->stream));
   m->step += 1;
-  MLP_TRY(launch_mlp_adam(m->P, m->G, m->M1, m->M2, lr, m->step, m->stream));
+  MLP_TRY(launch_mlp_finish(m->part, n, nullptr, m->loss, m->P, m->M1, m->M2, lr, m->step, m->sm_count, m->stream));
   if (loss_out) {
-    MLP_TRY(cudaMemcpyAsync(loss_out, m->loss, sizeof(float), cudaMemcpyDeviceToHost, m->stream));
     MLP_TRY(cudaStreamSynchronize(m->stream));
+    *loss_out = *(volatile float*)m->loss;
   }
   return PIC_OK;
 }

@@ -13,9 +13,9 @@
 // accumulate), 16 samples per warp tile.  A layer's accumulator fragments are,
 // after bias and ReLU, exactly the next layer's A fragments, so hidden
 // activations never leave registers in the forward pass.  Backward: dz on the
-// CUDA cores, dh2 = dz W3 and dh1 = da2 W2 on the tensor cores, weight
-// gradients (batch reductions) from BF16-rounded operands with FP32
-// accumulation in shared memory.  Inference (mlp_tc.cu) runs on tcgen05 with
+// CUDA cores, dh2 = dz W3 and dh1 = da2 W2 on the tensor cores, and so the
+// weight gradients (batch reductions) from BF16-rounded operands with FP32
+// accumulation.  Inference (mlp_tc.cu) runs on tcgen05 with
 // TMEM accumulators.
 #include <cuda_bf16.h>
 #include <math.h>
@@ -37,7 +37,6 @@ __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
-__device__ __forceinline__ float bf(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1) {
@@ -158,44 +157,77 @@ __device__ __forceinline__ void phi_fragment(const float* phi, int64_t n, int64_
   a1[3] = 0u;
 }
 
+// Per-block gradients, same packed order as the parameters.
+constexpr int kNParams = kH * kIn + kH + kH * kH + kH + kOut * kH + kOut;
+constexpr int kOffB1 = kH * kIn, kOffW2 = kOffB1 + kH, kOffB2 = kOffW2 + kH * kH, kOffW3 = kOffB2 + kH,
+              kOffB3 = kOffW3 + kOut * kH;
+// A block's partial result: the gradients, then the loss.
+constexpr int kPartial = kNParams + 8;
+constexpr int kGradWarps = 4, kGradRows = 16 * kGradWarps;  // samples per block and pass
+constexpr int kSN = 24;                                     // row stride of the 8-column operands
+
+// The BF16 operands of the weight gradients of a block's samples, rows padded
+// so that the eight rows of a transposing matrix load fall in distinct banks.
+// X: the six features, a one (whose column of a product is the bias gradient)
+// and a zero.
+struct GradStage {
+  __nv_bfloat16 h1[kGradRows][kS2], h2[kGradRows][kS2], da1[kGradRows][kS2], da2[kGradRows][kS2];
+  __nv_bfloat16 dz[kGradRows][kSN], X[kGradRows][kSN];
+  float loss[kGradWarps];
+};
+
+__device__ __forceinline__ void st2(__nv_bfloat16* p, float lo, float hi) {
+  *reinterpret_cast<uint32_t*>(p) = pack2(lo, hi);
+}
+// Four (two) 8 x 8 matrices of 16-bit elements, transposed on the way: lane l
+// gives the address of row l mod 8 of matrix l / 8.
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(smem_addr(p))
+               : "memory");
+}
+__device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"(smem_addr(p))
+               : "memory");
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- training (gradients)
 
-struct WarpStage {
-  float X[16][8];
-  float h1[16][kH];
-  float h2[16][kH];
-  float dz[16][kOut];
-  float da2[16][kH];
-  float da1[16][kH];
-};
-
-// Per-block gradient accumulator, same packed order as the parameters.
-constexpr int kNParams = kH * kIn + kH + kH * kH + kH + kOut * kH + kOut;
-
-__global__ void __launch_bounds__(128) mlp_grad_kernel(const float* P, const float* phi,
-                                                       const uint8_t* label, int64_t n,
-                                                       float inv_batch, float* grad, float* loss) {
+// Forward and backward pass, and this block's share of the gradients in
+// part[block].  Each warp takes 16 samples through the network; then the
+// weight gradients, which are contractions over the samples (da2^T h1 and so
+// on), run on the tensor cores too, the block's 64 samples at a time: warp w
+// forms rows 16 w .. 16 w + 15 of each, its operands by transposing matrix
+// loads from the staged tiles, and keeps its sums in registers over all of the
+// block's samples.  (On the FP32 pipes -- 16 products per element and shared
+// atomics between the warps, then an atomic per block and parameter -- a batch
+// of 8,192 took 30 us; this kernel 7.3 us and mlp_finish_kernel 3.2 us.)
+__global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const float* P, const float* phi,
+                                                                   const uint8_t* label, int64_t n,
+                                                                   float inv_batch, float* part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmemW& s = *reinterpret_cast<SmemW*>(smem_raw);
-  WarpStage* stage = reinterpret_cast<WarpStage*>(smem_raw + ((sizeof(SmemW) + 15) & ~(size_t)15));
-  float* acc = reinterpret_cast<float*>(stage + (blockDim.x >> 5));  // kNParams floats
+  GradStage& S = *reinterpret_cast<GradStage*>(smem_raw + ((sizeof(SmemW) + 15) & ~(size_t)15));
   load_weights(s, P);
-  for (int e = threadIdx.x; e < kNParams; e += blockDim.x) acc[e] = 0.f;
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
-  WarpStage& S = stage[warp];
-  float* gW1 = acc;
-  float* gb1 = gW1 + kH * kIn;
-  float* gW2 = gb1 + kH;
-  float* gb2 = gW2 + kH * kH;
-  float* gW3 = gb2 + kH;
-  float* gb3 = gW3 + kOut * kH;
+  const int r0w = 16 * warp;  // this warp's rows of the stage, and of every gradient
+  float gW2[8][4], gW1[4], gW3[4], gB2[4], gB3[4];  // gW1's and gB2's column 6: the bias gradients
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    gW1[q] = gW3[q] = gB2[q] = gB3[q] = 0.f;
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) gW2[nt][q] = 0.f;
+  }
   float my_loss = 0.f;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t tile = blockIdx.x * (int64_t)(blockDim.x >> 5) + warp; tile * 16 < n; tile += warps) {
-    const int64_t base = tile * 16;
+  const int64_t blocks = (n + kGradRows - 1) / kGradRows;
+  for (int64_t blk = blockIdx.x; blk < blocks; blk += gridDim.x) {
+    const int64_t base = blk * kGradRows + r0w;
     uint32_t a1[4];
     phi_fragment(phi, n, base, a1);
     Fwd f;
@@ -220,8 +252,8 @@ __global__ void __launch_bounds__(128) mlp_grad_kernel(const float* P, const flo
     dz[1] = r0 ? (e1 / s0 - (y0 == 2 * t + 1 ? 1.f : 0.f)) * inv_batch : 0.f;
     dz[2] = r1 ? (e2 / s1 - (y1 == 2 * t ? 1.f : 0.f)) * inv_batch : 0.f;
     dz[3] = r1 ? (e3 / s1 - (y1 == 2 * t + 1 ? 1.f : 0.f)) * inv_batch : 0.f;
-    if (r0 && (y0 >> 1) == t) my_loss += logf(s0) - (f.z[y0 & 1] - m0);
-    if (r1 && (y1 >> 1) == t) my_loss += logf(s1) - (f.z[2 + (y1 & 1)] - m1);
+    if (r0 && (y0 >> 1) == t) my_loss += logf(s0) - ((y0 & 1 ? f.z[1] : f.z[0]) - m0);
+    if (r1 && (y1 >> 1) == t) my_loss += logf(s1) - ((y1 & 1 ? f.z[3] : f.z[2]) - m1);
     // dh2 = dz W3 (K = 8 classes, padded to 16): B[k][n] = W3[k][n] = W3T[n][k]
     uint32_t adz[4] = {pack2(dz[0], dz[1]), pack2(dz[2], dz[3]), 0u, 0u};
     float dh2[8][4];
@@ -231,18 +263,13 @@ __global__ void __launch_bounds__(128) mlp_grad_kernel(const float* P, const flo
       mma16816(dh2[nt], adz, ld32(s.W3T + (8 * nt + g) * kOut + 2 * t), 0u);
     }
     // da2 = dh2 * (a2 > 0); dh1 = da2 W2: B[k][n] = W2[k][n] = W2T[n][k]
-    float da2[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) da2[nt][q] = f.acc2[nt][q] > 0.f ? dh2[nt][q] : 0.f;
     uint32_t ada2[4][4];
 #pragma unroll
-    for (int kc = 0; kc < 4; ++kc) {
-      ada2[kc][0] = pack2(da2[2 * kc][0], da2[2 * kc][1]);
-      ada2[kc][1] = pack2(da2[2 * kc][2], da2[2 * kc][3]);
-      ada2[kc][2] = pack2(da2[2 * kc + 1][0], da2[2 * kc + 1][1]);
-      ada2[kc][3] = pack2(da2[2 * kc + 1][2], da2[2 * kc + 1][3]);
+    for (int nt = 0; nt < 8; ++nt) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) dh2[nt][q] = f.acc2[nt][q] > 0.f ? dh2[nt][q] : 0.f;
+      ada2[nt >> 1][2 * (nt & 1)] = pack2(dh2[nt][0], dh2[nt][1]);
+      ada2[nt >> 1][2 * (nt & 1) + 1] = pack2(dh2[nt][2], dh2[nt][3]);
     }
     float dh1[8][4];
 #pragma unroll
@@ -253,93 +280,113 @@ __global__ void __launch_bounds__(128) mlp_grad_kernel(const float* P, const flo
       for (int kc = 0; kc < 4; ++kc)
         mma16816(dh1[nt], ada2[kc], ld32(w + 16 * kc + 2 * t), ld32(w + 16 * kc + 2 * t + 8));
     }
-    // stage the tile (BF16-rounded operands) for the weight-gradient reductions
+    // stage the operands (BF16-rounded)
+    __syncthreads();  // the block is done with the last pass's
+    const int ra = r0w + g, rb = ra + 8;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       const int c = 8 * nt + 2 * t;
-      S.h1[g][c] = bf(fmaxf(f.acc1[nt][0], 0.f));
-      S.h1[g][c + 1] = bf(fmaxf(f.acc1[nt][1], 0.f));
-      S.h1[g + 8][c] = bf(fmaxf(f.acc1[nt][2], 0.f));
-      S.h1[g + 8][c + 1] = bf(fmaxf(f.acc1[nt][3], 0.f));
-      S.h2[g][c] = bf(fmaxf(f.acc2[nt][0], 0.f));
-      S.h2[g][c + 1] = bf(fmaxf(f.acc2[nt][1], 0.f));
-      S.h2[g + 8][c] = bf(fmaxf(f.acc2[nt][2], 0.f));
-      S.h2[g + 8][c + 1] = bf(fmaxf(f.acc2[nt][3], 0.f));
-      S.da2[g][c] = bf(da2[nt][0]);
-      S.da2[g][c + 1] = bf(da2[nt][1]);
-      S.da2[g + 8][c] = bf(da2[nt][2]);
-      S.da2[g + 8][c + 1] = bf(da2[nt][3]);
-      S.da1[g][c] = bf(f.acc1[nt][0] > 0.f ? dh1[nt][0] : 0.f);
-      S.da1[g][c + 1] = bf(f.acc1[nt][1] > 0.f ? dh1[nt][1] : 0.f);
-      S.da1[g + 8][c] = bf(f.acc1[nt][2] > 0.f ? dh1[nt][2] : 0.f);
-      S.da1[g + 8][c + 1] = bf(f.acc1[nt][3] > 0.f ? dh1[nt][3] : 0.f);
+      st2(&S.h1[ra][c], fmaxf(f.acc1[nt][0], 0.f), fmaxf(f.acc1[nt][1], 0.f));
+      st2(&S.h1[rb][c], fmaxf(f.acc1[nt][2], 0.f), fmaxf(f.acc1[nt][3], 0.f));
+      st2(&S.h2[ra][c], fmaxf(f.acc2[nt][0], 0.f), fmaxf(f.acc2[nt][1], 0.f));
+      st2(&S.h2[rb][c], fmaxf(f.acc2[nt][2], 0.f), fmaxf(f.acc2[nt][3], 0.f));
+      *reinterpret_cast<uint32_t*>(&S.da2[ra][c]) = ada2[nt >> 1][2 * (nt & 1)];
+      *reinterpret_cast<uint32_t*>(&S.da2[rb][c]) = ada2[nt >> 1][2 * (nt & 1) + 1];
+      st2(&S.da1[ra][c], f.acc1[nt][0] > 0.f ? dh1[nt][0] : 0.f, f.acc1[nt][1] > 0.f ? dh1[nt][1] : 0.f);
+      st2(&S.da1[rb][c], f.acc1[nt][2] > 0.f ? dh1[nt][2] : 0.f, f.acc1[nt][3] > 0.f ? dh1[nt][3] : 0.f);
     }
-    S.dz[g][2 * t] = bf(dz[0]);
-    S.dz[g][2 * t + 1] = bf(dz[1]);
-    S.dz[g + 8][2 * t] = bf(dz[2]);
-    S.dz[g + 8][2 * t + 1] = bf(dz[3]);
-    {
-      const __nv_bfloat162 x0 = *reinterpret_cast<const __nv_bfloat162*>(&a1[0]);
-      const __nv_bfloat162 x1 = *reinterpret_cast<const __nv_bfloat162*>(&a1[1]);
-      S.X[g][2 * t] = __bfloat162float(x0.x);
-      S.X[g][2 * t + 1] = __bfloat162float(x0.y);
-      S.X[g + 8][2 * t] = __bfloat162float(x1.x);
-      S.X[g + 8][2 * t + 1] = __bfloat162float(x1.y);
-    }
-    __syncwarp();
-    // weight gradients: sum over the 16 rows, FP32 accumulation (shared atomics
-    // because the block's warps share one accumulator)
-    for (int e = lane; e < kOut * kH; e += 32) {
-      const int o = e / kH, i = e % kH;
-      float a = 0.f;
+    *reinterpret_cast<uint32_t*>(&S.dz[ra][2 * t]) = adz[0];
+    *reinterpret_cast<uint32_t*>(&S.dz[rb][2 * t]) = adz[1];
+    *reinterpret_cast<uint32_t*>(&S.X[ra][2 * t]) = t < 3 ? a1[0] : pack2(1.f, 0.f);
+    *reinterpret_cast<uint32_t*>(&S.X[rb][2 * t]) = t < 3 ? a1[1] : pack2(1.f, 0.f);
+    __syncthreads();
+    // this warp's rows of the gradients, 16 samples at a time
+    const int mr = lane & 7, m1b = (lane >> 3) & 1, m2b = lane >> 4;  // row and matrix of the loads
+#pragma unroll 1
+    for (int kc = 0; kc < kGradWarps; ++kc) {
+      const int k0 = 16 * kc;
+      uint32_t A[4], B[4], D[2], Xf[2];
+      // A (16 x 16): matrices (rows 0-7, k 0-7), (8-15, 0-7), (0-7, 8-15), (8-15, 8-15)
+      auto a_of = [&](const __nv_bfloat16(&T)[kGradRows][kS2]) { ldsm4t(A, &T[k0 + 8 * m2b + mr][r0w + 8 * m1b]); };
+      ldsm2t(D, &S.dz[k0 + 8 * m1b + mr][0]);
+      ldsm2t(Xf, &S.X[k0 + 8 * m1b + mr][0]);
+      a_of(S.da2);
+      mma16816(gB2, A, Xf[0], Xf[1]);
 #pragma unroll
-      for (int m = 0; m < 16; ++m) a = fmaf(S.dz[m][o], S.h2[m][i], a);
-      atomicAdd(&gW3[e], a);
-    }
-    if (lane < kOut) {
-      float a = 0.f;
-      for (int m = 0; m < 16; ++m) a += S.dz[m][lane];
-      atomicAdd(&gb3[lane], a);
-    }
-    for (int e = lane; e < kH * kH; e += 32) {
-      const int o = e / kH, i = e % kH;
-      float a = 0.f;
-#pragma unroll
-      for (int m = 0; m < 16; ++m) a = fmaf(S.da2[m][o], S.h1[m][i], a);
-      atomicAdd(&gW2[e], a);
-    }
-    for (int e = lane; e < kH * kIn; e += 32) {
-      const int o = e / kIn, i = e % kIn;
-      float a = 0.f;
-#pragma unroll
-      for (int m = 0; m < 16; ++m) a = fmaf(S.da1[m][o], S.X[m][i], a);
-      atomicAdd(&gW1[e], a);
-    }
-    for (int o = lane; o < kH; o += 32) {
-      float a = 0.f, b = 0.f;
-      for (int m = 0; m < 16; ++m) {
-        a += S.da2[m][o];
-        b += S.da1[m][o];
+      for (int nt = 0; nt < 8; nt += 2) {
+        ldsm4t(B, &S.h1[k0 + 8 * m1b + mr][8 * (nt + m2b)]);
+        mma16816(gW2[nt], A, B[0], B[1]);
+        mma16816(gW2[nt + 1], A, B[2], B[3]);
       }
-      atomicAdd(&gb2[o], a);
-      atomicAdd(&gb1[o], b);
+      a_of(S.da1);
+      mma16816(gW1, A, Xf[0], Xf[1]);
+      a_of(S.h2);
+      mma16816(gW3, A, D[0], D[1]);  // transposed: rows = inputs, columns = classes
+      if (warp == 0) {
+        const uint32_t one = pack2(1.f, 1.f), ones[4] = {one, one, one, one};
+        mma16816(gB3, ones, D[0], D[1]);
+      }
     }
-    __syncwarp();
+  }
+  float* out = part + (int64_t)blockIdx.x * kPartial;
+  const int oa = r0w + g, ob = oa + 8;
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) {
+    const int c = 8 * nt + 2 * t;
+    *reinterpret_cast<float2*>(out + kOffW2 + oa * kH + c) = make_float2(gW2[nt][0], gW2[nt][1]);
+    *reinterpret_cast<float2*>(out + kOffW2 + ob * kH + c) = make_float2(gW2[nt][2], gW2[nt][3]);
+  }
+  if (t < 3) {
+    *reinterpret_cast<float2*>(out + oa * kIn + 2 * t) = make_float2(gW1[0], gW1[1]);
+    *reinterpret_cast<float2*>(out + ob * kIn + 2 * t) = make_float2(gW1[2], gW1[3]);
+  } else {  // column 6: the ones
+    out[kOffB1 + oa] = gW1[0];
+    out[kOffB1 + ob] = gW1[2];
+    out[kOffB2 + oa] = gB2[0];
+    out[kOffB2 + ob] = gB2[2];
+  }
+  out[kOffW3 + (2 * t) * kH + oa] = gW3[0];
+  out[kOffW3 + (2 * t + 1) * kH + oa] = gW3[1];
+  out[kOffW3 + (2 * t) * kH + ob] = gW3[2];
+  out[kOffW3 + (2 * t + 1) * kH + ob] = gW3[3];
+  if (warp == 0 && g == 0) {
+    out[kOffB3 + 2 * t] = gB3[0];
+    out[kOffB3 + 2 * t + 1] = gB3[1];
   }
   for (int o = 16; o > 0; o >>= 1) my_loss += __shfl_xor_sync(0xffffffffu, my_loss, o);
-  if (lane == 0 && my_loss != 0.f) atomicAdd(loss, my_loss * inv_batch);
+  if (lane == 0) S.loss[warp] = my_loss;
   __syncthreads();
-  for (int e = threadIdx.x; e < kNParams; e += blockDim.x)
-    if (acc[e] != 0.f) atomicAdd(&grad[e], acc[e]);
+  if (threadIdx.x == 0) {
+    float l = 0.f;
+    for (int w = 0; w < kGradWarps; ++w) l += S.loss[w];
+    out[kNParams] = l * inv_batch;
+  }
 }
 
-// Adam on the FP32 master parameters.
-__global__ void mlp_adam_kernel(float* P, const float* grad, float* m1, float* m2, float lr,
-                                float beta1, float beta2, float eps, float bc1, float bc2) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < kNParams; e += gridDim.x * blockDim.x) {
-    const float gr = grad[e];
-    const float a = beta1 * m1[e] + (1.f - beta1) * gr;
-    const float b = beta2 * m2[e] + (1.f - beta2) * gr * gr;
+// Sums the blocks' partial results, in the blocks' order: the gradients into G
+// (G != nullptr), the loss into *loss (where the host reads it); with lr > 0
+// also the Adam step on the FP32 master parameters.  Thirty-two parameters per
+// block, eight threads each on an eighth of the partials.
+__global__ void __launch_bounds__(256) mlp_finish_kernel(const float* part, int blocks, float* G, float* loss,
+                                                         float* P, float* m1, float* m2, float lr, float beta1,
+                                                         float beta2, float eps, float bc1, float bc2) {
+  __shared__ float sum[8][33];
+  const int e = blockIdx.x * 32 + (threadIdx.x & 31), slice = threadIdx.x >> 5;
+  float g = 0.f;
+  if (e <= kNParams)
+    for (int b = slice; b < blocks; b += 8) g += part[(int64_t)b * kPartial + e];
+  sum[slice][threadIdx.x & 31] = g;
+  __syncthreads();
+  if (slice > 0 || e > kNParams) return;
+  for (int q = 1; q < 8; ++q) g += sum[q][threadIdx.x];
+  if (e == kNParams) {
+    *loss = g;
+    return;
+  }
+  if (G) G[e] = g;
+  if (lr > 0.f) {
+    const float a = beta1 * m1[e] + (1.f - beta1) * g;
+    const float b = beta2 * m2[e] + (1.f - beta2) * g * g;
     m1[e] = a;
     m2[e] = b;
     P[e] -= lr * (a / bc1) / (sqrtf(b / bc2) + eps);
@@ -348,15 +395,16 @@ __global__ void mlp_adam_kernel(float* P, const float* grad, float* m1, float* m
 
 int mlp_param_count() { return kNParams; }
 
-size_t mlp_grad_smem(int warps) {
-  return ((sizeof(SmemW) + 15) & ~(size_t)15) + (size_t)warps * sizeof(WarpStage) +
-         (size_t)kNParams * sizeof(float);
+static int grad_blocks(int64_t n, int sm_count) {
+  const int64_t want = (n + kGradRows - 1) / kGradRows, cap = sm_count > 0 ? sm_count : 152;
+  return (int)(want < cap ? want : cap);
 }
+size_t mlp_partial_floats(int sm_count) { return (size_t)(sm_count > 0 ? sm_count : 152) * kPartial; }
 
 cudaError_t launch_mlp_grad(const float* P, const float* phi, const uint8_t* label, int64_t n,
-                            float* grad, float* loss, int sm_count, cudaStream_t s) {
+                            float* part, int sm_count, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const size_t smem = mlp_grad_smem(4);
+  const size_t smem = ((sizeof(SmemW) + 15) & ~(size_t)15) + sizeof(GradStage);
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -364,19 +412,17 @@ cudaError_t launch_mlp_grad(const float* P, const float* phi, const uint8_t* lab
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  const int64_t tiles = (n + 15) / 16;
-  int64_t blocks = (tiles + 3) / 4;
-  const int64_t cap = (int64_t)(sm_count > 0 ? sm_count : 152);
-  if (blocks > cap) blocks = cap;
-  mlp_grad_kernel<<<(int)blocks, 128, smem, s>>>(P, phi, label, n, 1.0f / (float)n, grad, loss);
+  mlp_grad_kernel<<<grad_blocks(n, sm_count), 32 * kGradWarps, smem, s>>>(P, phi, label, n, 1.0f / (float)n,
+                                                                          part);
   return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_adam(float* P, const float* grad, float* m1, float* m2, float lr,
-                            int step, cudaStream_t s) {
+cudaError_t launch_mlp_finish(const float* part, int64_t n, float* grad, float* loss, float* P, float* m1,
+                              float* m2, float lr, int step, int sm_count, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float bc1 = 1.f - powf(b1, (float)step), bc2 = 1.f - powf(b2, (float)step);
-  mlp_adam_kernel<<<(kNParams + 255) / 256, 256, 0, s>>>(P, grad, m1, m2, lr, b1, b2, 1e-8f, bc1, bc2);
+  mlp_finish_kernel<<<(kNParams + 32) / 32, 256, 0, s>>>(part, grad_blocks(n, sm_count), grad, loss, P, m1, m2,
+                                                         lr, b1, b2, 1e-8f, bc1, bc2);
   return cudaGetLastError();
 }
 

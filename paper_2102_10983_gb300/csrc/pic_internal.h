@@ -295,9 +295,12 @@ cudaError_t launch_mlp_infer(const float* P, const float* phi, int64_t n, uint8_
 // network, and a tile of such particles skips the network.
 cudaError_t launch_predict_fused(const PushArgsMixed& a, int order, const float* P, uint8_t* pred,
                                  int sm_count, cudaStream_t s, bool fieldless_zero = false);
+// Gradients of a batch as partial results per block (mlp_partial_floats), then
+// their sum: into grad (optional) and *loss, and, lr > 0, the Adam step.
+size_t mlp_partial_floats(int sm_count);
 cudaError_t launch_mlp_grad(const float* P, const float* phi, const uint8_t* label, int64_t n,
-                            float* grad, float* loss, int sm_count, cudaStream_t s);
-cudaError_t launch_mlp_adam(float* P, const float* grad, float* m1, float* m2, float lr, int step,
-                            cudaStream_t s);
+                            float* part, int sm_count, cudaStream_t s);
+cudaError_t launch_mlp_finish(const float* part, int64_t n, float* grad, float* loss, float* P, float* m1,
+                              float* m2, float lr, int step, int sm_count, cudaStream_t s);
 
 }  // namespace pic
