@@ -38,7 +38,9 @@ struct pic_batch {
   int32_t* queue = nullptr;   // 2 x 7 x n_total
   int32_t* qcount = nullptr;  // 2 x n_ens x 8, then cursor, blocks done
   int64_t* prefix = nullptr;  // 7 n_ens + 1
-  float* half = nullptr;      // 2 x n_ens x W
+  float4* nodes = nullptr;    // n_ens x W: the step's node fields
+  int2* win = nullptr;        // 2 (step parity) x n_ens: the steps' windows
+  int32_t* chunk_ens = nullptr;  // the stream items' ensembles
   float* coef = nullptr;      // 2 (step parity) x n_ens x W x 2(p+1): node coefficient tables
   int32_t* lag_step = nullptr;  // per particle: the step a deferred particle is in (call-relative)
   uint16_t* lag_j = nullptr;    // and the sub-steps of it done
@@ -72,9 +74,30 @@ static void batch_free(pic_batch* b) {
   for (cudaEvent_t e : b->ev) cudaEventDestroy(e);
   void* ptrs[] = {b->ens_dev, b->cell, b->frac, b->px, b->py, b->pz, b->status, b->ring,
                   b->slot_i0, b->i0_dev, b->staging, b->wtab64, b->wtab32, b->dstats,
-                  b->queue, b->qcount, b->prefix, b->half, b->coef, b->lag_step, b->lag_j};
+                  b->queue, b->qcount, b->prefix, b->nodes, b->win, b->chunk_ens, b->coef, b->lag_step, b->lag_j};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+}
+
+// Tiles per stream item for a chunk length: whole tiles.
+static int32_t chunk_tiles(const pic_batch* b) { return (b->chunk + batch_tile() - 1) / batch_tile(); }
+
+// Divide the ensembles into stream items (which depend on the chunk length).
+static int set_chunk(pic_batch* b, int32_t chunk) {
+  b->chunk = chunk;
+  const int64_t T = batch_tile(), per = chunk_tiles(b);
+  int64_t chunk_first = 0;
+  for (int q = 0; q < b->n_ens; ++q) {
+    EnsDev& d = b->ens_dev_h[q];
+    d.chunk_first = chunk_first;
+    if (d.count > 0) chunk_first += ((d.first + d.count - 1) / T - d.first / T + per) / per;
+  }
+  b->n_chunks = chunk_first;
+  BATCH_TRY(b, cudaMemcpyAsync(b->ens_dev, b->ens_dev_h.data(), sizeof(EnsDev) * b->n_ens,
+                               cudaMemcpyHostToDevice, b->stream));
+  BATCH_TRY(b, launch_batch_chunks(b->ens_dev, b->n_ens, b->n_chunks, b->chunk_ens, b->stream));
+  BATCH_TRY(b, cudaStreamSynchronize(b->stream));
+  return PIC_OK;
 }
 
 extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t order,
@@ -136,7 +159,9 @@ extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t 
   A((void**)&b->queue, 2 * 7 * cap * 4);
   A((void**)&b->qcount, sizeof(int32_t) * (2 * 8 * (size_t)n_ens + 8));
   A((void**)&b->prefix, sizeof(int64_t) * (7 * (size_t)n_ens + 1));
-  A((void**)&b->half, sizeof(float) * 2 * (size_t)n_ens * window_cells);
+  A((void**)&b->nodes, sizeof(float4) * (size_t)n_ens * window_cells);
+  A((void**)&b->win, sizeof(int2) * 2 * (size_t)n_ens);
+  A((void**)&b->chunk_ens, sizeof(int32_t) * (cap / batch_tile() + 2 * (size_t)n_ens + 1));
   A((void**)&b->coef, sizeof(float) * 2 * (size_t)n_ens * window_cells * 2 * (size_t)(order + 1));
   A((void**)&b->lag_step, cap * 4);
   A((void**)&b->lag_j, cap * 2);
@@ -147,7 +172,7 @@ extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t 
     return bfail(nullptr, PIC_ENOMEM, "pic_batch_create: device allocation failed");
   }
   // ensemble table
-  int64_t first = 0, chunk_first = 0;
+  int64_t first = 0;
   b->ens_dev_h.resize(n_ens);
   for (int q = 0; q < n_ens; ++q) {
     const pic_ensemble& s = ens[q];
@@ -167,12 +192,9 @@ extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t 
     d.slot_i0 = b->slot_i0 + (size_t)q * ring_levels;
     d.first = first;
     d.count = s.n_particles;
-    d.chunk_first = chunk_first;
     first += s.n_particles;
-    chunk_first += (s.n_particles + b->chunk - 1) / b->chunk;
   }
-  b->n_chunks = chunk_first;
-  e = cudaMemcpy(b->ens_dev, b->ens_dev_h.data(), sizeof(EnsDev) * n_ens, cudaMemcpyHostToDevice);
+  if (set_chunk(b, b->chunk) != PIC_OK) e = cudaErrorUnknown;
   if (e == cudaSuccess) e = cudaMemset(b->qcount, 0, sizeof(int32_t) * (2 * 8 * (size_t)n_ens + 8));
   if (e == cudaSuccess) e = cudaMemset(b->dstats, 0, sizeof(DevStats));
   if (e == cudaSuccess) e = cudaMemset(b->status, 0, cap);
@@ -195,21 +217,6 @@ extern "C" int pic_batch_destroy(pic_batch* b) {
   cudaStreamSynchronize(b->stream);
   batch_free(b);
   delete b;
-  return PIC_OK;
-}
-
-// Re-chunk the ensembles (the chunk boundaries depend on the chunk length).
-static int set_chunk(pic_batch* b, int32_t chunk) {
-  b->chunk = chunk;
-  int64_t chunk_first = 0;
-  for (int q = 0; q < b->n_ens; ++q) {
-    b->ens_dev_h[q].chunk_first = chunk_first;
-    chunk_first += (b->ens_dev_h[q].count + chunk - 1) / chunk;
-  }
-  b->n_chunks = chunk_first;
-  BATCH_TRY(b, cudaMemcpyAsync(b->ens_dev, b->ens_dev_h.data(), sizeof(EnsDev) * b->n_ens,
-                               cudaMemcpyHostToDevice, b->stream));
-  BATCH_TRY(b, cudaStreamSynchronize(b->stream));
   return PIC_OK;
 }
 
@@ -343,7 +350,8 @@ static int queue_steps(pic_batch* b, int64_t n, int64_t n_steps) {
   base.ens = b->ens_dev;
   base.n_total = b->n_total;
   base.n_chunks = b->n_chunks;
-  base.chunk = b->chunk;
+  base.chunk_tiles = chunk_tiles(b);
+  base.chunk_ens = b->chunk_ens;
   base.cell = b->cell; base.frac = b->frac; base.px = b->px; base.py = b->py; base.pz = b->pz;
   base.status = b->status;
   base.R = b->R;
@@ -354,7 +362,7 @@ static int queue_steps(pic_batch* b, int64_t n, int64_t n_steps) {
   lagrange_monomials(p, base.mono);
   base.stats = b->dstats;
   base.prefix = b->prefix;
-  base.half = b->half;
+  base.nodes = b->nodes;
   base.cursor = (int*)(b->qcount + 16 * b->n_ens);
   base.blocks_done = (unsigned*)(b->qcount + 16 * b->n_ens + 2);
   const int64_t qsz = 7 * b->n_total;
@@ -382,6 +390,8 @@ static int queue_steps(pic_batch* b, int64_t n, int64_t n_steps) {
     const int64_t table = b->n_ens * b->W * 2 * (p + 1);
     a.coef = b->coef + (s & 1) * table;
     a.coef_p = (j > 0 && !fin) ? b->coef + ((s - 1) & 1) * table : a.coef;
+    a.win = b->win + (s & 1) * b->n_ens;
+    a.win_p = (j > 0 && !fin) ? b->win + ((s - 1) & 1) * b->n_ens : a.win;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (b->timing && !fin) {
       int rc = batch_timing_pair(b, &e0, &e1);

@@ -334,7 +334,7 @@ __device__ __forceinline__ void tc_end(TcSmem& s) {
 
 }  // namespace
 
-// pic_predict: features of every particle after step a (a.halfE / a.halfB: its
+// pic_predict: features of every particle after step a (a.featE / a.featB: its
 // feature nodes; the same code as the features kernel) and the network's
 // class, in one pass.
 template <int P>
@@ -354,7 +354,7 @@ __global__ void __launch_bounds__(kTcThreads) predict_tc_kernel(PushArgsMixed a,
     const int64_t tn = t + gridDim.x;
     const FeatureInput nxt = feature_input(a, tn < n_groups ? tn * kTcThreads + threadIdx.x : a.n);
     float f[6];
-    features_of(a, a.halfE, a.halfB, a.lo, a.hi, cur, f);
+    features_of(a, a.featE, a.featB, a.lo, a.hi, cur, f);
     // no field at the particle: no rotation, the criterion takes k = 0
     const bool fieldless = fieldless_zero && f[0] == 0.f && f[1] == 0.f;
     int c = 0;

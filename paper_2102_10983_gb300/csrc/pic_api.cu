@@ -40,7 +40,7 @@ struct pic_ctx {
   int32_t* qcount = nullptr;  // [0,16) deferred counts, 16 cursor, 18 blocks done, [32,40) predicted counts
   // predicted schedule
   uint8_t* pred = nullptr;
-  float* half = nullptr;  // mixed form: E_y, B_z of every window node at the step's t_n
+  float4* nodes = nullptr;  // mixed form: the step's node fields (PushArgsMixed::nodes)
   float* coef = nullptr;  // mixed form: per node monomial coefficients, two steps (parity of s)
   float* feat = nullptr;  // mixed form: the predictor's feature nodes (E_y, B_z at t_{n+1}), W + 1 each
   // binned mixed form: resumable long sub-cycles (per particle: the step it is
@@ -108,7 +108,7 @@ static void free_all(pic_ctx* c) {
 
   void* ptrs[] = {c->x, c->px, c->py, c->pz, c->cell, c->frac, c->fpx, c->fpy, c->fpz,
                   c->status, c->ringE, c->ringB, c->staging, c->wtab64, c->wtab32,
-                  c->dstats, c->queue, c->qcount, c->pred, c->pred_queue, c->half,
+                  c->dstats, c->queue, c->qcount, c->pred, c->pred_queue, c->nodes,
                   c->coef, c->lag_step, c->lag_j, c->dslot_i0, c->work, c->feat,
                   c->nodes64, c->k_sub, c->queue64, c->bin64};
   for (void* p : ptrs)
@@ -213,7 +213,7 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     if (e == cudaSuccess) e = cudaMalloc(p, bytes);
   };
   if (mixed) {
-    A((void**)&c->half, 2 * ((size_t)window_cells + 1) * 4);  // E_y, B_z: W + 1 nodes each
+    A((void**)&c->nodes, (size_t)window_cells * sizeof(float4));
     A((void**)&c->coef, 2 * (size_t)window_cells * 2 * (prm->order + 1) * 4);
     A((void**)&c->feat, 2 * ((size_t)window_cells + 1) * 4);
     A((void**)&c->cell, cap * 4);
@@ -646,8 +646,7 @@ static int close_open(pic_ctx* c) {
   const int64_t coef_stride = c->W * 2 * (c->prm.order + 1);
   const float* coef_s = c->coef + (S & 1) * coef_stride;
   a.coef = coef_s;
-  a.halfE = c->half;
-  a.halfB = c->half + c->W + 1;
+  a.nodes = c->nodes;
   const int64_t J = c->run_j - 1;
   a.parity_cur = (int)(J & 1);
   a.parity_next = (int)((J + 1) & 1);
@@ -758,11 +757,10 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
       const int64_t coef_stride = W * 2 * (p + 1);
       float* coef_cur = c->coef + (s & 1) * coef_stride;
       float* coef_prev = c->coef + ((s - 1) & 1) * coef_stride;
-      e = launch_halfstep(a, p, W, c->half, c->half + W + 1, coef_cur, c->stream);
+      e = launch_halfstep(a, p, W, c->nodes, coef_cur, c->stream);
       ++launches;
       if (e != cudaSuccess) return fail(c, PIC_ECUDA, "half-step launch: %s", cudaGetErrorString(e));
-      a.halfE = c->half;
-      a.halfB = c->half + W + 1;
+      a.nodes = c->nodes;
       a.coef = coef_cur;
       // deferred work of the previous step: from this call's last launch, or
       // carried from the last call
@@ -799,8 +797,8 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
             PushArgsMixed fa = a;
             fill_mixed(c, fa, s - 1, plo, phi, false);
             fa.coef = fa.coef_p = nullptr;
-            fa.halfE = c->feat;
-            fa.halfB = c->feat + W + 1;
+            fa.featE = c->feat;
+            fa.featB = c->feat + W + 1;
             e = launch_feature_nodes(fa, p, W, c->feat, c->feat + W + 1, c->stream);
             ++launches;
             if (e == cudaSuccess)
@@ -862,8 +860,8 @@ extern "C" int pic_features(pic_ctx* c, int64_t n, float* phi) {
   a.status = c->status;
   a.mask = (int32_t)(c->W - 1);
   fill_mixed(c, a, n, lo, hi, false);
-  a.halfE = c->feat;
-  a.halfB = c->feat + c->W + 1;
+  a.featE = c->feat;
+  a.featB = c->feat + c->W + 1;
   CUDA_TRY(c, launch_feature_nodes(a, c->prm.order, c->W, c->feat, c->feat + c->W + 1, c->stream));
   CUDA_TRY(c, launch_features_mixed(a, c->prm.order, phi, c->stream));
   c->launches += 2;
@@ -886,8 +884,8 @@ extern "C" int pic_predict(pic_ctx* c, const pic_mlp* mlp, int64_t n, uint8_t* p
   a.status = c->status;
   a.mask = (int32_t)(c->W - 1);
   fill_mixed(c, a, n, lo, hi, false);
-  a.halfE = c->feat;
-  a.halfB = c->feat + c->W + 1;
+  a.featE = c->feat;
+  a.featB = c->feat + c->W + 1;
   CUDA_TRY(c, launch_feature_nodes(a, c->prm.order, c->W, c->feat, c->feat + c->W + 1, c->stream));
   CUDA_TRY(c, launch_predict_fused(a, c->prm.order, mlp_device_params(mlp), pred, c->sm_count,
                                    c->stream));

@@ -111,11 +111,14 @@ struct PushArgsMixed {
   const float* B[kMaxOrder + 1];
   const float* Ep[kMaxOrder + 1];  // previous step's levels (binned: deferred work)
   const float* Bp[kMaxOrder + 1];
-  // E_y and B_z of every window node interpolated to t_n (theta = 1/2), written
-  // by the step's half-step kernel, W + 1 nodes each (node W repeats node 0);
-  // nullptr = not provided (gather the levels)
-  const float* halfE;
-  const float* halfB;
+  // per window node, E_y and B_z at t_n (theta = 1/2) and the steps to the next
+  // node, {E, dE, B, dB}, written by the step's half-step kernel; nullptr = not
+  // provided (gather the levels)
+  const float4* nodes;
+  // the predictor's feature nodes, E_y and B_z of every window node at t_{n+1}, W
+  // + 1 each (node W repeats node 0)
+  const float* featE;
+  const float* featB;
   // per window node, the monomial coefficients of the temporal interpolant of
   // E_y (p+1) then B_z (p+1) for this step (coef) and the previous one
   // (coef_p); nullptr = form them from the levels
@@ -183,7 +186,7 @@ struct EnsDev {
   const int64_t* slot_i0;  // [R] window origin of each ring slot
   double dx, inv_dx64;     // the cell and its reciprocal in FP64 (loading and reading particles)
   int64_t first, count;    // particle range in the concatenated store
-  int64_t chunk_first;     // index of its first stream chunk
+  int64_t chunk_first;     // index of its first stream item
 };
 
 // Arguments of one batched macro step.
@@ -191,7 +194,8 @@ struct BatchArgs {
   int32_t n_ens;
   const EnsDev* ens;
   int64_t n_total, n_chunks;
-  int32_t chunk;  // particles per stream chunk (multiple of 32)
+  int32_t chunk_tiles;       // tiles per stream item
+  const int32_t* chunk_ens;  // [n_chunks] the stream items' ensembles
   int32_t* cell;
   float* frac;
   float* px;
@@ -210,7 +214,9 @@ struct BatchArgs {
   int32_t* qcount_in;   // [n_ens][8]
   int32_t* qcount_out;
   const int64_t* prefix;  // [7*n_ens + 1] heavy-item prefix (filled per launch)
-  float* half;            // [2][n_ens][W]: E_y, B_z of every node at t_n (filled per launch)
+  float4* nodes;          // [n_ens][W]: step_node_f32 of every node (filled per launch)
+  int2* win;              // [n_ens] this step's windows [lo, hi] (filled per launch)
+  const int2* win_p;      // and the previous step's; two such tables, by step parity
   // [n_ens][W][2(p+1)]: every node's monomial coefficients of the temporal
   // interpolant (E_y then B_z) of this step (coef, filled per launch) and of
   // the previous one (coef_p); two such tables, by step parity
@@ -231,6 +237,9 @@ struct BatchArgs {
 cudaError_t launch_batch_step(const BatchArgs& a, int order, int blocks, cudaStream_t s,
                               int* launches);
 int batch_max_blocks_per_sm(int order);
+int batch_tile();  // particles per tile of the stream
+cudaError_t launch_batch_chunks(const EnsDev* ens, int32_t n_ens, int64_t n_chunks, int32_t* chunk_ens,
+                                cudaStream_t s);
 cudaError_t launch_batch_scatter(const EnsDev* ens, int32_t n_ens, int64_t slot, int64_t R,
                                  int64_t W, const double* Ey, const double* Bz, const int64_t* i0,
                                  int64_t* slot_i0_all, cudaStream_t s);
@@ -267,13 +276,13 @@ cudaError_t launch_binned_step(const PushArgsMixed& a, int order, int sm_count, 
                                int* launches);
 // E_y, B_z of every window node at t_n (the theta = 1/2 weights of a's step),
 // and (coef != nullptr) every node's monomial coefficients, 2(p+1) floats.
-cudaError_t launch_halfstep(const PushArgsMixed& a, int order, int64_t W, float* outE, float* outB,
-                            float* coef, cudaStream_t s);
+cudaError_t launch_halfstep(const PushArgsMixed& a, int order, int64_t W, float4* nodes, float* coef,
+                            cudaStream_t s);
 // E_y, B_z of every window node extrapolated to t_{n+1} (theta = 3/2) from step
 // a's levels, W + 1 nodes each: the predictor's field features.
 cudaError_t launch_feature_nodes(const PushArgsMixed& a, int order, int64_t W, float* outE,
                                  float* outB, cudaStream_t s);
-// Features of every particle (a.halfE / a.halfB: the feature nodes of a's step).
+// Features of every particle (a.featE / a.featB: the feature nodes of a's step).
 cudaError_t launch_features_mixed(const PushArgsMixed& a, int order, float* phi, cudaStream_t s);
 
 // Rebuilds the predicted queue: clears the old queue's marks, then bins and
@@ -288,7 +297,7 @@ const float* mlp_device_params(const struct ::pic_mlp* m);
 int mlp_param_count();
 cudaError_t launch_mlp_infer(const float* P, const float* phi, int64_t n, uint8_t* pred,
                              int sm_count, cudaStream_t s);
-// Features of step a's levels (theta = 3/2; a.halfE / a.halfB: the feature
+// Features of step a's levels (theta = 3/2; a.featE / a.featB: the feature
 // nodes) and the predicted class of every particle in one pass (the same
 // predictions as features + launch_mlp_infer).  fieldless_zero: a particle
 // that sees no field (E_y = B_z = 0 at its position) gets class 0 without the

@@ -6,8 +6,8 @@
 //
 // Work items, from one atomic cursor:
 //  1. deferred items (k >= kDeferMin) of every ensemble, largest k first;
-//  2. stream chunks; a chunk never spans two ensembles, so a warp streams one
-//     ensemble's particles at a time (k = 1, 2 go to the warp stashes, whose
+//  2. stream items: runs of tiles of one ensemble's particles, so a warp
+//     streams one ensemble at a time (k = 1, 2 go to the warp stashes, whose
 //     entries remember their ensemble).
 // The chunk length and the grid are launch parameters (tuned by
 // pic_batch_autotune).
@@ -19,15 +19,26 @@
 
 namespace pic {
 
-// Field view of ensemble e for the current (prev = false) or previous step.
+// Field view of ensemble e for the current (prev = false) or previous step;
+// the steps' windows are formed once per step and ensemble (batch_halfstep_kernel).
 template <int P>
 __device__ __forceinline__ void ens_fields(const BatchArgs& a, const EnsDev& e, bool prev,
                                            StepFields<P, true>& F) {
+  const int64_t q = &e - a.ens;
   const int64_t start = prev ? a.start_prev : a.start_cur;
   F.E.base = e.ringE + start * a.lstride;
   F.B.base = e.ringB + start * a.lstride;
   F.E.lstride = (int32_t)a.lstride;
   F.B.lstride = (int32_t)a.lstride;
+  F.coef = (prev ? a.coef_p : a.coef) + q * a.lstride * (2 * (P + 1));
+  const int2 win = __ldg((prev ? a.win_p : a.win) + q);
+  F.lo = win.x;
+  F.hi = win.y;
+}
+
+// The nodes all p + 1 levels from ring slot `start` cover, [lo, hi].
+template <int P>
+__device__ __forceinline__ int2 ens_window(const BatchArgs& a, const EnsDev& e, int64_t start) {
   int64_t lo = INT64_MIN, hi = INT64_MAX;
 #pragma unroll
   for (int l = 0; l <= P; ++l) {
@@ -35,10 +46,7 @@ __device__ __forceinline__ void ens_fields(const BatchArgs& a, const EnsDev& e, 
     lo = o > lo ? o : lo;
     hi = o + a.lstride - 1 < hi ? o + a.lstride - 1 : hi;
   }
-  // the step's node table of this ensemble (batch_halfstep_kernel)
-  F.coef = (prev ? a.coef_p : a.coef) + (int64_t)(&e - a.ens) * a.lstride * (2 * (P + 1));
-  F.lo = (int32_t)lo;
-  F.hi = (int32_t)hi;
+  return make_int2((int32_t)lo, (int32_t)hi);
 }
 
 __device__ __forceinline__ int64_t queue_slot(const BatchArgs& a, const EnsDev& e, int k,
@@ -63,49 +71,36 @@ __device__ __forceinline__ void batch_enqueue(const BatchArgs& a, int key, int32
 }
 
 struct BatchStash {
-  int32_t idx[kStashCap];
-  int32_t cell[kStashCap];
-  float frac[kStashCap], ux[kStashCap], uy[kStashCap], uz[kStashCap];
-  uint8_t kp[kStashCap];
+  Stash s;
   uint16_t ens[kStashCap];
 };
+static_assert(sizeof(BatchStash) % 16 == 0, "stashes follow each other in shared memory");
 
+// Push the last min(n, 32) stashed particles, one per lane (stash_drain of the
+// single-problem kernel, each particle with its ensemble's fields).
 template <int P>
-__device__ __forceinline__ void batch_stash_drain(const BatchArgs& a, BatchStash& S, int k, int& n,
-                                                  int cnt, unsigned long long* sh) {
+__device__ __forceinline__ void batch_stash_drain(const BatchArgs& a, const BatchStash& S, int k, int& n,
+                                                  unsigned long long* sh) {
   const int lane = threadIdx.x & 31;
+  const int cnt = n < 32 ? n : 32;
   if (lane < cnt) {
-    const EnsDev& e = a.ens[S.ens[lane]];
+    const int q = n - cnt + lane;
+    const EnsDev& e = a.ens[S.ens[q]];
     StepFields<P, true> F;
     ens_fields<P>(a, e, false, F);
-    MixedState s = {S.cell[lane], S.frac[lane], S.ux[lane], S.uy[lane], S.uz[lane]};
-    const int32_t i = S.idx[lane];
+    const float4 va = S.s.a[q];
+    const float2 vb = S.s.b[q];
+    const int32_t i = __float_as_int(vb.y);
+    MixedState s = {__float_as_int(va.x), va.y, va.z, va.w, vb.x};
     const bool ok = subcycle_f32<P, true, true>(F, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.mono,
-                                    k, S.kp[lane], 0.f, s);
+                                                k, S.s.kp[q], 0.f, s);
     normalize(s);
-    a.cell[i] = s.cell;
-    a.frac[i] = s.frac;
-    a.px[i] = s.ux;
-    a.py[i] = s.uy;
-    a.pz[i] = s.uz;
+    store_state(a, i, s);
     a.status[i] = ok ? (uint8_t)(k | (a.parity_next ? kParity : 0)) : (uint8_t)(k | PIC_STATUS_LOST);
     if (!ok) atomicAdd(&sh[11], 1ull);
   }
   __syncwarp();
-  const int rest = n - cnt;
-  if (lane < rest) {
-    const int q = cnt + lane;
-    S.idx[lane] = S.idx[q];
-    S.cell[lane] = S.cell[q];
-    S.frac[lane] = S.frac[q];
-    S.ux[lane] = S.ux[q];
-    S.uy[lane] = S.uy[q];
-    S.uz[lane] = S.uz[q];
-    S.kp[lane] = S.kp[q];
-    S.ens[lane] = S.ens[q];
-  }
-  __syncwarp();
-  n = rest;
+  n -= cnt;
 }
 
 // Field view of macro step s of ensemble e from its mirrored ring and the
@@ -122,15 +117,9 @@ __device__ __forceinline__ StepFields<P, true> ens_step_fields(const BatchArgs& 
   F.E.lstride = (int32_t)a.lstride;
   F.B.lstride = (int32_t)a.lstride;
   F.coef = nullptr;
-  int64_t lo = INT64_MIN, hi = INT64_MAX;
-#pragma unroll
-  for (int l = 0; l <= P; ++l) {
-    const int64_t o = e.slot_i0[(start + l) % R];
-    lo = o > lo ? o : lo;
-    hi = o + a.lstride - 1 < hi ? o + a.lstride - 1 : hi;
-  }
-  F.lo = (int32_t)lo;
-  F.hi = (int32_t)hi;
+  const int2 win = ens_window<P>(a, e, start);
+  F.lo = win.x;
+  F.hi = win.y;
   return F;
 }
 
@@ -265,11 +254,9 @@ __device__ __forceinline__ void batch_heavy(const BatchArgs& a, int ens, int64_t
   }
 }
 
-// Every ensemble's window nodes at t_n (theta = 1/2 weights): the same FMA
-// chain as a full gather takes at one node (see halfstep_kernel); and every
-// node's monomial coefficients of the temporal interpolant (to_monomial, the
-// values the sub-cycles would form from the levels), so that a sub-cycle reads
-// two 16-byte rows per grid instead of forming them.
+// Every ensemble's window nodes at t_n (step_node_f32), every node's monomial
+// coefficients of the temporal interpolant (to_monomial, the values the
+// sub-cycles would form from the levels), and the step's windows.
 template <int P>
 __global__ void batch_halfstep_kernel(BatchArgs a) {
   constexpr int stride = 2 * (P + 1);
@@ -280,66 +267,60 @@ __global__ void batch_halfstep_kernel(BatchArgs a) {
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total;
        q += (int64_t)gridDim.x * blockDim.x) {
     const EnsDev& e = a.ens[q / W];
-    const int64_t c = q % W;
-    const float* E = e.ringE + a.start_cur * W + c;
-    const float* B = e.ringB + a.start_cur * W + c;
-    float fe = __fmul_rn(wE[0], __ldg(E));
-    float fb = __fmul_rn(wB[0], __ldg(B));
-#pragma unroll
-    for (int l = 1; l <= P; ++l) {
-      fe = __fmaf_rn(wE[l], __ldg(E + l * W), fe);
-      fb = __fmaf_rn(wB[l], __ldg(B + l * W), fb);
-    }
-    a.half[q] = fe;
-    a.half[total + q] = fb;
+    const int32_t c = (int32_t)(q % W);
     StepFields<P, true> F;
     F.E.base = e.ringE + a.start_cur * W;
     F.B.base = e.ringB + a.start_cur * W;
     F.E.lstride = (int32_t)W;
     F.B.lstride = (int32_t)W;
-    float e0[P + 1], e1[P + 1], b0[P + 1], b1[P + 1];
-    to_monomial<P>(F.E, (int32_t)c, (int32_t)c, a.mono[0], e0, e1);
-    to_monomial<P>(F.B, (int32_t)c, (int32_t)c, a.mono[1], b0, b1);
+    a.nodes[q] = step_node_f32<P>(F.E, F.B, wE, wB, c, a.mask);
+    float e0[P + 1], b0[P + 1];
+    to_monomial1<P>(F.E, c, a.mono[0], e0);
+    to_monomial1<P>(F.B, c, a.mono[1], b0);
     float* r = a.coef + q * stride;
 #pragma unroll
     for (int k = 0; k <= P; ++k) {
       r[k] = e0[k];
       r[P + 1 + k] = b0[k];
     }
+    if (c == 0) a.win[q / W] = ens_window<P>(a, e, a.start_cur);
   }
 }
 
 // Heavy-item prefix: items of (k, ensemble) in the order k = 7..1, ensemble
 // ascending; prefix[q] = first item of entry q, prefix[7 * n_ens] = total.
-__global__ void batch_prefix_kernel(const int32_t* qcount_in, int32_t n_ens, int32_t k_lo,
-                                    int64_t* prefix) {
-  __shared__ long long part[1024];
-  const int n = 7 * n_ens;
-  const int per = (n + blockDim.x - 1) / blockDim.x;
-  const int q0 = threadIdx.x * per;
-  long long sum = 0;
-  for (int q = q0; q < q0 + per && q < n; ++q) {
-    const int k = 7 - q / n_ens, e = q % n_ens;
-    sum += k >= k_lo ? ((long long)qcount_in[e * 8 + k] + 31) / 32 : 0;
-  }
-  part[threadIdx.x] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    long long acc = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const long long v = part[t];
-      part[t] = acc;
-      acc += v;
+__global__ void __launch_bounds__(1024) batch_prefix_kernel(const int32_t* qcount_in, int32_t n_ens, int32_t k_lo,
+                                                            int64_t* prefix) {
+  __shared__ long long part[32];
+  const int n = 7 * n_ens, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  long long base = 0;  // items before this pass of 1,024 entries
+  for (int q0 = 0; q0 < n; q0 += 1024) {
+    const int q = q0 + threadIdx.x;
+    const int k = 7 - q / n_ens;
+    const long long c = q < n && k >= k_lo ? ((long long)qcount_in[(q % n_ens) * 8 + k] + 31) / 32 : 0;
+    long long v = c;  // inclusive scan: in the warp, then over the warps' sums
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long u = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += u;
     }
+    if (lane == 31) part[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+      long long w = part[lane];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long u = __shfl_up_sync(0xffffffffu, w, o);
+        if (lane >= o) w += u;
+      }
+      part[lane] = w;
+    }
+    __syncthreads();
+    if (q < n) prefix[q] = base + (warp ? part[warp - 1] : 0) + v - c;
+    base += part[31];
+    __syncthreads();
   }
-  __syncthreads();
-  long long acc = part[threadIdx.x];
-  for (int q = q0; q < q0 + per && q < n; ++q) {
-    prefix[q] = acc;
-    const int k = 7 - q / n_ens, e = q % n_ens;
-    acc += k >= k_lo ? ((long long)qcount_in[e * 8 + k] + 31) / 32 : 0;
-  }
-  if (threadIdx.x == blockDim.x - 1) prefix[n] = acc;
+  if (threadIdx.x == 0) prefix[n] = base;
 }
 
 // Block shape of the batched kernel: four blocks of five warps per SM (20
@@ -354,22 +335,44 @@ constexpr int kBatchWarps = kBatchThreads / 32;
 #ifndef PIC_BATCH_MIN_BLOCKS
 #define PIC_BATCH_MIN_BLOCKS 4
 #endif
+// Dynamic shared memory: the warps' staged tiles, then their stashes.
+constexpr size_t kBatchTileBytes = sizeof(Tile) * 2 * kBatchWarps;
+constexpr size_t kBatchSmem = kBatchTileBytes + sizeof(BatchStash) * kBatchWarps * kStashK;
+static_assert(kBatchTileBytes % 128 == 0, "stashes start aligned");
 
+// A stream item is a run of whole tiles of kTile particles of one ensemble
+// (tiles of the concatenated store: those at an ensemble's ends hold others'
+// particles too, which the item leaves alone), staged in shared memory by bulk
+// copies one tile ahead and pushed in rounds of 64, two particles per lane, as
+// the single-problem kernel's stream (push_mixed.cu).  (One particle per lane
+// from plain loads, the ensemble found by a search per chunk, its window from
+// the ring per chunk and per parked particle: 17.8 warp instructions per
+// particle of the 512-ensemble configuration, 13.8 so; 293 -> 265 us per step
+// of 11.9M particles.)
 template <int P>
 __global__ void __launch_bounds__(kBatchThreads, PIC_BATCH_MIN_BLOCKS) push_batch_kernel(BatchArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  BatchStash* stashes = reinterpret_cast<BatchStash*>(smem);  // [kBatchWarps][kStashK]
+  extern __shared__ __align__(128) unsigned char smem[];
+  Tile* tiles = reinterpret_cast<Tile*>(smem);  // [kBatchWarps][2]
+  BatchStash* stashes = reinterpret_cast<BatchStash*>(smem + kBatchTileBytes);  // [kBatchWarps][kStashK]
+  __shared__ __align__(8) uint64_t bars[kBatchWarps * 2];
   __shared__ unsigned long long sh[12];
-  __shared__ int s_task[kBatchWarps];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
   __syncthreads();
   constexpr int stride = 2 * (P + 1);
   const float* wcrit = a.wtab + a.crit_row * stride + (P + 1);
-  const float* w0 = a.wtab + wrow(0, 1) * stride;
   ThreadCounters tc;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
+  Tile* my_tiles = tiles + 2 * warp;
+  uint64_t* my_bars = bars + 2 * warp;
   BatchStash* my_stash = stashes + warp * kStashK;
+  if (lane == 0) {
+    mbar_init(my_bars);
+    mbar_init(my_bars + 1);
+    mbar_init_fence();
+  }
+  __syncwarp();
+  uint32_t phase = 0;  // bit s: parity of stage s's next completion
   int stash_n[kStashK];
 #pragma unroll
   for (int q = 0; q < kStashK; ++q) stash_n[q] = 0;
@@ -377,13 +380,29 @@ __global__ void __launch_bounds__(kBatchThreads, PIC_BATCH_MIN_BLOCKS) push_batc
   const uint8_t done = a.parity_next ? kParity : 0;
   const int64_t n_heavy = a.prefix[7 * a.n_ens];
   const int64_t n_items = n_heavy + (a.finalize ? 0 : a.n_chunks);
-  const int per_lane = a.chunk / 32;
+  const uint64_t policy = evict_first_policy();
+
+  auto drain = [&](bool all) {
+#pragma unroll 1
+    for (int q = 0; q < kStashK; ++q) {
+      int n = 0;
+#pragma unroll
+      for (int r = 0; r < kStashK; ++r)
+        if (r == q) n = stash_n[r];
+      const int keep = all ? 0 : 31;
+      if (n <= keep) continue;
+#pragma unroll 1
+      while (n > keep) batch_stash_drain<P>(a, my_stash[q], q + 1, n, sh);
+#pragma unroll
+      for (int r = 0; r < kStashK; ++r)
+        if (r == q) stash_n[r] = n;
+    }
+  };
 
   for (;;) {
-    if (lane == 0) s_task[warp] = atomicAdd(a.cursor, 1);
-    __syncwarp();
-    const int64_t t = s_task[warp];
-    __syncwarp();
+    int claim = 0;
+    if (lane == 0) claim = atomicAdd(a.cursor, 1);
+    const int64_t t = __shfl_sync(0xffffffffu, claim, 0);
     if (t >= n_items) break;
     if (t < n_heavy) {
       int lo = 0, hi = 7 * a.n_ens - 1;  // last entry q with prefix[q] <= t
@@ -402,104 +421,178 @@ __global__ void __launch_bounds__(kBatchThreads, PIC_BATCH_MIN_BLOCKS) push_batc
       batch_enqueue(a, key, i);
       continue;
     }
-    // stream chunk: which ensemble, which particles
+    // stream item: which ensemble, which tiles
     const int64_t c = t - n_heavy;
-    int lo = 0, hi = a.n_ens - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (a.ens[mid].chunk_first <= c) lo = mid; else hi = mid - 1;
-    }
-    const int ens = lo;
+    const int ens = __ldg(a.chunk_ens + c);
     const EnsDev& e = a.ens[ens];
-    StepFields<P, true> F;
-    ens_fields<P>(a, e, false, F);
-    const float hx0 = __fmul_rn(e.dt, e.inv_dx);
-    const int64_t first = e.first + (c - e.chunk_first) * a.chunk;
-    const int64_t end = e.first + e.count;
-    int64_t i = first + lane;
-    uint8_t st = PIC_STATUS_LOST;
-    MixedState s = {0, 0.5f, 0.f, 0.f, 0.f};
-    if (i < end) {
-      st = a.status[i];
-      s = {a.cell[i], a.frac[i], a.px[i], a.py[i], a.pz[i]};
-    }
+    const int64_t e_first = e.first, e_end = e.first + e.count;
+    const int64_t tile0 = e_first / kTile + (c - e.chunk_first) * a.chunk_tiles;
+    const int64_t tile_last = (e_end - 1) / kTile;
+    const int n_tiles = (int)(tile_last - tile0 + 1 < a.chunk_tiles ? tile_last - tile0 + 1 : a.chunk_tiles);
+    const int2 win = __ldg(a.win + ens);
+    const float dt = e.dt, qm = e.qm, qm_abs = e.qm_abs, psi_max = e.psi_max;
+    const int k_max = e.k_max, k_short = k_max < kDeferMin - 1 ? k_max : kDeferMin - 1;
+    const float hx0 = __fmul_rn(dt, e.inv_dx), qm_dt = __fmul_rn(qm_abs, dt);
+    const float tp = __fmul_rn(2.0f, psi_max), tp2 = __fmul_rn(tp, tp);
+    const float4* nodes = a.nodes + (int64_t)ens * a.lstride;
+
+    auto whole = [&](int64_t tile) { return (tile + 1) * kTile <= a.n_total; };
+    auto issue = [&](int stage, int r) {
+      if (r < n_tiles && whole(tile0 + r) && lane == 0)
+        tile_issue(a, my_tiles + stage, my_bars + stage, (tile0 + r) * kTile, policy);
+    };
+    issue(0, 0);
+    issue(1, 1);
+    bool gave_up = false;
 #pragma unroll 1
-    for (int r = 0; r < per_lane; ++r, i += 32) {
-      const int64_t inext = i + 32;
-      uint8_t st_n = PIC_STATUS_LOST;
-      MixedState s_n = {0, 0.5f, 0.f, 0.f, 0.f};
-      if (r + 1 < per_lane && inext < end) {
-        st_n = a.status[inext];
-        s_n = {a.cell[inext], a.frac[inext], a.px[inext], a.py[inext], a.pz[inext]};
+    for (int r = 0; r < n_tiles; ++r) {
+      const int stage = r & 1;
+      const int64_t first = (tile0 + r) * kTile;
+      const bool staged = whole(tile0 + r);
+      const Tile& T = my_tiles[stage];
+      if (staged) {
+        if (!mbar_wait(my_bars + stage, (phase >> stage) & 1u)) {
+          // the copies never completed: flag it for the host and leave the
+          // stream, after one more bounded wait for each stage in flight
+          if (lane == 0) atomicExch(&a.stats->error, 1);
+          mbar_wait(my_bars + stage, (phase >> stage) & 1u);
+          if (r + 1 < n_tiles && whole(tile0 + r + 1)) mbar_wait(my_bars + (stage ^ 1), (phase >> (stage ^ 1)) & 1u);
+          gave_up = true;
+          break;
+        }
+        phase ^= 1u << stage;
       }
-      const bool mine = i < end && !(st & PIC_STATUS_LOST) && !(st & kDeferMask) &&
-                        ((st & kParity) == want);
-      int key = -1, sk = 0;
-      if (mine) {
-        int32_t je, jb;
-        float we, wb;
-        const bool inwin = tent_coords(s.cell, s.frac, F.lo, F.hi, je, we, jb, wb);
-        const float* hE = a.half + (int64_t)ens * a.lstride;
-        const float* hB = hE + (int64_t)a.n_ens * a.lstride;
-        const float f0b = __ldg(hB + (jb & a.mask)), f1b = __ldg(hB + ((jb + 1) & a.mask));
-        const float f0e = __ldg(hE + (je & a.mask)), f1e = __ldg(hE + ((je + 1) & a.mask));
-        const float b0 = __fmaf_rn(wb, __fsub_rn(f1b, f0b), f0b);
-        const float ey = __fmaf_rn(we, __fsub_rn(f1e, f0e), f0e);
-        if (!inwin) {
-          a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
-          atomicAdd(&sh[11], 1ull);
+#pragma unroll 1
+      for (int h = 0; h < kTile / 64; ++h) {
+        const int q = h * 32 + lane;
+        const int64_t i = first + 2 * q;
+        uint8_t st0 = PIC_STATUS_LOST, st1 = PIC_STATUS_LOST;
+        MixedState2 s;
+        if (staged) {
+          const uint32_t st2 = reinterpret_cast<const uint16_t*>(T.st)[q];
+          st0 = (uint8_t)st2;
+          st1 = (uint8_t)(st2 >> 8);
+          s.cell = reinterpret_cast<const int2*>(T.cell)[q];
+          s.frac = reinterpret_cast<const float2*>(T.frac)[q];
+          s.ux = reinterpret_cast<const float2*>(T.px)[q];
+          s.uy = reinterpret_cast<const float2*>(T.py)[q];
+          s.uz = reinterpret_cast<const float2*>(T.pz)[q];
         } else {
-          bool capped;
-          const int k = psi_to_k(b0, s, e.qm_abs, e.dt, e.psi_max, e.k_max, capped);
-          count_step(tc, sh, k, capped);
-          const int k_prev = st & 7;
-          if (k == 0) {
-            const float h_old = pow4_down(e.dt, k_prev);
-            const float hp = __fmul_rn(0.5f, __fadd_rn(h_old, e.dt));
-            boris_f32(ey, b0, hp, hx0, e.qm, s);
-            normalize(s);
-            a.cell[i] = s.cell;
-            a.frac[i] = s.frac;
-            a.px[i] = s.ux;
-            a.py[i] = s.uy;
-            a.pz[i] = s.uz;
+          MixedState u0 = {0, 0.5f, 0.f, 0.f, 0.f}, u1 = u0;
+          if (i < a.n_total) {
+            st0 = a.status[i];
+            u0 = load_state(a, i);
+          }
+          if (i + 1 < a.n_total) {
+            st1 = a.status[i + 1];
+            u1 = load_state(a, i + 1);
+          }
+          s.cell = make_int2(u0.cell, u1.cell);
+          s.frac = make_float2(u0.frac, u1.frac);
+          s.ux = make_float2(u0.ux, u1.ux);
+          s.uy = make_float2(u0.uy, u1.uy);
+          s.uz = make_float2(u0.uz, u1.uz);
+        }
+        constexpr uint8_t kStreamMask = PIC_STATUS_LOST | kDeferMask | kParity;
+        const bool mine0 = (st0 & kStreamMask) == want && i >= e_first && i < e_end;
+        const bool mine1 = (st1 & kStreamMask) == want && i + 1 >= e_first && i + 1 < e_end;
+        const PairNodes pn = pair_nodes(s, win.x, win.y);
+        float2 ey, bz, a2, rhs;
+        pair_fields(nodes, a.mask, pn, ey, bz);
+        pair_psi(bz, s, qm_dt, tp2, a2, rhs);
+        const bool big0 = a2.x > rhs.x, big1 = a2.y > rhs.y;
+        bool push0 = mine0 && pn.in0 && !big0, push1 = mine1 && pn.in1 && !big1;
+        int k0 = 0, k1 = 0;
+        const bool side = !__all_sync(0xffffffffu, (push0 || !mine0) && (push1 || !mine1));
+        if (side) {
+          const int2 k = pair_short_k(a2, rhs);
+          k0 = mine0 && pn.in0 && big0 ? k.x : 0;
+          k1 = mine1 && pn.in1 && big1 ? k.y : 0;
+          if (__any_sync(0xffffffffu, k0 > k_short || k1 > k_short || (mine0 && !pn.in0) || (mine1 && !pn.in1))) {
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {  // long sub-cycles, caps below that, particles outside the window
+              int kk = p ? k1 : k0;
+              bool push = false;
+              const uint8_t st = p ? st1 : st0;
+              int key = -1;
+              if ((p ? mine1 : mine0) && !(p ? pn.in1 : pn.in0)) {
+                a.status[i + p] = (uint8_t)(st | PIC_STATUS_LOST);
+                atomicAdd(&sh[11], 1ull);
+              } else if (kk > k_short) {
+                bool capped;
+                const MixedState one = {0, 0.f, p ? s.ux.y : s.ux.x, p ? s.uy.y : s.uy.x, p ? s.uz.y : s.uz.x};
+                kk = psi_to_k(p ? bz.y : bz.x, one, qm_abs, dt, psi_max, k_max, capped);
+                tc.capped += capped ? 1u : 0u;
+                if (kk == 0) {
+                  push = true;  // capped at k_max = 0
+                } else if (kk >= kDeferMin) {
+                  atomicAdd(&sh[kk], 1ull);
+                  batch_defer_mark(a, i + p, st & 7, kk, a.step_cur);
+                  key = ens * 8 + kk;
+                  kk = 0;
+                }
+              }
+              batch_enqueue(a, key, (int32_t)(i + p));
+              k0 = p ? k0 : kk;
+              k1 = p ? kk : k1;
+              push0 |= !p && push;
+              push1 |= p && push;
+            }
+          }
+          tc.k1 += (k0 == 1 ? 1u : 0u) + (k1 == 1 ? 1u : 0u);
+          tc.k2 += (k0 == 2 ? 1u : 0u) + (k1 == 2 ? 1u : 0u);
+        }
+        tc.k0 += (push0 ? 1u : 0u) + (push1 ? 1u : 0u);
+        if (push0 || push1) {
+          const MixedState2 u = pair_push(s, ey, bz, st0, st1, dt, hx0, qm);
+          if (push0 && push1) {  // i even: 8-byte stores
+            __stcs(reinterpret_cast<int2*>(a.cell + i), u.cell);
+            __stcs(reinterpret_cast<float2*>(a.frac + i), u.frac);
+            __stcs(reinterpret_cast<float2*>(a.px + i), u.ux);
+            __stcs(reinterpret_cast<float2*>(a.py + i), u.uy);
+            __stcs(reinterpret_cast<float2*>(a.pz + i), u.uz);
+            *reinterpret_cast<uint16_t*>(a.status + i) = (uint16_t)(done | (done << 8));
+          } else if (push0) {
+            store_stream(a, (uint32_t)i, MixedState{u.cell.x, u.frac.x, u.ux.x, u.uy.x, u.uz.x});
             a.status[i] = done;
-          } else if (k < kDeferMin) {
-            sk = k;
           } else {
-            batch_defer_mark(a, i, k_prev, k, a.step_cur);
-            key = ens * 8 + k;
+            store_stream(a, (uint32_t)i + 1, MixedState{u.cell.y, u.frac.y, u.ux.y, u.uy.y, u.uz.y});
+            a.status[i + 1] = done;
           }
         }
-      }
-      batch_enqueue(a, key, (int32_t)i);
+        if (side) {  // park k = 1, 2 (push_mixed.cu), with the ensemble
+          const unsigned lt = (1u << lane) - 1u;
+          int pos0 = 0, pos1 = 0;
+          bool full = false;
 #pragma unroll
-      for (int q = 0; q < kStashK; ++q) {
-        const unsigned m = __ballot_sync(0xffffffffu, sk == q + 1);
-        if (m == 0u) continue;
-        BatchStash& S = my_stash[q];
-        if (sk == q + 1) {
-          const int pos = stash_n[q] + __popc(m & ((1u << lane) - 1u));
-          S.idx[pos] = (int32_t)i;
-          S.cell[pos] = s.cell;
-          S.frac[pos] = s.frac;
-          S.ux[pos] = s.ux;
-          S.uy[pos] = s.uy;
-          S.uz[pos] = s.uz;
-          S.kp[pos] = (uint8_t)(st & 7);
-          S.ens[pos] = (uint16_t)ens;
+          for (int v = 0; v < kStashK; ++v) {
+            const unsigned m0 = __ballot_sync(0xffffffffu, k0 == v + 1), m1 = __ballot_sync(0xffffffffu, k1 == v + 1);
+            const int n0 = stash_n[v], n1 = n0 + __popc(m0);
+            if (k0 == v + 1) pos0 = n0 + __popc(m0 & lt);
+            if (k1 == v + 1) pos1 = n1 + __popc(m1 & lt);
+            stash_n[v] = n1 + __popc(m1);
+            full |= stash_n[v] >= 32;
+          }
+          if (k0 > 0) {
+            BatchStash& S = my_stash[k0 - 1];
+            stash_put(S.s, pos0, (int32_t)i, MixedState{s.cell.x, s.frac.x, s.ux.x, s.uy.x, s.uz.x}, st0 & 7);
+            S.ens[pos0] = (uint16_t)ens;
+          }
+          if (k1 > 0) {
+            BatchStash& S = my_stash[k1 - 1];
+            stash_put(S.s, pos1, (int32_t)i + 1, MixedState{s.cell.y, s.frac.y, s.ux.y, s.uy.y, s.uz.y}, st1 & 7);
+            S.ens[pos1] = (uint16_t)ens;
+          }
+          __syncwarp();
+          if (full) drain(false);
         }
-        stash_n[q] += __popc(m);
-        __syncwarp();
-        if (stash_n[q] >= 32) batch_stash_drain<P>(a, S, q + 1, stash_n[q], 32, sh);
       }
-      st = st_n;
-      s = s_n;
+      __syncwarp();  // every lane is done with the stage before it is refilled
+      issue(stage, r + 2);
     }
+    if (gave_up) break;
   }
-#pragma unroll
-  for (int q = 0; q < kStashK; ++q)
-    if (stash_n[q] > 0) batch_stash_drain<P>(a, my_stash[q], q + 1, stash_n[q], stash_n[q], sh);
+  drain(true);
   flush_counters(tc, sh, a.stats);
 
   __syncthreads();
@@ -525,9 +618,26 @@ __global__ void batch_reset_status_kernel(uint8_t* status, int64_t n) {
   }
 }
 
-constexpr size_t kBatchStashBytes = sizeof(BatchStash) * kBatchWarps * kStashK;
-
-static_assert(kBatchStashBytes <= 48 * 1024, "stashes must fit the default shared-memory limit");
+// The stream items' ensembles (chunk_first of the table already set).
+__global__ void batch_chunk_kernel(const EnsDev* ens, int32_t n_ens, int64_t n_chunks, int32_t* chunk_ens) {
+  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n_chunks;
+       c += (int64_t)gridDim.x * blockDim.x) {
+    int lo = 0, hi = n_ens - 1;  // last one that starts at or before c
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (ens[mid].chunk_first <= c) lo = mid; else hi = mid - 1;
+    }
+    chunk_ens[c] = lo;
+  }
+}
+cudaError_t launch_batch_chunks(const EnsDev* ens, int32_t n_ens, int64_t n_chunks, int32_t* chunk_ens,
+                                cudaStream_t s) {
+  if (n_chunks <= 0) return cudaSuccess;
+  const int64_t want = (n_chunks + 255) / 256;
+  batch_chunk_kernel<<<(int)(want < 152 * 8 ? want : 152 * 8), 256, 0, s>>>(ens, n_ens, n_chunks, chunk_ens);
+  return cudaGetLastError();
+}
+int batch_tile() { return kTile; }
 
 template <int P>
 static cudaError_t launch_batch_p(const BatchArgs& a, int blocks, cudaStream_t s, int* launches) {
@@ -540,7 +650,7 @@ static cudaError_t launch_batch_p(const BatchArgs& a, int blocks, cudaStream_t s
     batch_halfstep_kernel<P><<<(int)(want < 152 * 16 ? want : 152 * 16), 256, 0, s>>>(a);
     ++n;
   }
-  push_batch_kernel<P><<<blocks, kBatchThreads, kBatchStashBytes, s>>>(a);
+  push_batch_kernel<P><<<blocks, kBatchThreads, kBatchSmem, s>>>(a);
   if (a.finalize) {
     const int64_t want = (a.n_total + 255) / 256;
     batch_reset_status_kernel<<<(int)(want < 152 * 8 ? want : 152 * 8), 256, 0, s>>>(a.status,
@@ -564,14 +674,24 @@ cudaError_t launch_batch_step(const BatchArgs& a, int order, int blocks, cudaStr
   }
 }
 
+template <int P>
+static int batch_occupancy() {
+  int occ = 0;
+  if (cudaFuncSetAttribute(push_batch_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem) ==
+      cudaSuccess)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<P>, kBatchThreads, kBatchSmem);
+  return occ;
+}
+
+// Called at pic_batch_create: also lets the kernel have its shared memory.
 int batch_max_blocks_per_sm(int order) {
   int occ = 0;
   switch (order) {
-    case 1: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<1>, kBatchThreads, kBatchStashBytes); break;
-    case 2: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<2>, kBatchThreads, kBatchStashBytes); break;
-    case 3: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<3>, kBatchThreads, kBatchStashBytes); break;
-    case 4: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<4>, kBatchThreads, kBatchStashBytes); break;
-    case 5: cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<5>, kBatchThreads, kBatchStashBytes); break;
+    case 1: occ = batch_occupancy<1>(); break;
+    case 2: occ = batch_occupancy<2>(); break;
+    case 3: occ = batch_occupancy<3>(); break;
+    case 4: occ = batch_occupancy<4>(); break;
+    case 5: occ = batch_occupancy<5>(); break;
     default: break;
   }
   return occ > 0 ? occ : 1;

@@ -230,6 +230,96 @@ __device__ __forceinline__ void boris_f32x2(float2 ey, float2 bz, float2 hp, flo
   s.frac = fma2(bc2(hx), mul2(ux, inv_g), s.frac);
 }
 
+// ---------------------------------------------------------------- m = 1 pushes from the step's node fields
+
+// Every node's E_y and B_z at t_n and the steps to the next node, {E, dE, B,
+// dB}: the FMA chains gather_f32 takes at the two nodes over the same levels
+// and their difference, so an m = 1 push (and the criterion) that reads them
+// and applies the tent weight gets exactly the bits of the full gather, from
+// one 8-byte load per grid instead of 2(p+1) scattered ones.
+template <int P, class LV>
+__device__ __forceinline__ float4 step_node_f32(const LV& E, const LV& B, const float* wE, const float* wB,
+                                                int32_t c, int32_t mask) {
+  const int32_t c1 = (c + 1) & mask;
+  float e0 = __fmul_rn(wE[0], __ldg(E.at(0) + c)), e1 = __fmul_rn(wE[0], __ldg(E.at(0) + c1));
+  float b0 = __fmul_rn(wB[0], __ldg(B.at(0) + c)), b1 = __fmul_rn(wB[0], __ldg(B.at(0) + c1));
+#pragma unroll
+  for (int l = 1; l <= P; ++l) {
+    e0 = __fmaf_rn(wE[l], __ldg(E.at(l) + c), e0);
+    e1 = __fmaf_rn(wE[l], __ldg(E.at(l) + c1), e1);
+    b0 = __fmaf_rn(wB[l], __ldg(B.at(l) + c), b0);
+    b1 = __fmaf_rn(wB[l], __ldg(B.at(l) + c1), b1);
+  }
+  return make_float4(e0, __fsub_rn(e1, e0), b0, __fsub_rn(b1, b0));
+}
+__device__ __forceinline__ float2 node_e(const float4* nodes, int32_t j) {
+  return __ldg(reinterpret_cast<const float2*>(nodes + j));
+}
+__device__ __forceinline__ float2 node_b(const float4* nodes, int32_t j) {
+  return __ldg(reinterpret_cast<const float2*>(nodes + j) + 1);
+}
+__device__ __forceinline__ float node_lerp_e(const float4* nodes, int32_t j, float w) {
+  const float2 v = node_e(nodes, j);
+  return __fmaf_rn(w, v.y, v.x);
+}
+__device__ __forceinline__ float node_lerp_b(const float4* nodes, int32_t j, float w) {
+  const float2 v = node_b(nodes, j);
+  return __fmaf_rn(w, v.y, v.x);
+}
+
+// tent_coords of two particles.
+struct PairNodes {
+  int2 je, jb;
+  float2 we, wb;
+  bool in0, in1;
+};
+__device__ __forceinline__ PairNodes pair_nodes(const MixedState2& s, int32_t lo, int32_t hi) {
+  PairNodes n;
+  const float2 fe = floor2(s.frac);
+  const float2 fbm = add2(s.frac, bc2(-0.5f));
+  const float2 fb = floor2(fbm);
+  n.we = sub2(s.frac, fe);
+  n.wb = sub2(fbm, fb);
+  n.je = make_int2(s.cell.x + (int32_t)fe.x, s.cell.y + (int32_t)fe.y);
+  n.jb = make_int2(s.cell.x + (int32_t)fb.x, s.cell.y + (int32_t)fb.y);
+  n.in0 = n.jb.x >= lo && n.je.x < hi;
+  n.in1 = n.jb.y >= lo && n.je.y < hi;
+  return n;
+}
+__device__ __forceinline__ void pair_fields(const float4* nodes, int32_t mask, const PairNodes& n, float2& ey,
+                                            float2& bz) {
+  const float2 e0 = node_e(nodes, n.je.x & mask), e1 = node_e(nodes, n.je.y & mask);
+  const float2 b0 = node_b(nodes, n.jb.x & mask), b1 = node_b(nodes, n.jb.y & mask);
+  ey = fma2(n.we, make_float2(e0.y, e1.y), make_float2(e0.x, e1.x));
+  bz = fma2(n.wb, make_float2(b0.y, b1.y), make_float2(b0.x, b1.x));
+}
+// psi_terms of each; qm_dt = |q/m| dt, tp2 = (2 Psi_max)^2.
+__device__ __forceinline__ void pair_psi(float2 bz, const MixedState2& s, float qm_dt, float tp2, float2& a2,
+                                         float2& rhs) {
+  const float2 av = mul2(bc2(qm_dt), bz);
+  a2 = mul2(av, av);
+  rhs = mul2(bc2(tp2), add2(bc2(1.0f), fma2(s.uz, s.uz, fma2(s.uy, s.uy, mul2(s.ux, s.ux)))));
+}
+// psi_to_k of particles with k >= 1, uncapped, as far as 3 (= 3 or more).
+__device__ __forceinline__ int2 pair_short_k(float2 a2, float2 rhs) {
+  const float2 r16 = mul2(rhs, bc2(16.0f)), r256 = mul2(r16, bc2(16.0f));
+  return make_int2(1 + (a2.x > r16.x ? 1 : 0) + (a2.x > r256.x ? 1 : 0),
+                   1 + (a2.y > r16.y ? 1 : 0) + (a2.y > r256.y ? 1 : 0));
+}
+// The m = 1 push of two particles, k_prev in bits 0-2 of their status.
+__device__ __forceinline__ MixedState2 pair_push(const MixedState2& s, float2 ey, float2 bz, uint8_t st0,
+                                                 uint8_t st1, float dt, float hx0, float qm) {
+  const float2 h_old = make_float2(pow4_down(dt, st0 & 7), pow4_down(dt, st1 & 7));
+  const float2 hp = mul2(bc2(0.5f), add2(h_old, bc2(dt)));
+  MixedState2 u = s;
+  boris_f32x2(ey, bz, hp, hx0, qm, u);
+  const float2 fl = floor2(u.frac);  // normalize each
+  u.cell.x += (int32_t)fl.x;
+  u.cell.y += (int32_t)fl.y;
+  u.frac = sub2(u.frac, fl);
+  return u;
+}
+
 // Reciprocal of prod_{k != j} (j - k), the denominator of L_{p,j} (Sec. VI).
 __host__ __device__ constexpr float lagrange_inv_den(int p, int j) {
   float d = 1.f;
@@ -689,7 +779,8 @@ __device__ __forceinline__ void flush_counters(const ThreadCounters& tc, unsigne
   }
 }
 
-__device__ __forceinline__ MixedState load_state(const PushArgsMixed& a, int64_t i) {
+template <class ARGS>
+__device__ __forceinline__ MixedState load_state(const ARGS& a, int64_t i) {
   MixedState s;
   s.cell = a.cell[i];
   s.frac = a.frac[i];
@@ -699,7 +790,8 @@ __device__ __forceinline__ MixedState load_state(const PushArgsMixed& a, int64_t
   return s;
 }
 
-__device__ __forceinline__ void store_state(const PushArgsMixed& a, int64_t i, const MixedState& s) {
+template <class ARGS>
+__device__ __forceinline__ void store_state(const ARGS& a, int64_t i, const MixedState& s) {
   a.cell[i] = s.cell;
   a.frac[i] = s.frac;
   a.px[i] = s.ux;
@@ -725,7 +817,8 @@ __device__ __forceinline__ void fetch_stream(const PushArgsMixed& a, uint32_t i,
   }
 }
 
-__device__ __forceinline__ void store_stream(const PushArgsMixed& a, uint32_t i, const MixedState& s) {
+template <class ARGS>
+__device__ __forceinline__ void store_stream(const ARGS& a, uint32_t i, const MixedState& s) {
   __stcs(a.cell + i, s.cell);
   __stcs(a.frac + i, s.frac);
   __stcs(a.px + i, s.ux);
@@ -800,7 +893,8 @@ __device__ __forceinline__ void bulk_to_smem(void* dst, const void* src, uint32_
 }
 // One lane: stage particles [first, first + kTile) into t (all of them exist,
 // the arrays are 16-byte aligned and first is a multiple of kTile).
-__device__ __forceinline__ void tile_issue(const PushArgsMixed& a, Tile* t, uint64_t* bar,
+template <class ARGS>
+__device__ __forceinline__ void tile_issue(const ARGS& a, Tile* t, uint64_t* bar,
                                            int64_t first, uint64_t policy) {
   mbar_expect(bar, kTileBytes);
   bulk_to_smem(t->cell, a.cell + first, kTile * 4, bar, policy);

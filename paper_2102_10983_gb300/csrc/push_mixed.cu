@@ -84,15 +84,11 @@ void lagrange_monomials(int p, float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1]) {
 // ---------------------------------------------------------------- half-step fields
 
 // Every window node's E_y and B_z interpolated to t_n with the theta = 1/2
-// weights: the same FMA chain over the same levels as gather_f32 takes at one
-// node, so an m = 1 push (and the criterion) that reads these two nodes and
-// applies the tent weight gets exactly the bits of the full gather, from two
-// loads per grid instead of 2(p+1).
-//
-// With coef set, the same pass also writes each node's monomial coefficients
-// (to_monomial over the same levels, so the same bits): E_y's p+1 then B_z's.
+// weights, and the steps to the next node (step_node_f32).  With coef set, the
+// same pass also writes each node's monomial coefficients (to_monomial over
+// the same levels, so the same bits): E_y's p+1 then B_z's.
 template <int P>
-__global__ void halfstep_kernel(PushArgsMixed a, int64_t W, float* outE, float* outB, float* coef) {
+__global__ void halfstep_kernel(PushArgsMixed a, int64_t W, float4* nodes, float* coef) {
   constexpr int stride = 2 * (P + 1);
   const float* wB = a.wtab + a.crit_row * stride + (P + 1);
   const float* wE = a.wtab + wrow(0, 1) * stride;
@@ -100,23 +96,11 @@ __global__ void halfstep_kernel(PushArgsMixed a, int64_t W, float* outE, float* 
   load_fields<P, true>(F, a, false);
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < W;
        c += (int64_t)gridDim.x * blockDim.x) {
-    float fe = __fmul_rn(wE[0], __ldg(F.E.at(0) + c));
-    float fb = __fmul_rn(wB[0], __ldg(F.B.at(0) + c));
-#pragma unroll
-    for (int l = 1; l <= P; ++l) {
-      fe = __fmaf_rn(wE[l], __ldg(F.E.at(l) + c), fe);
-      fb = __fmaf_rn(wB[l], __ldg(F.B.at(l) + c), fb);
-    }
-    outE[c] = fe;
-    outB[c] = fb;
-    if (c == 0) {  // padding node W: the circular successor of node W - 1
-      outE[W] = fe;
-      outB[W] = fb;
-    }
+    nodes[c] = step_node_f32<P>(F.E, F.B, wE, wB, (int32_t)c, a.mask);
     if (coef) {
-      float e0[P + 1], e1[P + 1], b0[P + 1], b1[P + 1];
-      to_monomial<P>(F.E, (int32_t)c, (int32_t)c, a.mono[0], e0, e1);
-      to_monomial<P>(F.B, (int32_t)c, (int32_t)c, a.mono[1], b0, b1);
+      float e0[P + 1], b0[P + 1];
+      to_monomial1<P>(F.E, (int32_t)c, a.mono[0], e0);
+      to_monomial1<P>(F.B, (int32_t)c, a.mono[1], b0);
       float* r = coef + c * stride;
 #pragma unroll
       for (int q = 0; q <= P; ++q) {
@@ -127,28 +111,19 @@ __global__ void halfstep_kernel(PushArgsMixed a, int64_t W, float* outE, float* 
   }
 }
 
-cudaError_t launch_halfstep(const PushArgsMixed& a, int order, int64_t W, float* outE, float* outB,
-                            float* coef, cudaStream_t s) {
+cudaError_t launch_halfstep(const PushArgsMixed& a, int order, int64_t W, float4* nodes, float* coef,
+                            cudaStream_t s) {
   const int64_t want = (W + 255) / 256;
   const int blocks = (int)(want < 152 * 8 ? want : 152 * 8);
   switch (order) {
-    case 1: halfstep_kernel<1><<<blocks, 256, 0, s>>>(a, W, outE, outB, coef); break;
-    case 2: halfstep_kernel<2><<<blocks, 256, 0, s>>>(a, W, outE, outB, coef); break;
-    case 3: halfstep_kernel<3><<<blocks, 256, 0, s>>>(a, W, outE, outB, coef); break;
-    case 4: halfstep_kernel<4><<<blocks, 256, 0, s>>>(a, W, outE, outB, coef); break;
-    case 5: halfstep_kernel<5><<<blocks, 256, 0, s>>>(a, W, outE, outB, coef); break;
+    case 1: halfstep_kernel<1><<<blocks, 256, 0, s>>>(a, W, nodes, coef); break;
+    case 2: halfstep_kernel<2><<<blocks, 256, 0, s>>>(a, W, nodes, coef); break;
+    case 3: halfstep_kernel<3><<<blocks, 256, 0, s>>>(a, W, nodes, coef); break;
+    case 4: halfstep_kernel<4><<<blocks, 256, 0, s>>>(a, W, nodes, coef); break;
+    case 5: halfstep_kernel<5><<<blocks, 256, 0, s>>>(a, W, nodes, coef); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
-}
-
-// Tent interpolation of a half-step field between nodes j, j+1.  The array
-// holds W + 1 nodes, node W repeating node 0, so the pair never wraps.
-__device__ __forceinline__ float half_lerp(const float* f, int32_t j, float w, int32_t mask) {
-  const float* q = f + (j & mask);
-  const float f0 = __ldg(q);
-  const float f1 = __ldg(q + 1);
-  return __fmaf_rn(w, __fsub_rn(f1, f0), f0);
 }
 
 // ---------------------------------------------------------------- PLAIN schedule
@@ -178,8 +153,8 @@ __global__ void __launch_bounds__(256) push_mixed_plain_kernel(PushArgsMixed a) 
     bool capped;
     float b0;
     int k;
-    if (a.halfE) {
-      b0 = half_lerp(a.halfB, jb, wb, a.mask);
+    if (a.nodes) {
+      b0 = node_lerp_b(a.nodes, jb & a.mask, wb);
       k = psi_to_k(b0, s, a.qm_abs, a.dt, a.psi_max, a.k_max, capped);
     } else {
       k = criterion_f32<P>(F.B, wcrit, jb, wb, a.mask, s, a.qm_abs, a.dt, a.psi_max, a.k_max,
@@ -187,10 +162,10 @@ __global__ void __launch_bounds__(256) push_mixed_plain_kernel(PushArgsMixed a) 
     }
     count_step(tc, sh, k, capped);
     bool ok = true;
-    if (k == 0 && a.halfE) {
+    if (k == 0 && a.nodes) {
       const float h_old = pow4_down(a.dt, st & 0x7f);
       const float hp = __fmul_rn(0.5f, __fadd_rn(h_old, a.dt));
-      boris_f32(half_lerp(a.halfE, je, we, a.mask), b0, hp, __fmul_rn(a.dt, a.inv_dx), a.qm, s);
+      boris_f32(node_lerp_e(a.nodes, je & a.mask, we), b0, hp, __fmul_rn(a.dt, a.inv_dx), a.qm, s);
     } else {
       ok = subcycle_f32<P>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.mono, k,
                            st & 0x7f, b0, s);
@@ -482,35 +457,19 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
       s.uz = make_float2(u0.uz, u1.uz);
     }
     const bool mine0 = (st0 & kStreamMask) == want, mine1 = (st1 & kStreamMask) == want;
-    const float2 fe = floor2(s.frac);  // tent_coords of each
-    const float2 fbm = add2(s.frac, bc2(-0.5f));
-    const float2 fb = floor2(fbm);
-    const float2 we = sub2(s.frac, fe), wb = sub2(fbm, fb);
-    const int32_t je0 = s.cell.x + (int32_t)fe.x, je1 = s.cell.y + (int32_t)fe.y;
-    const int32_t jb0 = s.cell.x + (int32_t)fb.x, jb1 = s.cell.y + (int32_t)fb.y;
-    const bool in0 = jb0 >= F.lo && je0 < F.hi, in1 = jb1 >= F.lo && je1 < F.hi;
-    float2 ey, bz;  // half_lerp of each, or gather_f32 without half-step fields
-    if (a.halfE) {
-      const float* e0 = a.halfE + (je0 & a.mask);
-      const float* e1 = a.halfE + (je1 & a.mask);
-      const float* b0 = a.halfB + (jb0 & a.mask);
-      const float* b1 = a.halfB + (jb1 & a.mask);
-      const float2 elo = make_float2(__ldg(e0), __ldg(e1));
-      const float2 ehi = make_float2(__ldg(e0 + 1), __ldg(e1 + 1));
-      const float2 blo = make_float2(__ldg(b0), __ldg(b1));
-      const float2 bhi = make_float2(__ldg(b0 + 1), __ldg(b1 + 1));
-      ey = fma2(we, sub2(ehi, elo), elo);
-      bz = fma2(wb, sub2(bhi, blo), blo);
+    const PairNodes pn = pair_nodes(s, F.lo, F.hi);
+    float2 ey, bz;
+    if (RING || a.nodes) {
+      pair_fields(a.nodes, a.mask, pn, ey, bz);
     } else {
-      ey = make_float2(gather_f32<P>(F.E, w0, je0, we.x, a.mask),
-                       gather_f32<P>(F.E, w0, je1, we.y, a.mask));
-      bz = make_float2(gather_f32<P>(F.B, wcrit, jb0, wb.x, a.mask),
-                       gather_f32<P>(F.B, wcrit, jb1, wb.y, a.mask));
+      ey = make_float2(gather_f32<P>(F.E, w0, pn.je.x, pn.we.x, a.mask),
+                       gather_f32<P>(F.E, w0, pn.je.y, pn.we.y, a.mask));
+      bz = make_float2(gather_f32<P>(F.B, wcrit, pn.jb.x, pn.wb.x, a.mask),
+                       gather_f32<P>(F.B, wcrit, pn.jb.y, pn.wb.y, a.mask));
     }
-    const float2 av = mul2(bc2(qm_dt), bz);  // psi_terms of each
-    const float2 a2 = mul2(av, av);
-    const float2 rhs =
-        mul2(bc2(tp2), add2(bc2(1.0f), fma2(s.uz, s.uz, fma2(s.uy, s.uy, mul2(s.ux, s.ux)))));
+    const bool in0 = pn.in0, in1 = pn.in1;
+    float2 a2, rhs;
+    pair_psi(bz, s, qm_dt, tp2, a2, rhs);
     const bool big0 = a2.x > rhs.x, big1 = a2.y > rhs.y;
     bool push0 = mine0 && in0 && !big0;
     bool push1 = mine1 && in1 && !big1;
@@ -518,10 +477,9 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
     int k0 = 0, k1 = 0;  // k of the particles that sub-cycle
     bool rare = false;
     if (side) {
-      // the rest of the criterion's comparisons (psi_to_k): k = 1, 2, or more
-      const float2 r16 = mul2(rhs, bc2(16.0f)), r256 = mul2(r16, bc2(16.0f));
-      k0 = mine0 && in0 && big0 ? 1 + (a2.x > r16.x ? 1 : 0) + (a2.x > r256.x ? 1 : 0) : 0;
-      k1 = mine1 && in1 && big1 ? 1 + (a2.y > r16.y ? 1 : 0) + (a2.y > r256.y ? 1 : 0) : 0;
+      const int2 k = pair_short_k(a2, rhs);
+      k0 = mine0 && in0 && big0 ? k.x : 0;
+      k1 = mine1 && in1 && big1 ? k.y : 0;
       // long sub-cycles, caps below that and particles outside the window
       rare = __any_sync(0xffffffffu, k0 > k_short || k1 > k_short || (mine0 && !in0) || (mine1 && !in1));
       if (rare) {
@@ -563,14 +521,7 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
     const MixedState p0 = {s.cell.x, s.frac.x, s.ux.x, s.uy.x, s.uz.x};  // as loaded, for the stash
     const MixedState p1 = {s.cell.y, s.frac.y, s.ux.y, s.uy.y, s.uz.y};
     if (push0 || push1) {
-      const float2 h_old = make_float2(pow4_down(a.dt, st0 & 7), pow4_down(a.dt, st1 & 7));
-      const float2 hp = mul2(bc2(0.5f), add2(h_old, bc2(a.dt)));
-      MixedState2 u = s;
-      boris_f32x2(ey, bz, hp, hx0, a.qm, u);
-      const float2 fl = floor2(u.frac);  // normalize each
-      u.cell.x += (int32_t)fl.x;
-      u.cell.y += (int32_t)fl.y;
-      u.frac = sub2(u.frac, fl);
+      const MixedState2 u = pair_push(s, ey, bz, st0, st1, a.dt, hx0, a.qm);
       if (push0 && push1 && a.tma) {  // 16-byte aligned arrays, i even: 8-byte stores
         __stcs(reinterpret_cast<int2*>(a.cell + i), u.cell);
         __stcs(reinterpret_cast<float2*>(a.frac + i), u.frac);
@@ -808,13 +759,13 @@ cudaError_t launch_feature_nodes(const PushArgsMixed& a, int order, int64_t W, f
   return cudaGetLastError();
 }
 
-// phi of every particle after macro step n (see particle_features; a.halfE,
-// a.halfB: the feature nodes of step n).
+// phi of every particle after macro step n (see particle_features; a.featE,
+// a.featB: the feature nodes of step n).
 __global__ void features_kernel(PushArgsMixed a, float* phi) {
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
        i += (int64_t)gridDim.x * blockDim.x) {
     float f[6];
-    particle_features(a, a.halfE, a.halfB, a.lo, a.hi, i, f);
+    particle_features(a, a.featE, a.featB, a.lo, a.hi, i, f);
 #pragma unroll
     for (int q = 0; q < 6; ++q) phi[i * 6 + q] = f[q];
   }
