@@ -39,9 +39,10 @@ struct pic_batch {
   int32_t* qcount = nullptr;  // 2 x n_ens x 8, then cursor, blocks done
   int64_t* prefix = nullptr;  // 7 n_ens + 1
   float4* nodes = nullptr;    // n_ens x W: the step's node fields
-  int2* win = nullptr;        // 2 (step parity) x n_ens: the steps' windows
+  int2* win = nullptr;        // T x n_ens: the steps' windows
+  int32_t T = 2;              // steps whose tables and windows are kept (coef_steps_kept)
   int32_t* chunk_ens = nullptr;  // the stream items' ensembles
-  float* coef = nullptr;      // 2 (step parity) x n_ens x W x 2(p+1): node coefficient tables
+  float* coef = nullptr;      // T x n_ens x W x 2(p+1): node coefficient tables, step s's s mod T
   int32_t* lag_step = nullptr;  // per particle: the step a deferred particle is in (call-relative)
   uint16_t* lag_j = nullptr;    // and the sub-steps of it done
   int32_t heavy_budget = 1024;  // sub-steps of long sub-cycles per particle and launch
@@ -160,9 +161,11 @@ extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t 
   A((void**)&b->qcount, sizeof(int32_t) * (2 * 8 * (size_t)n_ens + 8));
   A((void**)&b->prefix, sizeof(int64_t) * (7 * (size_t)n_ens + 1));
   A((void**)&b->nodes, sizeof(float4) * (size_t)n_ens * window_cells);
-  A((void**)&b->win, sizeof(int2) * 2 * (size_t)n_ens);
+  const size_t table_bytes = sizeof(float) * (size_t)n_ens * window_cells * 2 * (size_t)(order + 1);
+  b->T = coef_steps_kept(table_bytes);
+  A((void**)&b->win, sizeof(int2) * b->T * (size_t)n_ens);
   A((void**)&b->chunk_ens, sizeof(int32_t) * (cap / batch_tile() + 2 * (size_t)n_ens + 1));
-  A((void**)&b->coef, sizeof(float) * 2 * (size_t)n_ens * window_cells * 2 * (size_t)(order + 1));
+  A((void**)&b->coef, b->T * table_bytes);
   A((void**)&b->lag_step, cap * 4);
   A((void**)&b->lag_j, cap * 2);
   if (e != cudaSuccess) {
@@ -386,12 +389,18 @@ static int queue_steps(pic_batch* b, int64_t n, int64_t n_steps) {
     a.step0 = n;
     a.step_cur = fin ? s + 1 : s;  // the closing launch brings every particle to the end of s
     a.heavy_budget = b->heavy_budget;
-    // node tables by step parity; the closing launch finishes step s with its own
+    // node tables and windows by step; the closing launch finishes step s with its own
     const int64_t table = b->n_ens * b->W * 2 * (p + 1);
-    a.coef = b->coef + (s & 1) * table;
-    a.coef_p = (j > 0 && !fin) ? b->coef + ((s - 1) & 1) * table : a.coef;
-    a.win = b->win + (s & 1) * b->n_ens;
-    a.win_p = (j > 0 && !fin) ? b->win + ((s - 1) & 1) * b->n_ens : a.win;
+    const int64_t at = ((s % b->T) + b->T) % b->T, before = (((s - 1) % b->T) + b->T) % b->T;
+    a.coef_all = b->coef;
+    a.win_all = b->win;
+    a.coef_stride = table;
+    a.steps_kept = b->T;
+    a.oldest_kept = s - b->T + 1;  // a deferred particle is in a step of this call
+    a.coef = b->coef + at * table;
+    a.coef_p = (j > 0 && !fin) ? b->coef + before * table : a.coef;
+    a.win = b->win + at * b->n_ens;
+    a.win_p = (j > 0 && !fin) ? b->win + before * b->n_ens : a.win;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (b->timing && !fin) {
       int rc = batch_timing_pair(b, &e0, &e1);

@@ -41,7 +41,8 @@ struct pic_ctx {
   // predicted schedule
   uint8_t* pred = nullptr;
   float4* nodes = nullptr;  // mixed form: the step's node fields (PushArgsMixed::nodes)
-  float* coef = nullptr;  // mixed form: per node monomial coefficients, two steps (parity of s)
+  float* coef = nullptr;  // mixed form: per node monomial coefficients, step s's in table s mod T
+  int32_t T = 2;          // tables kept (coef_steps_kept)
   float* feat = nullptr;  // mixed form: the predictor's feature nodes (E_y, B_z at t_{n+1}), W + 1 each
   // binned mixed form: resumable long sub-cycles (per particle: the step it is
   // in and the sub-steps done), and a device copy of slot_i0 for the kernel
@@ -214,7 +215,9 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
   };
   if (mixed) {
     A((void**)&c->nodes, (size_t)window_cells * sizeof(float4));
-    A((void**)&c->coef, 2 * (size_t)window_cells * 2 * (prm->order + 1) * 4);
+    const size_t table = (size_t)window_cells * 2 * (prm->order + 1) * 4;
+    c->T = prm->schedule == PIC_SCHED_PLAIN ? 2 : coef_steps_kept(table);
+    A((void**)&c->coef, c->T * table);
     A((void**)&c->feat, 2 * ((size_t)window_cells + 1) * 4);
     A((void**)&c->cell, cap * 4);
     A((void**)&c->frac, cap * 4);
@@ -572,6 +575,10 @@ static void fill_mixed(pic_ctx* c, PushArgsMixed& a, int64_t s, int64_t lo, int6
   }
 }
 
+static float* coef_table(const pic_ctx* c, int64_t s) {
+  return c->coef + (((s % c->T) + c->T) % c->T) * (c->W * 2 * (c->prm.order + 1));
+}
+
 // Launch arguments of the mixed form common to every launch of a call.
 static void mixed_base(pic_ctx* c, PushArgsMixed& base) {
   memset(&base, 0, sizeof(base));
@@ -604,6 +611,9 @@ static void mixed_base(pic_ctx* c, PushArgsMixed& base) {
     base.heavy_budget = c->heavy_budget;
     base.ring_R = c->R;
     base.slot_i0 = c->dslot_i0;  // kept current by pic_fields_upload, in stream order
+    base.coef_all = c->coef;
+    base.coef_stride = c->W * 2 * (c->prm.order + 1);
+    base.coef_steps = c->T;
   }
 }
 
@@ -643,9 +653,9 @@ static int close_open(pic_ctx* c) {
   a.step0 = c->open_step0;
   a.step_cur = S;
   fill_mixed(c, a, S, lo, hi, false);
-  const int64_t coef_stride = c->W * 2 * (c->prm.order + 1);
-  const float* coef_s = c->coef + (S & 1) * coef_stride;
+  const float* coef_s = coef_table(c, S);
   a.coef = coef_s;
+  a.coef_oldest = S - c->T + 1;
   a.nodes = c->nodes;
   const int64_t J = c->run_j - 1;
   a.parity_cur = (int)(J & 1);
@@ -752,16 +762,18 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
       a.step_cur = s;
       fill_mixed(c, a, s, lo, hi, false);
       // this step's fields at t_n on every window node (the m = 1 pushes) and
-      // its node coefficient table (the sub-cycles); the previous step's table
-      // is the other half of c->coef
-      const int64_t coef_stride = W * 2 * (p + 1);
-      float* coef_cur = c->coef + (s & 1) * coef_stride;
-      float* coef_prev = c->coef + ((s - 1) & 1) * coef_stride;
+      // its node coefficient table (the sub-cycles); the previous steps' tables
+      // stay
+      float* coef_cur = coef_table(c, s);
+      float* coef_prev = coef_table(c, s - 1);
       e = launch_halfstep(a, p, W, c->nodes, coef_cur, c->stream);
       ++launches;
       if (e != cudaSuccess) return fail(c, PIC_ECUDA, "half-step launch: %s", cudaGetErrorString(e));
       a.nodes = c->nodes;
       a.coef = coef_cur;
+      // a deferred particle is in a step of this run, whose table this run made
+      // and whose levels pic_fields_upload has kept
+      a.coef_oldest = s - c->T + 1;
       // deferred work of the previous step: from this call's last launch, or
       // carried from the last call
       const bool has_prev = j > 0 || cont;

@@ -124,6 +124,12 @@ struct PushArgsMixed {
   // (coef_p); nullptr = form them from the levels
   const float* coef;
   const float* coef_p;
+  // the tables of the last coef_steps steps, step s's at (s mod coef_steps)
+  // coef_stride; a deferred particle in a step before coef_oldest (or the run's
+  // first) forms its coefficients from the levels
+  const float* coef_all;
+  int64_t coef_stride, coef_oldest;
+  int32_t coef_steps;
   int32_t lo, hi;      // tent node j must satisfy lo <= j and j+1 <= hi
   int32_t lo_p, hi_p;  // same for the previous step
   int32_t mask;
@@ -174,6 +180,14 @@ struct PushArgsMixed {
 // Fills PushArgsMixed::mono for order p (host side, FP64 expansion).
 void lagrange_monomials(int p, float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1]);
 
+// Steps whose node coefficient tables (table_bytes each) a context keeps: a
+// deferred particle a few steps behind the stream then reads a table as the
+// others of its warp do, instead of a path of its own; as many as 256 MB hold.
+inline int32_t coef_steps_kept(size_t table_bytes) {
+  const size_t n = ((size_t)256 << 20) / (table_bytes > 0 ? table_bytes : 1);
+  return (int32_t)(n < 2 ? 2 : n > 16 ? 16 : n);
+}
+
 // Sets the reason pic_last_error(NULL) reports.
 void set_global_error(const char* msg);
 
@@ -216,12 +230,17 @@ struct BatchArgs {
   const int64_t* prefix;  // [7*n_ens + 1] heavy-item prefix (filled per launch)
   float4* nodes;          // [n_ens][W]: step_node_f32 of every node (filled per launch)
   int2* win;              // [n_ens] this step's windows [lo, hi] (filled per launch)
-  const int2* win_p;      // and the previous step's; two such tables, by step parity
+  const int2* win_p;      // and the previous step's
+  const int2* win_all;    // the steps' kept, as coef_all, n_ens apart
   // [n_ens][W][2(p+1)]: every node's monomial coefficients of the temporal
   // interpolant (E_y then B_z) of this step (coef, filled per launch) and of
-  // the previous one (coef_p); two such tables, by step parity
+  // the previous one (coef_p); coef_all: the tables of the last steps kept,
+  // step s's at (s mod steps_kept) coef_stride, from step oldest_kept on
   float* coef;
   const float* coef_p;
+  const float* coef_all;
+  int64_t coef_stride, oldest_kept;
+  int32_t steps_kept;
   int* cursor;
   unsigned* blocks_done;
   int parity_cur, parity_next, finalize;

@@ -103,21 +103,28 @@ __device__ __forceinline__ void batch_stash_drain(const BatchArgs& a, const Batc
   n -= cnt;
 }
 
-// Field view of macro step s of ensemble e from its mirrored ring and the
-// device copy of its slots' window origins: for a deferred particle that runs
-// behind the stream (no node table).
+// Field view of macro step s of ensemble e from its mirrored ring: for a
+// deferred particle that runs behind the stream.  With the step's table and
+// window where they are kept, else from the slots' window origins.
 template <int P>
 __device__ __forceinline__ StepFields<P, true> ens_step_fields(const BatchArgs& a, const EnsDev& e,
                                                                int64_t s) {
   StepFields<P, true> F;
-  const int64_t R = a.R;
+  const int64_t R = a.R, T = a.steps_kept, q = &e - a.ens;
   const int64_t start = ((s - P) % R + R) % R;
   F.E.base = e.ringE + start * a.lstride;
   F.B.base = e.ringB + start * a.lstride;
   F.E.lstride = (int32_t)a.lstride;
   F.B.lstride = (int32_t)a.lstride;
   F.coef = nullptr;
-  const int2 win = ens_window<P>(a, e, start);
+  int2 win;
+  if (s >= a.oldest_kept) {
+    const int64_t at = (s % T + T) % T;
+    F.coef = a.coef_all + at * a.coef_stride + q * a.lstride * (2 * (P + 1));
+    win = __ldg(a.win_all + at * a.n_ens + q);
+  } else {
+    win = ens_window<P>(a, e, start);
+  }
   F.lo = win.x;
   F.hi = win.y;
   return F;
@@ -174,15 +181,14 @@ __device__ __forceinline__ void batch_heavy(const BatchArgs& a, int ens, int64_t
     int j1 = m;
     if (k >= kDeferMin && m - j0 > budget) j1 = j0 + budget;
     bool ok;
-    if (si >= a.step_cur - 1) {  // the previous or the current step: node tables
-      const StepFields<P, true> Fs = si == a.step_cur ? Fc : Fp;
+    StepFields<P, true> Fs = si == a.step_cur ? Fc : Fp;
+    if (si < a.step_cur - 1) Fs = ens_step_fields<P>(a, e, si);
+    if (Fs.coef)
       ok = subcycle_f32<P, true, true>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.mono,
                                        k, k_prev, b0, s, j0, j1);
-    } else {
-      const StepFields<P, true> Fs = ens_step_fields<P>(a, e, si);
+    else  // further behind than the tables kept
       ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time,
                                         a.mono, k, k_prev, b0, s, j0, j1);
-    }
     if (k >= kDeferMin) budget -= j1 - j0;
     if (!ok) {
       lose();
@@ -231,7 +237,7 @@ __device__ __forceinline__ void batch_heavy(const BatchArgs& a, int ens, int64_t
     }
     // behind the stream: the next step's criterion, then its sub-cycle
     si += 1;
-    const StepFields<P, true> Fs = si == a.step_cur - 1 ? Fp : ens_step_fields<P>(a, e, si);
+    Fs = si == a.step_cur - 1 ? Fp : ens_step_fields<P>(a, e, si);
     int32_t je, jb;
     float we, wb;
     if (!tent_coords(s.cell, s.frac, Fs.lo, Fs.hi, je, we, jb, wb)) {

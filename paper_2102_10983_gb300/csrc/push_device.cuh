@@ -999,7 +999,7 @@ __device__ __forceinline__ void particle_features(const PushArgsMixed& a, const 
 
 // Field view of macro step s from the mirrored ring and the device copy of
 // the slots' window origins (the host's step_slots / fill_mixed, on the GPU):
-// for a deferred particle that runs behind the stream.  No node table.
+// for a deferred particle that runs behind the stream.
 template <int P>
 __device__ __forceinline__ StepFields<P, true> ring_step_fields(const PushArgsMixed& a, int64_t s) {
   StepFields<P, true> F;
@@ -1009,7 +1009,8 @@ __device__ __forceinline__ StepFields<P, true> ring_step_fields(const PushArgsMi
   F.B.base = a.ringB + start * a.lstride;
   F.E.lstride = (int32_t)a.lstride;
   F.B.lstride = (int32_t)a.lstride;
-  F.coef = nullptr;
+  const int64_t T = a.coef_steps;
+  F.coef = s >= a.coef_oldest ? a.coef_all + ((s % T + T) % T) * a.coef_stride : nullptr;
   int64_t lo = INT64_MIN, hi = INT64_MAX;
 #pragma unroll
   for (int l = 0; l <= P; ++l) {
@@ -1161,19 +1162,20 @@ __device__ __forceinline__ void heavy_particle(const PushArgsMixed& a, const Ste
     const int m = 1 << (2 * k);
     int j1 = m;
     if (k >= kDeferMin && m - j0 > budget && si >= a.keep_step) j1 = j0 + budget;
-    bool ok;
-    if (si >= a.step_cur - 1) {  // the previous or the current step: node tables
-      const StepFields<P, RING> Fs = si == a.step_cur ? Fc : Fp;
+    bool ok = false;
+    // the particle's own step's fields, so that a warp whose particles are in
+    // different steps still runs their sub-steps together
+    StepFields<P, RING> Fs = si == a.step_cur ? Fc : Fp;
+    if constexpr (RING) {
+      if (si < a.step_cur - 1) Fs = ring_step_fields<P>(a, si);
+    }
+    if (!RING || Fs.coef) {
       ok = subcycle_site<P, RING, RING>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time,
                                         a.mono, k, k_prev, b0, s, j0, j1);
-    } else {
-      if constexpr (RING) {
-        const StepFields<P, true> Fs = ring_step_fields<P>(a, si);
+    } else {  // further behind than the tables kept
+      if constexpr (RING)
         ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time,
                                           a.mono, k, k_prev, b0, s, j0, j1);
-      } else {
-        ok = false;  // unreachable: without the lag arrays si is always the previous step
-      }
     }
     if (k >= kDeferMin) budget -= j1 - j0;
     if (!ok) {
