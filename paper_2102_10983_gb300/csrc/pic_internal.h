@@ -130,6 +130,7 @@ struct PushArgsMixed {
   const float* coef_all;
   int64_t coef_stride, coef_oldest;
   int32_t coef_steps;
+  int32_t item_tiles;  // tiles per stream item
   int32_t lo, hi;      // tent node j must satisfy lo <= j and j+1 <= hi
   int32_t lo_p, hi_p;  // same for the previous step
   int32_t mask;

@@ -1044,15 +1044,11 @@ __device__ __forceinline__ void defer_mark(const PushArgsMixed& a, int64_t i, in
 #endif
 constexpr int kThreads = PIC_THREADS;
 constexpr int kWarps = kThreads / 32;
-#ifndef PIC_CHUNK
-#define PIC_CHUNK 512
-#endif
 #ifndef PIC_STAGES
 #define PIC_STAGES 2
 #endif
-constexpr int kChunk = PIC_CHUNK;    // particles per stream item (kChunk / kTile tiles)
 constexpr int kStages = PIC_STAGES;  // staged tiles per warp (one in flight while one is pushed)
-static_assert(kChunk % kTile == 0 && kTile % 64 == 0, "a stream item is whole tiles of whole rounds");
+static_assert(kTile % 64 == 0, "a tile is whole rounds");
 constexpr int kStashK = kDeferMin - 1;
 constexpr int kStashCap = 96;  // up to 31 left over and a round's 64
 constexpr uint8_t kParity = 0x08;
