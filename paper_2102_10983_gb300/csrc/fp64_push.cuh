@@ -277,10 +277,12 @@ static __device__ __noinline__ Push64 push64_any(double ex, double ey, double bz
 }
 // The same bits with the integer roots and quotients, in one straight line (no
 // branch between the FP64 operations, so their latencies overlap what is
-// independent); operands outside those routines' domain are seen at the end
-// and the push is taken again by push64_any.
+// independent); q: the momentum after it.  False: operands outside those
+// routines' domain, the push is to be taken again by push64_any.  A serial
+// chain forms its next position before it looks at that.
 template <bool UNIT, bool EX>
-__device__ __forceinline__ Push64 push64(double ex, double ey, double bz, double half, double qm, Mom64& p) {
+__device__ __forceinline__ bool push64_try(double ex, double ey, double bz, double half, double qm,
+                                           const Mom64& p, Mom64& q, Push64& r) {
   const double dpx = EX ? times_qm<UNIT>(qm, ex) * half : 0.0;
   const double dpy = times_qm<UNIT>(qm, ey) * half;
   const double mx = EX ? p.x + dpx : p.x, mx2 = EX ? mx * mx : p.x2;
@@ -291,16 +293,21 @@ __device__ __forceinline__ Push64 push64(double ex, double ey, double bz, double
   const double ppx = mx + my * tz;
   const double ppy = my - mx * tz;
   ok &= div2_try(tz, 1.0 + tz * tz, sz);
-  Mom64 q;
   q.x = EX ? (mx + ppy * sz) + dpx : mx + ppy * sz;
   q.y = (my - ppx * sz) + dpy;
   q.z = p.z;
   q.z2 = p.z2;
   q.x2 = q.x * q.x;
-  Push64 r;
   r.vy = 0.0;
   ok &= div_sqrt_try<EX>(q.x, q.y, 1.0 + (q.x2 + q.y * q.y + q.z2), r.vx, r.vy, r.gam);
-  if (!ok) return push64_any<UNIT, EX>(ex, ey, bz, half, qm, &p);
+  return ok;
+}
+template <bool UNIT, bool EX>
+__device__ __forceinline__ Push64 push64(double ex, double ey, double bz, double half, double qm, Mom64& p) {
+  Mom64 q;
+  Push64 r;
+  if (!push64_try<UNIT, EX>(ex, ey, bz, half, qm, p, q, r))
+    return push64_any<UNIT, EX>(ex, ey, bz, half, qm, &p);
   p = q;
   return r;
 }

@@ -159,18 +159,34 @@ __device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first
       bd = B.d;
     }
   };
+  // No branch on the chain but the vote, which the gather's first two
+  // operations overlap: they are taken with the nodes as they were, and again
+  // in the rare case.  An electron that is lost is written out there; its
+  // lanes' later values are not used.
 #pragma unroll 1
   for (int j = 0; j < m; ++j) {
+    const double s = xi * a.inv_dx;
     Coords64 c;
-    const bool in = live && locate(a, xi * a.inv_dx, c);
-    const int32_t ne = in ? (int32_t)(c.je & a.mask) : E.at, nb = in ? (int32_t)(c.jb & a.mask) : B.at;
-    live = in;
-    const bool moved = ne != E.at || nb != B.at;
-    if (__any_sync(0xffffffffu, moved || j >= at + have)) {
+    const bool in = coords64_fast(s, c) & live & (c.jb >= a.lo_i) & (c.je < a.hi_i);  // as locate
+    double ey = ef + c.we * ed, bz = bf + c.wb * bd;
+    bool moved = in & (((int32_t)(c.je & a.mask) != E.at) | ((int32_t)(c.jb & a.mask) != B.at));
+    if (__any_sync(0xffffffffu, moved | (in != live) | (j >= at + have))) {
+      if (in != live) {
+        live = locate(a, s, c);
+        moved = live && ((int32_t)(c.je & a.mask) != E.at || (int32_t)(c.jb & a.mask) != B.at);
+        if (!live && copy == 0) {
+          if (diag) a.work[i] = work;
+          a.x[i] = xi;
+          a.px[i] = p.x;
+          a.py[i] = p.y;
+          a.status[i] = (uint8_t)(k | PIC_STATUS_LOST);
+          atomicAdd(&sh[11], 1ull);
+        }
+      }
       if (!__any_sync(0xffffffffu, live)) break;
       if (moved) {
-        E.load(a.E, ne, mask);
-        B.load(a.B, nb, mask);
+        E.load(a.E, (int32_t)(c.je & a.mask), mask);
+        B.load(a.B, (int32_t)(c.jb & a.mask), mask);
       }
       at = j;
       have = rows;
@@ -178,28 +194,35 @@ __device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first
       E.sums(wr);
       B.sums(wr + (P + 1));
       take(0);
+      ey = ef + c.we * ed;
+      bz = bf + c.wb * bd;
     }
-    const double ey = ef + c.we * ed, bz = bf + c.wb * bd;
     take(j + 1 - at);  // the next sub-step's, unless the electron changes node
-    if (live) {
-      const Push64 r = push64<UNIT, false>(0.0, ey, bz, half, a.qm, p);
-      xi = xi + h * r.vx;
-      if (diag) {  // (q hp / 2) E . (v_before + v_after) (App. B)
-        const double v = div_rn(p.y, r.gam);
-        work = work + ((a.qm * hp) * 0.5) * (ey * (vy + v));
-        vy = v;
-        hp = h;
-      }
-      half = 0.5 * h;
+    Mom64 q;
+    Push64 r;
+    const bool ok = push64_try<UNIT, false>(0.0, ey, bz, half, a.qm, p, q, r);
+    double xn = xi + h * r.vx;
+    if (live && !ok) {
+      q = p;
+      r = push64_any<UNIT, false>(0.0, ey, bz, half, a.qm, &q);
+      xn = xi + h * r.vx;
     }
+    p = q;
+    xi = xn;
+    if (diag) {  // (q hp / 2) E . (v_before + v_after) (App. B)
+      const double v = div_rn(p.y, r.gam);
+      work = work + ((a.qm * hp) * 0.5) * (ey * (vy + v));
+      vy = v;
+      hp = h;
+    }
+    half = 0.5 * h;
   }
-  if (valid && copy == 0) {
+  if (live && copy == 0) {
     if (diag) a.work[i] = work;
     a.x[i] = xi;
     a.px[i] = p.x;
     a.py[i] = p.y;
-    a.status[i] = (uint8_t)(live ? k : k | PIC_STATUS_LOST);
-    if (!live) atomicAdd(&sh[11], 1ull);
+    a.status[i] = (uint8_t)k;
   }
 }
 

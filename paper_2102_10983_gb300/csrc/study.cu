@@ -228,9 +228,17 @@ __device__ __forceinline__ void study_electron(const pic_study_case& q, double x
       const int src = first + (j & 31);
       const double ey = __shfl_sync(0xffffffffu, E.f, src) + c.we * __shfl_sync(0xffffffffu, E.d, src);
       const double bz = __shfl_sync(0xffffffffu, B.f, src) + c.wb * __shfl_sync(0xffffffffu, B.d, src);
-      r = push64<UNIT, false>(0.0, ey, bz, half, q.qm, p);
+      Mom64 pn;
+      const bool ok = push64_try<UNIT, false>(0.0, ey, bz, half, q.qm, p, pn, r);
+      double xn = xi + h * r.vx;
+      if (!ok) {
+        pn = p;
+        r = push64_any<UNIT, false>(0.0, ey, bz, half, q.qm, &pn);
+        xn = xi + h * r.vx;
+      }
+      p = pn;
+      xi = xn;
       half = 0.5 * h;
-      xi = xi + h * r.vx;
     }
     k_prev = k;
     const double dR = fabs((r.gam - p.x) - 1.0);
