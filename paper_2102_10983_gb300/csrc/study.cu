@@ -200,34 +200,46 @@ __device__ __forceinline__ void study_electron(const pic_study_case& q, double x
     }
     const int first = k == 0 ? 31 : k == 1 ? 16 : 0;  // the lane with the first sub-step's sums
     Push64 r;
+    double ef, ed, bf, bd;  // sub-step j's sums
+    auto take = [&](int j) {
+      const int src = (first + (j & 31)) & 31;
+      ef = __shfl_sync(0xffffffffu, E.f, src);
+      ed = __shfl_sync(0xffffffffu, E.d, src);
+      bf = __shfl_sync(0xffffffffu, B.f, src);
+      bd = __shfl_sync(0xffffffffu, B.d, src);
+    };
+    take(0);
     for (int j = 0; j < m; ++j) {
       if (j > 0) locate(c);
-      const bool moved = c.je != je || c.jb != jb;
-      if (k > 2 && (j & 31) == 0) {  // the next 32 sub-steps' weights
-        const double th = theta_of(q.field_time, j + lane, k);
-        lagrange<P>(true, th, wE);
-        lagrange<P>(false, th, wB);
-      }
-      if (moved) {
-        // one node on is in the tile; anything else (a step of more than a
-        // node, c dt > dx, or a turn back) is evaluated anew
-        if (c.je < te || c.je > te + 1 || c.jb < tb || c.jb > tb + 1) {
-          te = c.je;
-          tb = c.jb;
-          tile.fill(q, sm, te, tb, n, xi_diag);
+      // the gather overlaps the tests: taken again where they find new sums
+      double ey = ef + c.we * ed, bz = bf + c.wb * bd;
+      const bool moved = c.je != je || c.jb != jb, more = k > 2 && (j & 31) == 0;
+      if (moved || more) {
+        if (more) {  // the next 32 sub-steps' weights
+          const double th = theta_of(q.field_time, j + lane, k);
+          lagrange<P>(true, th, wE);
+          lagrange<P>(false, th, wB);
         }
-        je = c.je;
-        jb = c.jb;
-        tile.read(sm, false, je, n, E.v0, E.v1);
-        tile.read(sm, true, jb, n, B.v0, B.v1);
-      }
-      if (moved || (k > 2 && (j & 31) == 0)) {
+        if (moved) {
+          // one node on is in the tile; anything else (a step of more than a
+          // node, c dt > dx, or a turn back) is evaluated anew
+          if (c.je < te || c.je > te + 1 || c.jb < tb || c.jb > tb + 1) {
+            te = c.je;
+            tb = c.jb;
+            tile.fill(q, sm, te, tb, n, xi_diag);
+          }
+          je = c.je;
+          jb = c.jb;
+          tile.read(sm, false, je, n, E.v0, E.v1);
+          tile.read(sm, true, jb, n, B.v0, B.v1);
+        }
         E.sums(wE);
         B.sums(wB);
+        take(j);
+        ey = ef + c.we * ed;
+        bz = bf + c.wb * bd;
       }
-      const int src = first + (j & 31);
-      const double ey = __shfl_sync(0xffffffffu, E.f, src) + c.we * __shfl_sync(0xffffffffu, E.d, src);
-      const double bz = __shfl_sync(0xffffffffu, B.f, src) + c.wb * __shfl_sync(0xffffffffu, B.d, src);
+      take(j + 1);
       Mom64 pn;
       const bool ok = push64_try<UNIT, false>(0.0, ey, bz, half, q.qm, p, pn, r);
       double xn = xi + h * r.vx;
