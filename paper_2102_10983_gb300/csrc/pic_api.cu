@@ -55,8 +55,7 @@ struct pic_ctx {
   double* nodes64 = nullptr;
   uint8_t* k_sub = nullptr;
   int32_t* queue64 = nullptr;
-  int32_t* bin64 = nullptr;  // two sets of 32 counters, used in turn
-  int bin64_at = 0;
+  int32_t* bin64 = nullptr;
   int32_t* pred_queue = nullptr;
   const pic_mlp* mlp = nullptr;
   int32_t predict_every = 1;
@@ -244,7 +243,7 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     if (prm->diagnostics == PIC_DIAG_WORK) A((void**)&c->work, cap * 8);
     A((void**)&c->k_sub, cap);
     A((void**)&c->queue64, cap * 4);
-    A((void**)&c->bin64, 64 * 4);
+    A((void**)&c->bin64, kBinF64 * 4);
   }
   A((void**)&c->status, cap);
   // the mixed form's ring is mirrored (2R slots, see PushArgsMixed)
@@ -273,7 +272,6 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     cudaGetLastError();
   }
   e = cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream);
-  if (e == cudaSuccess && c->bin64) e = cudaMemsetAsync(c->bin64, 0, 64 * 4, c->stream);
   if (e == cudaSuccess && c->qcount) e = cudaMemsetAsync(c->qcount, 0, 64 * 4, c->stream);
   if (e == cudaSuccess && c->pred) e = cudaMemsetAsync(c->pred, 0, cap, c->stream);
 
@@ -752,9 +750,7 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
       a.nodes = c->nodes64;
       a.k_sub = c->k_sub;
       a.queue = c->queue64;
-      a.bin = c->bin64 + 32 * c->bin64_at;
-      c->bin64_at ^= 1;
-      a.bin_next = c->bin64 + 32 * c->bin64_at;
+      a.bin = c->bin64;
       e = mark(ev0);
       if (e == cudaSuccess) e = launch_push_f64(a, p, c->stream, &launches);
     } else {

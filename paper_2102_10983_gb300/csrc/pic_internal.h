@@ -54,6 +54,7 @@ __host__ __device__ inline float criterion_f64_scale(double qm_abs, double dt, d
 
 // The electrons of a step that sub-cycle: k_sub[i] = their k (else 0), bin[1..7]
 // the counts per k, bin[8..15] places taken so far, bin[16] the item cursor.
+constexpr int kBinF64 = 32;  // counters in bin
 struct BinF64 {
   int64_t n;
   const uint8_t* k_sub;
@@ -84,8 +85,7 @@ struct PushArgsF64 {
   double* nodes;      // nullptr, or 4 W: each node's fields at t_n (nodes_f64_kernel)
   uint8_t* k_sub;     // per particle: k of the step where k > 0 (written every step)
   int32_t* queue;     // particles with k > 0, grouped by k
-  int32_t* bin;       // [32] this step's counts and cursors, zero on entry
-  int32_t* bin_next;  // [32] the next step's: zeroed by this one
+  int32_t* bin;       // [kBinF64] the step's counts and cursors, zeroed by its first launch
   int sms;            // set by the launcher
 };
 

@@ -66,7 +66,6 @@ struct Sc1dArgs {
   uint8_t* k_sub;     // as in PushArgsF64
   int32_t* queue;
   int32_t* bin;
-  int32_t* bin_next;
   int sms;
 };
 
@@ -154,6 +153,7 @@ __device__ __forceinline__ void face_flux(int64_t Q, int64_t ia, double wa, int6
 template <int P>
 __global__ void __launch_bounds__(128) nodes_kernel(Sc1dArgs a) {
   constexpr int stride = 2 * (P + 1);
+  if (blockIdx.x == 0 && threadIdx.x < kBinF64) a.bin[threadIdx.x] = 0;  // the step's counts
   const double* wE = a.wtab + wrow(0, 1) * stride;
   const double* wB = a.wtab + a.crit_row * stride + (P + 1);
   for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < 3 * a.M;
@@ -179,7 +179,6 @@ template <bool UNIT>
 __global__ void __launch_bounds__(256) push_deposit_kernel(Sc1dArgs a) {
   __shared__ unsigned long long sh[12];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
-  if (blockIdx.x == 0 && threadIdx.x < 32) a.bin_next[threadIdx.x] = 0;  // the next step's counts
   __syncthreads();
   unsigned k0 = 0, k1 = 0;
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < a.n; b += (int64_t)gridDim.x * blockDim.x) {
@@ -493,8 +492,7 @@ struct pic_sc1d {
   double2* nodes = nullptr;  // [M][3] fields at t_n
   uint8_t* k_sub = nullptr;  // the electrons of a step that sub-cycle (push_deposit_kernel)
   int32_t* queue = nullptr;
-  int32_t* bin = nullptr;    // two sets of 32 counters, used in turn
-  int bin_at = 0;
+  int32_t* bin = nullptr;
   DevStats* dstats = nullptr;
   double* staging = nullptr;  // 3 M host-upload staging
   int64_t launches = 0;
@@ -575,7 +573,7 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   ok &= cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) == cudaSuccess;
   ok &= cudaMalloc(&c->k_sub, cap) == cudaSuccess;
   ok &= cudaMalloc(&c->queue, cap * 4) == cudaSuccess;
-  ok &= cudaMalloc(&c->bin, 64 * 4) == cudaSuccess;
+  ok &= cudaMalloc(&c->bin, kBinF64 * 4) == cudaSuccess;
   if (!ok) {
     pic_sc1d_destroy(c);
     return sc_fail(nullptr, PIC_ENOMEM, "pic_sc1d_create: device allocation failed");
@@ -583,7 +581,6 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   cudaError_t e = cudaMemsetAsync(c->ring, 0, (int64_t)c->R * 3 * c->M * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->acc, 0, (6 * c->M + 2) * 8, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->dstats, 0, sizeof(DevStats), c->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->bin, 0, 64 * 4, c->stream);
   if (e == cudaSuccess) e = build_wtab_f64(c->wtab, prm->order, prm->k_max, prm->field_time, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) {
@@ -771,9 +768,7 @@ extern "C" int pic_sc1d_step(pic_sc1d* c, int64_t n0, int64_t n_steps, pic_sc1d_
       a.nodes = c->nodes;
       a.k_sub = c->k_sub;
       a.queue = c->queue;
-      a.bin = c->bin + 32 * c->bin_at;
-      c->bin_at ^= 1;
-      a.bin_next = c->bin + 32 * c->bin_at;
+      a.bin = c->bin;
       a.sms = c->sm_count > 0 ? c->sm_count : 152;
       switch (p) {
         case 1: launch_push<1>(c, a); break;

@@ -87,6 +87,7 @@ __device__ __forceinline__ double tsum64(const double* const* lv, const double* 
 
 template <int P>
 __global__ void __launch_bounds__(128) nodes_f64_kernel(PushArgsF64 a) {
+  if (blockIdx.x == 0 && threadIdx.x < kBinF64) a.bin[threadIdx.x] = 0;  // the step's counts
   const double* wE = a.wtab + wrow(0, 1) * (2 * (P + 1));
   const double* wB = a.wtab + a.crit_row * (2 * (P + 1)) + (P + 1);
   for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c <= a.mask;
@@ -245,7 +246,6 @@ template <int P, bool UNIT>
 __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) {
   __shared__ unsigned long long sh[12];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
-  if (blockIdx.x == 0 && threadIdx.x < 32) a.bin_next[threadIdx.x] = 0;  // the next step's counts
   __syncthreads();
   unsigned k0 = 0, k1 = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
@@ -308,6 +308,7 @@ __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) 
     atomicAdd(&a.bin[threadIdx.x], (int32_t)sh[threadIdx.x]);
 }
 
+// Every step starts from counts of zero, so that a captured step can be replayed.
 // bin[1..7]: the step's counts per k; bin[8 + k]: entries of k placed so far;
 // bin[16]: the sub-cycle kernel's item cursor.  Queue order: k = 7 first.
 __global__ void __launch_bounds__(256) bin_f64_kernel(BinF64 a) {
@@ -389,6 +390,8 @@ static void launch_f64_p(PushArgsF64 a, int sms, cudaStream_t s, int* launches) 
     const int64_t want = (a.mask + 128) / 128;
     nodes_f64_kernel<P><<<(int)(want < sms * 8 ? want : sms * 8), 128, 0, s>>>(a);
     ++n;
+  } else {
+    cudaMemsetAsync(a.bin, 0, kBinF64 * sizeof(int32_t), s);
   }
   // small ensembles in small blocks: every SM's FP64 unit takes part
   const int threads = a.n >= (int64_t)sms * 256 ? 256 : a.n >= (int64_t)sms * 64 ? 64 : 32;
