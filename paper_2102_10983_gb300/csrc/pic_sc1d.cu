@@ -519,6 +519,10 @@ static int sc_fail(pic_sc1d* c, int code, const char* msg, const char* detail = 
     if (e_ != cudaSuccess) return sc_fail((c), PIC_ECUDA, #call ": ", cudaGetErrorString(e_)); \
   } while (0)
 
+// The queue's entries and counts are 32-bit numbers: electrons beyond kSlice are
+// pushed in further rounds of the passes.
+constexpr int64_t kSlice = (int64_t)1 << 30;
+
 static double* slot_field(pic_sc1d* c, int slot, int f) {
   return c->ring + ((int64_t)slot * 3 + f) * c->M;
 }
@@ -571,8 +575,9 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   ok &= cudaMalloc(&c->dstats, sizeof(DevStats)) == cudaSuccess;
   ok &= cudaMalloc(&c->staging, 3 * c->M * 8) == cudaSuccess;
   ok &= cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) == cudaSuccess;
-  ok &= cudaMalloc(&c->k_sub, cap) == cudaSuccess;
-  ok &= cudaMalloc(&c->queue, cap * 4) == cudaSuccess;
+  const int64_t slice = cap < kSlice ? cap : kSlice;
+  ok &= cudaMalloc(&c->k_sub, slice) == cudaSuccess;
+  ok &= cudaMalloc(&c->queue, slice * 4) == cudaSuccess;
   ok &= cudaMalloc(&c->bin, kBinF64 * 4) == cudaSuccess;
   if (!ok) {
     pic_sc1d_destroy(c);
@@ -700,10 +705,16 @@ static int sc_gauss(pic_sc1d* c) {
 }
 
 template <int P>
-static void launch_push(pic_sc1d* c, const Sc1dArgs& a) {
+static void launch_push(pic_sc1d* c, const Sc1dArgs& all, int64_t off = 0) {
   const cudaStream_t s = c->stream;
+  Sc1dArgs a = all;
+  a.x += off; a.px += off; a.py += off; a.pz += off; a.status += off; a.Q += off;
+  a.n = all.n - off < kSlice ? all.n - off : kSlice;
   const bool unit = a.qm_abs == 1.0;
-  nodes_kernel<P><<<grid_for(c, 2 * 3 * c->M), 128, 0, s>>>(a);
+  if (off == 0)
+    nodes_kernel<P><<<grid_for(c, 2 * 3 * c->M), 128, 0, s>>>(a);
+  else
+    cudaMemsetAsync(a.bin, 0, kBinF64 * sizeof(int32_t), s);
   // small ensembles in small blocks: every SM's FP64 unit takes part
   const int threads = a.n >= (int64_t)a.sms * 256 ? 256 : a.n >= (int64_t)a.sms * 64 ? 64 : 32;
   const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)a.sms * 8;
@@ -719,7 +730,8 @@ static void launch_push(pic_sc1d* c, const Sc1dArgs& a) {
     subcycle_deposit_kernel<P, true><<<warps, 32, 0, s>>>(a);
   else
     subcycle_deposit_kernel<P, false><<<warps, 32, 0, s>>>(a);
-  c->launches += 4;
+  c->launches += off == 0 ? 4 : 3;
+  if (off + a.n < all.n) launch_push<P>(c, all, off + a.n);
 }
 
 extern "C" int pic_sc1d_step(pic_sc1d* c, int64_t n0, int64_t n_steps, pic_sc1d_stats* stats) {
