@@ -341,15 +341,13 @@ def run_batched(args, dev, stream, sms):
 
 # ---------------------------------------------------------------- our arm
 
-# FP64 pipe cost of the FP64 form (push_f64_kernel<3>), counted from its source
-# in DFMA issue slots: per Boris sub-step 77 FP64 add/mul/compare/floor
-# operations (two order-3 gathers 34, Boris and position 33, coordinates and
-# window test 10) plus 2 square roots and 3 divisions; per macro step the
-# criterion adds one gather, a square root and a division (27 operations).  A
-# square root or division occupies the pipe ~10 DFMA slots (measured 0.19 of
-# them per clock per SM against 1.92 DFMAs).
-F64_SLOTS_PER_SUBSTEP = 77 + 5 * 10
-F64_SLOTS_PER_STEP = 27 + 2 * 10
+# FP64 pipe cost of the FP64 form at order 3, counted from its source in DFMA
+# issue slots: a sub-step of a sub-cycled electron takes 34 additions and
+# products for its two order-3 gathers and 33 for the Boris push and position; a
+# macro step 25 (the criterion and, for m = 1, the push from the step's node
+# fields).  Roots, quotients, floors and comparisons are on the integer pipes.
+F64_SLOTS_PER_SUBSTEP = 34 + 33
+F64_SLOTS_PER_STEP = 25
 DFMA_PER_CLK_PER_SM = 1.92
 
 
@@ -362,13 +360,14 @@ def device_props(local):
 def fp64_roofline(st, steps_particles, ms, sms, sm_mhz):
     """FP64-pipe roofline of the FP64 form: DFMA slots the run needed over the
     time, against sms x 1.92 x clock."""
-    slots = st["substeps"] * F64_SLOTS_PER_SUBSTEP + steps_particles * F64_SLOTS_PER_STEP
+    sub = st["substeps"] - st["k_hist"][0]  # those of the sub-cycled electrons
+    slots = sub * F64_SLOTS_PER_SUBSTEP + steps_particles * F64_SLOTS_PER_STEP
     achieved = slots / (ms / 1e3)
     peak = sms * DFMA_PER_CLK_PER_SM * sm_mhz * 1e6
     return {"bound": "alu (FP64 pipe)", "achieved": achieved, "peak": peak,
             "unit": "DFMA slots/s", "frac": achieved / peak,
-            "model": f"{F64_SLOTS_PER_SUBSTEP} slots per Boris sub-step + {F64_SLOTS_PER_STEP} per "
-                     "macro step (sqrt/div = 10 slots); peak = SMs x 1.92 DFMA/clk x SM clock"}
+            "model": f"{F64_SLOTS_PER_SUBSTEP} slots per sub-step of a sub-cycle + {F64_SLOTS_PER_STEP} per "
+                     "macro step; peak = SMs x 1.92 DFMA/clk x SM clock"}
 
 
 def snapshot(integ, n_e, dev):
