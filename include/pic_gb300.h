@@ -339,7 +339,9 @@ int pic_batch_fields_upload(pic_batch* b, int64_t level, const int64_t* i0, cons
                             const double* Bz, int32_t where);
 
 /* Macro steps n .. n+n_steps-1 of every ensemble (stats: totals over the
- * batch; as for pic_push_step). */
+ * batch; as for pic_push_step).  Errors: PIC_EINVAL, PIC_ECUDA, PIC_ERANGE,
+ * PIC_EKMAX, PIC_ETIMEOUT (a bounded device wait gave up, in this call or in
+ * an earlier one without stats: particle state is not trustworthy). */
 int pic_batch_push_step(pic_batch* b, int64_t n, int64_t n_steps, pic_step_stats* stats);
 
 /* Event timing of each pushed step: on/off; with non-NULL outputs, also return
@@ -353,9 +355,15 @@ int64_t pic_batch_launch_count(const pic_batch* b);
  * macro steps from step n, each from the same saved particle state (restored
  * afterwards); the fastest is kept and returned (ms per step in ms_out).  The
  * levels of steps n .. n+steps-1 must be in the ring.  Allocates a temporary
- * copy of the particle state. */
+ * copy of the particle state.  PIC_ETIMEOUT (as for pic_batch_push_step; the
+ * configuration stays as it was): a trial, or an earlier call without stats,
+ * gave up. */
 int pic_batch_autotune(pic_batch* b, int64_t n, int32_t steps, int32_t* chunk_out,
                        int32_t* blocks_out, double* ms_out);
+
+/* pic_inject_error for a batch: the next pic_batch_push_step with stats, or
+ * pic_batch_autotune, reports it.  Errors: PIC_EINVAL, PIC_ECUDA. */
+int pic_batch_inject_error(pic_batch* b, int32_t word);
 
 const char* pic_batch_last_error(const pic_batch* b);
 

@@ -463,6 +463,7 @@ extern "C" int pic_batch_push_step(pic_batch* b, int64_t n, int64_t n_steps, pic
   stats->clamped = (int64_t)h.clamped;
   stats->out_of_window = (int64_t)h.lost;
   stats->error = h.error;
+  if (h.error) return bfail(b, PIC_ETIMEOUT, "device error word set");
   if (stats->out_of_window) return bfail(b, PIC_ERANGE, "particles left the field window");
   if (stats->clamped) return bfail(b, PIC_EKMAX, "criterion capped at k_max");
   return PIC_OK;
@@ -513,7 +514,8 @@ extern "C" int pic_batch_autotune(pic_batch* b, int64_t n, int32_t steps, int32_
   const int32_t chunks[4] = {128, 256, 512, 1024};
   const int maxb = batch_max_blocks_per_sm(b->order);
   double best = 1e300;
-  int32_t best_c = b->chunk, best_b = b->blocks_per_sm;
+  const int32_t old_c = b->chunk, old_b = b->blocks_per_sm;
+  int32_t best_c = old_c, best_b = old_b;
   const bool graph = b->use_graph, timing = b->timing;
   b->use_graph = false;
   cudaEvent_t t0 = nullptr, t1 = nullptr;
@@ -541,6 +543,10 @@ extern "C" int pic_batch_autotune(pic_batch* b, int64_t n, int32_t steps, int32_
     }
   }
   if (e == cudaSuccess) e = copy_state(false);
+  // the error word first: a trial that gave up is fast, and an earlier call
+  // without stats may have left one
+  DevStats h{};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, b->dstats, sizeof(DevStats), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->dstats, 0, sizeof(DevStats), b->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
   if (t0) cudaEventDestroy(t0);
@@ -549,6 +555,11 @@ extern "C" int pic_batch_autotune(pic_batch* b, int64_t n, int32_t steps, int32_
   b->use_graph = graph;
   b->timing = timing;
   if (e != cudaSuccess) return bfail(b, PIC_ECUDA, "pic_batch_autotune: a trial failed");
+  if (h.error) {
+    b->blocks_per_sm = old_b;
+    const int rc = set_chunk(b, old_c);
+    return rc != PIC_OK ? rc : bfail(b, PIC_ETIMEOUT, "pic_batch_autotune: device error word set");
+  }
   b->blocks_per_sm = best_b;
   int rc = set_chunk(b, best_c);
   if (rc != PIC_OK) return rc;
@@ -563,5 +574,12 @@ extern "C" const char* pic_batch_last_error(const pic_batch* b) { return b ? b->
 extern "C" int pic_batch_heavy_budget(pic_batch* b, int32_t budget) {
   if (!b) return PIC_EINVAL;
   b->heavy_budget = budget == 0 ? 1024 : budget;
+  return PIC_OK;
+}
+
+extern "C" int pic_batch_inject_error(pic_batch* b, int32_t word) {
+  if (!b) return PIC_EINVAL;
+  // pageable source: the copy is staged before cudaMemcpyAsync returns
+  BATCH_TRY(b, cudaMemcpyAsync(&b->dstats->error, &word, sizeof(int32_t), cudaMemcpyHostToDevice, b->stream));
   return PIC_OK;
 }

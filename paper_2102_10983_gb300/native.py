@@ -142,6 +142,7 @@ SIGNATURES = {
     "pic_batch_launch_count": (ctypes.c_int64, [_VP]),
     "pic_batch_autotune": (ctypes.c_int, [_VP, _I64, _I32, ctypes.POINTER(_I32), ctypes.POINTER(_I32),
                                           ctypes.POINTER(_D)]),
+    "pic_batch_inject_error": (ctypes.c_int, [_VP, _I32]),
     "pic_batch_last_error": (ctypes.c_char_p, [_VP]),
     "pic_push_mixed_noalloc": (ctypes.c_int, [ctypes.POINTER(PicParams), _I64, _VP, _VP, _VP, _VP,
                                               _VP, _VP, _VP, _VP, _VP, _I64, _I64, _I64, _VP,
@@ -476,6 +477,9 @@ class Batch:
 
     def launches(self) -> int:
         return int(lib().pic_batch_launch_count(self.h))
+
+    def inject_error(self, word: int = 1):
+        self._chk(lib().pic_batch_inject_error(self.h, int(word)))
 
     def autotune(self, n, steps=4):
         c, b, ms = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_double()
