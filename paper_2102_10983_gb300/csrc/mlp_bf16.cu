@@ -46,6 +46,13 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+// d += a b: the product's sum from zero, then an FP32 addition.
+__device__ __forceinline__ void add_product(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  mma16816(s, a, b0, b1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) d[q] = __fadd_rn(d[q], s[q]);
+}
 
 // Weights as the kernels read them from shared memory (BF16):
 //   W1p [64][16] (cols 6..15 zero), W2 [64][64], W2T [64][64], W3 [8][64] (rows at the
@@ -204,9 +211,14 @@ __device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], const __nv_bfloat16* p)
 // on), run on the tensor cores too, the block's 64 samples at a time: warp w
 // forms rows 16 w .. 16 w + 15 of each, its operands by transposing matrix
 // loads from the staged tiles, and keeps its sums in registers over all of the
-// block's samples.  (On the FP32 pipes -- 16 products per element and shared
-// atomics between the warps, then an atomic per block and parameter -- a batch
-// of 8,192 took 30 us; this kernel 7.3 us and mlp_finish_kernel 3.2 us.)
+// block's samples.  The tensor cores truncate where they add into an
+// accumulator, a bias that grows with the number of additions: so they sum 16
+// samples from zero, and those sums are added in FP32, to nearest (a batch of
+// 1,048,576, against 64-bit sums of the same operands: relative error 2.0e-5 if
+// the accumulators run on, 7e-8 so; 2e-7 on the FP32 pipes).
+// (On the FP32 pipes -- 16 products per element and shared atomics between the
+// warps, then an atomic per block and parameter -- a batch of 8,192 took 30 us;
+// this kernel 7.3 us and mlp_finish_kernel 3.2 us.)
 __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const float* P, const float* phi,
                                                                    const uint8_t* label, int64_t n,
                                                                    float inv_batch, float* part) {
@@ -311,20 +323,20 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const float* 
       ldsm2t(D, &S.dz[k0 + 8 * m1b + mr][0]);
       ldsm2t(Xf, &S.X[k0 + 8 * m1b + mr][0]);
       a_of(S.da2);
-      mma16816(gB2, A, Xf[0], Xf[1]);
+      add_product(gB2, A, Xf[0], Xf[1]);
 #pragma unroll
       for (int nt = 0; nt < 8; nt += 2) {
         ldsm4t(B, &S.h1[k0 + 8 * m1b + mr][8 * (nt + m2b)]);
-        mma16816(gW2[nt], A, B[0], B[1]);
-        mma16816(gW2[nt + 1], A, B[2], B[3]);
+        add_product(gW2[nt], A, B[0], B[1]);
+        add_product(gW2[nt + 1], A, B[2], B[3]);
       }
       a_of(S.da1);
-      mma16816(gW1, A, Xf[0], Xf[1]);
+      add_product(gW1, A, Xf[0], Xf[1]);
       a_of(S.h2);
-      mma16816(gW3, A, D[0], D[1]);  // transposed: rows = inputs, columns = classes
+      add_product(gW3, A, D[0], D[1]);  // transposed: rows = inputs, columns = classes
       if (warp == 0) {
         const uint32_t one = pack2(1.f, 1.f), ones[4] = {one, one, one, one};
-        mma16816(gB3, ones, D[0], D[1]);
+        add_product(gB3, ones, D[0], D[1]);
       }
     }
   }
