@@ -265,9 +265,10 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     return fail(nullptr, e == cudaErrorMemoryAllocation ? PIC_ENOMEM : PIC_ECUDA,
                 "pic_create: device allocation failed: %s", cudaGetErrorString(e));
   }
-  // the node fields save the FP64 push its gathers; without room for them it
-  // gathers the levels
-  if (!mixed && cudaMalloc((void**)&c->nodes64, (size_t)window_cells * 32) != cudaSuccess) {
+  // the node fields save the FP64 push its gathers; without them (a window that
+  // no ensemble of this capacity pays for, no room) it gathers the levels
+  if (!mixed && node_fields_pay(capacity, window_cells) &&
+      cudaMalloc((void**)&c->nodes64, (size_t)window_cells * 32) != cudaSuccess) {
     c->nodes64 = nullptr;
     cudaGetLastError();
   }
@@ -747,7 +748,7 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
       a.lo_i = (int32_t)(lo < -i32 ? -i32 : lo > i32 ? i32 : lo);
       a.hi_i = (int32_t)(hi < -i32 ? -i32 : hi > i32 ? i32 : hi);
       a.crit_scale = crit64;
-      a.nodes = c->nodes64;
+      a.nodes = node_fields_pay(c->n, W) ? c->nodes64 : nullptr;
       a.k_sub = c->k_sub;
       a.queue = c->queue64;
       a.bin = c->bin64;

@@ -52,6 +52,17 @@ __host__ __device__ inline float criterion_f64_scale(double qm_abs, double dt, d
   return (c >= 0x1p-60 && c <= 0x1p60 && psi_max >= 0x1p-500 && psi_max <= 0x1p500) ? (float)c : 0.0f;
 }
 
+// Whether the FP64 forms' node fields pay: one pass over the grid's entries per
+// step, then one multiplication and one addition per grid and electron instead
+// of its gather.  Per entry that pass costs what an electron's gather does (57
+// ps: 30 FP64 operations), so a grid of more entries than electrons is not worth
+// it.  Steps of m = 1 pushes, with the pass and without: 256 electrons in a
+// window of 2^22 nodes 276 and 16 us; 1,048,576 electrons in 2^15 128 and 196;
+// as many nodes as electrons, 131,072 41 and 40, 1,048,576 190 and 197.
+__host__ __device__ inline bool node_fields_pay(int64_t electrons, int64_t entries) {
+  return electrons >= entries;
+}
+
 // The electrons of a step that sub-cycle: k_sub[i] = their k (else 0), bin[1..7]
 // the counts per k, bin[8..15] places taken so far, bin[16] the item cursor.
 constexpr int kBinF64 = 32;  // counters in bin
@@ -82,7 +93,7 @@ struct PushArgsF64 {
   DevStats* stats;
   double* work;  // nullptr, or per particle the accumulated work of E (App. B)
   float crit_scale;   // criterion_f64_scale: 0 = the exact criterion only
-  double* nodes;      // nullptr, or 4 W: each node's fields at t_n (nodes_f64_kernel)
+  double* nodes;      // nullptr, or 4 W: each node's fields at t_n (nodes_f64_kernel; node_fields_pay)
   uint8_t* k_sub;     // per particle: k of the step where k > 0 (written every step)
   int32_t* queue;     // particles with k > 0, grouped by k
   int32_t* bin;       // [kBinF64] the step's counts and cursors, zeroed by its first launch
