@@ -112,24 +112,22 @@ __device__ __forceinline__ bool locate(const PushArgsF64& a, double s, Coords64&
   return true;
 }
 
-// All 4^k sub-steps of one macro step of g electrons (g a power of two; entries
-// first .. of the queue, those from `end` on absent).  Lane l works on electron
-// l mod g, in 32 / g equal copies: every copy takes the electron's serial chain
-// (about 21 dependent FP64 operations of 64 clocks and five divisions and
-// roots per sub-step), which costs the FP64 unit nothing, its time being per
-// warp instruction.  What does not depend on where the electron goes while it
+// All 4^k sub-steps of one macro step of g electrons (g a power of two; lane l
+// has electron i of index l mod g, if `valid`).  Each is worked on in 32 / g
+// equal copies: every copy takes the electron's serial chain (about 21
+// dependent FP64 operations of 64 clocks and five divisions and roots per
+// sub-step), which costs the FP64 unit nothing, its time being per warp
+// instruction.  What does not depend on where the electron goes while it
 // keeps its nodes -- the temporal sums at its nodes, 28 operations at order 3
 // -- the copies share: copy r forms those of the r-th sub-step to come, so a
 // warp pays for them once in 32 / g sub-steps, or when one of its electrons
 // changes node.
 template <int P, bool UNIT>
-__device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first, int64_t end, int g, int k,
+__device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t i, bool valid, int g, int k,
                                              unsigned long long* sh) {
   constexpr int stride = 2 * (P + 1);
   const int lane = threadIdx.x & 31, mine = lane & (g - 1), rows = 32 / g;
   const int copy = lane / g;
-  const bool valid = first + mine < end;
-  const int64_t i = valid ? a.queue[first + mine] : 0;
   const uint8_t st = valid ? a.status[i] : 0;
   double xi = valid ? a.x[i] : 0.0;
   Mom64 p = valid ? mom64(a.px[i], a.py[i], a.pz[i]) : Mom64{0.0, 0.0, 0.0, 0.0, 0.0};
@@ -242,6 +240,50 @@ __device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t first
 // 2.6 us before); 256 electrons at the a0 = 100 front 2.98 -> 1.2 ms, the chain
 // likewise.
 
+// Electron i's criterion and, with k = 0, its m = 1 push: its k, or -1 if it is
+// lost (or is now).
+template <int P, bool UNIT>
+__device__ __forceinline__ int criterion_push_f64(const PushArgsF64& a, int64_t i, unsigned long long* sh) {
+  const uint8_t st = a.status[i];
+  if (st & PIC_STATUS_LOST) return -1;
+  const double x = a.x[i];
+  Mom64 p = mom64(a.px[i], a.py[i], a.pz[i]);
+  Coords64 c;
+  if (!locate(a, x * a.inv_dx, c)) {
+    a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
+    atomicAdd(&sh[11], 1ull);
+    return -1;
+  }
+  double ey, bz;
+  if (a.nodes) {
+    const double2 e = __ldg(reinterpret_cast<const double2*>(a.nodes) + 2 * (c.je & a.mask));
+    const double2 b = __ldg(reinterpret_cast<const double2*>(a.nodes) + 2 * (c.jb & a.mask) + 1);
+    ey = e.x + c.we * e.y;
+    bz = b.x + c.wb * b.y;
+  } else {
+    const double* wE = a.wtab + wrow(0, 1) * (2 * (P + 1));
+    const double* wB = a.wtab + a.crit_row * (2 * (P + 1)) + (P + 1);
+    const int64_t e0 = c.je & a.mask, b0 = c.jb & a.mask;
+    const double fe = tsum64<P>(a.E, wE, e0), fb = tsum64<P>(a.B, wB, b0);
+    ey = fe + c.we * (tsum64<P>(a.E, wE, (e0 + 1) & a.mask) - fe);
+    bz = fb + c.wb * (tsum64<P>(a.B, wB, (b0 + 1) & a.mask) - fb);
+  }
+  bool capped;
+  const int k = criterion_f64(a.crit_scale, a.qm_abs, a.dt, a.psi_max, a.k_max, bz, p.x, p.y, p.z, capped);
+  if (capped) atomicAdd(&sh[10], 1ull);
+  if (k > 0) return k;
+  const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
+  double vy = 0.0;
+  if (a.work) vy = div_rn(p.y, sqrt_rn(1.0 + (p.x2 + p.y * p.y + p.z2)));
+  const Push64 r = push64<UNIT, false>(0.0, ey, bz, 0.5 * hp, a.qm, p);
+  a.x[i] = x + a.dt * r.vx;
+  if (a.work) a.work[i] = a.work[i] + ((a.qm * hp) * 0.5) * (ey * (vy + div_rn(p.y, r.gam)));
+  a.px[i] = p.x;
+  a.py[i] = p.y;
+  a.status[i] = 0;
+  return 0;
+}
+
 template <int P, bool UNIT>
 __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) {
   __shared__ unsigned long long sh[12];
@@ -250,55 +292,11 @@ __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) 
   unsigned k0 = 0, k1 = 0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.n;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const uint8_t st = a.status[i];
-    int k_sub = 0;
-    if (!(st & PIC_STATUS_LOST)) {
-      const double x = a.x[i];
-      Mom64 p = mom64(a.px[i], a.py[i], a.pz[i]);
-      Coords64 c;
-      if (!locate(a, x * a.inv_dx, c)) {
-        a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
-        atomicAdd(&sh[11], 1ull);
-      } else {
-        double ey, bz;
-        if (a.nodes) {
-          const double2 e = __ldg(reinterpret_cast<const double2*>(a.nodes) + 2 * (c.je & a.mask));
-          const double2 b = __ldg(reinterpret_cast<const double2*>(a.nodes) + 2 * (c.jb & a.mask) + 1);
-          ey = e.x + c.we * e.y;
-          bz = b.x + c.wb * b.y;
-        } else {
-          const double* wE = a.wtab + wrow(0, 1) * (2 * (P + 1));
-          const double* wB = a.wtab + a.crit_row * (2 * (P + 1)) + (P + 1);
-          const int64_t e0 = c.je & a.mask, b0 = c.jb & a.mask;
-          const double fe = tsum64<P>(a.E, wE, e0), fb = tsum64<P>(a.B, wB, b0);
-          ey = fe + c.we * (tsum64<P>(a.E, wE, (e0 + 1) & a.mask) - fe);
-          bz = fb + c.wb * (tsum64<P>(a.B, wB, (b0 + 1) & a.mask) - fb);
-        }
-        bool capped;
-        const int k = criterion_f64(a.crit_scale, a.qm_abs, a.dt, a.psi_max, a.k_max, bz, p.x, p.y, p.z,
-                                    capped);
-        if (capped) atomicAdd(&sh[10], 1ull);
-        if (k > 0) {
-          k_sub = k;
-          if (k == 1)
-            ++k1;
-          else
-            atomicAdd(&sh[k], 1ull);
-        } else {
-          ++k0;
-          const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
-          double vy = 0.0;
-          if (a.work) vy = div_rn(p.y, sqrt_rn(1.0 + (p.x2 + p.y * p.y + p.z2)));
-          const Push64 r = push64<UNIT, false>(0.0, ey, bz, 0.5 * hp, a.qm, p);
-          a.x[i] = x + a.dt * r.vx;
-          if (a.work) a.work[i] = a.work[i] + ((a.qm * hp) * 0.5) * (ey * (vy + div_rn(p.y, r.gam)));
-          a.px[i] = p.x;
-          a.py[i] = p.y;
-          a.status[i] = 0;
-        }
-      }
-    }
-    a.k_sub[i] = (uint8_t)k_sub;
+    const int k = criterion_push_f64<P, UNIT>(a, i, sh);
+    k0 += k == 0 ? 1u : 0u;
+    k1 += k == 1 ? 1u : 0u;
+    if (k > 1) atomicAdd(&sh[k], 1ull);
+    a.k_sub[i] = (uint8_t)(k > 0 ? k : 0);
   }
   const unsigned k0w = __reduce_add_sync(0xffffffffu, k0), k1w = __reduce_add_sync(0xffffffffu, k1);
   if ((threadIdx.x & 31) == 0 && k0w) atomicAdd(&sh[0], (unsigned long long)k0w);
@@ -306,6 +304,30 @@ __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) 
   flush_f64(sh, a.stats);
   if (threadIdx.x > 0 && threadIdx.x < 8 && sh[threadIdx.x])
     atomicAdd(&a.bin[threadIdx.x], (int32_t)sh[threadIdx.x]);
+}
+
+// The whole step of a small ensemble in one launch, a warp (and a block) per
+// electron: its criterion and m = 1 push by one lane, a sub-cycle by all.  The
+// four launches of the three passes are most of such a step, and a few warps per
+// SM leave the FP64 unit idle between their chains' operations.  Steps of m = 1
+// pushes: 1 electron 17 us by the passes and 8.4 so (11.5 once, as one thread per
+// electron), 608 17 and 8.5, 1,216 17.5 and 12.3, 2,432 17.5 and 16.7; with
+// sub-cycles, 256 electrons 1,071 and 1,024, 1,216 1,461 and 1,413.
+constexpr int kEachF64 = 8;  // electrons per SM
+template <int P, bool UNIT>
+__global__ void __launch_bounds__(32) each_f64_kernel(PushArgsF64 a) {
+  __shared__ unsigned long long sh[12];
+  if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
+  __syncwarp();
+  const int64_t i = blockIdx.x;
+  int k = 0;
+  if (threadIdx.x == 0) {
+    k = criterion_push_f64<P, UNIT>(a, i, sh);
+    if (k >= 0) atomicAdd(&sh[k], 1ull);
+  }
+  k = __shfl_sync(0xffffffffu, k, 0);
+  if (k > 0) subcycle_f64<P, UNIT>(a, i, true, 1, k, sh);
+  flush_f64(sh, a.stats);
 }
 
 // Every step starts from counts of zero, so that a captured step can be replayed.
@@ -373,7 +395,8 @@ __global__ void __launch_bounds__(32) subcycle_f64_kernel(PushArgsF64 a) {
     int64_t first, end;
     int k, g;
     if (!item_f64(a.bin, a.sms, t, first, end, k, g)) break;
-    subcycle_f64<P, UNIT>(a, first, end, g, k, sh);
+    const int64_t q = first + (threadIdx.x & (g - 1));
+    subcycle_f64<P, UNIT>(a, q < end ? a.queue[q] : 0, q < end, g, k, sh);
     int next = 0;
     if (threadIdx.x == 0) next = atomicAdd(&a.bin[16], 1);
     t = (int64_t)gridDim.x + __shfl_sync(0xffffffffu, next, 0);
@@ -385,6 +408,12 @@ __global__ void __launch_bounds__(32) subcycle_f64_kernel(PushArgsF64 a) {
 template <int P, bool UNIT>
 static void launch_f64_p(PushArgsF64 a, int sms, cudaStream_t s, int* launches) {
   a.sms = sms;
+  if (a.n <= (int64_t)sms * kEachF64) {
+    a.nodes = nullptr;
+    each_f64_kernel<P, UNIT><<<(int)a.n, 32, 0, s>>>(a);
+    if (launches) ++*launches;
+    return;
+  }
   int n = 3;
   if (a.nodes) {
     const int64_t want = (a.mask + 128) / 128;

@@ -1,6 +1,6 @@
-"""The FP64 push with and without its node fields (a window with more nodes than
-electrons gathers the levels), against the oracle bit for bit; and what a large
-window costs a small ensemble."""
+"""The FP64 push by its routes, against the oracle bit for bit: with and without
+its node fields (a window with more nodes than electrons gathers the levels),
+small ensembles in one launch; and what a large window costs a small ensemble."""
 from __future__ import annotations
 
 import numpy as np
@@ -88,3 +88,23 @@ def test_a_large_window_does_not_slow_a_small_ensemble():
         ms[lw] = sorted(t)[4]
         it.close()
     assert ms[22] < 3.0 * ms[12], ms
+
+
+# one warp per electron up to eight per SM, in one launch; the three passes beyond
+@pytest.mark.parametrize("n", [1, 2, 33, 8 * 152, 8 * 152 + 1])
+@pytest.mark.parametrize("order,work", [(1, False), (3, True), (5, False)])
+def test_small_ensembles(n, order, work):
+    _both(n, 64, order, k_max=5 if n < 100 else 3, work=work, qm=-1.0 if order < 5 else -0.37)
+
+
+def test_small_ensembles_take_one_launch():
+    it = native.Integrator(W.DT75, W.DT75 / 0.99, 0.01, precision=native.PIC_FP64, capacity=100, window=64,
+                           ring_levels=8)
+    z = np.zeros(100)
+    it.pic_particles_write(z + 3.0, z, z, z)
+    for r in range(7):
+        it.pic_fields_upload(r - 3, -8, np.ones(64), np.ones(64))
+    before = it.launches()
+    it.pic_push_step(0, 4)
+    assert it.launches() - before == 4
+    it.close()
