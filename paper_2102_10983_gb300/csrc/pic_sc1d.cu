@@ -17,7 +17,8 @@
 //     (h/dt) v_y S(x_mid) of every sub-step to per-node FP64 sums, and at the
 //     end of the macro step one rounded fixed-point value per node to J_y, and
 //     the charge flux of its move (start -> end or frozen position) to J_x.
-//     As in push_f64.cu: node fields at t_n once per step (nodes_kernel), the
+//     As in push_f64.cu: node fields at t_n once per step (nodes_kernel; a grid
+//     of more entries than electrons is gathered from instead), the
 //     m = 1 electrons in order (push_deposit_kernel), the others in warps of
 //     equal k (subcycle_deposit_kernel), and roots, quotients, floors and
 //     conversions off the FP64 unit, which bounds the kernels (19 clocks per
@@ -62,7 +63,7 @@ struct Sc1dArgs {
   int64_t crit_row;
   DevStats* stats;
   float crit_scale;   // criterion_f64_scale
-  double2* nodes;     // [M][3]: {f, f_next - f} of E_x, E_y, B_z at t_n
+  double2* nodes;     // nullptr, or [M][3]: {f, f_next - f} of E_x, E_y, B_z at t_n (node_fields_pay)
   uint8_t* k_sub;     // as in PushArgsF64
   int32_t* queue;
   int32_t* bin;
@@ -172,10 +173,80 @@ __global__ void __launch_bounds__(128) nodes_kernel(Sc1dArgs a) {
   }
 }
 
+// What an electron adds to the grid sums: d0, d1 to D at node jd and the next,
+// f0, f1 to F after node jf and the next.
+struct Deposit {
+  int64_t jd = 0, d0 = 0, d1 = 0, jf = 0, f0 = 0, f1 = 0;
+};
+
+// One grid's field at t_n about the array index q, offset w, from the levels.
+template <int P>
+__device__ __forceinline__ double gather_tn(const double* const* lv, const double* wt, int64_t q, double w) {
+  double f0 = wt[0] * __ldg(lv[0] + q), f1 = wt[0] * __ldg(lv[0] + q + 1);
+#pragma unroll
+  for (int l = 1; l <= P; ++l) {
+    f0 = f0 + wt[l] * __ldg(lv[l] + q);
+    f1 = f1 + wt[l] * __ldg(lv[l] + q + 1);
+  }
+  return f0 + w * (f1 - f0);
+}
+
+// Electron i's criterion and, with k = 0, its m = 1 push and deposit: its k, or
+// -1 if it is lost (or is now).
+template <int P, bool UNIT>
+__device__ __forceinline__ int criterion_deposit(const Sc1dArgs& a, int64_t i, unsigned long long* sh, Deposit& dep) {
+  const uint8_t st = a.status[i];
+  if (st & PIC_STATUS_LOST) return -1;
+  const double x = a.x[i];
+  Mom64 p = mom64(a.px[i], a.py[i], a.pz[i]);
+  Coords64 c;
+  if (!locate(a, x * a.inv_dx, c)) {
+    a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
+    atomicAdd(&sh[11], 1ull);
+    return -1;
+  }
+  double ex, ey, bz;
+  if (a.nodes) {
+    const double2 nx = __ldg(a.nodes + 3 * (c.jb + 2)), ny = __ldg(a.nodes + 3 * (c.je + 2) + 1),
+                  nb = __ldg(a.nodes + 3 * (c.jb + 2) + 2);
+    ex = nx.x + c.wb * nx.y;
+    ey = ny.x + c.we * ny.y;
+    bz = nb.x + c.wb * nb.y;
+  } else {
+    const double* wE = a.wtab + wrow(0, 1) * (2 * (P + 1));
+    ex = gather_tn<P>(a.Ex, wE, c.jb + 2, c.wb);
+    ey = gather_tn<P>(a.Ey, wE, c.je + 2, c.we);
+    bz = gather_tn<P>(a.Bz, a.wtab + a.crit_row * (2 * (P + 1)) + (P + 1), c.jb + 2, c.wb);
+  }
+  bool capped;
+  const int k = criterion_f64(a.crit_scale, a.qm_abs, a.dt, a.psi_max, a.k_max, bz, p.x, p.y, p.z, capped);
+  if (capped) atomicAdd(&sh[10], 1ull);
+  if (k > 0) return k;
+  const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
+  const Push64 r = push64<UNIT, true>(ex, ey, bz, 0.5 * hp, a.qm, p);
+  const double hv = a.dt * r.vx;
+  const double xn = x + hv;
+  a.x[i] = xn;
+  a.px[i] = p.x;
+  a.py[i] = p.y;
+  a.status[i] = 0;
+  const int64_t Q = a.Q[i];
+  const double Qd = ll_to_double(Q);
+  double w;
+  floor_frac64((x + half64(hv)) * a.inv_dx, dep.jd, w);
+  const double t = r.vy * w;
+  dep.d0 = -double_to_ll((r.vy - t) * Qd);
+  dep.d1 = -double_to_ll(t * Qd);
+  int64_t ib;
+  floor_frac64(xn * a.inv_dx, ib, w);
+  face_flux(Q, c.je, c.we, ib, w, dep.jf, dep.f0, dep.f1);
+  return 0;
+}
+
 // The three passes of push_f64.cu with E_x and the deposit: (1) here, every
 // electron's criterion, the m = 1 push and its deposit; (2) bin_f64_kernel;
 // (3) subcycle_deposit_kernel.
-template <bool UNIT>
+template <int P, bool UNIT>
 __global__ void __launch_bounds__(256) push_deposit_kernel(Sc1dArgs a) {
   __shared__ unsigned long long sh[12];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
@@ -183,57 +254,16 @@ __global__ void __launch_bounds__(256) push_deposit_kernel(Sc1dArgs a) {
   unsigned k0 = 0, k1 = 0;
   for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < a.n; b += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = b + threadIdx.x;
-    const uint8_t st = i < a.n ? a.status[i] : PIC_STATUS_LOST;
-    int k_sub = 0;
-    int64_t jd = 0, d0 = 0, d1 = 0, jf = 0, f0 = 0, f1 = 0;
-    if (!(st & PIC_STATUS_LOST)) {
-      const double x = a.x[i];
-      Mom64 p = mom64(a.px[i], a.py[i], a.pz[i]);
-      Coords64 c;
-      if (!locate(a, x * a.inv_dx, c)) {
-        a.status[i] = (uint8_t)(st | PIC_STATUS_LOST);
-        atomicAdd(&sh[11], 1ull);
-      } else {
-        const double2 nx = __ldg(a.nodes + 3 * (c.jb + 2)), ny = __ldg(a.nodes + 3 * (c.je + 2) + 1),
-                      nb = __ldg(a.nodes + 3 * (c.jb + 2) + 2);
-        const double bz = nb.x + c.wb * nb.y;
-        bool capped;
-        const int k = criterion_f64(a.crit_scale, a.qm_abs, a.dt, a.psi_max, a.k_max, bz, p.x, p.y, p.z,
-                                    capped);
-        if (capped) atomicAdd(&sh[10], 1ull);
-        if (k > 0) {
-          k_sub = k;
-          if (k == 1)
-            ++k1;
-          else
-            atomicAdd(&sh[k], 1ull);
-        } else {
-          ++k0;
-          const double ex = nx.x + c.wb * nx.y, ey = ny.x + c.we * ny.y;
-          const double hp = 0.5 * (pow4_down64(a.dt, st & 0x7f) + a.dt);
-          const Push64 r = push64<UNIT, true>(ex, ey, bz, 0.5 * hp, a.qm, p);
-          const double hv = a.dt * r.vx;
-          const double xn = x + hv;
-          a.x[i] = xn;
-          a.px[i] = p.x;
-          a.py[i] = p.y;
-          a.status[i] = 0;
-          const int64_t Q = a.Q[i];
-          const double Qd = ll_to_double(Q);
-          double w;
-          floor_frac64((x + half64(hv)) * a.inv_dx, jd, w);
-          const double t = r.vy * w;
-          d0 = -double_to_ll((r.vy - t) * Qd);
-          d1 = -double_to_ll(t * Qd);
-          int64_t ib;
-          floor_frac64(xn * a.inv_dx, ib, w);
-          face_flux(Q, c.je, c.we, ib, w, jf, f0, f1);
-        }
-      }
+    Deposit dep;
+    if (i < a.n) {
+      const int k = criterion_deposit<P, UNIT>(a, i, sh, dep);
+      k0 += k == 0 ? 1u : 0u;
+      k1 += k == 1 ? 1u : 0u;
+      if (k > 1) atomicAdd(&sh[k], 1ull);
+      a.k_sub[i] = (uint8_t)(k > 0 ? k : 0);
     }
-    if (i < a.n) a.k_sub[i] = (uint8_t)k_sub;
-    add_pair_warp(a.D, jd + 2, a.M, d0, d1);
-    add_pair_warp(a.F, jf + 2, a.M, f0, f1);
+    add_pair_warp(a.D, dep.jd + 2, a.M, dep.d0, dep.d1);
+    add_pair_warp(a.F, dep.jf + 2, a.M, dep.f0, dep.f1);
   }
   const unsigned k0w = __reduce_add_sync(0xffffffffu, k0), k1w = __reduce_add_sync(0xffffffffu, k1);
   if ((threadIdx.x & 31) == 0 && k0w) atomicAdd(&sh[0], (unsigned long long)k0w);
@@ -272,16 +302,14 @@ struct NodeSums {
   }
 };
 
-// The sub-cycles, g equal-k electrons per warp (subcycle_f64 of push_f64.cu,
-// with E_x and the deposit).
+// The sub-cycles, g equal-k electrons per warp, each lane's i (subcycle_f64 of
+// push_f64.cu, with E_x and the deposit).
 template <int P, bool UNIT>
-__device__ __forceinline__ void subcycle_deposit(const Sc1dArgs& a, int64_t first, int64_t end, int g, int k,
+__device__ __forceinline__ void subcycle_deposit(const Sc1dArgs& a, int64_t i, bool valid, int g, int k,
                                                  unsigned long long* sh) {
   constexpr int stride = 2 * (P + 1);
   const int lane = threadIdx.x & 31, mine = lane & (g - 1), rows = 32 / g;
   const int copy = lane / g;
-  const bool valid = first + mine < end;
-  const int64_t i = valid ? a.queue[first + mine] : 0;
   const uint8_t st = valid ? a.status[i] : 0;
   double xi = valid ? a.x[i] : 0.0;
   Mom64 p = valid ? mom64(a.px[i], a.py[i], a.pz[i]) : Mom64{0.0, 0.0, 0.0, 0.0, 0.0};
@@ -369,13 +397,39 @@ __global__ void __launch_bounds__(32) subcycle_deposit_kernel(Sc1dArgs a) {
     int64_t first, end;
     int k, g;
     if (!item_f64(a.bin, a.sms, t, first, end, k, g)) break;
-    subcycle_deposit<P, UNIT>(a, first, end, g, k, sh);
+    const int64_t q = first + (threadIdx.x & (g - 1));
+    subcycle_deposit<P, UNIT>(a, q < end ? a.queue[q] : 0, q < end, g, k, sh);
     int next = 0;
     if (threadIdx.x == 0) next = atomicAdd(&a.bin[16], 1);
     t = (int64_t)gridDim.x + __shfl_sync(0xffffffffu, next, 0);
   }
   __syncwarp();
   if (threadIdx.x == 0 && sh[11]) atomicAdd(&a.stats->lost, sh[11]);
+}
+
+// A small ensemble's step in one launch, a warp per electron (each_f64_kernel of
+// push_f64.cu).  100 electrons on 20,000 cells, m = 1: 32 us per step by the
+// passes, 18 so (28 once, as one thread per electron).
+constexpr int kEachSc1d = 8;  // electrons per SM
+template <int P, bool UNIT>
+__global__ void __launch_bounds__(32) each_deposit_kernel(Sc1dArgs a) {
+  __shared__ unsigned long long sh[12];
+  if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
+  __syncwarp();
+  const int64_t i = blockIdx.x;
+  int k = 0;
+  if (threadIdx.x == 0) {
+    Deposit dep;
+    k = criterion_deposit<P, UNIT>(a, i, sh, dep);
+    if (k >= 0) atomicAdd(&sh[k], 1ull);
+    if (dep.d0) add_i64(a.D, dep.jd + 2, a.M, dep.d0);
+    if (dep.d1) add_i64(a.D, dep.jd + 3, a.M, dep.d1);
+    if (dep.f0) add_i64(a.F, dep.jf + 2, a.M, dep.f0);
+    if (dep.f1) add_i64(a.F, dep.jf + 3, a.M, dep.f1);
+  }
+  k = __shfl_sync(0xffffffffu, k, 0);
+  if (k > 0) subcycle_deposit<P, UNIT>(a, i, true, 1, k, sh);
+  flush_f64(sh, a.stats);
 }
 
 struct FieldArgs {
@@ -574,7 +628,12 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   ok &= cudaMalloc(&c->wtab, wcount * 8) == cudaSuccess;
   ok &= cudaMalloc(&c->dstats, sizeof(DevStats)) == cudaSuccess;
   ok &= cudaMalloc(&c->staging, 3 * c->M * 8) == cudaSuccess;
-  ok &= cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) == cudaSuccess;
+  // without node fields (a grid that no ensemble of this capacity pays for, no
+  // room) the push gathers the levels
+  if (node_fields_pay(cap, c->M) && cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) != cudaSuccess) {
+    c->nodes = nullptr;
+    cudaGetLastError();
+  }
   const int64_t slice = cap < kSlice ? cap : kSlice;
   ok &= cudaMalloc(&c->k_sub, slice) == cudaSuccess;
   ok &= cudaMalloc(&c->queue, slice * 4) == cudaSuccess;
@@ -711,7 +770,17 @@ static void launch_push(pic_sc1d* c, const Sc1dArgs& all, int64_t off = 0) {
   a.x += off; a.px += off; a.py += off; a.pz += off; a.status += off; a.Q += off;
   a.n = all.n - off < kSlice ? all.n - off : kSlice;
   const bool unit = a.qm_abs == 1.0;
-  if (off == 0)
+  if (all.n <= (int64_t)a.sms * kEachSc1d) {
+    a.nodes = nullptr;
+    if (unit)
+      each_deposit_kernel<P, true><<<(int)a.n, 32, 0, s>>>(a);
+    else
+      each_deposit_kernel<P, false><<<(int)a.n, 32, 0, s>>>(a);
+    ++c->launches;
+    return;
+  }
+  const bool fill = off == 0 && a.nodes;
+  if (fill)
     nodes_kernel<P><<<grid_for(c, 2 * 3 * c->M), 128, 0, s>>>(a);
   else
     cudaMemsetAsync(a.bin, 0, kBinF64 * sizeof(int32_t), s);
@@ -720,9 +789,9 @@ static void launch_push(pic_sc1d* c, const Sc1dArgs& all, int64_t off = 0) {
   const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)a.sms * 8;
   const int blocks = (int)(want < cap ? want : cap);
   if (unit)
-    push_deposit_kernel<true><<<blocks, threads, 0, s>>>(a);
+    push_deposit_kernel<P, true><<<blocks, threads, 0, s>>>(a);
   else
-    push_deposit_kernel<false><<<blocks, threads, 0, s>>>(a);
+    push_deposit_kernel<P, false><<<blocks, threads, 0, s>>>(a);
   launch_bin_f64(BinF64{a.n, a.k_sub, a.queue, a.bin}, a.sms, s);
   const int64_t most = (int64_t)a.sms * 12;
   const int warps = (int)(a.n < most ? a.n : most);
@@ -730,7 +799,7 @@ static void launch_push(pic_sc1d* c, const Sc1dArgs& all, int64_t off = 0) {
     subcycle_deposit_kernel<P, true><<<warps, 32, 0, s>>>(a);
   else
     subcycle_deposit_kernel<P, false><<<warps, 32, 0, s>>>(a);
-  c->launches += off == 0 ? 4 : 3;
+  c->launches += fill ? 4 : 3;
   if (off + a.n < all.n) launch_push<P>(c, all, off + a.n);
 }
 
@@ -777,7 +846,7 @@ extern "C" int pic_sc1d_step(pic_sc1d* c, int64_t n0, int64_t n_steps, pic_sc1d_
     a.stats = c->dstats;
     if (c->n > 0) {
       a.crit_scale = criterion_f64_scale(a.qm_abs, a.dt, a.psi_max);
-      a.nodes = c->nodes;
+      a.nodes = node_fields_pay(c->n, c->M) ? c->nodes : nullptr;
       a.k_sub = c->k_sub;
       a.queue = c->queue;
       a.bin = c->bin;
