@@ -4,19 +4,21 @@
 // the field sampled on the grid (the "perfectly propagating PIC" of Sec. III):
 // E_y at nodes i dx and times n dt, B_z at (i + 1/2) dx and (n + 1/2) dt.
 //
-// One warp per electron: each integrates its whole trajectory with the method
-// (Algorithm 1 of Sec. IV, order-p Lagrange in time of Sec. VI, tent in space,
-// Boris), in FP64 compiled with -fmad=false in the order of a serial
-// evaluation.  A trajectory is one serial chain, and the FP64 unit takes 19
-// clocks for a warp instruction with one active lane as with 32, so a warp of
-// 32 electrons (as this once was) ran all of them as long as its largest 4^k,
-// at 2 us per sub-step.  Here the chain is taken by every lane alike and the
-// work beside it is dealt to the lanes: the field at the nodes about the
-// electron (the formula's exp, sin, cos: one evaluation of the warp per macro
-// step serves all levels, grids and nodes, and the diagnostic's a), the
-// Lagrange weights and the temporal sums of 32 sub-steps at a time.  Orders 1,
-// 3 and 5, a0 = 5, lambda/75, 64 electrons each, 2,000 macro steps: 264 ms
-// with 32 electrons per warp, 25 ms so.
+// Each electron integrates its whole trajectory with the method (Algorithm 1 of
+// Sec. IV, order-p Lagrange in time of Sec. VI, tent in space, Boris), in FP64
+// compiled with -fmad=false in the order of a serial evaluation.  A trajectory
+// is one serial chain, and the FP64 unit takes 19 clocks for a warp instruction
+// with one active lane as with 32.  So there are two forms of the same bits:
+//  study_kernel, one warp per electron: the chain is taken by every lane alike
+//    and the work beside it is dealt to the lanes: the field at the nodes about
+//    the electron (the formula's exp, sin, cos: one evaluation of the warp per
+//    macro step serves all levels, grids and nodes, and the diagnostic's a), the
+//    Lagrange weights and the temporal sums of 32 sub-steps at a time (orders 1,
+//    3 and 5, a0 = 5, lambda/75, 64 electrons each, 2,000 macro steps: 25 ms, 264
+//    as one thread per electron);
+//  study_many_kernel, one thread per electron: 32 chains for the unit's time of
+//    one, where there are more electrons than the unit has time for.
+// pic_study_run chooses by the cases' steps and electrons (study_by_warp).
 //
 // Per electron and macro step (Sec. IV, Eqs. R error, gamma error): R = gamma
 // - p_x, the energy error |gamma - gamma_th| / gamma_th with gamma_th = 1 +
@@ -273,6 +275,116 @@ __device__ __forceinline__ void study_electron(const pic_study_case& q, double x
   *k_count = count;
 }
 
+// The field values of one grid at a node pair for the levels n - P .. n (E:
+// times l dt; B: half a step on), from the formula as the electron comes to
+// them: a macro step that keeps the nodes computes only the newest level.
+template <int P, bool IS_B>
+struct FieldPair {
+  NodePair<P> v;
+  int64_t node = INT64_MIN, level = INT64_MIN;
+  static __device__ __forceinline__ double at(const pic_study_case& q, int64_t l, int64_t i) {
+    const double off = IS_B ? 0.5 : 0.0;
+    const double xi = (ll_to_double(l) + off) * q.dt - (ll_to_double(i) + off) * q.dx;
+    const double d = xi - q.xi0, ss = q.sigma * q.sigma;
+    const double env = q.a0 * exp(div_rn(-(d * d), 2.0 * q.sigma * q.sigma));
+    double sn, cs;
+    sincos(xi, &sn, &cs);
+    return -(env * (cs - div_rn(d, ss) * sn));  // as FieldTile::fill
+  }
+  __device__ __forceinline__ void ensure(const pic_study_case& q, int64_t j, int64_t n) {
+    if (j == node && n == level) return;
+    int first = 0;
+    if (j == node && n == level + 1) {
+#pragma unroll
+      for (int l = 0; l < P; ++l) {
+        v.v0[l] = v.v0[l + 1];
+        v.v1[l] = v.v1[l + 1];
+      }
+      first = P;
+    }
+#pragma unroll 1
+    for (int l = first; l <= P; ++l) {
+      const double a = at(q, n - P + l, j), b = at(q, n - P + l, j + 1);
+#pragma unroll
+      for (int r = 0; r <= P; ++r)
+        if (r == l) {
+          v.v0[r] = a;
+          v.v1[r] = b;
+        }
+    }
+    node = j;
+    level = n;
+  }
+};
+
+// study_electron by one thread.
+template <int P, bool UNIT>
+__device__ __forceinline__ void study_electron_alone(const pic_study_case& q, double x0, double* out_eps_r,
+                                                     double* out_eps_e, double* out_gmax, int64_t* n_star,
+                                                     int64_t* substeps, int64_t* k_count) {
+  const double dt = q.dt, inv_dx = 1.0 / q.dx;
+  const double qm_abs = fabs(q.qm);
+  const float scale = criterion_f64_scale(qm_abs, dt, q.psi_max);
+  FieldPair<P, false> E;
+  FieldPair<P, true> B;
+  Mom64 p = mom64(0.0, 0.0, 0.0);
+  double xi = x0;
+  int k_prev = 0;
+  double eps_r = 0.0, eps_e = 0.0, gmax = 1.0;
+  int64_t ns = 0, sub = 0;
+  double w[P + 1];
+  Coords64 c;
+  auto locate = [&]() {
+    const double s = xi * inv_dx;
+    if (!coords64_fast(s, c)) coords64_any(s, c);
+  };
+  auto gather = [&](auto& F, bool is_b, int64_t j, int64_t n, double theta, double off) {
+    F.ensure(q, j, n);
+    lagrange<P>(is_b ? false : true, theta, w);
+    F.v.sums(w);
+    return F.v.f + off * F.v.d;
+  };
+  for (int64_t n = 0; n < q.n_steps; ++n) {
+    locate();
+    const double b0 = gather(B, true, c.jb, n, 0.5, c.wb);
+    bool capped;
+    const int k = criterion_f64(scale, qm_abs, dt, q.psi_max, q.k_max, b0, p.x, p.y, p.z, capped);
+    const int m = 1 << (2 * k);
+    const double h = pow4_down64(dt, k), h_old = pow4_down64(dt, k_prev);
+    k_count[k] += 1;
+    sub += m;
+    if (k > 0) ns += m;
+    double half = 0.5 * (0.5 * (h_old + h));
+    Push64 r;
+#pragma unroll 1
+    for (int j = 0; j < m; ++j) {
+      if (j > 0) locate();
+      const double th = theta_of(q.field_time, j, k);
+      const double ey = gather(E, false, c.je, n, th, c.we), bz = gather(B, true, c.jb, n, th, c.wb);
+      r = push64<UNIT, false>(0.0, ey, bz, half, q.qm, p);
+      xi = xi + h * r.vx;
+      half = 0.5 * h;
+    }
+    k_prev = k;
+    const double dR = fabs((r.gam - p.x) - 1.0);
+    if (dR > eps_r) eps_r = dR;
+    if (r.gam > gmax) gmax = r.gam;
+    const double t_p = ll_to_double(n + 1) * dt - 0.5 * h;
+    const double ph = t_p - (xi - 0.5 * h * r.vx), d = ph - q.xi0;
+    double sn, cs;
+    sincos(ph, &sn, &cs);
+    const double a = q.a0 * exp(div_rn(-(d * d), 2.0 * q.sigma * q.sigma)) * sn;
+    const double g_th = 1.0 + 0.5 * a * a;
+    const double de = div_rn(fabs(r.gam - g_th), g_th);
+    if (de > eps_e) eps_e = de;
+  }
+  *out_eps_r = eps_r;
+  *out_eps_e = eps_e;
+  *out_gmax = gmax;
+  *n_star = ns;
+  *substeps = sub;
+}
+
 __device__ __forceinline__ void atomic_max_pos(unsigned long long* a, double v) {
   atomicMax(a, (unsigned long long)__double_as_longlong(v));  // v >= 0
 }
@@ -290,6 +402,31 @@ __device__ __forceinline__ void study_order(const pic_study_case& q, double x0, 
     study_electron<P, true>(q, x0, sm, er, ee, gm, ns, sub, kc);
   else
     study_electron<P, false>(q, x0, sm, er, ee, gm, ns, sub, kc);
+}
+
+template <int P>
+__device__ __forceinline__ void study_order_alone(const pic_study_case& q, double x0, double* er, double* ee,
+                                                  double* gm, int64_t* ns, int64_t* sub, int64_t* kc) {
+  if (fabs(q.qm) == 1.0)
+    study_electron_alone<P, true>(q, x0, er, ee, gm, ns, sub, kc);
+  else
+    study_electron_alone<P, false>(q, x0, er, ee, gm, ns, sub, kc);
+}
+
+// An electron's part in its case's results.
+__device__ __forceinline__ void study_report(StudyAcc& A, pic_study_result& r, int e, double er, double ee,
+                                             double gm, int64_t ns, int64_t sub) {
+  atomic_max_pos(&A.eps_r, er);
+  atomic_max_pos(&A.eps_e, ee);
+  atomic_max_pos(&A.gmax, gm);
+  atomicAdd(&A.n_star_sum, (unsigned long long)ns);
+  atomicAdd(&A.substeps_sum, (unsigned long long)sub);
+  if (e == 0) {
+    r.eps_dephasing_first = er;
+    r.eps_energy_first = ee;
+    r.gamma_max_first = gm;
+    r.n_star_first = ns;
+  }
 }
 
 // One warp per CTA and electron: block b runs electron b mod per_case of case
@@ -314,19 +451,51 @@ __global__ void __launch_bounds__(32) study_kernel(const pic_study_case* cases, 
   }
   StudyAcc& A = acc[c];
   if (threadIdx.x < 8 && kc) atomicAdd(&A.k_hist[threadIdx.x], (unsigned long long)kc);
-  if (threadIdx.x > 0) return;
-  atomic_max_pos(&A.eps_r, er);
-  atomic_max_pos(&A.eps_e, ee);
-  atomic_max_pos(&A.gmax, gm);
-  atomicAdd(&A.n_star_sum, (unsigned long long)ns);
-  atomicAdd(&A.substeps_sum, (unsigned long long)sub);
-  if (e == 0) {
-    pic_study_result& r = out[c];
-    r.eps_dephasing_first = er;
-    r.eps_energy_first = ee;
-    r.gamma_max_first = gm;
-    r.n_star_first = ns;
+  if (threadIdx.x == 0) study_report(A, out[c], e, er, ee, gm, ns, sub);
+}
+
+// One thread per electron, one warp per CTA: block b runs electrons 32 (b mod
+// per_case) .. + 31 of case b / per_case.
+__global__ void __launch_bounds__(32) study_many_kernel(const pic_study_case* cases, pic_study_result* out,
+                                                        StudyAcc* acc, int per_case) {
+  const int c = blockIdx.x / per_case;
+  const pic_study_case q = cases[c];
+  const int e = (blockIdx.x % per_case) * 32 + (int)threadIdx.x;
+  if (e >= q.n_electrons) return;
+  const double x0 = (2.0 * M_PI) * (double)e / (double)q.n_electrons;
+  double er, ee, gm;
+  int64_t ns, sub;
+  int64_t kc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  switch (q.order) {
+    case 1: study_order_alone<1>(q, x0, &er, &ee, &gm, &ns, &sub, kc); break;
+    case 2: study_order_alone<2>(q, x0, &er, &ee, &gm, &ns, &sub, kc); break;
+    case 3: study_order_alone<3>(q, x0, &er, &ee, &gm, &ns, &sub, kc); break;
+    case 4: study_order_alone<4>(q, x0, &er, &ee, &gm, &ns, &sub, kc); break;
+    default: study_order_alone<5>(q, x0, &er, &ee, &gm, &ns, &sub, kc); break;
   }
+  StudyAcc& A = acc[c];
+  for (int k = 0; k < 8; ++k)
+    if (kc[k]) atomicAdd(&A.k_hist[k], (unsigned long long)kc[k]);
+  study_report(A, out[c], e, er, ee, gm, ns, sub);
+}
+
+// Whether a warp per electron is the faster form.  It takes the FP64 unit's time
+// for every electron and macro step; a thread per electron takes the longest
+// case's chain.  Per macro step on the GB300 (a0 from 2 to 100, lambda/50 and /75):
+// 17.5 ns per electron and a chain of 75 us with sub-cycles (a warp runs as long
+// as its largest 4^k), 12.3 ns and 26 us without.  256 electrons per case, a0 = 25:
+// 15 cases 259 ms by warps and 309 by threads, 20 cases 339 and 308, 60 cases 939
+// and 346.
+bool study_by_warp(const pic_study_case* cases, int32_t n, int sms) {
+  double by_warp = 0.0, by_thread = 0.0;  // us
+  for (int32_t i = 0; i < n; ++i) {
+    const pic_study_case& q = cases[i];
+    const bool sub = q.k_max > 0 && fabs(q.qm * q.a0) * q.dt > 2.0 * q.psi_max;
+    const double steps = (double)q.n_steps, chain = steps * (sub ? 75.0 : 26.0);
+    by_warp += steps * (double)q.n_electrons * (sub ? 17.5e-3 : 12.3e-3) * 152.0 / (double)(sms > 0 ? sms : 152);
+    by_thread = chain > by_thread ? chain : by_thread;
+  }
+  return by_warp <= by_thread;
 }
 
 }  // namespace
@@ -373,7 +542,15 @@ extern "C" int pic_study_run(const pic_study_case* cases, int32_t n_cases, pic_s
   for (int32_t i = 0; i < n_cases; ++i)
     per_case = cases[i].n_electrons > per_case ? cases[i].n_electrons : per_case;
   if (e == cudaSuccess) {
-    study_kernel<<<(unsigned)(n_cases * per_case), 32, 0, st>>>(dcases, dout, dacc, per_case);
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (study_by_warp(cases, n_cases, sms)) {
+      study_kernel<<<(unsigned)(n_cases * per_case), 32, 0, st>>>(dcases, dout, dacc, per_case);
+    } else {
+      per_case = (per_case + 31) / 32;
+      study_many_kernel<<<(unsigned)(n_cases * per_case), 32, 0, st>>>(dcases, dout, dacc, per_case);
+    }
     e = cudaGetLastError();
   }
   std::vector<StudyAcc> acc(n_cases);
