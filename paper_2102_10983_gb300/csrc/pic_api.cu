@@ -42,7 +42,7 @@ struct pic_ctx {
   uint8_t* pred = nullptr;
   float4* nodes = nullptr;  // mixed form: the step's node fields (PushArgsMixed::nodes)
   float* coef = nullptr;  // mixed form: per node monomial coefficients, step s's in table s mod T
-  int32_t T = 2;          // tables kept (coef_steps_kept)
+  int32_t T = 2;          // tables kept (coef_steps_kept; none where nothing reads them)
   float* feat = nullptr;  // mixed form: the predictor's feature nodes (E_y, B_z at t_{n+1}), W + 1 each
   // binned mixed form: resumable long sub-cycles (per particle: the step it is
   // in and the sub-steps done), and a device copy of slot_i0 for the kernel
@@ -215,8 +215,9 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
   if (mixed) {
     A((void**)&c->nodes, (size_t)window_cells * sizeof(float4));
     const size_t table = (size_t)window_cells * 2 * (prm->order + 1) * 4;
-    c->T = prm->schedule == PIC_SCHED_PLAIN ? 2 : coef_steps_kept(table);
-    A((void**)&c->coef, c->T * table);
+    // the plain schedule reads this step's table, at order 3 only
+    c->T = prm->schedule != PIC_SCHED_PLAIN ? coef_steps_kept(table) : prm->order == 3 ? 1 : 0;
+    if (c->T > 0) A((void**)&c->coef, c->T * table);
     A((void**)&c->feat, 2 * ((size_t)window_cells + 1) * 4);
     A((void**)&c->cell, cap * 4);
     A((void**)&c->frac, cap * 4);
@@ -575,6 +576,7 @@ static void fill_mixed(pic_ctx* c, PushArgsMixed& a, int64_t s, int64_t lo, int6
 }
 
 static float* coef_table(const pic_ctx* c, int64_t s) {
+  if (!c->coef) return nullptr;
   return c->coef + (((s % c->T) + c->T) % c->T) * (c->W * 2 * (c->prm.order + 1));
 }
 

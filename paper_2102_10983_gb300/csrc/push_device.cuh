@@ -627,8 +627,10 @@ __device__ __forceinline__ bool cycle_near(const StepFields<P, RING>& F, int32_t
 // three -> with stretches: 300 electrons at the front 119 -> 117 -> 95 us,
 // 16.8M electrons 249 -> 219 -> 199 us, 1,000,003 at fifth order 120 -> 118 ->
 // 90 us.
+// A warp of mixed k (the plain schedule) would run both loops one after the
+// other: it takes NEAR = 1, all of them cycle_near.
 constexpr int kNearMin = 2, kHalfMin = 3;
-template <int P, bool RING, bool TABLE = false>
+template <int P, bool RING, bool TABLE = false, int NEAR = kNearMin>
 __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const float* wtab,
                                              int32_t mask, float dt, float inv_dx, float qm,
                                              int field_time,
@@ -654,7 +656,7 @@ __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const
   for (int j = j0; j < j_end && ok;) {
     int n = j_end - j;
     bool done = false;
-    if (k >= kNearMin) {
+    if (k >= NEAR) {
       float back = c.s.ux < 0.f ? 1.0f : 0.0f;
       if (k >= kHalfMin) {
         n = min(n, m >> 1);
