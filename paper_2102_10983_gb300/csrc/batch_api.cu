@@ -40,7 +40,7 @@ struct pic_batch {
   int64_t* prefix = nullptr;  // 7 n_ens + 1
   float4* nodes = nullptr;    // n_ens x W: the step's node fields
   int2* win = nullptr;        // T x n_ens: the steps' windows
-  int32_t T = 2;              // steps whose tables and windows are kept (coef_steps_kept)
+  int32_t T = 2;              // steps whose tables and windows are kept (alloc_coef_tables: 16 at most)
   int32_t* chunk_ens = nullptr;  // the stream items' ensembles
   float* coef = nullptr;      // T x n_ens x W x 2(p+1): node coefficient tables, step s's s mod T
   int32_t* lag_step = nullptr;  // per particle: the step a deferred particle is in (call-relative)
@@ -161,13 +161,12 @@ extern "C" int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t 
   A((void**)&b->qcount, sizeof(int32_t) * (2 * 8 * (size_t)n_ens + 8));
   A((void**)&b->prefix, sizeof(int64_t) * (7 * (size_t)n_ens + 1));
   A((void**)&b->nodes, sizeof(float4) * (size_t)n_ens * window_cells);
-  const size_t table_bytes = sizeof(float) * (size_t)n_ens * window_cells * 2 * (size_t)(order + 1);
-  b->T = coef_steps_kept(table_bytes);
-  A((void**)&b->win, sizeof(int2) * b->T * (size_t)n_ens);
   A((void**)&b->chunk_ens, sizeof(int32_t) * (cap / batch_tile() + 2 * (size_t)n_ens + 1));
-  A((void**)&b->coef, b->T * table_bytes);
   A((void**)&b->lag_step, cap * 4);
   A((void**)&b->lag_j, cap * 2);
+  A((void**)&b->win, sizeof(int2) * 16 * (size_t)n_ens);
+  if (e == cudaSuccess)
+    e = alloc_coef_tables(sizeof(float) * (size_t)n_ens * window_cells * 2 * (size_t)(order + 1), &b->coef, &b->T);
   if (e != cudaSuccess) {
     batch_free(b);
     delete b;

@@ -42,7 +42,7 @@ struct pic_ctx {
   uint8_t* pred = nullptr;
   float4* nodes = nullptr;  // mixed form: the step's node fields (PushArgsMixed::nodes)
   float* coef = nullptr;  // mixed form: per node monomial coefficients, step s's in table s mod T
-  int32_t T = 2;          // tables kept (coef_steps_kept; none where nothing reads them)
+  int32_t T = 1;          // tables kept (alloc_coef_tables; none where nothing reads them)
   float* feat = nullptr;  // mixed form: the predictor's feature nodes (E_y, B_z at t_{n+1}), W + 1 each
   // binned mixed form: resumable long sub-cycles (per particle: the step it is
   // in and the sub-steps done), and a device copy of slot_i0 for the kernel
@@ -53,8 +53,9 @@ struct pic_ctx {
   double* work = nullptr;  // FP64 form with PIC_DIAG_WORK: per-particle work of E
   // FP64 form: node fields at t_n (4 W, optional), k > 0 electrons of a step
   double* nodes64 = nullptr;
-  uint8_t* k_sub = nullptr;
   int32_t* queue64 = nullptr;
+  uint8_t* k_sub = nullptr;  // in queue64's allocation
+  int64_t slice64 = 0;
   int32_t* bin64 = nullptr;
   int32_t* pred_queue = nullptr;
   const pic_mlp* mlp = nullptr;
@@ -110,7 +111,7 @@ static void free_all(pic_ctx* c) {
                   c->status, c->ringE, c->ringB, c->staging, c->wtab64, c->wtab32,
                   c->dstats, c->queue, c->qcount, c->pred, c->pred_queue, c->nodes,
                   c->coef, c->lag_step, c->lag_j, c->dslot_i0, c->work, c->feat,
-                  c->nodes64, c->k_sub, c->queue64, c->bin64};
+                  c->nodes64, c->queue64, c->bin64};
   for (void* p : ptrs)
     if (p) cudaFree(p);
 }
@@ -214,10 +215,6 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
   };
   if (mixed) {
     A((void**)&c->nodes, (size_t)window_cells * sizeof(float4));
-    const size_t table = (size_t)window_cells * 2 * (prm->order + 1) * 4;
-    // the plain schedule reads this step's table, at order 3 only
-    c->T = prm->schedule != PIC_SCHED_PLAIN ? coef_steps_kept(table) : prm->order == 3 ? 1 : 0;
-    if (c->T > 0) A((void**)&c->coef, c->T * table);
     A((void**)&c->feat, 2 * ((size_t)window_cells + 1) * 4);
     A((void**)&c->cell, cap * 4);
     A((void**)&c->frac, cap * 4);
@@ -242,8 +239,6 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
     A((void**)&c->py, cap * 8);
     A((void**)&c->pz, cap * 8);
     if (prm->diagnostics == PIC_DIAG_WORK) A((void**)&c->work, cap * 8);
-    A((void**)&c->k_sub, cap);
-    A((void**)&c->queue64, cap * 4);
     A((void**)&c->bin64, kBinF64 * 4);
   }
   A((void**)&c->status, cap);
@@ -259,6 +254,13 @@ extern "C" int pic_create(const pic_params* prm, int64_t capacity, int64_t windo
   A((void**)&c->wtab64, (size_t)wcount * 8);
   if (mixed) A((void**)&c->wtab32, (size_t)wcount * 4);
   A((void**)&c->dstats, sizeof(DevStats));
+  const size_t table = (size_t)window_cells * 2 * (prm->order + 1) * 4;
+  if (e == cudaSuccess && !mixed)
+    e = alloc_bin_f64((int64_t)cap, (int64_t)1 << 31, &c->queue64, &c->k_sub, &c->slice64);
+  else if (e == cudaSuccess && prm->schedule != PIC_SCHED_PLAIN)
+    e = alloc_coef_tables(table, &c->coef, &c->T);
+  else if (prm->order == 3)  // the plain schedule reads this step's table, at order 3 only
+    A((void**)&c->coef, table);
   if (e != cudaSuccess) {
     free_all(c);
     delete c;
@@ -751,6 +753,7 @@ extern "C" int pic_push_step(pic_ctx* c, int64_t n, int64_t n_steps, pic_step_st
       a.hi_i = (int32_t)(hi < -i32 ? -i32 : hi > i32 ? i32 : hi);
       a.crit_scale = crit64;
       a.nodes = node_fields_pay(c->n, W) ? c->nodes64 : nullptr;
+      a.slice = c->slice64;
       a.k_sub = c->k_sub;
       a.queue = c->queue64;
       a.bin = c->bin64;

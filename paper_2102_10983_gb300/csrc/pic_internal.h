@@ -73,6 +73,25 @@ struct BinF64 {
   int32_t* bin;
 };
 
+// Device memory for that, of at most `most` electrons (a power of two): queue,
+// then k_sub, 5 bytes each in one allocation.  Without room for all of them
+// (down to 65,536) for fewer, *slice: the passes then take that many at a time.
+inline cudaError_t alloc_bin_f64(int64_t electrons, int64_t most, int32_t** queue, uint8_t** k_sub, int64_t* slice) {
+  int64_t n = electrons < most ? electrons : most;
+  for (;; n /= 2) {
+    n = (n + 15) & ~(int64_t)15;  // k_sub is read in 16-byte words
+    const cudaError_t e = cudaMalloc((void**)queue, (size_t)n * 5);
+    if (e == cudaSuccess) {
+      *k_sub = (uint8_t*)(*queue + n);
+      *slice = n;
+      return e;
+    }
+    *queue = nullptr;
+    if (e != cudaErrorMemoryAllocation || n <= 65536) return e;
+    cudaGetLastError();
+  }
+}
+
 // Arguments of the FP64 push (one macro step).
 struct PushArgsF64 {
   int64_t n;
@@ -94,8 +113,9 @@ struct PushArgsF64 {
   double* work;  // nullptr, or per particle the accumulated work of E (App. B)
   float crit_scale;   // criterion_f64_scale: 0 = the exact criterion only
   double* nodes;      // nullptr, or 4 W: each node's fields at t_n (nodes_f64_kernel; node_fields_pay)
-  uint8_t* k_sub;     // per particle: k of the step where k > 0 (written every step)
-  int32_t* queue;     // particles with k > 0, grouped by k
+  int64_t slice;      // particles the passes take at a time (alloc_bin_f64)
+  uint8_t* k_sub;     // per particle of a slice: k of the step where k > 0 (written every step)
+  int32_t* queue;     // the slice's particles with k > 0, grouped by k
   int32_t* bin;       // [kBinF64] the step's counts and cursors, zeroed by its first launch
   int sms;            // set by the launcher
 };
@@ -192,12 +212,20 @@ struct PushArgsMixed {
 // Fills PushArgsMixed::mono for order p (host side, FP64 expansion).
 void lagrange_monomials(int p, float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1]);
 
-// Steps whose node coefficient tables (table_bytes each) a context keeps: a
+// The node coefficient tables (table_bytes each) of the steps a context keeps: a
 // deferred particle a few steps behind the stream then reads a table as the
-// others of its warp do, instead of a path of its own; as many as 256 MB hold.
-inline int32_t coef_steps_kept(size_t table_bytes) {
-  const size_t n = ((size_t)256 << 20) / (table_bytes > 0 ? table_bytes : 1);
-  return (int32_t)(n < 2 ? 2 : n > 16 ? 16 : n);
+// others of its warp do, instead of a path of its own; as many as 256 MB hold,
+// fewer (two at least) where there is no room.  Allocated after everything else
+// that a context cannot do without.
+inline cudaError_t alloc_coef_tables(size_t table_bytes, float** coef, int32_t* steps) {
+  const size_t most = ((size_t)256 << 20) / (table_bytes > 0 ? table_bytes : 1);
+  for (*steps = (int32_t)(most < 2 ? 2 : most > 16 ? 16 : most);; *steps = *steps > 4 ? *steps / 2 : 2) {
+    const cudaError_t e = cudaMalloc((void**)coef, *steps * table_bytes);
+    if (e == cudaSuccess) return e;
+    *coef = nullptr;
+    if (e != cudaErrorMemoryAllocation || *steps <= 2) return e;
+    cudaGetLastError();
+  }
 }
 
 // Sets the reason pic_last_error(NULL) reports.

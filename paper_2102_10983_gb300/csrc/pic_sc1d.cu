@@ -544,11 +544,11 @@ struct pic_sc1d {
   unsigned long long* acc = nullptr;  // [2 parities][F, D][M], then C, C_ion [M] each, gauss [2]
   double* wtab = nullptr;
   double2* nodes = nullptr;  // [M][3] fields at t_n
-  uint8_t* k_sub = nullptr;  // the electrons of a step that sub-cycle (push_deposit_kernel)
-  int32_t* queue = nullptr;
+  int32_t* queue = nullptr;  // the electrons of a step that sub-cycle (push_deposit_kernel)
+  uint8_t* k_sub = nullptr;  // in queue's allocation
+  int64_t slice = 0;
   int32_t* bin = nullptr;
   DevStats* dstats = nullptr;
-  double* staging = nullptr;  // 3 M host-upload staging
   int64_t launches = 0;
   double gauss_res = 0.0, rho_max = 0.0;
   int32_t checks = 0;
@@ -573,8 +573,9 @@ static int sc_fail(pic_sc1d* c, int code, const char* msg, const char* detail = 
     if (e_ != cudaSuccess) return sc_fail((c), PIC_ECUDA, #call ": ", cudaGetErrorString(e_)); \
   } while (0)
 
-// The queue's entries and counts are 32-bit numbers: electrons beyond kSlice are
-// pushed in further rounds of the passes.
+// The queue's entries and counts are 32-bit numbers: electrons beyond this (or
+// than there is room for, alloc_bin_f64) are pushed in further rounds of the
+// passes.
 constexpr int64_t kSlice = (int64_t)1 << 30;
 
 static double* slot_field(pic_sc1d* c, int slot, int f) {
@@ -627,17 +628,14 @@ extern "C" int pic_sc1d_create(const pic_sc1d_params* prm, int64_t capacity, voi
   const int64_t wcount = wrows_total(prm->k_max) * 2 * (prm->order + 1);
   ok &= cudaMalloc(&c->wtab, wcount * 8) == cudaSuccess;
   ok &= cudaMalloc(&c->dstats, sizeof(DevStats)) == cudaSuccess;
-  ok &= cudaMalloc(&c->staging, 3 * c->M * 8) == cudaSuccess;
+  ok &= cudaMalloc(&c->bin, kBinF64 * 4) == cudaSuccess;
+  ok = ok && alloc_bin_f64(cap, kSlice, &c->queue, &c->k_sub, &c->slice) == cudaSuccess;
   // without node fields (a grid that no ensemble of this capacity pays for, no
   // room) the push gathers the levels
-  if (node_fields_pay(cap, c->M) && cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) != cudaSuccess) {
+  if (ok && node_fields_pay(cap, c->M) && cudaMalloc(&c->nodes, 3 * c->M * sizeof(double2)) != cudaSuccess) {
     c->nodes = nullptr;
     cudaGetLastError();
   }
-  const int64_t slice = cap < kSlice ? cap : kSlice;
-  ok &= cudaMalloc(&c->k_sub, slice) == cudaSuccess;
-  ok &= cudaMalloc(&c->queue, slice * 4) == cudaSuccess;
-  ok &= cudaMalloc(&c->bin, kBinF64 * 4) == cudaSuccess;
   if (!ok) {
     pic_sc1d_destroy(c);
     return sc_fail(nullptr, PIC_ENOMEM, "pic_sc1d_create: device allocation failed");
@@ -660,8 +658,8 @@ extern "C" int pic_sc1d_destroy(pic_sc1d* c) {
   if (!c) return PIC_OK;
   cudaFree(c->x); cudaFree(c->px); cudaFree(c->py); cudaFree(c->pz); cudaFree(c->w_stage);
   cudaFree(c->status); cudaFree(c->Q); cudaFree(c->ring); cudaFree(c->acc); cudaFree(c->wtab);
-  cudaFree(c->dstats); cudaFree(c->staging);
-  cudaFree(c->nodes); cudaFree(c->k_sub); cudaFree(c->queue); cudaFree(c->bin);
+  cudaFree(c->dstats);
+  cudaFree(c->nodes); cudaFree(c->queue); cudaFree(c->bin);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   delete c;
@@ -768,7 +766,7 @@ static void launch_push(pic_sc1d* c, const Sc1dArgs& all, int64_t off = 0) {
   const cudaStream_t s = c->stream;
   Sc1dArgs a = all;
   a.x += off; a.px += off; a.py += off; a.pz += off; a.status += off; a.Q += off;
-  a.n = all.n - off < kSlice ? all.n - off : kSlice;
+  a.n = all.n - off < c->slice ? all.n - off : c->slice;
   const bool unit = a.qm_abs == 1.0;
   if (all.n <= (int64_t)a.sms * kEachSc1d) {
     a.nodes = nullptr;

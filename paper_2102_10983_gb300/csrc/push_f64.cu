@@ -414,22 +414,27 @@ static void launch_f64_p(PushArgsF64 a, int sms, cudaStream_t s, int* launches) 
     if (launches) ++*launches;
     return;
   }
-  int n = 3;
-  if (a.nodes) {
-    const int64_t want = (a.mask + 128) / 128;
-    nodes_f64_kernel<P><<<(int)(want < sms * 8 ? want : sms * 8), 128, 0, s>>>(a);
-    ++n;
-  } else {
-    cudaMemsetAsync(a.bin, 0, kBinF64 * sizeof(int32_t), s);
+  const int64_t all = a.n;
+  for (int64_t off = 0; off < all; off += a.slice) {
+    a.n = all - off < a.slice ? all - off : a.slice;
+    if (off == 0 && a.nodes) {
+      const int64_t want = (a.mask + 128) / 128;
+      nodes_f64_kernel<P><<<(int)(want < sms * 8 ? want : sms * 8), 128, 0, s>>>(a);
+      if (launches) ++*launches;
+    } else {
+      cudaMemsetAsync(a.bin, 0, kBinF64 * sizeof(int32_t), s);
+    }
+    // small ensembles in small blocks: every SM's FP64 unit takes part
+    const int threads = a.n >= (int64_t)sms * 256 ? 256 : a.n >= (int64_t)sms * 64 ? 64 : 32;
+    const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)sms * 8;
+    criterion_push_f64_kernel<P, UNIT><<<(int)(want < cap ? want : cap), threads, 0, s>>>(a);
+    launch_bin_f64(BinF64{a.n, a.k_sub, a.queue, a.bin}, sms, s);
+    const int64_t most = (int64_t)sms * 12;
+    subcycle_f64_kernel<P, UNIT><<<(int)(a.n < most ? a.n : most), 32, 0, s>>>(a);
+    if (launches) *launches += 3;
+    a.x += a.n; a.px += a.n; a.py += a.n; a.pz += a.n; a.status += a.n;
+    if (a.work) a.work += a.n;
   }
-  // small ensembles in small blocks: every SM's FP64 unit takes part
-  const int threads = a.n >= (int64_t)sms * 256 ? 256 : a.n >= (int64_t)sms * 64 ? 64 : 32;
-  const int64_t want = (a.n + threads - 1) / threads, cap = (int64_t)sms * 8;
-  criterion_push_f64_kernel<P, UNIT><<<(int)(want < cap ? want : cap), threads, 0, s>>>(a);
-  launch_bin_f64(BinF64{a.n, a.k_sub, a.queue, a.bin}, sms, s);
-  const int64_t most = (int64_t)sms * 12;
-  subcycle_f64_kernel<P, UNIT><<<(int)(a.n < most ? a.n : most), 32, 0, s>>>(a);
-  if (launches) *launches += n;
 }
 
 cudaError_t launch_push_f64(const PushArgsF64& a, int order, cudaStream_t s, int* launches) {
