@@ -63,7 +63,8 @@ __device__ __forceinline__ float fp64i_top(uint64_t u, uint32_t field) {
   return __int_as_float((int32_t)(((uint32_t)(u >> 29) & 0x7fffffu) | (field << 23)));
 }
 
-// 2^SH a / (B 2^(eb - 1075)), B in [2^52, 2^53], eb in 1 .. 2046, given y =
+// 2^SH a / (B 2^(eb - 1075)) (SH = 0, 1: a power of two does not change the
+// rounding), B in [2^52, 2^53], eb in 1 .. 2046, given y =
 // (2^52 / B)(1 + e), |e| <= 2^-21.9; neg: the divisor's sign bit in place.
 //
 // Digits q1 (2^-21), q2 (2^-41), q3 (2^-54) of the significands' quotient A / B
@@ -99,20 +100,15 @@ __device__ __forceinline__ bool fp64i_quot(uint64_t ua, uint64_t B, int eb, floa
   return zero || ((unsigned)(ea - 1) < 2046u && (unsigned)de < 2044u);
 }
 
-// 2^SH a / b (SH = 0, 1: a power of two does not change the rounding).
-template <int SH>
-__device__ __forceinline__ double fp64i_div(double a, double b) {
+__device__ __forceinline__ double div_rn(double a, double b) {
   const uint64_t ub = (uint64_t)__double_as_longlong(b);
   const uint32_t hb = (uint32_t)(ub >> 32);
   const int eb = (int)((hb >> 20) & 0x7ffu);
   double q;
-  const bool ok = fp64i_quot<SH>((uint64_t)__double_as_longlong(a), fp64i_sig(ub), eb,
-                                 fp64i_rcp(fp64i_top(ub, 127)), hb, q);
-  if (ok && (unsigned)(eb - 1) < 2046u) return q;
-  return fp64i_div_any(SH ? 2.0 * a : a, b);
+  const bool ok = fp64i_quot<0>((uint64_t)__double_as_longlong(a), fp64i_sig(ub), eb,
+                                fp64i_rcp(fp64i_top(ub, 127)), hb, q);
+  return ok && (unsigned)(eb - 1) < 2046u ? q : fp64i_div_any(a, b);
 }
-__device__ __forceinline__ double div_rn(double a, double b) { return fp64i_div<0>(a, b); }
-__device__ __forceinline__ double div2_rn(double a, double b) { return fp64i_div<1>(a, b); }
 
 // The rounded significand (53 bits, or 2^53) of sqrt(a), its exponent field
 // (for a significand below 2^53) and y = 1 / (significand / 2^52) to 2^-22;
@@ -156,7 +152,9 @@ __device__ __forceinline__ double sqrt_rn(double a) {
 
 // The same without branches, for a caller that strings several together and
 // looks at the result's validity once (false: an operand or a result outside
-// the domain, the values are to be ignored): 2 a / b; and g = sqrt(a) with
+// the domain, the values are to be ignored): 2 a / b rounded once (also where 2 a
+// would overflow: the push's b = 1 + a^2 is then infinite, outside the domain);
+// and g = sqrt(a) with
 // t / g (TWO: and u / g), which start from the root's own reciprocal.
 __device__ __forceinline__ bool div2_try(double a, double b, double& q) {
   const uint64_t ub = (uint64_t)__double_as_longlong(b);

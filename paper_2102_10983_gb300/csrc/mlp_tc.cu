@@ -383,7 +383,6 @@ __device__ __forceinline__ void tc_end(TcSmem& s, DevStats* stats) {
 // pic_predict: features of every particle after step a (a.featE / a.featB: its
 // feature nodes; the same code as the features kernel) and the network's
 // class, in one pass.
-template <int P>
 __global__ void __launch_bounds__(kTcThreads, 1) predict_tc_kernel(PushArgsMixed a, const float* Pm, uint8_t* pred,
                                                                 int fieldless_zero) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -481,17 +480,11 @@ cudaError_t launch_predict_fused(const PushArgsMixed& a, int order, const float*
                                  int sm_count, cudaStream_t st, bool fieldless_zero) {
   const int fz = fieldless_zero ? 1 : 0;
   if (a.n <= 0) return cudaSuccess;
+  if (order < 1 || order > kMaxOrder) return cudaErrorInvalidValue;
   const int blocks = tc_grid(a.n, sm_count);
-  cudaError_t e = cudaSuccess;
-  switch (order) {
-    case 1: e = tc_configure(predict_tc_kernel<1>); if (e == cudaSuccess) predict_tc_kernel<1><<<blocks, kTcThreads, kTcSmemBytes, st>>>(a, P, pred, fz); break;
-    case 2: e = tc_configure(predict_tc_kernel<2>); if (e == cudaSuccess) predict_tc_kernel<2><<<blocks, kTcThreads, kTcSmemBytes, st>>>(a, P, pred, fz); break;
-    case 3: e = tc_configure(predict_tc_kernel<3>); if (e == cudaSuccess) predict_tc_kernel<3><<<blocks, kTcThreads, kTcSmemBytes, st>>>(a, P, pred, fz); break;
-    case 4: e = tc_configure(predict_tc_kernel<4>); if (e == cudaSuccess) predict_tc_kernel<4><<<blocks, kTcThreads, kTcSmemBytes, st>>>(a, P, pred, fz); break;
-    case 5: e = tc_configure(predict_tc_kernel<5>); if (e == cudaSuccess) predict_tc_kernel<5><<<blocks, kTcThreads, kTcSmemBytes, st>>>(a, P, pred, fz); break;
-    default: return cudaErrorInvalidValue;
-  }
+  cudaError_t e = tc_configure(predict_tc_kernel);
   if (e != cudaSuccess) return e;
+  predict_tc_kernel<<<blocks, kTcThreads, kTcSmemBytes, st>>>(a, P, pred, fz);
   return cudaGetLastError();
 }
 
