@@ -46,13 +46,6 @@ __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], 
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// d += a b: the product's sum from zero, then an FP32 addition.
-__device__ __forceinline__ void add_product(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  float s[4] = {0.f, 0.f, 0.f, 0.f};
-  mma16816(s, a, b0, b1);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) d[q] = __fadd_rn(d[q], s[q]);
-}
 
 // Weights as the kernels read them from shared memory (BF16):
 //   W1p [64][16] (cols 6..15 zero), W2 [64][64], W2T [64][64], W3 [8][64] (rows at the
@@ -212,10 +205,11 @@ __device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], const __nv_bfloat16* p)
 // forms rows 16 w .. 16 w + 15 of each, its operands by transposing matrix
 // loads from the staged tiles, and keeps its sums in registers over all of the
 // block's samples.  The tensor cores truncate where they add into an
-// accumulator, a bias that grows with the number of additions: so they sum 16
-// samples from zero, and those sums are added in FP32, to nearest (a batch of
-// 1,048,576, against 64-bit sums of the same operands: relative error 2.0e-5 if
-// the accumulators run on, 7e-8 so; 2e-7 on the FP32 pipes).
+// accumulator, a bias that grows with the number of additions: so they sum the
+// 64 samples of a pass from zero, and the passes' sums are added in FP32, to
+// nearest (a batch of 1,048,576, against 64-bit sums of the same operands:
+// relative error 2.0e-5 if the accumulators run on, 5e-8 so, 1.8e-7 on the FP32
+// pipes).
 // (On the FP32 pipes -- 16 products per element and shared atomics between the
 // warps, then an atomic per block and parameter -- a batch of 8,192 took 30 us;
 // this kernel 7.3 us and mlp_finish_kernel 3.2 us.)
@@ -229,16 +223,27 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const float* 
   __syncthreads();
   const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, warp = threadIdx.x >> 5;
   const int r0w = 16 * warp;  // this warp's rows of the stage, and of every gradient
-  float gW2[8][4], gW1[4], gW3[4], gB2[4], gB3[4];  // gW1's and gB2's column 6: the bias gradients
+  // the gradients of a pass, and of the passes before it: W2 in 0 .. 7, then W1,
+  // W3, b2 and b3 (W1's and b2's column 6: the bias gradients)
+  float g4[12][4], sum[12][4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    gW1[q] = gW3[q] = gB2[q] = gB3[q] = 0.f;
+  for (int r = 0; r < 12; ++r)
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) gW2[nt][q] = 0.f;
-  }
+    for (int q = 0; q < 4; ++q) g4[r][q] = sum[r][q] = 0.f;
+  float (&gW1)[4] = g4[8], (&gW3)[4] = g4[9], (&gB2)[4] = g4[10], (&gB3)[4] = g4[11];
+  auto add_pass = [&]() {
+#pragma unroll
+    for (int r = 0; r < 12; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        sum[r][q] = __fadd_rn(sum[r][q], g4[r][q]);
+        g4[r][q] = 0.f;
+      }
+  };
   float my_loss = 0.f;
   const int64_t blocks = (n + kGradRows - 1) / kGradRows;
   for (int64_t blk = blockIdx.x; blk < blocks; blk += gridDim.x) {
+    if (blk != blockIdx.x) add_pass();
     const int64_t base = blk * kGradRows + r0w;
     uint32_t a1[4];
     phi_fragment(phi, n, base, a1);
@@ -323,30 +328,37 @@ __global__ void __launch_bounds__(32 * kGradWarps) mlp_grad_kernel(const float* 
       ldsm2t(D, &S.dz[k0 + 8 * m1b + mr][0]);
       ldsm2t(Xf, &S.X[k0 + 8 * m1b + mr][0]);
       a_of(S.da2);
-      add_product(gB2, A, Xf[0], Xf[1]);
+      mma16816(gB2, A, Xf[0], Xf[1]);
 #pragma unroll
       for (int nt = 0; nt < 8; nt += 2) {
         ldsm4t(B, &S.h1[k0 + 8 * m1b + mr][8 * (nt + m2b)]);
-        add_product(gW2[nt], A, B[0], B[1]);
-        add_product(gW2[nt + 1], A, B[2], B[3]);
+        mma16816(g4[nt], A, B[0], B[1]);
+        mma16816(g4[nt + 1], A, B[2], B[3]);
       }
       a_of(S.da1);
-      add_product(gW1, A, Xf[0], Xf[1]);
+      mma16816(gW1, A, Xf[0], Xf[1]);
       a_of(S.h2);
-      add_product(gW3, A, D[0], D[1]);  // transposed: rows = inputs, columns = classes
+      mma16816(gW3, A, D[0], D[1]);  // transposed: rows = inputs, columns = classes
       if (warp == 0) {
         const uint32_t one = pack2(1.f, 1.f), ones[4] = {one, one, one, one};
-        add_product(gB3, ones, D[0], D[1]);
+        mma16816(gB3, ones, D[0], D[1]);
       }
     }
+  }
+  if (blocks > gridDim.x) {  // several passes
+    add_pass();
+#pragma unroll
+    for (int r = 0; r < 12; ++r)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) g4[r][q] = sum[r][q];
   }
   float* out = part + (int64_t)blockIdx.x * kPartial;
   const int oa = r0w + g, ob = oa + 8;
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt) {
     const int c = 8 * nt + 2 * t;
-    *reinterpret_cast<float2*>(out + kOffW2 + oa * kH + c) = make_float2(gW2[nt][0], gW2[nt][1]);
-    *reinterpret_cast<float2*>(out + kOffW2 + ob * kH + c) = make_float2(gW2[nt][2], gW2[nt][3]);
+    *reinterpret_cast<float2*>(out + kOffW2 + oa * kH + c) = make_float2(g4[nt][0], g4[nt][1]);
+    *reinterpret_cast<float2*>(out + kOffW2 + ob * kH + c) = make_float2(g4[nt][2], g4[nt][3]);
   }
   if (t < 3) {
     *reinterpret_cast<float2*>(out + oa * kIn + 2 * t) = make_float2(gW1[0], gW1[1]);
