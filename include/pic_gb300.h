@@ -282,7 +282,10 @@ int pic_mlp_train_step(pic_mlp* mlp, const float* phi, const uint8_t* label, int
                        float lr, float* loss_out);
 
 /* Predicted class (argmax of the logits; ties go to the smaller k) of n
- * samples: pred is device n uint8.  Asynchronous. */
+ * samples: pred is device n uint8.  Asynchronous.  The network (here, in
+ * pic_predict and in the predicted schedule's refresh) takes the whole tensor
+ * memory of the SMs it runs on: beside a kernel of another stream that holds
+ * tensor memory it starts on an SM when that kernel has left it. */
 int pic_mlp_infer(pic_mlp* mlp, const float* phi, int64_t n, uint8_t* pred);
 
 /* pic_features of every loaded particle after macro step n followed by
@@ -313,8 +316,9 @@ int pic_batch_create(const pic_ensemble* ens, int32_t n_ens, int32_t order,
                      int64_t window_cells, int32_t ring_levels, void* stream, pic_batch** out);
 int pic_batch_destroy(pic_batch* b);
 
-/* Stream chunk length (a multiple of 32 in [32, 8192]), resident blocks per SM
- * (1 .. the kernel's occupancy) and whether multi-step pic_batch_push_step
+/* Stream chunk length (a multiple of 32 in [32, 8192]; rounded up to whole tiles
+ * of 128 particles, so 32, 64, 96 and 128 are one setting), resident blocks per
+ * SM (1 .. the kernel's occupancy) and whether multi-step pic_batch_push_step
  * calls are captured into one CUDA graph and launched as such (needs a
  * non-NULL stream). */
 int pic_batch_config(pic_batch* b, int32_t chunk, int32_t blocks_per_sm, int32_t use_graph);

@@ -237,8 +237,8 @@ __device__ __forceinline__ void subcycle_f64(const PushArgsF64& a, int64_t i, bo
 // Measured per step (order 3): 1,048,576 electrons of the a0 = 150 ensemble 6.2
 // ms as one thread per particle, 1.9 ms so (pass 1 0.09 ms = 25 FP64 slots per
 // warp, pass 2 6 us, the rest the longest chain: 1,024 sub-steps of 1.7 us,
-// 2.6 us before); 256 electrons at the a0 = 100 front 2.98 -> 1.2 ms, the chain
-// likewise.
+// 2.6 us before); 2,432 electrons at the a0 = 100 front 4.24 -> 1.54 ms, the chain
+// likewise.  Small ensembles go without the passes (each_f64_kernel).
 
 // Electron i's criterion and, with k = 0, its m = 1 push: its k, or -1 if it is
 // lost (or is now).

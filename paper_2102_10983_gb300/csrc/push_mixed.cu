@@ -177,9 +177,9 @@ __global__ void __launch_bounds__(256, plain_blocks(P)) push_mixed_plain_kernel(
       boris_f32(node_lerp_e(a.nodes, je & a.mask, we), b0, hp, __fmul_rn(a.dt, a.inv_dx), a.qm, s);
     } else {
       // Order 3 reads its nodes' coefficients from the step's table in aligned
-      // 16-byte loads: 16.8M electrons 1.369 -> 1.334 ms per step.  Rows of the
-      // other orders are not aligned: they form them from the levels (100,003
-      // electrons at order 5: 0.092 ms, 0.096 by the table).
+      // 16-byte loads: 16.8M electrons over steps 2405 to 4404 0.965 ms per step,
+      // 1.026 from the levels.  Rows of the other orders are not aligned: they form
+      // them from the levels (100,003 electrons at order 5: 89 us, 95 by the table).
       ok = subcycle_f32<P, RING, P == 3, 1>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.mono, k,
                                          st & 0x7f, b0, s);
     }
