@@ -408,9 +408,10 @@ __global__ void __launch_bounds__(32) subcycle_deposit_kernel(Sc1dArgs a) {
 }
 
 // A small ensemble's step in one launch, a warp per electron (each_f64_kernel of
-// push_f64.cu).  100 electrons on 20,000 cells, m = 1: 32 us per step by the
-// passes, 18 so (28 once, as one thread per electron).
-constexpr int kEachSc1d = 8;  // electrons per SM
+// push_f64.cu).  us per step by the passes and so: 100 electrons on 20,000 cells,
+// m = 1, 32 and 18 (28 once, as one thread per electron); every electron k = 5, 456
+// 2,569 and 2,434, 608 2,566 and 2,613, 1,216 2,780 and 4,013.
+constexpr int kEachSc1d = 3;  // electrons per SM
 template <int P, bool UNIT>
 __global__ void __launch_bounds__(32) each_deposit_kernel(Sc1dArgs a) {
   __shared__ unsigned long long sh[12];

@@ -308,12 +308,13 @@ __global__ void __launch_bounds__(256) criterion_push_f64_kernel(PushArgsF64 a) 
 
 // The whole step of a small ensemble in one launch, a warp (and a block) per
 // electron: its criterion and m = 1 push by one lane, a sub-cycle by all.  The
-// four launches of the three passes are most of such a step, and a few warps per
-// SM leave the FP64 unit idle between their chains' operations.  Steps of m = 1
-// pushes: 1 electron 17 us by the passes and 8.4 so (11.5 once, as one thread per
-// electron), 608 17 and 8.5, 1,216 17.5 and 12.3, 2,432 17.5 and 16.7; with
-// sub-cycles, 256 electrons 1,071 and 1,024, 1,216 1,461 and 1,413.
-constexpr int kEachF64 = 8;  // electrons per SM
+// four launches of the three passes are most of such a step, and four warps per
+// SM leave the FP64 unit idle between their chains' operations (more do not: the
+// passes put several electrons into a warp).  us per step by the passes and so:
+// m = 1, 1 electron 17 and 8.4 (12.5 once, as one thread per electron), 608 17 and
+// 8.5; every electron k = 5, 152 1,613 and 1,555, 608 1,743 and 1,685, 1,216 1,907
+// and 2,603.
+constexpr int kEachF64 = 4;  // electrons per SM
 template <int P, bool UNIT>
 __global__ void __launch_bounds__(32) each_f64_kernel(PushArgsF64 a) {
   __shared__ unsigned long long sh[12];

@@ -90,8 +90,8 @@ def test_a_large_window_does_not_slow_a_small_ensemble():
     assert ms[22] < 3.0 * ms[12], ms
 
 
-# one warp per electron up to eight per SM, in one launch; the three passes beyond
-@pytest.mark.parametrize("n", [1, 2, 33, 8 * 152, 8 * 152 + 1])
+# one warp per electron up to four per SM, in one launch; the three passes beyond
+@pytest.mark.parametrize("n", [1, 2, 33, 4 * 152, 4 * 152 + 1])
 @pytest.mark.parametrize("order,work", [(1, False), (3, True), (5, False)])
 def test_small_ensembles(n, order, work):
     _both(n, 64, order, k_max=5 if n < 100 else 3, work=work, qm=-1.0 if order < 5 else -0.37)

@@ -1,5 +1,5 @@
 """The coupled loop by its routes, against the oracle bit for bit: small ensembles
-in one launch (a warp per electron, up to eight per SM), electrons fewer than
+in one launch (a warp per electron, up to three per SM), electrons fewer than
 the grid's entries (levels gathered), as many (node fields); and what a large
 grid costs a small ensemble."""
 from __future__ import annotations
@@ -20,7 +20,7 @@ from test_gpu_sc1d_paths import test_sc1d_unsorted_electrons_and_odd_charges as 
 
 
 @pytest.mark.parametrize("n,cells,qm,order", [
-    (2, 16, -1.0, 2), (700, 300, -0.4, 4), (8 * 152, 900, -1.0, 3), (8 * 152 + 1, 900, -1.0, 3),
+    (2, 16, -1.0, 2), (700, 300, -0.4, 4), (3 * 152, 300, -1.0, 3), (3 * 152 + 1, 600, -1.0, 3),
     (1500, 4000, -1.0, 1), (1500, 4000, 0.3, 2), (1500, 4000, 1.0, 4), (1500, 4000, -1.0, 5),
     (3004, 3000, -1.0, 3), (3005, 3000, -1.0, 3)])
 def test_routes(n, cells, qm, order):
