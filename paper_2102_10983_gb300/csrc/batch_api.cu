@@ -362,6 +362,9 @@ static int queue_steps(pic_batch* b, int64_t n, int64_t n_steps) {
   base.wtab = b->wtab32;
   base.crit_row = wrows_total(kMaxK) - 1;
   lagrange_monomials(p, base.mono);
+  double cells = 0.0;
+  for (const pic_ensemble& q : b->ens_h) cells = q.dt / q.dx > cells ? q.dt / q.dx : cells;
+  base.near = stretches(cells, kNearMin);
   base.stats = b->dstats;
   base.prefix = b->prefix;
   base.nodes = b->nodes;

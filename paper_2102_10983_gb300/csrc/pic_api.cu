@@ -598,6 +598,7 @@ static void mixed_base(pic_ctx* c, PushArgsMixed& base) {
   base.inv_dx = (float)(1.0 / c->prm.dx);
   base.k_max = c->prm.k_max;
   base.field_time = c->prm.field_time;
+  base.near = stretches(c->prm.dt / c->prm.dx, c->prm.schedule == PIC_SCHED_PLAIN ? 1 : kNearMin);
   lagrange_monomials(c->prm.order, base.mono);
   base.wtab = c->wtab32;
   base.crit_row = wrows_total(c->prm.k_max) - 1;

@@ -120,6 +120,28 @@ struct PushArgsF64 {
   int sms;            // set by the launcher
 };
 
+// From which k on, and in stretches of 4^k >> half sub-steps, the mixed form's
+// sub-cycles run without a branch (subcycle_f32).
+struct Stretches {
+  int k_min, half;
+};
+constexpr int kNearMin = 2, kHalfMin = 3, kStretchMin = 8;
+// cells: c dt / dx; k_min: the smallest k where that is at most one (kNearMin; 1
+// for the plain schedule, whose warps of mixed k would run both loops one after the
+// other).  With more cells per macro step a stretch of half a cell is a smaller part
+// of it; k whose stretch would be shorter than kStretchMin, and k < kHalfMin, whose
+// one stretch an electron could leave, look at the nodes in each sub-step.  262,144
+// gyrating electrons at c dt = 4 dx, us per step, before these loops, in halves of a
+// macro step (which nearly all electrons left, to be taken again), and so: plain
+// schedule, k = 4 251, 335, 169; binned, k = 4 292, 380, 191; batch, k = 2 92, 120, 95.
+inline Stretches stretches(double cells, int k_min) {
+  Stretches r{k_min, 1};
+  while (cells > (double)(1 << (r.half - 1)) && r.half < 16) ++r.half;
+  if (r.half > 1)
+    for (r.k_min = kHalfMin; r.k_min <= kMaxK && ((1 << (2 * r.k_min)) >> r.half) < kStretchMin;) ++r.k_min;
+  return r;
+}
+
 // Arguments of the mixed-precision push.  Position = (cell + frac) * dx with
 // an exact int32 cell and an FP32 offset.
 struct PushArgsMixed {
@@ -169,6 +191,7 @@ struct PushArgsMixed {
   float inv_dx;
   int k_max;
   int field_time;  // 0: theta_j = 1/2 + (j-1)/m; 1: theta_j = (j - 1/2)/m
+  Stretches near;
   // monomial coefficients, in u = theta - 1, of the Lagrange basis polynomials:
   // L^E_{p,l}(theta) = sum_q mono[0][l][q] u^q, L^B likewise with mono[1]
   float mono[2][kMaxOrder + 1][kMaxOrder + 1];
@@ -259,6 +282,7 @@ struct BatchArgs {
   int64_t R, lstride;  // ring slots, W
   int32_t mask;
   int64_t start_cur, start_prev;
+  Stretches near;  // for the ensemble with the most cells per macro step
   const float* wtab;
   int64_t crit_row;
   float mono[2][kMaxOrder + 1][kMaxOrder + 1];

@@ -92,7 +92,7 @@ __device__ __forceinline__ void batch_stash_drain(const BatchArgs& a, const Batc
     const float2 vb = S.s.b[q];
     const int32_t i = __float_as_int(vb.y);
     MixedState s = {__float_as_int(va.x), va.y, va.z, va.w, vb.x};
-    const bool ok = subcycle_f32<P, true, true>(F, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.mono,
+    const bool ok = subcycle_f32<P, true, true>(F, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.near, a.mono,
                                                 k, S.s.kp[q], 0.f, s);
     normalize(s);
     store_state(a, i, s);
@@ -184,10 +184,10 @@ __device__ __forceinline__ void batch_heavy(const BatchArgs& a, int ens, int64_t
     StepFields<P, true> Fs = si == a.step_cur ? Fc : Fp;
     if (si < a.step_cur - 1) Fs = ens_step_fields<P>(a, e, si);
     if (Fs.coef)
-      ok = subcycle_f32<P, true, true>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.mono,
+      ok = subcycle_f32<P, true, true>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.near, a.mono,
                                        k, k_prev, b0, s, j0, j1);
     else  // further behind than the tables kept
-      ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time,
+      ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.near,
                                         a.mono, k, k_prev, b0, s, j0, j1);
     if (k >= kDeferMin) budget -= j1 - j0;
     if (!ok) {

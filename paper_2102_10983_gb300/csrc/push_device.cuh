@@ -619,21 +619,19 @@ __device__ __forceinline__ bool cycle_near(const StepFields<P, RING>& F, int32_t
 // each, and the nodes' values formed after it, made that 200.  So k >= kNearMin
 // runs without a branch (cycle_near), the next sub-step's values formed in the
 // shadow of this one's push: 153.  k >= kHalfMin goes in stretches of at most
-// half a macro step, half a cell, from the middle of the kept nodes, which an
-// electron cannot leave either way; k = 2 in one stretch, the nodes ahead of
-// the electron kept (its 16 sub-steps would not pay for a second load).  What
-// does not fit (a turn back, c dt > dx, the window's ends) takes cycle_any, as
-// does k = 1, whose four sub-steps gain nothing.  Per step, two nodes ->
+// half a cell (half a macro step where c dt <= dx), from the middle of the kept
+// nodes, which an electron cannot leave either way; k = 2 in one stretch, the
+// nodes ahead of the electron kept (its 16 sub-steps would not pay for a second
+// load).  What does not fit (a turn back, the window's ends) takes cycle_any, as
+// does k = 1, whose four sub-steps gain nothing.  near: the rule for the grid
+// (stretches), a launch argument: a register for it costs the kernels 1 to 5 %.  Per step, two nodes ->
 // three -> with stretches: 300 electrons at the front 119 -> 117 -> 95 us,
 // 16.8M electrons 249 -> 219 -> 199 us, 1,000,003 at fifth order 120 -> 118 ->
 // 90 us.
-// A warp of mixed k (the plain schedule) would run both loops one after the
-// other: it takes NEAR = 1, all of them cycle_near.
-constexpr int kNearMin = 2, kHalfMin = 3;
-template <int P, bool RING, bool TABLE = false, int NEAR = kNearMin>
+template <int P, bool RING, bool TABLE = false>
 __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const float* wtab,
                                              int32_t mask, float dt, float inv_dx, float qm,
-                                             int field_time,
+                                             int field_time, const Stretches& near,
                                              const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1],
                                              int k, int k_prev, float b0, MixedState& s,
                                              int j0 = 0, int j1 = -1) {
@@ -656,10 +654,10 @@ __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const
   for (int j = j0; j < j_end && ok;) {
     int n = j_end - j;
     bool done = false;
-    if (k >= NEAR) {
+    if (k >= near.k_min) {
       float back = c.s.ux < 0.f ? 1.0f : 0.0f;
       if (k >= kHalfMin) {
-        n = min(n, m >> 1);
+        n = min(n, m >> near.half);
         back = 0.5f;
       }
       const CycleState before = c;
@@ -684,31 +682,31 @@ struct SubOut {
 template <int P>
 __device__ __noinline__ SubOut subcycle_table_call(StepFields<P, true> F, const float* wtab,
                                                    int32_t mask, float dt, float inv_dx, float qm,
-                                                   int field_time, int k, int k_prev, float b0,
+                                                   int field_time, Stretches near, int k, int k_prev, float b0,
                                                    MixedState s, int j0, int j1) {
   float no_mono[2][kMaxOrder + 1][kMaxOrder + 1];  // the table form never reads it
   SubOut o;
   o.s = s;
-  o.ok = subcycle_f32<P, true, true>(F, wtab, mask, dt, inv_dx, qm, field_time, no_mono, k, k_prev,
+  o.ok = subcycle_f32<P, true, true>(F, wtab, mask, dt, inv_dx, qm, field_time, near, no_mono, k, k_prev,
                                      b0, o.s, j0, j1);
   return o;
 }
 template <int P, bool RING, bool TABLE>
 __device__ __forceinline__ bool subcycle_site(const StepFields<P, RING>& F, const float* wtab,
                                               int32_t mask, float dt, float inv_dx, float qm,
-                                              int field_time,
+                                              int field_time, const Stretches& near,
                                               const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1],
                                               int k, int k_prev, float b0, MixedState& s,
                                               int j0 = 0, int j1 = -1) {
 #ifdef PIC_SUBCYCLE_NOINLINE
   if constexpr (RING && TABLE) {
-    const SubOut o = subcycle_table_call<P>(F, wtab, mask, dt, inv_dx, qm, field_time, k, k_prev, b0,
+    const SubOut o = subcycle_table_call<P>(F, wtab, mask, dt, inv_dx, qm, field_time, near, k, k_prev, b0,
                                             s, j0, j1);
     s = o.s;
     return o.ok;
   }
 #endif
-  return subcycle_f32<P, RING, TABLE>(F, wtab, mask, dt, inv_dx, qm, field_time, mono, k, k_prev,
+  return subcycle_f32<P, RING, TABLE>(F, wtab, mask, dt, inv_dx, qm, field_time, near, mono, k, k_prev,
                                       b0, s, j0, j1);
 }
 
@@ -1110,7 +1108,7 @@ __device__ __forceinline__ void stash_drain(const PushArgsMixed& a, const StepFi
     const int32_t i = __float_as_int(vb.y);
     MixedState s = {__float_as_int(va.x), va.y, va.z, va.w, vb.x};
     const bool ok = subcycle_site<P, RING, RING>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm,
-                                                 a.field_time, a.mono, k, kp & 7, 0.f, s);
+                                                 a.field_time, a.near, a.mono, k, kp & 7, 0.f, s);
     normalize(s);
     store_state(a, i, s);
     a.status[i] = ok ? (uint8_t)(k | (kp & 8 ? kOwned : 0) | (a.parity_next ? kParity : 0))
@@ -1168,11 +1166,11 @@ __device__ __forceinline__ void heavy_particle(const PushArgsMixed& a, const Ste
       if (si < a.step_cur - 1) Fs = ring_step_fields<P>(a, si);
     }
     if (!RING || Fs.coef) {
-      ok = subcycle_site<P, RING, RING>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time,
+      ok = subcycle_site<P, RING, RING>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.near,
                                         a.mono, k, k_prev, b0, s, j0, j1);
     } else {  // further behind than the tables kept
       if constexpr (RING)
-        ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time,
+        ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.near,
                                           a.mono, k, k_prev, b0, s, j0, j1);
     }
     if (k >= kDeferMin) budget -= j1 - j0;
@@ -1291,7 +1289,7 @@ __device__ __forceinline__ void predicted_particle(const PushArgsMixed& a, const
   count_step(tc, sh, k, capped);
   if (k == 0 || (k == k_pred && k < kDeferMin)) {
     const bool ok = subcycle_site<P, RING, RING>(Fc, a.wtab, a.mask, a.dt, a.inv_dx, a.qm,
-                                                 a.field_time, a.mono, k, k_prev, b0, s);
+                                                 a.field_time, a.near, a.mono, k, k_prev, b0, s);
     normalize(s);
     store_state(a, i, s);
     a.status[i] = ok ? (uint8_t)(k | kOwned | (a.parity_next ? kParity : 0))

@@ -129,14 +129,13 @@ cudaError_t launch_halfstep(const PushArgsMixed& a, int order, int64_t W, float4
 // ---------------------------------------------------------------- PLAIN schedule
 
 // A warp runs as long as its largest 4^k, so what counts is one loop for all k
-// (subcycle_f32's NEAR = 1) and enough warps: four blocks per SM at 64 registers
+// (stretches from k = 1 on) and enough warps: four blocks per SM at 64 registers
 // up to order 3 (16 bytes of spills there), three at order 4, and as many
-// registers as it takes at order 5 (64 there spill 112 bytes: 100,003 electrons
-// 100 us, 91 so).  ms per step, steps 2405 to 4404, before the three-node
-// sub-cycles, with them in two loops at 74 registers, and so: 16.8M electrons
-// 1.029, 1.065, 0.963; 67.1M at a0 = 300 3.06, 3.17, 2.89; 1,048,576 0.166, 0.165,
-// 0.158.
-constexpr int plain_blocks(int order) { return order <= 3 ? 4 : order == 4 ? 3 : 0; }
+// registers as it takes at order 5 (100,003 electrons at 128 registers 87 us, 104 at
+// 80).  ms per step, steps 2405 to 4404, before the three-node sub-cycles, with them
+// in two loops at 74 registers, and so: 16.8M electrons 1.029, 1.065, 0.965; 67.1M
+// at a0 = 300 3.06, 3.17, 2.90; 1,048,576 0.166, 0.165, 0.158.
+constexpr int plain_blocks(int order) { return order <= 3 ? 4 : order == 4 ? 3 : 1; }
 template <int P, bool RING>
 __global__ void __launch_bounds__(256, plain_blocks(P)) push_mixed_plain_kernel(PushArgsMixed a) {
   __shared__ unsigned long long sh[12];
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(256, plain_blocks(P)) push_mixed_plain_kernel(
       // 16-byte loads: 16.8M electrons over steps 2405 to 4404 0.965 ms per step,
       // 1.026 from the levels.  Rows of the other orders are not aligned: they form
       // them from the levels (100,003 electrons at order 5: 89 us, 95 by the table).
-      ok = subcycle_f32<P, RING, P == 3, 1>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.mono, k,
+      ok = subcycle_f32<P, RING, P == 3>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.near, a.mono, k,
                                          st & 0x7f, b0, s);
     }
     normalize(s);

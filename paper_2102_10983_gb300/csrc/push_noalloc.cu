@@ -185,6 +185,7 @@ extern "C" int pic_push_mixed_noalloc(const pic_params* prm, int64_t n_particles
   base.inv_dx = (float)(1.0 / prm->dx);
   base.k_max = prm->k_max;
   base.field_time = prm->field_time;
+  base.near = stretches(prm->dt / prm->dx, kNearMin);
   lagrange_monomials(p, base.mono);
   base.wtab = wtab;
   base.crit_row = kRows - 1;  // theta = 1/2, the same weights as the cap's own criterion row
