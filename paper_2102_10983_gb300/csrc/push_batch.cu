@@ -78,7 +78,7 @@ static_assert(sizeof(BatchStash) % 16 == 0, "stashes follow each other in shared
 
 // Push the last min(n, 32) stashed particles, one per lane (stash_drain of the
 // single-problem kernel, each particle with its ensemble's fields).
-template <int P>
+template <int P, bool WIDE>
 __device__ __forceinline__ void batch_stash_drain(const BatchArgs& a, const BatchStash& S, int k, int& n,
                                                   unsigned long long* sh) {
   const int lane = threadIdx.x & 31;
@@ -92,7 +92,7 @@ __device__ __forceinline__ void batch_stash_drain(const BatchArgs& a, const Batc
     const float2 vb = S.s.b[q];
     const int32_t i = __float_as_int(vb.y);
     MixedState s = {__float_as_int(va.x), va.y, va.z, va.w, vb.x};
-    const bool ok = subcycle_f32<P, true, true>(F, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.near, a.mono,
+    const bool ok = subcycle_f32<P, true, true>(F, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, NearRule<WIDE>(a.near), a.mono,
                                                 k, S.s.kp[q], 0.f, s);
     normalize(s);
     store_state(a, i, s);
@@ -146,7 +146,7 @@ __device__ __forceinline__ void batch_defer_mark(const BatchArgs& a, int64_t i, 
 // stays deferred where it is and resumes in the next launch.  finalize: bring
 // it to the end of the last step only (public status).  key: ens * 8 + k of
 // a re-deferral, else -1.
-template <int P>
+template <int P, bool WIDE>
 __device__ __forceinline__ void batch_heavy(const BatchArgs& a, int ens, int64_t i,
                                             const float* wcrit, ThreadCounters& tc,
                                             unsigned long long* sh, int& key) {
@@ -184,10 +184,10 @@ __device__ __forceinline__ void batch_heavy(const BatchArgs& a, int ens, int64_t
     StepFields<P, true> Fs = si == a.step_cur ? Fc : Fp;
     if (si < a.step_cur - 1) Fs = ens_step_fields<P>(a, e, si);
     if (Fs.coef)
-      ok = subcycle_f32<P, true, true>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.near, a.mono,
+      ok = subcycle_f32<P, true, true>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, NearRule<WIDE>(a.near), a.mono,
                                        k, k_prev, b0, s, j0, j1);
     else  // further behind than the tables kept
-      ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, a.near,
+      ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, e.dt, e.inv_dx, e.qm, e.field_time, NearRule<WIDE>(a.near),
                                         a.mono, k, k_prev, b0, s, j0, j1);
     if (k >= kDeferMin) budget -= j1 - j0;
     if (!ok) {
@@ -355,7 +355,7 @@ static_assert(kBatchTileBytes % 128 == 0, "stashes start aligned");
 // the ring per chunk and per parked particle: 17.8 warp instructions per
 // particle of the 512-ensemble configuration, 13.8 so; 293 -> 265 us per step
 // of 11.9M particles.)
-template <int P>
+template <int P, bool WIDE>
 __global__ void __launch_bounds__(kBatchThreads, PIC_BATCH_MIN_BLOCKS) push_batch_kernel(BatchArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
   Tile* tiles = reinterpret_cast<Tile*>(smem);  // [kBatchWarps][2]
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kBatchThreads, PIC_BATCH_MIN_BLOCKS) push_batc
       const int keep = all ? 0 : 31;
       if (n <= keep) continue;
 #pragma unroll 1
-      while (n > keep) batch_stash_drain<P>(a, my_stash[q], q + 1, n, sh);
+      while (n > keep) batch_stash_drain<P, WIDE>(a, my_stash[q], q + 1, n, sh);
 #pragma unroll
       for (int r = 0; r < kStashK; ++r)
         if (r == q) stash_n[r] = n;
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(kBatchThreads, PIC_BATCH_MIN_BLOCKS) push_batc
       int32_t i = 0;
       if (entry < a.qcount_in[ens * 8 + k]) {
         i = a.queue_in[queue_slot(a, a.ens[ens], k, entry)];
-        batch_heavy<P>(a, ens, i, wcrit, tc, sh, key);
+        batch_heavy<P, WIDE>(a, ens, i, wcrit, tc, sh, key);
       }
       batch_enqueue(a, key, i);
       continue;
@@ -656,7 +656,10 @@ static cudaError_t launch_batch_p(const BatchArgs& a, int blocks, cudaStream_t s
     batch_halfstep_kernel<P><<<(int)(want < 152 * 16 ? want : 152 * 16), 256, 0, s>>>(a);
     ++n;
   }
-  push_batch_kernel<P><<<blocks, kBatchThreads, kBatchSmem, s>>>(a);
+  if (a.near.half > 1)  // c dt > dx in an ensemble
+    push_batch_kernel<P, true><<<blocks, kBatchThreads, kBatchSmem, s>>>(a);
+  else
+    push_batch_kernel<P, false><<<blocks, kBatchThreads, kBatchSmem, s>>>(a);
   if (a.finalize) {
     const int64_t want = (a.n_total + 255) / 256;
     batch_reset_status_kernel<<<(int)(want < 152 * 8 ? want : 152 * 8), 256, 0, s>>>(a.status,
@@ -680,13 +683,18 @@ cudaError_t launch_batch_step(const BatchArgs& a, int order, int blocks, cudaStr
   }
 }
 
+template <int P, bool WIDE>
+static int batch_occupancy_of() {
+  int occ = 0;
+  if (cudaFuncSetAttribute(push_batch_kernel<P, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)kBatchSmem) == cudaSuccess)
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<P, WIDE>, kBatchThreads, kBatchSmem);
+  return occ;
+}
 template <int P>
 static int batch_occupancy() {
-  int occ = 0;
-  if (cudaFuncSetAttribute(push_batch_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBatchSmem) ==
-      cudaSuccess)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_batch_kernel<P>, kBatchThreads, kBatchSmem);
-  return occ;
+  const int a = batch_occupancy_of<P, false>(), b = batch_occupancy_of<P, true>();
+  return a < b ? a : b;
 }
 
 // Called at pic_batch_create: also lets the kernel have its shared memory.

@@ -624,14 +624,26 @@ __device__ __forceinline__ bool cycle_near(const StepFields<P, RING>& F, int32_t
 // nodes ahead of the electron kept (its 16 sub-steps would not pay for a second
 // load).  What does not fit (a turn back, the window's ends) takes cycle_any, as
 // does k = 1, whose four sub-steps gain nothing.  near: the rule for the grid
-// (stretches), a launch argument: a register for it costs the kernels 1 to 5 %.  Per step, two nodes ->
+// (stretches), fixed at compile time where c dt <= dx: as a value of its own it
+// cost the kernels 1 to 5 % (16.8M electrons over steps 2405 to 4404, binned, push
+// kernel 0.254 and 0.263 ms).  Per step, two nodes ->
 // three -> with stretches: 300 electrons at the front 119 -> 117 -> 95 us,
 // 16.8M electrons 249 -> 219 -> 199 us, 1,000,003 at fifth order 120 -> 118 ->
 // 90 us.
-template <int P, bool RING, bool TABLE = false>
+template <bool WIDE, int K_MIN = kNearMin>
+struct NearRule {
+  static constexpr int k_min = K_MIN, half = 1;
+  __device__ __forceinline__ explicit NearRule(const Stretches&) {}
+};
+template <int K_MIN>
+struct NearRule<true, K_MIN> {
+  int k_min, half;
+  __device__ __forceinline__ explicit NearRule(const Stretches& s) : k_min(s.k_min), half(s.half) {}
+};
+template <int P, bool RING, bool TABLE = false, class NEAR>
 __device__ __forceinline__ bool subcycle_f32(const StepFields<P, RING>& F, const float* wtab,
                                              int32_t mask, float dt, float inv_dx, float qm,
-                                             int field_time, const Stretches& near,
+                                             int field_time, const NEAR& near,
                                              const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1],
                                              int k, int k_prev, float b0, MixedState& s,
                                              int j0 = 0, int j1 = -1) {
@@ -679,10 +691,10 @@ struct SubOut {
   MixedState s;
   bool ok;
 };
-template <int P>
+template <int P, class NEAR>
 __device__ __noinline__ SubOut subcycle_table_call(StepFields<P, true> F, const float* wtab,
                                                    int32_t mask, float dt, float inv_dx, float qm,
-                                                   int field_time, Stretches near, int k, int k_prev, float b0,
+                                                   int field_time, NEAR near, int k, int k_prev, float b0,
                                                    MixedState s, int j0, int j1) {
   float no_mono[2][kMaxOrder + 1][kMaxOrder + 1];  // the table form never reads it
   SubOut o;
@@ -691,10 +703,10 @@ __device__ __noinline__ SubOut subcycle_table_call(StepFields<P, true> F, const 
                                      b0, o.s, j0, j1);
   return o;
 }
-template <int P, bool RING, bool TABLE>
+template <int P, bool RING, bool TABLE, class NEAR>
 __device__ __forceinline__ bool subcycle_site(const StepFields<P, RING>& F, const float* wtab,
                                               int32_t mask, float dt, float inv_dx, float qm,
-                                              int field_time, const Stretches& near,
+                                              int field_time, const NEAR& near,
                                               const float (&mono)[2][kMaxOrder + 1][kMaxOrder + 1],
                                               int k, int k_prev, float b0, MixedState& s,
                                               int j0 = 0, int j1 = -1) {
@@ -1095,7 +1107,7 @@ __device__ __forceinline__ void stash_put(Stash& S, int pos, int32_t i, const Mi
 // Push the last min(n, 32) stashed particles, one per lane, with 4^k sub-steps
 // each.  Warp-collective.  Stash entry kp: k_prev in bits 0-2, bit 3 set for a
 // predicted-queue particle (which stays in that queue).
-template <int P, bool RING>
+template <int P, bool RING, bool WIDE>
 __device__ __forceinline__ void stash_drain(const PushArgsMixed& a, const StepFields<P, RING>& F,
                                             const Stash& S, int k, int& n, unsigned long long* sh) {
   const int lane = threadIdx.x & 31;
@@ -1108,7 +1120,7 @@ __device__ __forceinline__ void stash_drain(const PushArgsMixed& a, const StepFi
     const int32_t i = __float_as_int(vb.y);
     MixedState s = {__float_as_int(va.x), va.y, va.z, va.w, vb.x};
     const bool ok = subcycle_site<P, RING, RING>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm,
-                                                 a.field_time, a.near, a.mono, k, kp & 7, 0.f, s);
+                                                 a.field_time, NearRule<WIDE>(a.near), a.mono, k, kp & 7, 0.f, s);
     normalize(s);
     store_state(a, i, s);
     a.status[i] = ok ? (uint8_t)(k | (kp & 8 ? kOwned : 0) | (a.parity_next ? kParity : 0))
@@ -1131,7 +1143,7 @@ __device__ __forceinline__ void stash_drain(const PushArgsMixed& a, const StepFi
 // into the next call: the steps whose levels the ring must keep), which it
 // finishes regardless of the budget.  finalize: bring it
 // to the end of the last step only (public status).
-template <int P, bool RING>
+template <int P, bool RING, bool WIDE>
 __device__ __forceinline__ void heavy_particle(const PushArgsMixed& a, const StepFields<P, RING>& Fp,
                                             const StepFields<P, RING>& Fc, const float* wcrit,
                                             int64_t i, ThreadCounters& tc,
@@ -1166,11 +1178,11 @@ __device__ __forceinline__ void heavy_particle(const PushArgsMixed& a, const Ste
       if (si < a.step_cur - 1) Fs = ring_step_fields<P>(a, si);
     }
     if (!RING || Fs.coef) {
-      ok = subcycle_site<P, RING, RING>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.near,
+      ok = subcycle_site<P, RING, RING>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, NearRule<WIDE>(a.near),
                                         a.mono, k, k_prev, b0, s, j0, j1);
     } else {  // further behind than the tables kept
       if constexpr (RING)
-        ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.near,
+        ok = subcycle_f32<P, true, false>(Fs, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, NearRule<WIDE>(a.near),
                                           a.mono, k, k_prev, b0, s, j0, j1);
     }
     if (k >= kDeferMin) budget -= j1 - j0;
@@ -1264,7 +1276,7 @@ __device__ __forceinline__ void heavy_particle(const PushArgsMixed& a, const Ste
 // particle code, at most heavy_budget sub-steps in this launch -- so a warp of
 // right predictions runs dense from the start of the launch -- else it is
 // deferred to the next launch (key), as the stream would.
-template <int P, bool RING>
+template <int P, bool RING, bool WIDE>
 __device__ __forceinline__ void predicted_particle(const PushArgsMixed& a, const StepFields<P, RING>& Fc,
                                                    const float* wcrit, int64_t i, int k_pred,
                                                    ThreadCounters& tc, unsigned long long* sh,
@@ -1289,7 +1301,7 @@ __device__ __forceinline__ void predicted_particle(const PushArgsMixed& a, const
   count_step(tc, sh, k, capped);
   if (k == 0 || (k == k_pred && k < kDeferMin)) {
     const bool ok = subcycle_site<P, RING, RING>(Fc, a.wtab, a.mask, a.dt, a.inv_dx, a.qm,
-                                                 a.field_time, a.near, a.mono, k, k_prev, b0, s);
+                                                 a.field_time, NearRule<WIDE>(a.near), a.mono, k, k_prev, b0, s);
     normalize(s);
     store_state(a, i, s);
     a.status[i] = ok ? (uint8_t)(k | kOwned | (a.parity_next ? kParity : 0))

@@ -136,7 +136,7 @@ cudaError_t launch_halfstep(const PushArgsMixed& a, int order, int64_t W, float4
 // in two loops at 74 registers, and so: 16.8M electrons 1.029, 1.065, 0.965; 67.1M
 // at a0 = 300 3.06, 3.17, 2.90; 1,048,576 0.166, 0.165, 0.158.
 constexpr int plain_blocks(int order) { return order <= 3 ? 4 : order == 4 ? 3 : 1; }
-template <int P, bool RING>
+template <int P, bool RING, bool WIDE>
 __global__ void __launch_bounds__(256, plain_blocks(P)) push_mixed_plain_kernel(PushArgsMixed a) {
   __shared__ unsigned long long sh[12];
   if (threadIdx.x < 12) sh[threadIdx.x] = 0ull;
@@ -179,7 +179,8 @@ __global__ void __launch_bounds__(256, plain_blocks(P)) push_mixed_plain_kernel(
       // 16-byte loads: 16.8M electrons over steps 2405 to 4404 0.965 ms per step,
       // 1.026 from the levels.  Rows of the other orders are not aligned: they form
       // them from the levels (100,003 electrons at order 5: 89 us, 95 by the table).
-      ok = subcycle_f32<P, RING, P == 3>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, a.near, a.mono, k,
+      ok = subcycle_f32<P, RING, P == 3>(F, a.wtab, a.mask, a.dt, a.inv_dx, a.qm, a.field_time, NearRule<WIDE, 1>(a.near),
+                                         a.mono, k,
                                          st & 0x7f, b0, s);
     }
     normalize(s);
@@ -322,7 +323,8 @@ static_assert(kStashBytes % 128 == 0, "tiles start on a 128-byte boundary");
 #define PIC_BINNED_MIN_BLOCKS 2
 #endif
 
-template <int P, bool RING>
+// WIDE: c dt > dx (stretches).
+template <int P, bool RING, bool WIDE>
 __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_kernel(PushArgsMixed a) {
   extern __shared__ __align__(128) unsigned char smem[];
   Stash* stashes = reinterpret_cast<Stash*>(smem);  // [kWarps][kStashK]
@@ -403,7 +405,7 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
       const int keep = all ? 0 : 31;
       if (n <= keep) continue;
 #pragma unroll 1
-      while (n > keep) stash_drain<P, RING>(a, F, my_stash[q], q + 1, n, sh);
+      while (n > keep) stash_drain<P, RING, WIDE>(a, F, my_stash[q], q + 1, n, sh);
       stash_set(q, n);
     }
   };
@@ -607,10 +609,10 @@ __global__ void __launch_bounds__(kThreads, PIC_BINNED_MIN_BLOCKS) push_binned_k
       const int64_t e = (t - first) * 32 + lane;
       if (e < a.pred_count[k]) {
         i = a.pred_queue[(int64_t)(k - 1) * a.qcap + e];
-        predicted_particle<P, RING>(a, F, wcrit, i, k, tc, sh, key, sk, s, kp, heavy);
+        predicted_particle<P, RING, WIDE>(a, F, wcrit, i, k, tc, sh, key, sk, s, kp, heavy);
       }
     }
-    if (heavy) heavy_particle<P, RING>(a, Fp, F, wcrit, i, tc, sh, key);
+    if (heavy) heavy_particle<P, RING, WIDE>(a, Fp, F, wcrit, i, tc, sh, key);
     enqueue(a, key, i);
     park(sk, 0, i, s, s, kp, kp);
     t = claim();
@@ -800,19 +802,23 @@ static cudaError_t launch_p(const PushArgsMixed& a, int schedule, int sm_count, 
   if (schedule == PIC_SCHED_PLAIN) {
     const int64_t want = (a.n + 255) / 256;
     const int64_t cap = (int64_t)sms * 8;
-    push_mixed_plain_kernel<P, false><<<(int)(want < cap ? want : cap), 256, 0, s>>>(a);
+    const int blocks = (int)(want < cap ? want : cap);
+    if (a.near.half > 1)
+      push_mixed_plain_kernel<P, false, true><<<blocks, 256, 0, s>>>(a);
+    else
+      push_mixed_plain_kernel<P, false, false><<<blocks, 256, 0, s>>>(a);
     if (launches) ++*launches;
   }
   return cudaGetLastError();
 }
 
-template <int P, bool RING>
+template <int P, bool RING, bool WIDE>
 static cudaError_t launch_binned_p(PushArgsMixed a, int sm_count, cudaStream_t main,
                                    int* launches) {
   const int sms = sm_count > 0 ? sm_count : 152;
   static int occ = 0;
   if (occ == 0) {
-    cudaError_t e = cudaFuncSetAttribute(push_binned_kernel<P, RING>,
+    cudaError_t e = cudaFuncSetAttribute(push_binned_kernel<P, RING, WIDE>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBinnedSmem);
     if (e != cudaSuccess) return e;
 #ifdef PIC_MIN_CARVEOUT
@@ -820,12 +826,12 @@ static cudaError_t launch_binned_p(PushArgsMixed a, int sm_count, cudaStream_t m
       const int need = PIC_BINNED_MIN_BLOCKS * ((int)kBinnedSmem + 1024 + 512);
       int pct = (need * 100 + 228 * 1024 - 1) / (228 * 1024);
       if (pct > 100) pct = 100;
-      e = cudaFuncSetAttribute(push_binned_kernel<P, RING>,
+      e = cudaFuncSetAttribute(push_binned_kernel<P, RING, WIDE>,
                                cudaFuncAttributePreferredSharedMemoryCarveout, pct);
       if (e != cudaSuccess) return e;
     }
 #endif
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_binned_kernel<P, RING>, kThreads,
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, push_binned_kernel<P, RING, WIDE>, kThreads,
                                                   kBinnedSmem);
     if (occ < 1) occ = 1;
   }
@@ -839,7 +845,7 @@ static cudaError_t launch_binned_p(PushArgsMixed a, int sm_count, cudaStream_t m
   a.item_tiles = tiles >= 8 * blocks * kWarps ? 2 : 1;
   const int64_t items = (tiles + a.item_tiles - 1) / a.item_tiles;
   if (!a.finalize && blocks > (items + kWarps - 1) / kWarps + sms) blocks = (items + kWarps - 1) / kWarps + sms;
-  push_binned_kernel<P, RING><<<(int)blocks, kThreads, kBinnedSmem, main>>>(a);
+  push_binned_kernel<P, RING, WIDE><<<(int)blocks, kThreads, kBinnedSmem, main>>>(a);
   int n = 1;
   if (a.finalize) {
     const int64_t want = (a.n + 255) / 256;
@@ -864,28 +870,30 @@ cudaError_t launch_push_mixed(const PushArgsMixed& a, int order, int schedule, i
   }
 }
 
+template <bool RING, bool WIDE>
+static cudaError_t launch_binned_order(const PushArgsMixed& a, int order, int sm_count, cudaStream_t main,
+                                       int* launches) {
+  switch (order) {
+    case 1: return launch_binned_p<1, RING, WIDE>(a, sm_count, main, launches);
+    case 2: return launch_binned_p<2, RING, WIDE>(a, sm_count, main, launches);
+    case 3: return launch_binned_p<3, RING, WIDE>(a, sm_count, main, launches);
+    case 4: return launch_binned_p<4, RING, WIDE>(a, sm_count, main, launches);
+    case 5: return launch_binned_p<5, RING, WIDE>(a, sm_count, main, launches);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t launch_binned_step(const PushArgsMixed& a, int order, int sm_count, cudaStream_t main,
                                int* launches) {
   if (a.n <= 0) return cudaSuccess;
+  const bool wide = a.near.half > 1;
   if (a.ringE) {
     if (!a.coef || !a.coef_p) return cudaErrorInvalidValue;  // the ring form reads the node tables
-    switch (order) {
-      case 1: return launch_binned_p<1, true>(a, sm_count, main, launches);
-      case 2: return launch_binned_p<2, true>(a, sm_count, main, launches);
-      case 3: return launch_binned_p<3, true>(a, sm_count, main, launches);
-      case 4: return launch_binned_p<4, true>(a, sm_count, main, launches);
-      case 5: return launch_binned_p<5, true>(a, sm_count, main, launches);
-      default: return cudaErrorInvalidValue;
-    }
+    return wide ? launch_binned_order<true, true>(a, order, sm_count, main, launches)
+                : launch_binned_order<true, false>(a, order, sm_count, main, launches);
   }
-  switch (order) {
-    case 1: return launch_binned_p<1, false>(a, sm_count, main, launches);
-    case 2: return launch_binned_p<2, false>(a, sm_count, main, launches);
-    case 3: return launch_binned_p<3, false>(a, sm_count, main, launches);
-    case 4: return launch_binned_p<4, false>(a, sm_count, main, launches);
-    case 5: return launch_binned_p<5, false>(a, sm_count, main, launches);
-    default: return cudaErrorInvalidValue;
-  }
+  return wide ? launch_binned_order<false, true>(a, order, sm_count, main, launches)
+              : launch_binned_order<false, false>(a, order, sm_count, main, launches);
 }
 
 }  // namespace pic
