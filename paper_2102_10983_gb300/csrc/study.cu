@@ -481,21 +481,26 @@ __global__ void __launch_bounds__(32) study_many_kernel(const pic_study_case* ca
 
 // Whether a warp per electron is the faster form.  It takes the FP64 unit's time
 // for every electron and macro step; a thread per electron takes the longest
-// case's chain.  Per macro step on the GB300 (a0 from 2 to 100, lambda/50 and /75):
-// 17.5 ns per electron and a chain of 75 us with sub-cycles (a warp runs as long
-// as its largest 4^k), 12.3 ns and 26 us without.  256 electrons per case, a0 = 25:
-// 15 cases 259 ms by warps and 309 by threads, 20 cases 339 and 308, 60 cases 939
-// and 346.
+// case's chain, in which a warp runs as long as its largest 4^k.  Measured per macro
+// step and order, a0 = 25, lambda/75 (5 to 100 likewise): without and with sub-cycles,
+// which an electron from rest takes once the pulse's envelope reaches four times the
+// criterion's threshold.  4,352 electrons at order 3: 72 us by warps and 77 by
+// threads, 10,240 162 and 79; without sub-cycles 49 and 25, 111 and 25.
 bool study_by_warp(const pic_study_case* cases, int32_t n, int sms) {
+  static const double chain_us[2][kMaxOrder] = {{16.7, 20.6, 24.6, 28.4, 32.3}, {42.0, 61.0, 77.0, 94.0, 111.0}};
+  static const double warp_ns[2][kMaxOrder] = {{10.4, 10.8, 11.3, 11.9, 15.8}, {15.1, 15.9, 16.6, 17.3, 22.0}};
   double by_warp = 0.0, by_thread = 0.0;  // us
   for (int32_t i = 0; i < n; ++i) {
     const pic_study_case& q = cases[i];
-    const bool sub = q.k_max > 0 && fabs(q.qm * q.a0) * q.dt > 2.0 * q.psi_max;
-    const double steps = (double)q.n_steps, chain = steps * (sub ? 75.0 : 26.0);
-    by_warp += steps * (double)q.n_electrons * (sub ? 17.5e-3 : 12.3e-3) * 152.0 / (double)(sms > 0 ? sms : 152);
+    const double steps = (double)q.n_steps, top = fabs(q.qm * q.a0) * q.dt / (8.0 * q.psi_max);
+    double plain = steps;  // macro steps before the sub-cycles
+    if (q.k_max > 0 && top > 1.0) plain = fmin(steps, fmax(0.0, (q.xi0 - q.sigma * sqrt(2.0 * log(top))) / q.dt));
+    const int o = q.order - 1;
+    const double chain = plain * chain_us[0][o] + (steps - plain) * chain_us[1][o];
+    by_warp += (plain * warp_ns[0][o] + (steps - plain) * warp_ns[1][o]) * (double)q.n_electrons;
     by_thread = chain > by_thread ? chain : by_thread;
   }
-  return by_warp <= by_thread;
+  return by_warp * 1e-3 * 152.0 / (double)(sms > 0 ? sms : 152) <= by_thread;
 }
 
 }  // namespace
